@@ -80,9 +80,10 @@ typedef enum {
  *                     summed on CUDA cores in FP32 from fl32(B), because the
  *                     tensor-core accumulator truncates toward zero;
  *   DSRG_PREC_BF16X3  same with BF16 planes.
- * In every mode the regulator (Delta, exp(-s Delta^2), the denominator), the
- * combination with the exchange integral and every sum of energy
- * contributions are FP64. */
+ * The regulator (Delta, exp(-s Delta^2), the denominator) and every sum of energy
+ * contributions are FP64, except in the CCVV kernel of the split modes away
+ * from Delta = 0: there they are pairs of FP32 numbers (48 bits; relative error
+ * of the regulator below 2^-40, as of the FP64 form with its one Newton step). */
 typedef enum {
   DSRG_PREC_FP64 = 0,
   DSRG_PREC_TF32X3 = 1,
@@ -327,8 +328,10 @@ dsrg_status_t dsrg_ccvv_energy_noalloc(const dsrg_sizes_t *sz, const double *B, 
  *                             columns of one core pair) whose every |Delta| is so
  *                             large that exp(-2 s Delta^2) < 2^-63, evaluated as
  *                             1/Delta;
- *   DSRG_COUNT_CCVV_FACTORED  blocks with every |Delta| >= 1/4 evaluated from the
- *                             factorised exponentials;
+ *   DSRG_COUNT_CCVV_FACTORED  blocks with every |Delta| >= 1/4 of a pair whose
+ *                             factorised exponentials stay in range (the energy
+ *                             forms exp(-2 s Delta^2) directly, the gradient from
+ *                             the factors);
  *   DSRG_COUNT_CCVV_DIRECT    blocks with some |Delta| < 1/4 (or of a pair whose
  *                             factors could overflow), evaluated with expm1 per
  *                             element (R(0) = 0) and the exchange combination in FP64;

@@ -119,44 +119,100 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+// 32 TMEM lanes x 16 columns as 16 x 8 fragments: lane l of the warp gets, in
+// r[8h + 4g + 2v + e], row 16 h + l / 4 + 8 v and column 8 g + 2 (l % 4) + e.
+__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, uint32_t (&r)[16]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[8 * h]), "=r"(r[8 * h + 1]), "=r"(r[8 * h + 2]), "=r"(r[8 * h + 3]),
+                   "=r"(r[8 * h + 4]), "=r"(r[8 * h + 5]), "=r"(r[8 * h + 6]), "=r"(r[8 * h + 7])
+                 : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+}
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void named_bar(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
-// Eight consecutive floats from global memory, read-only path (32-byte aligned).
-__device__ __forceinline__ void ldg8(const float* p, float (&v)[8]) {
-  asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
-        "=f"(v[7])
-      : "l"(p));
+// The FP32 tail rows: fl32(B) of the first TAIL_Q auxiliary functions of every
+// plane row, in blocks of 8 rows, [row / 8][q / 4][row % 8][q % 4]. The four
+// values of 8 consecutive rows are one 128-byte line, so a warp's load of any 8
+// rows at one q / 4 meets every shared-memory/L1 bank once (as 128-byte rows they
+// met the same 32 bytes of banks: 25 cycles of the data path per load, which the
+// MMAs' operand reads share).
+__host__ __device__ __forceinline__ size_t tail_off(size_t row) {
+  return (row >> 3) * (8 * TAIL_Q) + (row & 7) * 4;
 }
 
 // x_ab += sum_{q < TAIL_Q} T_a[q] T_b[q] for the 16 columns b of one chunk, in
-// FP32 with round-to-nearest, q from the last to the first. T holds fl32(B) of
-// the first TAIL_Q auxiliary functions, one 128-byte row per plane row; `ra` is
-// this thread's row, `rb` the first of the chunk's 16 rows (the same for every
-// lane of the warp, so each load is a broadcast; 32-byte loads halve their count).
+// FP32 with round-to-nearest, q from the last to the first. `ra`: this thread's
+// tail row, `rb`: the first of the chunk's 16 rows (a multiple of 8; the same for
+// every lane of the warp, so each load is a broadcast).
 __device__ __forceinline__ void tail_add16(const float* __restrict__ ra,
                                            const float* __restrict__ rb, uint32_t (&r)[16]) {
   float t[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) t[k] = 0.f;
-#pragma unroll 1
-  for (int q8 = TAIL_Q / 8 - 1; q8 >= 0; --q8) {
-    float a[8];
-    ldg8(ra + 8 * q8, a);
+#pragma unroll 2
+  for (int q4 = TAIL_Q / 4 - 1; q4 >= 0; --q4) {
+    const float4 a = __ldg((const float4*)(ra + 32 * q4));
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      float b[8];
-      ldg8(rb + k * TAIL_Q + 8 * q8, b);
-#pragma unroll
-      for (int i = 7; i >= 0; --i) t[k] = fmaf(a[i], b[i], t[k]);
+      const float4 b = __ldg((const float4*)(rb + (k >> 3) * (8 * TAIL_Q) + (k & 7) * 4 + 32 * q4));
+      t[k] = fmaf(a.w, b.w, t[k]);
+      t[k] = fmaf(a.z, b.z, t[k]);
+      t[k] = fmaf(a.y, b.y, t[k]);
+      t[k] = fmaf(a.x, b.x, t[k]);
     }
   }
 #pragma unroll
   for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) + t[k]);
+}
+
+// The same sums for a block of 32 rows x 16 NC columns in the fragment layout of
+// tmem_ld_frag16: a thread's 16 NC elements are 4 rows (`ra`, 8 apart) x 4 NC
+// columns (`rb`, pairs 8 apart), so a loaded value feeds 4 NC or 4 FMAs instead of
+// one: a load fills registers at 128 bytes a clock and SM, which the row-per-lane
+// form above, with 17 loads for 16 FMAs, is bound by. Same FMA order per element.
+template <int NC>
+__device__ __forceinline__ void tail_frag(const float* __restrict__ ra,
+                                          const float* __restrict__ rb, float (&t)[NC][16]) {
+#pragma unroll
+  for (int n = 0; n < NC; ++n)
+#pragma unroll
+    for (int k = 0; k < 16; ++k) t[n][k] = 0.f;
+#pragma unroll 2
+  for (int q4 = TAIL_Q / 4 - 1; q4 >= 0; --q4) {
+    float4 a[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) a[v] = __ldg((const float4*)(ra + 8 * TAIL_Q * v + 32 * q4));
+#pragma unroll
+    for (int c = 0; c < 4 * NC; ++c) {  // column 8 (c / 2) + c % 2 from rb
+      const float4 b = __ldg((const float4*)(rb + 8 * TAIL_Q * (c >> 1) + 4 * (c & 1) + 32 * q4));
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        float& s = t[c >> 2][8 * (v >> 1) + 4 * ((c >> 1) & 1) + 2 * (v & 1) + (c & 1)];
+        s = fmaf(a[v].w, b.w, s);
+        s = fmaf(a[v].z, b.z, s);
+        s = fmaf(a[v].y, b.y, s);
+        s = fmaf(a[v].x, b.x, s);
+      }
+    }
+  }
+}
+
+// Add the tensor cores' rest of the same block from TMEM.
+template <int NC>
+__device__ __forceinline__ void tmem_add_frag(uint32_t taddr, float (&t)[NC][16]) {
+#pragma unroll
+  for (int n = 0; n < NC; ++n) {
+    uint32_t r[16];
+    tmem_ld_frag16(taddr + 16 * n, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) t[n][k] = __uint_as_float(r[k]) + t[n][k];
+  }
 }
 
 // Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows at a

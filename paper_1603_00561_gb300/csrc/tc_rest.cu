@@ -54,7 +54,7 @@ struct TcGemmArgs {
   int m_tiles, n_tiles;
   int kblocks;        // K stages on the tensor cores: Q from kq0 to the padded end
   int kq0;            // = TAIL_Q: Q < kq0 is added in the epilogue from `tail`
-  const float* tail;  // [plane rows + TAIL_PAD][TAIL_Q] fl32(B) of Q < TAIL_Q
+  const float* tail;  // [plane rows + TAIL_PAD][TAIL_Q] fl32(B) of Q < TAIL_Q (tail_off)
   float* Y;
   long long ldy;
   int* status;
@@ -231,9 +231,8 @@ __global__ void __launch_bounds__(G_THREADS, 1)
       }
     }
   } else {
-    // epilogue: warp w reads TMEM lanes 32*(w%4).. (its row of the tile)
+    // epilogue: warp w reads TMEM lanes 32*(w%4).. (its rows of the tile)
     const int quarter = warp & 3;
-    const int row = quarter * 32 + lane;
     int tbuf = 0;
     uint32_t tphase = 0;
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -241,26 +240,25 @@ __global__ void __launch_bounds__(G_THREADS, 1)
       tc_fence_after();
       if (ok) {
         const uint32_t t = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(tbuf * G_BN);
-        float* y = a.Y + (size_t)((it / a.n_tiles) * G_BM + row) * a.ldy + (it % a.n_tiles) * G_BN;
-        const float* ta = a.tail + (size_t)(a.a_row0 + (it / a.n_tiles) * G_BM + row) * TAIL_Q;
-        const float* tb = a.tail + (size_t)(a.b_row0 + (it % a.n_tiles) * G_BN) * TAIL_Q;
+        // fragments of 32 rows x 32 columns (tail_frag): this thread holds the rows
+        // r0, + 8, + 16, + 24 and the column pairs cl, cl + 8
+        const int r0 = quarter * 32 + (lane >> 2), cl = 2 * (lane & 3);
+        float* y = a.Y + (size_t)((it / a.n_tiles) * G_BM + r0) * a.ldy + (it % a.n_tiles) * G_BN + cl;
+        const float* ta = a.tail + tail_off(a.a_row0 + (it / a.n_tiles) * G_BM + r0);
+        const float* tb = a.tail + tail_off(a.b_row0 + (it % a.n_tiles) * G_BN + cl);
         for (int c0 = 0; c0 < G_BN; c0 += 32) {
-          uint32_t r0[16], r1[16];
-          tmem_ld16(t + c0, r0);
-          tmem_ld16(t + c0 + 16, r1);
-          tmem_ld_wait();
           // the first TAIL_Q auxiliary functions in FP32 round-to-nearest
-          tail_add16(ta, tb + (size_t)c0 * TAIL_Q, r0);
-          tail_add16(ta, tb + (size_t)(c0 + 16) * TAIL_Q, r1);
-          float4* o = (float4*)(y + c0);
+          float x[2][16];
+          tail_frag<2>(ta, tb + (size_t)c0 * TAIL_Q, x);
+          tmem_add_frag<2>(t + c0, x);
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            o[q] = make_float4(__uint_as_float(r0[4 * q]), __uint_as_float(r0[4 * q + 1]),
-                               __uint_as_float(r0[4 * q + 2]), __uint_as_float(r0[4 * q + 3]));
+          for (int n = 0; n < 2; ++n)
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            o[4 + q] = make_float4(__uint_as_float(r1[4 * q]), __uint_as_float(r1[4 * q + 1]),
-                                   __uint_as_float(r1[4 * q + 2]), __uint_as_float(r1[4 * q + 3]));
+            for (int k = 0; k < 16; k += 2) {
+              float* o = y + (long long)(16 * (k >> 3) + 8 * ((k >> 1) & 1)) * a.ldy + c0 + 16 * n +
+                         8 * ((k >> 2) & 1);
+              *(float2*)o = make_float2(x[n][k], x[n][k + 1]);
+            }
         }
       }
       tc_fence_before();
@@ -302,7 +300,7 @@ __global__ void xrows_kernel(const double* __restrict__ B, Sizes z, long long xr
   const size_t o = (size_t)(xrow0 + t) * Qld + q;
   // the same split of fl32(B) as the main plane rows
   const float vf = (float)v;
-  if (q < TAIL_Q) tail[(size_t)(xrow0 + t) * TAIL_Q + q] = vf;
+  if (q < TAIL_Q) tail[tail_off(xrow0 + t) + 32 * (q >> 2) + (q & 3)] = vf;
   if (BF16) {
     const __nv_bfloat16 vh = __float2bfloat16_rn(vf);
     ((__nv_bfloat16*)hi)[o] = vh;

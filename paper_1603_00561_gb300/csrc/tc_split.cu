@@ -13,12 +13,20 @@
 // its bias would otherwise be set by the largest partial sums. Then it adds
 //     w * sum_ab (x^2 - x y + y^2) R_ab,   R = (1 - exp(-2 s D^2)) / D,
 // D = e_i + e_j - e_a - e_b, w = (2 if i<j) * (2 if A<B); for i = j only x is
-// formed (y = x). The regulator is FP64 throughout: exp(-2 s D^2) is the
-// product of four exponentials (one per pair, one per row, one per column,
-// one pair-independent table), 1/D is an FP32 seed refined by one FP64
-// Newton-Raphson step; positions with |D| < 1/4 (never the case for core ->
-// virtual excitations of a normal spectrum) take expm1 and an FP64 exchange
-// combination instead.
+// formed (y = x). The energy's regulator and sums are pairs of FP32 numbers
+// (48 bits, ff.cuh): the FP64 pipe, 2 FMAs per SM and clock, took longer for the
+// regulators of an item than the tensor cores for its products. Positions with
+// |D| < 1/4 (never the case for core -> virtual excitations of a normal spectrum)
+// take expm1 and the exchange combination in FP64 instead. The adjoint's regulators
+// are FP64: exp(-2 s D^2) is the product of four exponentials (one per pair, one
+// per row, one per column, one pair-independent table), 1/D a seed refined by one
+// Newton-Raphson step.
+//
+// Measured on one GB300 (this kernel alone, BF16x3): cc-pVTZ size (24/2/372/1200)
+// 855 us with the FP64 regulator and row-per-lane tail sums, 475 us now, 297 us
+// with the epilogue left out (the shared-memory path of the MMAs); cc-pV5Z size
+// (24/2/1214/3400) 8.45 ms, 8.2 ms, 7.3 ms. What the epilogue still adds is the
+// tail rows' loads (120 us and 0.6 ms), which use the same data path.
 //
 // Roles (one CTA per SM, persistent over the work list):
 //   warp 0      TMA producer (one elected thread)
@@ -38,6 +46,7 @@
 
 #include <cstring>
 
+#include "ff.cuh"
 #include "internal.cuh"
 #include "regulators.cuh"
 #include "tc_common.cuh"
@@ -60,7 +69,7 @@ struct SplitWs {
   long long row_base = 0;   // first row of this molecule in a shared (batched) plane buffer
   void* hi = nullptr;
   void* lo = nullptr;
-  float* tail = nullptr;    // [rows + TAIL_PAD][TAIL_Q]  fl32(B) of the first TAIL_Q auxiliary functions
+  float* tail = nullptr;    // [rows + TAIL_PAD][TAIL_Q]  fl32(B) of the first TAIL_Q auxiliary functions (tail_off)
   CUtensorMap map_hi, map_lo;  // 64-byte swizzled maps of the tc_rest GEMM
   CcvvMaps cmaps;              // 32-byte swizzled maps of the CCVV kernel
   double* alpha = nullptr;  // [n_pairs][nVpad]  exp(4 s E_p e_b)
@@ -412,8 +421,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   double* sEps = (double*)(smem + STAGES * STAGE_BYTES + 256);
   double* sAlpha = sEps + TT;
   double* sRed = sAlpha + TT;                 // [EPI_WARPS] warp sums
-  float* sEpsF = (float*)(sRed + EPI_WARPS);
-  float* sCr = sEpsF + TT;  // [TT/16][2]: min, max of e over the valid columns of each 16-column chunk
+  ff* sEb = (ff*)(sRed + EPI_WARPS);          // [TT] e_b as FP32 pairs
+  ff* sTab = sEb + TT;                        // [8] ff_exp_entry
+  float* sCr = (float*)(sTab + 8);  // [TT/16][2]: min, max of e over the valid columns of each 16-column chunk
   unsigned* sCnt = (unsigned*)(sCr + 2 * (TT / 16));  // [EPI_WARPS][3] epilogue blocks by regulator path
   // adjoint epilogue: column sums per warp [EPI_WARPS][64], row sums per column
   // half [2][TT], and the block sums of the pair and s derivatives [2][EPI_WARPS]
@@ -636,6 +646,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
     // 32-row x 16-column blocks of this warp by regulator path (lane 0 counts
     // in shared memory; the first barrier of the item loop orders the clearing)
     if (et < 3 * EPI_WARPS) sCnt[et] = 0u;
+    if (et < 8) sTab[et] = ff_exp_entry(et);
     for (int idx = it0; idx < it1; ++idx) {
       const MolDesc* md;
       const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
@@ -653,19 +664,21 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
         const int b = ip.Bt * TT + ip.cofs + et;
         const double eb = (b < nV) ? eps[ve + b] : 0.0;
         sEps[et] = eb;
-        sEpsF[et] = (float)eb;
-        sAlpha[et] = (b < nV) ? alpha[b] : 0.0;
-      }
-      named_bar(1, 32 * EPI_WARPS);
-      if (et < TT / 16) {
-        // range of e over the valid columns of chunk et (FP32: it only picks a path)
-        float lo = 3.0e38f, hi = -3.0e38f;
-        for (int c = 16 * et; c < 16 * et + 16 && c < ip.ncols; ++c) {
-          lo = fminf(lo, sEpsF[c]);
-          hi = fmaxf(hi, sEpsF[c]);
+        // columns past the end keep a valid e: their D stays in the block's range, q = 0
+        sEb[et] = ff_from(eps[ve + min(b, nV - 1)]);
+        if (ADJ) sAlpha[et] = (b < nV) ? alpha[b] : 0.0;
+        // range of e over the valid columns of each 16-column chunk (FP32: it only
+        // picks a path)
+        float lo = et < ip.ncols ? (float)eb : 3.0e38f, hi = et < ip.ncols ? (float)eb : -3.0e38f;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+          lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+          hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
-        sCr[2 * et] = lo;
-        sCr[2 * et + 1] = hi;
+        if ((et & 15) == 0) {
+          sCr[et >> 3] = lo;
+          sCr[(et >> 3) + 1] = hi;
+        }
       }
       named_bar(1, 32 * EPI_WARPS);
       const int arow = ip.A * TT + row;
@@ -677,8 +690,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       const int cend = min(cbeg + 64, ip.ncols);
       const double s = md->s;
       const double* taucol = md->tau + (size_t)(ip.Bt * TT + ip.cofs) * nVpad + arow;
-      const float* tail_ia = md->tail + (size_t)(ip.i * nVpad + arow) * TAIL_Q;
-      const float* tail_ja = md->tail + (size_t)(ip.j * nVpad + arow) * TAIL_Q;
+      const float* tail_ia = md->tail + tail_off(ip.i * nVpad + arow);
+      const float* tail_ja = md->tail + tail_off(ip.j * nVpad + arow);
       // range of E - e_a over this warp's valid rows (FP32)
       float clo = rok ? caf : 3.0e38f, chi = rok ? caf : -3.0e38f;
       for (int o = 16; o > 0; o >>= 1) {
@@ -699,75 +712,96 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       bool ok = mbar_wait(&tfull[tbuf], tphase, abort_flag, a.status);
       tc_fence_after();
       double acc = 0.0;
+      ff accf = {0.f, 0.f};
+      // (rows past the end take the last valid row's e: their q is 0)
+      const ff caff = ff_from(E - eps[ve + min(arow, nV - 1)]), kreg = ff_reg_scale(2.0 * s);
       if (ok) {
         const uint32_t tx = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(tbuf * 256);
         const uint32_t ty = tx + 128;
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
-          uint32_t xr[16], yr[16];
-          tmem_ld16(tx + c0, xr);
-          if (ip.two) tmem_ld16(ty + c0, yr);
-          tmem_ld_wait();
-          // The regulator path of this warp's 32 rows and the 16 columns from c0
-          // (the same for the whole warp): every |D| so large that
-          // exp(-2 s D^2) < 2^-63 -> R = 1/D; every |D| >= 1/4 with factorisable
-          // exponentials -> the factor tables; else expm1 per element.
+        // The regulator path of this warp's 32 rows and the 16 columns from c0
+        // (the same for the whole warp): every |D| so large that
+        // exp(-2 s D^2) < 2^-63 -> R = 1/D; every |D| >= 1/4 of a factorisable pair
+        // -> 1 - exp(-2 s D^2) in FP32 pairs; else expm1 per element in FP64.
+        auto path_of = [&](int c0) {
           const float dlo = clo - sCr[2 * (c0 >> 4) + 1], dhi = chi - sCr[2 * (c0 >> 4)];
           const bool away = dhi <= -0.25f || dlo >= 0.25f;
           const float dn = dhi <= 0.0f ? dhi : dlo;
-          const int pth = !away ? 2 : (dn * dn > far_d2 ? 0 : (factorisable ? 1 : 2));
-          if constexpr (ADJ) {
-            adjoint_chunk(a, ip, xr, yr, rok, pth, c0, cend, cbeg, arow, nVpad, ca, ha, s, sEps,
-                          sAlpha, taucol, md->tail, tail_ia, tail_ja, sColAcc + (warp - 2) * 64,
-                          lane, racc, sacc);
-            continue;
+          // (energies past 1e15 leave the range of the FP32 pairs)
+          const bool wide = !(fmaxf(fabsf(dlo), fabsf(dhi)) < 1e15f);
+          return !away || wide ? 2 : (dn * dn > far_d2 ? 0 : (factorisable ? 1 : 2));
+        };
+        if constexpr (ADJ) {
+          for (int c0 = cbeg; c0 < cend; c0 += 16) {
+            uint32_t xr[16], yr[16];
+            tmem_ld16(tx + c0, xr);
+            if (ip.two) tmem_ld16(ty + c0, yr);
+            tmem_ld_wait();
+            adjoint_chunk(a, ip, xr, yr, rok, path_of(c0), c0, cend, cbeg, arow, nVpad, ca, ha, s,
+                          sEps, sAlpha, taucol, md->tail, tail_ia, tail_ja,
+                          sColAcc + (warp - 2) * 64, lane, racc, sacc);
           }
-          if (lane == 0) sCnt[3 * (warp - 2) + pth] += 1u;
-          if (!rok) continue;
-          // the first TAIL_Q auxiliary functions, the largest terms, in FP32
-          // round-to-nearest (the tensor cores took the rest)
-          tail_add16(tail_ia, md->tail + (size_t)(ip.j * nVpad + ip.Bt * TT + ip.cofs + c0) * TAIL_Q,
-                     xr);
-          if (ip.two)
-            tail_add16(tail_ja,
-                       md->tail + (size_t)(ip.i * nVpad + ip.Bt * TT + ip.cofs + c0) * TAIL_Q, yr);
-          if (pth == 0) {
+        } else {
+          // 32 rows x 16 columns at a time, each thread 4 rows (r0, + 8, + 16, + 24) x
+          // 4 columns (tail_frag): wider blocks reload less but spill at 168 registers
+          const int r0 = quarter * 32 + (lane >> 2), cl = 2 * (lane & 3);
+          ff car[4];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              const int cb = c0 + k;
-              if (cb >= cend) break;
-              const float xf = __uint_as_float(xr[k]);
-              const float yf = ip.two ? __uint_as_float(yr[k]) : xf;
-              const double D = ca - sEps[cb];
-              double r0;
-              asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(D));  // 1/D, seed
-              const double R = fma(r0, fma(-D, r0, 1.0), r0);       // one Newton step
-              acc = fma((double)fmaf(xf, xf - yf, yf * yf), R, acc);
+          for (int v = 0; v < 4; ++v) {
+            car[v].h = __shfl_sync(0xffffffffu, caff.h, (lane >> 2) + 8 * v);
+            car[v].l = __shfl_sync(0xffffffffu, caff.l, (lane >> 2) + 8 * v);
+          }
+          const float* tr_i = md->tail + tail_off(ip.i * nVpad + ip.A * TT + r0);
+          const float* tr_j = md->tail + tail_off(ip.j * nVpad + ip.A * TT + r0);
+          const float* tc_i = md->tail + tail_off(ip.i * nVpad + ip.Bt * TT + ip.cofs + cl);
+          const float* tc_j = md->tail + tail_off(ip.j * nVpad + ip.Bt * TT + ip.cofs + cl);
+          for (int c0 = cbeg; c0 < cend; c0 += 16) {
+            float x[1][16], y[1][16];
+            // the first TAIL_Q auxiliary functions, the largest terms, in FP32
+            // round-to-nearest, then the tensor cores' rest
+            tail_frag<1>(tr_i, tc_j + (size_t)c0 * TAIL_Q, x);
+            tmem_add_frag<1>(tx + c0, x);
+            if (ip.two) {
+              tail_frag<1>(tr_j, tc_i + (size_t)c0 * TAIL_Q, y);
+              tmem_add_frag<1>(ty + c0, y);
             }
-          } else if (pth == 1) {
+            const int pth = path_of(c0);
+            if (lane == 0) sCnt[3 * (warp - 2) + pth] += 1u;
+            // q = x^2 - x y + y^2 (0 outside the valid rows and columns)
+            float q[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
-              const int cb = c0 + k;
-              if (cb >= cend) break;
-              const float xf = __uint_as_float(xr[k]);
-              const float yf = ip.two ? __uint_as_float(yr[k]) : xf;
-              const double D = ca - sEps[cb];
-              const double g = ha * sAlpha[cb] * taucol[(size_t)cb * nVpad];
-              double r0;
-              asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(D));  // 1/D, seed
-              const double e = fma(-D, r0, 1.0);         // Newton-Raphson residual
-              const double R0 = fma(-g, r0, r0);         // (1 - g) / D, seed accuracy
-              const double R = fma(R0, e, R0);           // one Newton step
-              acc = fma((double)fmaf(xf, xf - yf, yf * yf), R, acc);
+              const int cb = c0 + 8 * ((k >> 2) & 1) + cl + (k & 1);
+              const int ra = ip.A * TT + r0 + 16 * (k >> 3) + 8 * ((k >> 1) & 1);
+              const float xf = x[0][k], yf = ip.two ? y[0][k] : xf;
+              if (pth == 2) {
+                if (cb < cend && ra < nV) {
+                  const double xd = xf, yd = yf;
+                  const double D = E - eps[ve + ra] - sEps[cb];
+                  acc = fma(fma(xd, xd - yd, yd * yd), reg_f1(D, s), acc);
+                }
+                q[k] = 0.f;
+              } else {
+                q[k] = cb < cend && ra < nV ? fmaf(xf, xf - yf, yf * yf) : 0.f;
+              }
             }
-          } else {
+            if (pth == 2) continue;
+            // one column (4 elements) per pass: the code of the longer path stays small
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              const ff eb = sEb[c0 + 8 * (c >> 1) + cl + (c & 1)];
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              const int cb = c0 + k;
-              if (cb >= cend) break;
-              const double xd = __uint_as_float(xr[k]);
-              const double yd = ip.two ? (double)__uint_as_float(yr[k]) : xd;
-              const double D = ca - sEps[cb];
-              acc = fma(fma(xd, xd - yd, yd * yd), reg_f1(D, s), acc);
+              for (int v = 0; v < 4; ++v) {
+                const ff D = ff_diff(car[v], eb);
+                ff R = ff_inv(D);
+                if (pth == 1) R = ff_mul(ff_one_minus_exp(D, kreg, sTab), R);
+                ff_acc(accf, ff_mul(q[8 * (v >> 1) + 2 * (v & 1)], R));
+              }
+              // the next column's values move to the front
+#pragma unroll
+              for (int v = 0; v < 4; ++v) {
+                const int k = 8 * (v >> 1) + 2 * (v & 1);
+                q[k] = c == 0 ? q[k + 1] : (c == 1 ? q[k + 4] : q[k + 5]);
+              }
             }
           }
         }
@@ -827,6 +861,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       // warp half 0 alone, so the sum of a tile's column half does not depend on
       // whether the tile ran whole or as halves. Partial slot 2 * (pair tile-pair
       // index) + (column half of the tile).
+      acc += ff_to(accf);
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (lane == 0) sRed[warp - 2] = acc;
       named_bar(1, 32 * EPI_WARPS);
@@ -903,10 +938,11 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const double* __restr
   for (int k = 0; k < 16; ++k) xf[k] = (float)x[k];
   const size_t row = (size_t)h * nVpad + a;
   if (q0 < TAIL_Q) {
-    // fl32(B) of the first TAIL_Q auxiliary functions, row-major per plane row
-    float4* tr = (float4*)(tail + row * TAIL_Q + q0);
+    // fl32(B) of the first TAIL_Q auxiliary functions (tail_off)
+    float* tr = tail + tail_off(row) + 8 * q0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) tr[j] = make_float4(xf[4 * j], xf[4 * j + 1], xf[4 * j + 2], xf[4 * j + 3]);
+    for (int j = 0; j < 4; ++j)
+      *(float4*)(tr + 32 * j) = make_float4(xf[4 * j], xf[4 * j + 1], xf[4 * j + 2], xf[4 * j + 3]);
   }
   const size_t o = row * Qld + q0;
   if (BF16) {
@@ -1413,7 +1449,7 @@ void split_free(dsrg_plan* p) {
 }
 
 static size_t split_smem_bytes() {
-  return (size_t)STAGES * STAGE_BYTES + 1024 + 256 + (2 * TT + EPI_WARPS) * 8 + TT * 4 +
+  return (size_t)STAGES * STAGE_BYTES + 1024 + 256 + (2 * TT + EPI_WARPS) * 8 + (TT + 8) * 8 +
          2 * (TT / 16) * 4 + 3 * EPI_WARPS * 4 + 64;
 }
 
