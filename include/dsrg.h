@@ -81,9 +81,10 @@ typedef enum {
  *                     tensor-core accumulator truncates toward zero;
  *   DSRG_PREC_BF16X3  same with BF16 planes.
  * The regulator (Delta, exp(-s Delta^2), the denominator) and every sum of energy
- * contributions are FP64, except in the CCVV kernel of the split modes away
- * from Delta = 0: there they are pairs of FP32 numbers (48 bits; relative error
- * of the regulator below 2^-40, as of the FP64 form with its one Newton step). */
+ * contributions are FP64, except in the CCVV, CAVV, CCAV and (A,A|V,V) kernels of
+ * the split modes away from Delta = 0: there they are pairs of FP32 numbers (48
+ * bits; relative error of the regulator below 2^-40, as of the FP64 form with its
+ * one Newton step). */
 typedef enum {
   DSRG_PREC_FP64 = 0,
   DSRG_PREC_TF32X3 = 1,

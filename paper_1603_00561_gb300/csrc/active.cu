@@ -24,6 +24,7 @@
 // -L[u,v,y,x]; (beta alpha|alpha beta) -L[v,u,x,y].
 #include <type_traits>
 
+#include "ff.cuh"
 #include "internal.cuh"
 #include "regulators.cuh"
 
@@ -387,33 +388,16 @@ __global__ void __launch_bounds__(256) gram_aavv_kernel(const double* __restrict
 constexpr int ACTVV_BLOCKS = 152;
 constexpr int ACTVV_CH = 64;      // positions (e, f) per chunk of the active VV sums
 
-// Factor tables of exp(-s D_p^2), D_p = E_p - e_e - e_f for the active pairs
-// p = (x, u), E_p = e_x + e_u: exp(-s E_p^2) exp(2 s E_p e_e) exp(2 s E_p e_f)
-// exp(-s (e_e + e_f)^2). alpha == nullptr: evaluate exp directly.
-struct ActFact {
-  const double* alpha;  // [nA^2][ld]  exp(2 s E_p e_e)
-  const double* pinfo;  // [nA^2][4]   E_p, exp(-s E_p^2), factorisable flag
-  const double* tau;    // [ld][ld]    exp(-s (e_e + e_f)^2)
-  int ld;
-};
-
-// Rv = 1 + exp(-s D^2), Rt = (1 - exp(-s D^2)) / D in FP64; g = exp(-s D^2)
-// from the factor tables when fact, 1/D as an FP32 seed and one Newton step;
-// |D| < 1/4 takes expm1 and an FP64 divide.
-__device__ __forceinline__ void reg_pair(double D, double s, bool fact, double g, double& rv,
-                                         double& rt) {
-  if (fact && fabs(D) >= 0.25) {
-    float r0f;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0f) : "f"((float)D));
-    const double r0 = (double)r0f;
-    const double en = fma(-D, r0, 1.0);
-    const double R0 = fma(-g, r0, r0);
-    rt = fma(R0, en, R0);
-    rv = 1.0 + g;
-  } else {
-    rt = reg_t(D, s);
-    rv = reg_v(D, s);
-  }
+// Rv = 1 + exp(-s D^2) and Rt = (1 - exp(-s D^2)) / D as FP32 pairs (split-precision
+// plans; 7 FP64 instructions less per pair and position): true if |D| >= 1/4 and in
+// range, else the caller takes the FP64 forms.
+__device__ __forceinline__ bool reg_pair_ff(ff D, ff kreg, const ff* tab, ff& rv, ff& rt) {
+  if (!(fabsf(D.h) >= 0.25f && fabsf(D.h) < 1e15f)) return false;
+  const ff om = ff_one_minus_exp(D, kreg, tab);
+  rt = ff_mul(om, ff_inv(D));
+  rv = ff_fast_sum(2.0f, -om.h);
+  rv.l = rv.l - om.l;
+  return true;
 }
 
 __global__ void __launch_bounds__(256) actvv_kernel(const double* __restrict__ eps, double s,
@@ -455,19 +439,23 @@ __global__ void __launch_bounds__(256) actvv_kernel(const double* __restrict__ e
 template <int NA, bool F32>
 __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restrict__ eps, double s,
                                                           Sizes z, const double* __restrict__ M,
-                                                          ActFact F, double* __restrict__ part) {
+                                                          double* __restrict__ part) {
   constexpr int NA2 = NA * NA, NA4 = NA2 * NA2;
   __shared__ double red[8];
   const size_t nV2 = (size_t)z.nV * z.nV;
   const int ve = z.nC + z.nA;
-  double Ep[NA2], Bp[NA2];
-  bool fact = F.alpha != nullptr;
+  double Ep[NA2];
+  ff Epf[NA2];
 #pragma unroll
   for (int p = 0; p < NA2; ++p) {
     Ep[p] = eps[z.nC + p / NA] + eps[z.nC + p % NA];
-    Bp[p] = fact ? F.pinfo[4 * p + 1] : 0.0;
-    fact = fact && F.pinfo[4 * p + 2] != 0.0;
+    Epf[p] = ff_from(Ep[p]);
   }
+  __shared__ ff sTab[8];
+  if (threadIdx.x < 8) sTab[threadIdx.x] = ff_exp_entry(threadIdx.x);
+  __syncthreads();
+  const ff kreg = ff_reg_scale(s);
+  const bool pairs = s <= 1e3;  // keeps the exponent's scale in FP32 range
   double acc1[NA4], acc2[NA4];
   float f1[NA4], f2[NA4];
   int cnt = 0;
@@ -479,27 +467,29 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
   for (size_t k = (size_t)blockIdx.x * 256 + threadIdx.x; k < nV2; k += (size_t)gridDim.x * 256) {
     const int e = (int)(k / z.nV), f = (int)(k % z.nV);
     const double ef = eps[ve + e] + eps[ve + f];
-    const double tau = fact ? F.tau[(size_t)e * F.ld + f] : 0.0;
-    double mr[NA2], mq[NA2], m[NA2];
+    double m[NA2];
 #pragma unroll
     for (int p = 0; p < NA2; ++p) m[p] = M[(size_t)p * nV2 + k];
-#pragma unroll
-    for (int p = 0; p < NA2; ++p) {
-      const double D = Ep[p] - ef;
-      const double g = fact ? Bp[p] * F.alpha[(size_t)p * F.ld + e] * F.alpha[(size_t)p * F.ld + f] * tau : 0.0;
-      double rv, rt;
-      reg_pair(D, s, fact, g, rv, rt);
-      mr[p] = m[p] * rv;
-      mq[p] = rt;
-    }
     if constexpr (F32) {
+      // M holds FP32 values (tc_rest.cu), so its products with the pairs round once
       float a[NA2], b[NA2], c[NA2];
+      const ff eff = ff_from(ef);
 #pragma unroll
       for (int p = 0; p < NA2; ++p) {
         const int pt = (p % NA) * NA + p / NA;
-        a[p] = (float)mr[p];
-        b[p] = (float)(m[p] * mq[p]);
-        c[p] = (float)(m[pt] * mq[p]);
+        const float mp = (float)m[p], mt = (float)m[pt];
+        ff rv, rt;
+        if (pairs && reg_pair_ff(ff_diff(Epf[p], eff), kreg, sTab, rv, rt)) {
+          a[p] = ff_round(ff_mul(mp, rv));
+          b[p] = ff_round(ff_mul(mp, rt));
+          c[p] = ff_round(ff_mul(mt, rt));
+        } else {
+          const double D = Ep[p] - ef;
+          const double rtd = reg_t(D, s);
+          a[p] = (float)(m[p] * reg_v(D, s));
+          b[p] = (float)(m[p] * rtd);
+          c[p] = (float)(m[pt] * rtd);
+        }
       }
 #pragma unroll
       for (int p = 0; p < NA2; ++p)
@@ -518,6 +508,13 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
         }
       }
     } else {
+      double mr[NA2], mq[NA2];
+#pragma unroll
+      for (int p = 0; p < NA2; ++p) {
+        const double D = Ep[p] - ef;
+        mr[p] = m[p] * reg_v(D, s);
+        mq[p] = reg_t(D, s);
+      }
 #pragma unroll
       for (int p = 0; p < NA2; ++p)
 #pragma unroll
@@ -559,7 +556,7 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
 template <int NA, bool F32>
 __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict__ eps, double s,
                                                         Sizes z, const double* __restrict__ M,
-                                                        ActFact F, double* __restrict__ part) {
+                                                        double* __restrict__ part) {
   using T = typename std::conditional<F32, float, double>::type;
   constexpr int NA2 = NA * NA, NA4 = NA2 * NA2;
   constexpr int PER = (NA4 + 255) / 256;  // (p,q) outputs per thread
@@ -570,8 +567,10 @@ __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict
   __shared__ double red[8];
   const size_t nV2 = (size_t)z.nV * z.nV;
   const int ve = z.nC + z.nA;
-  bool fact = F.alpha != nullptr;
-  for (int p = 0; fact && p < NA2; ++p) fact = F.pinfo[4 * p + 2] != 0.0;
+  __shared__ ff sTab[8];
+  if (threadIdx.x < 8) sTab[threadIdx.x] = ff_exp_entry(threadIdx.x);  // (the loop's first barrier orders it)
+  const ff kreg = ff_reg_scale(s);
+  const bool pairs = F32 && s <= 1e3;  // keeps the exponent's scale in FP32 range
   double acc1[PER], acc2[PER];
 #pragma unroll
   for (int r = 0; r < PER; ++r) acc1[r] = acc2[r] = 0.0;
@@ -582,25 +581,29 @@ __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict
     for (int it = threadIdx.x; it < NA2 * ACTVV_CH; it += 256) {
       const int pidx = it / ACTVV_CH, kk = it % ACTVV_CH;
       const size_t k = k0 + kk;
-      double a = 0.0, b = 0.0, c = 0.0;
+      T a = 0, b = 0, c = 0;
       if (k < nV2) {
         const int x = pidx / NA, u = pidx % NA;
         const int e = (int)(k / z.nV), f = (int)(k % z.nV);
         const double D = eps[z.nC + x] + eps[z.nC + u] - eps[ve + e] - eps[ve + f];
         const double m = M[(size_t)pidx * nV2 + k];
         const double mt = M[(size_t)(u * NA + x) * nV2 + k];
-        const double g = fact ? F.pinfo[4 * pidx + 1] * F.alpha[(size_t)pidx * F.ld + e] *
-                                    F.alpha[(size_t)pidx * F.ld + f] * F.tau[(size_t)e * F.ld + f]
-                              : 0.0;
-        double rv, rt;
-        reg_pair(D, s, fact, g, rv, rt);
-        a = m * rv;
-        b = m * rt;
-        c = mt * rt;
+        ff rvf, rtf;
+        if (pairs && reg_pair_ff(ff_from(D), kreg, sTab, rvf, rtf)) {
+          // M holds FP32 values (tc_rest.cu), so its products with the pairs round once
+          a = (T)ff_round(ff_mul((float)m, rvf));
+          b = (T)ff_round(ff_mul((float)m, rtf));
+          c = (T)ff_round(ff_mul((float)mt, rtf));
+        } else {
+          const double rv = reg_v(D, s), rt = reg_t(D, s);
+          a = (T)(m * rv);
+          b = (T)(m * rt);
+          c = (T)(mt * rt);
+        }
       }
-      sa[it] = (T)a;
-      sb[it] = (T)b;
-      sc[it] = (T)c;
+      sa[it] = a;
+      sb[it] = b;
+      sc[it] = c;
     }
     __syncthreads();
 #pragma unroll
@@ -644,13 +647,16 @@ __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict
   (void)red;
 }
 
+// One warp per output: lanes take every 32nd CTA's partial, then a fixed butterfly
+// (one thread per output, 152 dependent loads and FP64 adds, took 18-21 us).
 __global__ void actvv_reduce_kernel(int nA4, int nblk, const double* __restrict__ part,
                                     double* __restrict__ P12) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (k >= 2 * nA4) return;
   double acc = 0.0;
-  for (int b = 0; b < nblk; ++b) acc += part[(size_t)b * 2 * nA4 + k];
-  P12[k] = acc;
+  for (int b = lane; b < nblk; b += 32) acc += part[(size_t)b * 2 * nA4 + k];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) P12[k] = acc;
 }
 
 // ---------------------------------------------------------------------------
@@ -987,6 +993,12 @@ __global__ void __launch_bounds__(TERM_NT) terms_kernel(Sizes z, TermArgs t,
   if (term == T_F6 || term == T_F7) return;  // term_f6_kernel, term_f7_kernel
   if (term == T_I && z.nA <= 6) return;      // term_i_kernel
   const long n = term_count(term, d);
+  if ((long)blockIdx.x * TERM_NT >= n || ((term == T_J || term == T_K) && !t.lam3)) {
+    // nothing for this CTA: no block sum (its FP64 adds are what most CTAs of a small
+    // system would spend their time on)
+    if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = 0.0;
+    return;
+  }
   double v = 0.0;
   for (long o = (long)blockIdx.x * TERM_NT + threadIdx.x; o < n; o += (long)gridDim.x * TERM_NT)
     v += term_value(term, o, z, d, t);
@@ -1288,31 +1300,28 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   const int nA4 = z.nA * z.nA * z.nA * z.nA;
   {
     const size_t smg = (size_t)3 * z.nA * z.nA * ACTVV_CH * sizeof(double);
-    // factor tables of the split path (tc_rest.cu) when this call formed them
-    ActFact F{nullptr, nullptr, nullptr, 0};
-    if (ints_ready) rest_act_tables(p, &F.alpha, &F.pinfo, &F.tau, &F.ld);
 #define ACTVV_GEN(NA_)                                                                       \
   case NA_:                                                                                  \
     if (ints_ready) {                                                                        \
       raise_smem_limit((const void*)actvv_gen_kernel<NA_, true>, smg);                       \
-      actvv_gen_kernel<NA_, true><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, F, w.P12part); \
+      actvv_gen_kernel<NA_, true><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     } else {                                                                                 \
       raise_smem_limit((const void*)actvv_gen_kernel<NA_, false>, smg);                      \
-      actvv_gen_kernel<NA_, false><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, F, w.P12part); \
+      actvv_gen_kernel<NA_, false><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     }                                                                                        \
     break;
     switch (z.nA) {
       case 1:
         if (ints_ready)
-          actvv_small_kernel<1, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, F, w.P12part);
+          actvv_small_kernel<1, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         else
-          actvv_small_kernel<1, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, F, w.P12part);
+          actvv_small_kernel<1, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         break;
       case 2:
         if (ints_ready)
-          actvv_small_kernel<2, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, F, w.P12part);
+          actvv_small_kernel<2, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         else
-          actvv_small_kernel<2, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, F, w.P12part);
+          actvv_small_kernel<2, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         break;
       ACTVV_GEN(3) ACTVV_GEN(4) ACTVV_GEN(5) ACTVV_GEN(6) ACTVV_GEN(7) ACTVV_GEN(8)
       default: {
@@ -1322,7 +1331,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     }
 #undef ACTVV_GEN
     DSRG_LAUNCH_CHECK(p);
-    actvv_reduce_kernel<<<(2 * nA4 + 127) / 128, 128, 0, st>>>(nA4, ACTVV_BLOCKS, w.P12part, w.P12);
+    actvv_reduce_kernel<<<(2 * nA4 + 3) / 4, 128, 0, st>>>(nA4, ACTVV_BLOCKS, w.P12part, w.P12);
     DSRG_LAUNCH_CHECK(p);
   }
   {

@@ -67,6 +67,12 @@ FF_FN ff ff_diff(ff a, ff b) {
   return ff_fast_sum(t.h, FF_ADD(t.l, FF_SUB(a.l, b.l)));
 }
 
+// a + b
+FF_FN ff ff_add(ff a, ff b) {
+  const ff t = ff_two_sum(a.h, b.h);
+  return ff_fast_sum(t.h, FF_ADD(t.l, FF_ADD(a.l, b.l)));
+}
+
 // a += b: the heads exactly, the tails in FP32, renormalised
 FF_FN void ff_acc(ff& a, ff b) {
   const ff t = ff_two_sum(a.h, b.h);
@@ -85,6 +91,9 @@ FF_FN ff ff_mul(float a, ff b) {
   r.l = FF_FMA(a, b.l, FF_FMA(a, b.h, -r.h));
   return r;
 }
+
+// the pair rounded to FP32 (a product's head alone lacks its tail)
+FF_FN float ff_round(ff a) { return FF_ADD(a.h, a.l); }
 
 // 1/D: an FP32 seed r (error e < 2^-22) and r (1 + e + e^2), remainder e^3
 FF_FN ff ff_inv(ff D) {
@@ -163,7 +172,7 @@ FF_FN ff ff_one_minus_exp(ff D, ff k, const ff* tab) {
   const ff P = ff_mul(T, em);
   const ff a = ff_fast_sum(1.0f, -T.h);
   const ff g = ff_fast_sum(a.h, -P.h);
-  return ff{g.h, FF_ADD(g.l, FF_SUB(FF_SUB(a.l, T.l), P.l))};
+  return ff_fast_sum(g.h, FF_ADD(g.l, FF_SUB(FF_SUB(a.l, T.l), P.l)));
 }
 
 }  // namespace dsrg

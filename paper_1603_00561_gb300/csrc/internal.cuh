@@ -32,7 +32,8 @@ enum Block { BLK_CCVV = 0, BLK_CAVV = 1, BLK_CCAV = 2, BLK_ACTIVE = 3 };
 struct Segment {
   int begin, count, block;
 };
-constexpr int RED_CHUNK = 4096;  // partials per CTA of the first reduction level
+constexpr int RED_CHUNK = 256;   // partials per CTA of the first reduction level
+constexpr int RED_THREADS = 64;  // its threads
 
 // Active-block workspace (spin-orbital tables and spatial integrals).
 struct ActiveWs {

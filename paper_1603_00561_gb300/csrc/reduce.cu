@@ -14,93 +14,87 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
   s = t;
 }
 
-// Level 1: one CTA of 256 threads per chunk of RED_CHUNK partials of one
-// segment. Each thread sums a fixed strided subset with Neumaier compensation;
-// warp 0 then folds the 256 (sum, compensation) pairs in a fixed order: lane l
-// takes pairs 8l .. 8l+7 in index order, and the 32 lane results meet in a
-// fixed butterfly of compensated additions (lane l with lane l ^ o). Every lane
-// ends with the same (sum, compensation); lane 0 stores the chunk's pair.
-__global__ void __launch_bounds__(256) reduce_chunks_kernel(const double* __restrict__ partials,
-                                                            const Segment* __restrict__ segs,
-                                                            const int2* __restrict__ chunks,
-                                                            double* __restrict__ red) {
-  __shared__ double sh_s[256], sh_c[256];
+// (a, ca) += (b, cb) of the lane o away; the lower lane's sum comes first in both, so
+// both get the same operands in the same order.
+__device__ __forceinline__ void neumaier_xor(double& S, double& C, int o) {
+  const double oS = __shfl_xor_sync(0xffffffffu, S, o);
+  const double oC = __shfl_xor_sync(0xffffffffu, C, o);
+  const bool low = (threadIdx.x & o) == 0;
+  double a = low ? S : oS;
+  const double b = low ? oS : S;
+  double cc = (low ? C : oC) + (low ? oC : C);
+  neumaier_add(a, cc, b);
+  S = a;
+  C = cc;
+}
+
+// Level 1: one CTA of RED_THREADS threads per chunk of RED_CHUNK partials of one
+// segment. Each thread sums a fixed strided subset with Neumaier compensation, the
+// lanes of a warp meet in a fixed butterfly, thread 0 adds the warps in order. Small
+// chunks on many SMs: a compensated add is 7 FP64 instructions, each 64 clocks of a
+// scheduler's FP64 pipe (chunks of 4096 on 256 threads took 16 us, of which the
+// partials' reads are under 1).
+__global__ void __launch_bounds__(RED_THREADS) reduce_chunks_kernel(
+    const double* __restrict__ partials, const Segment* __restrict__ segs,
+    const int2* __restrict__ chunks, double* __restrict__ red) {
+  __shared__ double sh_s[RED_THREADS / 32], sh_c[RED_THREADS / 32];
   const int2 ch = chunks[blockIdx.x];
   const Segment sg = segs[ch.x];
   const int k0 = ch.y * RED_CHUNK;
   const int k1 = min(sg.count, k0 + RED_CHUNK);
   const double* p = partials + sg.begin;
   double s = 0.0, c = 0.0;
-  for (int k = k0 + threadIdx.x; k < k1; k += 256) neumaier_add(s, c, p[k]);
-  sh_s[threadIdx.x] = s;
-  sh_c[threadIdx.x] = c;
+  for (int k = k0 + threadIdx.x; k < k1; k += RED_THREADS) neumaier_add(s, c, p[k]);
+  for (int o = 1; o < 32; o <<= 1) neumaier_xor(s, c, o);
+  if ((threadIdx.x & 31) == 0) {
+    sh_s[threadIdx.x >> 5] = s;
+    sh_c[threadIdx.x >> 5] = c;
+  }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double S = 0.0, C = 0.0;
-    for (int k = 8 * threadIdx.x; k < 8 * threadIdx.x + 8; ++k) {
-      neumaier_add(S, C, sh_s[k]);
-      C += sh_c[k];
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < RED_THREADS / 32; ++w) {
+      neumaier_add(s, c, sh_s[w]);
+      c += sh_c[w];
     }
-    for (int o = 1; o < 32; o <<= 1) {
-      // the lower lane of each pair adds the upper one's sum, and vice versa: both
-      // get the same operands in the same order (a + b with b from the higher lane)
-      const double oS = __shfl_xor_sync(0xffffffffu, S, o);
-      const double oC = __shfl_xor_sync(0xffffffffu, C, o);
-      const bool low = (threadIdx.x & o) == 0;
-      double a = low ? S : oS, b = low ? oS : S;
-      const double ca = low ? C : oC, cb = low ? oC : C;
-      double cc = ca + cb;
-      neumaier_add(a, cc, b);
-      S = a;
-      C = cc;
-    }
-    if (threadIdx.x == 0) {
-      red[2 * blockIdx.x] = S;
-      red[2 * blockIdx.x + 1] = C;
-    }
+    red[2 * blockIdx.x] = s;
+    red[2 * blockIdx.x + 1] = c;
   }
 }
 
-// Level 2 (one CTA): the chunk pairs and their block ids are staged in shared
-// memory, then one thread folds the chunk pairs of each block in chunk order.
-// out[0..3] = blocks, out[4] = their total.
-constexpr int RED2_MAX = 2048;  // chunks staged in shared memory
-__global__ void reduce_blocks_kernel(const Segment* __restrict__ segs, const int2* __restrict__ chunks,
-                                     int nchunks, const double* __restrict__ red,
-                                     double* __restrict__ out) {
-  __shared__ double sr[2 * RED2_MAX];
-  __shared__ int sb[RED2_MAX];
-  const bool staged = nchunks <= RED2_MAX;
-  if (staged)
-    for (int k = threadIdx.x; k < nchunks; k += blockDim.x) {
-      sb[k] = segs[chunks[k].x].block;
-      sr[2 * k] = red[2 * k];
-      sr[2 * k + 1] = red[2 * k + 1];
-    }
+// Level 2 (one CTA): warp b folds the chunk pairs of block b, lanes in chunk order
+// and then a fixed butterfly. out[0..3] = blocks, out[4] = their total.
+__global__ void __launch_bounds__(128) reduce_blocks_kernel(const Segment* __restrict__ segs,
+                                                            const int2* __restrict__ chunks,
+                                                            int nchunks,
+                                                            const double* __restrict__ red,
+                                                            double* __restrict__ out) {
+  __shared__ double blk[4];
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double S = 0.0, C = 0.0;
+  for (int k = lane; k < nchunks; k += 32) {
+    if (segs[chunks[k].x].block != b) continue;
+    neumaier_add(S, C, red[2 * k]);
+    C += red[2 * k + 1];
+  }
+  for (int o = 1; o < 32; o <<= 1) neumaier_xor(S, C, o);
+  if (lane == 0) blk[b] = S + C;
   __syncthreads();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (threadIdx.x != 0) return;
   double T = 0.0, TC = 0.0;
-  for (int b = 0; b < 4; ++b) {
-    double S = 0.0, C = 0.0;
-    for (int k = 0; k < nchunks; ++k) {
-      const int kb = staged ? sb[k] : segs[chunks[k].x].block;
-      if (kb != b) continue;
-      neumaier_add(S, C, staged ? sr[2 * k] : red[2 * k]);
-      C += staged ? sr[2 * k + 1] : red[2 * k + 1];
-    }
-    out[b] = S + C;
-    neumaier_add(T, TC, out[b]);
+  for (int k = 0; k < 4; ++k) {
+    out[k] = blk[k];
+    neumaier_add(T, TC, blk[k]);
   }
   out[4] = T + TC;
 }
 
 cudaError_t launch_final_reduce(dsrg_plan* p, double* out) {
   if (p->n_chunks > 0) {
-    reduce_chunks_kernel<<<p->n_chunks, 256, 0, p->stream>>>(p->d_partials, p->d_segs, p->d_chunks,
+    reduce_chunks_kernel<<<p->n_chunks, RED_THREADS, 0, p->stream>>>(p->d_partials, p->d_segs, p->d_chunks,
                                                             p->d_red);
     DSRG_LAUNCH_CHECK(p);
   }
-  reduce_blocks_kernel<<<1, 256, 0, p->stream>>>(p->d_segs, p->d_chunks, p->n_chunks, p->d_red, out);
+  reduce_blocks_kernel<<<1, 128, 0, p->stream>>>(p->d_segs, p->d_chunks, p->n_chunks, p->d_red, out);
   DSRG_LAUNCH_CHECK(p);
   return cudaSuccess;
 }
