@@ -246,97 +246,98 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    const uint32_t leader = tc_elect();
+    if (leader) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_s_hi) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_s_lo) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_bt_hi) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_bt_lo) : "memory");
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
-        int mt, nt;
-        ag_item(it, g.m_tiles, g.n_tiles, &mt, &nt);
-        for (int kb = 0; kb < g.kblocks; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.status)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = tiles + stage * AG_STAGE_BYTES;
-          mbar_expect_tx(&full[stage], (uint32_t)AG_STAGE_BYTES);
-          const int kq = kb * (AG_KB / 2);
-          tma_load_2d(st, &map_s_hi, &full[stage], kq, mt * AG_BM);
-          tma_load_2d(st + AG_TILE, &map_s_lo, &full[stage], kq, mt * AG_BM);
-          tma_load_2d(st + 2 * AG_TILE, &map_bt_hi, &full[stage], kq, nt * AG_BN);
-          tma_load_2d(st + 3 * AG_TILE, &map_bt_lo, &full[stage], kq, nt * AG_BN);
-          if (++stage == AG_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
+    }
+    __syncwarp();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
+      int mt, nt;
+      ag_item(it, g.m_tiles, g.n_tiles, &mt, &nt);
+      for (int kb = 0; kb < g.kblocks; ++kb) {
+        if (!TC_WARP_WAIT(&empty[stage], phase ^ 1u, abort_flag, g.status)) {
+          ok = false;
+          break;
+        }
+        uint8_t* st = tiles + stage * AG_STAGE_BYTES;
+        mbar_expect_tx_if(leader, &full[stage], (uint32_t)AG_STAGE_BYTES);
+        const int kq = kb * (AG_KB / 2);
+        tma_load_2d_if(leader, st, &map_s_hi, &full[stage], kq, mt * AG_BM);
+        tma_load_2d_if(leader, st + AG_TILE, &map_s_lo, &full[stage], kq, mt * AG_BM);
+        tma_load_2d_if(leader, st + 2 * AG_TILE, &map_bt_hi, &full[stage], kq, nt * AG_BN);
+        tma_load_2d_if(leader, st + 3 * AG_TILE, &map_bt_lo, &full[stage], kq, nt * AG_BN);
+        if (++stage == AG_STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok) {
-        int s = stage;
-        uint32_t ph = phase;
-        for (int k = 0; k < AG_STAGES; ++k) {
-          if (--s < 0) {
-            s = AG_STAGES - 1;
-            ph ^= 1u;
-          }
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
-          }
+    }
+    if (!ok && leader) {
+      int s = stage;
+      uint32_t ph = phase;
+      for (int k = 0; k < AG_STAGES; ++k) {
+        if (--s < 0) {
+          s = AG_STAGES - 1;
+          ph ^= 1u;
+        }
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_128x128<true>();
-      int stage = 0, tb = 0;
-      uint32_t phase = 0, tphase = 0;
-      bool ok = true, issued = false;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
-        for (int kb = 0; kb < g.kblocks; ++kb) {
-          const int sub = kb % AG_CH;  // stage within the TMEM accumulation
-          if ((sub == 0 && !mbar_wait(&tempty[tb], tphase ^ 1u, abort_flag, g.status)) ||
-              !mbar_wait(&full[stage], phase, abort_flag, g.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d = tmem_base + (uint32_t)(tb * AG_BN);
-          const uint32_t sa = su32(tiles + stage * AG_STAGE_BYTES);
+    constexpr uint32_t idesc = idesc_128x128<true>();
+    const uint32_t leader = tc_elect(), tmem_u = tc_uniform(tmem_base);
+    int stage = 0, tb = 0;
+    uint32_t phase = 0, tphase = 0;
+    bool ok = true, issued = false;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
+      for (int kb = 0; kb < g.kblocks; ++kb) {
+        const int sub = kb % AG_CH;  // stage within the TMEM accumulation
+        if ((sub == 0 && !TC_WARP_WAIT(&tempty[tb], tphase ^ 1u, abort_flag, g.status)) ||
+            !TC_WARP_WAIT(&full[stage], phase, abort_flag, g.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem_u + (uint32_t)(tb * AG_BN);
+        const uint32_t sa = su32(tiles) + (uint32_t)(stage * AG_STAGE_BYTES);
 #pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            const uint32_t off = (uint32_t)(k * 32);
-            const uint64_t ah = desc_sw64(sa + off), al = desc_sw64(sa + AG_TILE + off);
-            const uint64_t bh = desc_sw64(sa + 2 * AG_TILE + off);
-            const uint64_t bl = desc_sw64(sa + 3 * AG_TILE + off);
-            // a fresh accumulation every AG_CH stages: lo.hi, hi.lo (keeps A), hi.hi (reuses it)
-            tc_mma<true>(d, al, bh, idesc, (sub > 0 || k > 0) ? 1u : 0u);
-            tc_mma<true, 1>(d, ah, bl, idesc, 1u);
-            tc_mma<true, 2>(d, ah, bh, idesc, 1u);
-          }
-          issued = true;
-          tc_commit(&empty[stage]);
-          if (++stage == AG_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
-          if (sub == AG_CH - 1) {
-            tc_commit(&tfull[tb]);
-            if (++tb == AG_NBUF) {
-              tb = 0;
-              tphase ^= 1u;
-            }
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t off = (uint32_t)(k * 32);
+          const uint64_t ah = desc_sw64(sa + off), al = desc_sw64(sa + AG_TILE + off);
+          const uint64_t bh = desc_sw64(sa + 2 * AG_TILE + off);
+          const uint64_t bl = desc_sw64(sa + 3 * AG_TILE + off);
+          // a fresh accumulation every AG_CH stages: lo.hi, hi.lo (keeps A), hi.hi (reuses it)
+          tc_mma_if<true>(leader, d, al, bh, idesc, (sub > 0 || k > 0) ? 1u : 0u);
+          tc_mma_if<true, 1>(leader, d, ah, bl, idesc, 1u);
+          tc_mma_if<true, 2>(leader, d, ah, bh, idesc, 1u);
+        }
+        issued = true;
+        tc_commit_if(leader, &empty[stage]);
+        if (++stage == AG_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+        if (sub == AG_CH - 1) {
+          tc_commit_if(leader, &tfull[tb]);
+          if (++tb == AG_NBUF) {
+            tb = 0;
+            tphase ^= 1u;
           }
         }
       }
-      if (!ok && issued) {
-        tc_commit(drain);
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
-        }
+    }
+    if (!ok && issued && leader) {
+      tc_commit(drain);
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
       }
     }
   } else {

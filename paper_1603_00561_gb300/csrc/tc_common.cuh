@@ -68,6 +68,22 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
       "l"((unsigned long long)map), "r"(su32(bar)), "r"(c0), "r"(c1)
       : "memory");
 }
+// ... of a whole converged warp, issued by its leader lane (tc_elect).
+__device__ __forceinline__ void mbar_expect_tx_if(uint32_t leader, uint64_t* b, uint32_t bytes) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+               " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(su32(b)),
+               "r"(bytes), "r"(leader)
+               : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_if(uint32_t leader, void* dst, const CUtensorMap* map,
+                                               uint64_t* bar, int c0, int c1) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n"
+      " @q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
+      "%4}], [%2];\n}\n" ::"r"(su32(dst)),
+      "l"((unsigned long long)map), "r"(su32(bar)), "r"(c0), "r"(c1), "r"(leader)
+      : "memory");
+}
 // Bring a box of the tensor into L2 ahead of its load (no shared-memory write).
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
@@ -80,6 +96,28 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// One lane of a converged warp (the same one every time); 1 there, 0 elsewhere. An MMA
+// issuer runs with its whole warp and predicates the MMAs and commits on this: its
+// descriptors are then warp-uniform values the compiler keeps in uniform registers, where
+// the MMA reads them. Issued from inside `if (lane == 0)`, every operand is first moved
+// there, about 90 clocks an MMA, more than a 128 x 64 one takes.
+__device__ __forceinline__ uint32_t tc_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+  return p;
+}
+// A value that is the same in every lane, as a warp-uniform one.
+__device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+// Bounded wait of a whole warp (uniform result).
+#define TC_WARP_WAIT(...) __all_sync(0xffffffffu, mbar_wait(__VA_ARGS__))
+__device__ __forceinline__ void tc_commit_if(uint32_t leader, uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          su32(bar)),
+      "r"(leader)
+      : "memory");
 }
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -98,6 +136,26 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
   asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"                               \
                " tcgen05.mma.cta_group::1.kind::" KIND CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
                "l"(a), "l"(b), "r"(idesc), "r"(acc)                                          \
+               : "memory")
+  if (BF16) {
+    if (COL == 1) DSRG_MMA("f16", ".collector::a::fill");
+    else if (COL == 2) DSRG_MMA("f16", ".collector::a::lastuse");
+    else DSRG_MMA("f16", "");
+  } else {
+    if (COL == 1) DSRG_MMA("tf32", ".collector::a::fill");
+    else if (COL == 2) DSRG_MMA("tf32", ".collector::a::lastuse");
+    else DSRG_MMA("tf32", "");
+  }
+#undef DSRG_MMA
+}
+// tc_mma of a whole converged warp, issued by its leader lane (tc_elect).
+template <bool BF16, int COL = 0>
+__device__ __forceinline__ void tc_mma_if(uint32_t leader, uint32_t d, uint64_t a, uint64_t b,
+                                          uint32_t idesc, uint32_t acc) {
+#define DSRG_MMA(KIND, CU)                                                                      \
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"        \
+               " @q tcgen05.mma.cta_group::1.kind::" KIND CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
+               "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(leader)                                 \
                : "memory")
   if (BF16) {
     if (COL == 1) DSRG_MMA("f16", ".collector::a::fill");

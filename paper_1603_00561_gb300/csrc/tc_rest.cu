@@ -22,8 +22,8 @@
 // has no virtual index, is formed in FP64 from B directly.
 //
 // The GEMM kernel (one CTA per SM, persistent, tiles 128 x 256):
-//   warp 0      TMA producer (one elected thread)
-//   warp 1      TMEM allocator and MMA issuer (one elected thread)
+//   warp 0      TMA producer (the whole warp runs the loop, an elected lane issues)
+//   warp 1      TMEM allocator and MMA issuer (likewise)
 //   warps 2-5   epilogue: TMEM -> registers -> FP32 stores of Y
 // Shared memory: 4 stages x (A 128 rows + B 256 rows) x 2 planes x 64 B, 64-byte
 // swizzle. TMEM: 2 buffers x 256 columns. Every wait is bounded (about 2 s).
@@ -73,7 +73,8 @@ __host__ __device__ constexpr uint32_t idesc_mn(bool bf16, uint32_t m, uint32_t 
 // arrive. GRAM (the tile's A rows and B rows overlap, so its diagonal holds
 // squares sum_Q P_r^2) also keeps lo*lo, whose omission would bias them low.
 template <bool BF16, bool GRAM>
-__device__ __forceinline__ void gemm_stage_mmas(uint32_t d, uint32_t sa, uint32_t sb, int kb) {
+__device__ __forceinline__ void gemm_stage_mmas(uint32_t leader, uint32_t d, uint32_t sa, uint32_t sb,
+                                                int kb) {
   constexpr uint32_t idesc = idesc_mn(BF16, G_BM, G_BN);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -82,13 +83,13 @@ __device__ __forceinline__ void gemm_stage_mmas(uint32_t d, uint32_t sa, uint32_
     const uint64_t bh = desc_sw64(sb + off), bl = desc_sw64(sb + G_B_BYTES + off);
     const uint32_t acc0 = (kb > 0 || k > 0) ? 1u : 0u;
     if (GRAM) {
-      tc_mma<BF16>(d, al, bl, idesc, acc0);
-      tc_mma<BF16>(d, al, bh, idesc, 1u);
+      tc_mma_if<BF16>(leader, d, al, bl, idesc, acc0);
+      tc_mma_if<BF16>(leader, d, al, bh, idesc, 1u);
     } else {
-      tc_mma<BF16>(d, al, bh, idesc, acc0);
+      tc_mma_if<BF16>(leader, d, al, bh, idesc, acc0);
     }
-    tc_mma<BF16, 1>(d, ah, bl, idesc, 1u);
-    tc_mma<BF16, 2>(d, ah, bh, idesc, 1u);
+    tc_mma_if<BF16, 1>(leader, d, ah, bl, idesc, 1u);
+    tc_mma_if<BF16, 2>(leader, d, ah, bh, idesc, 1u);
   }
 }
 
@@ -136,99 +137,100 @@ __global__ void __launch_bounds__(G_THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    const uint32_t leader = tc_elect();
+    if (leader) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_hi) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_lo) : "memory");
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
-        const int arow = a.a_row0 + (it / a.n_tiles) * G_BM;
-        const int brow = a.b_row0 + (it % a.n_tiles) * G_BN;
-        for (int kb = 0; kb < a.kblocks; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = tiles + stage * G_STAGE_BYTES;
-          mbar_expect_tx(&full[stage], (uint32_t)G_STAGE_BYTES);
-          // the last auxiliary functions first (see the K order of the MMA issuer)
-          const int kq = a.kq0 + (a.kblocks - 1 - kb) * (G_KB / (BF16 ? 2 : 4));
-          tma_load_2d(st, &map_hi, &full[stage], kq, arow);
-          tma_load_2d(st + G_A_BYTES, &map_lo, &full[stage], kq, arow);
-          uint8_t* sb = st + 2 * G_A_BYTES;
-          tma_load_2d(sb, &map_hi, &full[stage], kq, brow);
-          tma_load_2d(sb + G_A_BYTES, &map_hi, &full[stage], kq, brow + G_BM);
-          tma_load_2d(sb + G_B_BYTES, &map_lo, &full[stage], kq, brow);
-          tma_load_2d(sb + G_B_BYTES + G_A_BYTES, &map_lo, &full[stage], kq, brow + G_BM);
-          if (++stage == G_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
+    }
+    __syncwarp();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
+      const int arow = a.a_row0 + (it / a.n_tiles) * G_BM;
+      const int brow = a.b_row0 + (it % a.n_tiles) * G_BN;
+      for (int kb = 0; kb < a.kblocks; ++kb) {
+        if (!TC_WARP_WAIT(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        uint8_t* st = tiles + stage * G_STAGE_BYTES;
+        mbar_expect_tx_if(leader, &full[stage], (uint32_t)G_STAGE_BYTES);
+        // the last auxiliary functions first (see the K order of the MMA issuer)
+        const int kq = a.kq0 + (a.kblocks - 1 - kb) * (G_KB / (BF16 ? 2 : 4));
+        tma_load_2d_if(leader, st, &map_hi, &full[stage], kq, arow);
+        tma_load_2d_if(leader, st + G_A_BYTES, &map_lo, &full[stage], kq, arow);
+        uint8_t* sb = st + 2 * G_A_BYTES;
+        tma_load_2d_if(leader, sb, &map_hi, &full[stage], kq, brow);
+        tma_load_2d_if(leader, sb + G_A_BYTES, &map_hi, &full[stage], kq, brow + G_BM);
+        tma_load_2d_if(leader, sb + G_B_BYTES, &map_lo, &full[stage], kq, brow);
+        tma_load_2d_if(leader, sb + G_B_BYTES + G_A_BYTES, &map_lo, &full[stage], kq, brow + G_BM);
+        if (++stage == G_STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok) {
-        int s = stage;
-        uint32_t ph = phase;
-        for (int k = 0; k < G_STAGES; ++k) {
-          if (--s < 0) {
-            s = G_STAGES - 1;
-            ph ^= 1u;
-          }
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
-          }
+    }
+    if (!ok && leader) {
+      int s = stage;
+      uint32_t ph = phase;
+      for (int k = 0; k < G_STAGES; ++k) {
+        if (--s < 0) {
+          s = G_STAGES - 1;
+          ph ^= 1u;
+        }
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int tbuf = 0;
-      uint32_t tphase = 0;
-      bool ok = true, issued = false;
-      for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
-        if (!mbar_wait(&tempty[tbuf], tphase ^ 1u, abort_flag, a.status)) {
+    const uint32_t leader = tc_elect(), tmem_u = tc_uniform(tmem_base);
+    int stage = 0;
+    uint32_t phase = 0;
+    int tbuf = 0;
+    uint32_t tphase = 0;
+    bool ok = true, issued = false;
+    for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
+      if (!TC_WARP_WAIT(&tempty[tbuf], tphase ^ 1u, abort_flag, a.status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d = tmem_u + (uint32_t)(tbuf * G_BN);
+      const int arow = a.a_row0 + (it / a.n_tiles) * G_BM;
+      const int brow = a.b_row0 + (it % a.n_tiles) * G_BN;
+      const bool gram = arow < brow + G_BN && brow < arow + G_BM;
+      for (int kb = 0; kb < a.kblocks; ++kb) {
+        if (!TC_WARP_WAIT(&full[stage], phase, abort_flag, a.status)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(tbuf * G_BN);
-        const int arow = a.a_row0 + (it / a.n_tiles) * G_BM;
-        const int brow = a.b_row0 + (it % a.n_tiles) * G_BN;
-        const bool gram = arow < brow + G_BN && brow < arow + G_BM;
-        for (int kb = 0; kb < a.kblocks; ++kb) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sa = su32(tiles + stage * G_STAGE_BYTES);
-          const uint32_t sb = sa + 2 * G_A_BYTES;
-          if (gram)
-            gemm_stage_mmas<BF16, true>(d, sa, sb, kb);
-          else
-            gemm_stage_mmas<BF16, false>(d, sa, sb, kb);
-          issued = true;
-          tc_commit(&empty[stage]);
-          if (++stage == G_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-        if (!ok) break;
-        tc_commit(&tfull[tbuf]);
-        if (++tbuf == 2) {
-          tbuf = 0;
-          tphase ^= 1u;
+        const uint32_t sa = su32(tiles) + (uint32_t)(stage * G_STAGE_BYTES);
+        const uint32_t sb = sa + 2 * G_A_BYTES;
+        if (gram)
+          gemm_stage_mmas<BF16, true>(leader, d, sa, sb, kb);
+        else
+          gemm_stage_mmas<BF16, false>(leader, d, sa, sb, kb);
+        issued = true;
+        tc_commit_if(leader, &empty[stage]);
+        if (++stage == G_STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok && issued) {
-        tc_commit(drain);
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
-        }
+      if (!ok) break;
+      tc_commit_if(leader, &tfull[tbuf]);
+      if (++tbuf == 2) {
+        tbuf = 0;
+        tphase ^= 1u;
+      }
+    }
+    if (!ok && issued && leader) {
+      tc_commit(drain);
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
       }
     }
   } else {

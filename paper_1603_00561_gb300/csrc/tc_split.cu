@@ -23,14 +23,16 @@
 // Newton-Raphson step.
 //
 // Measured on one GB300 (this kernel alone, BF16x3): cc-pVTZ size (24/2/372/1200)
-// 855 us with the FP64 regulator and row-per-lane tail sums, 475 us now, 297 us
-// with the epilogue left out (the shared-memory path of the MMAs); cc-pV5Z size
-// (24/2/1214/3400) 8.45 ms, 8.2 ms, 7.3 ms. What the epilogue still adds is the
-// tail rows' loads (120 us and 0.6 ms), which use the same data path.
+// 855 us with the FP64 regulator and row-per-lane tail sums, 475 us with FP32 pairs,
+// 454 us with the MMAs and copies issued from a converged warp (tc_elect); cc-pV5Z
+// size (24/2/1214/3400) 8.45 ms, 8.2 ms, 6.88 ms; TF32x3 at 31/5/467/1609
+// 2.41 ms to 1.83 ms by that last change. Without the epilogue the MMAs
+// took 297 us and 7.3 ms before it: what the epilogue adds is mostly the
+// tail rows' loads, which use the same shared-memory path.
 //
 // Roles (one CTA per SM, persistent over the work list):
-//   warp 0      TMA producer (one elected thread)
-//   warp 1      TMEM allocator and MMA issuer (one elected thread)
+//   warp 0      TMA producer (the whole warp runs the loop, an elected lane issues)
+//   warp 1      TMEM allocator and MMA issuer (likewise)
 //   warps 2-9   epilogue: 256 threads; warp w reads TMEM lanes 32*(w%4).. and
 //               columns 64*((w-2)/4).. of the tile (two warps per lane quarter)
 // Shared memory: 3 stages x 4 operand slots x 2 planes x (128 rows x 64 B),
@@ -214,29 +216,28 @@ __device__ __forceinline__ int slot_row(const ItemPlan& ip, int slot, int nVpad)
 // the accumulator small until the largest terms arrive, so few truncations act
 // on the full-size sum. hi*lo and hi*hi share their A operand, which the second
 // takes from the collector buffer. N is the item's tile width (nB).
+// shared-memory offsets of the A and B operand slots of both products.
+struct MmaSlots {
+  uint32_t a1, b1, a2, b2;
+};
 template <bool BF16>
-__device__ __forceinline__ void ccvv_stage_mmas(uint32_t dx, uint32_t dy, uint32_t sb,
-                                                const ItemPlan& ip, int kb) {
-  const uint32_t idesc = idesc_128xn<BF16>((uint32_t)ip.nB);
+__device__ __forceinline__ void ccvv_stage_mmas(uint32_t leader, uint32_t dx, uint32_t dy, uint32_t sb,
+                                                const MmaSlots& o, uint32_t idesc, bool two, int kb) {
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const uint32_t off = (uint32_t)((1 - k) * 32);
-    const uint64_t a1h = desc_sw64(sb + (ip.g1a * 2 + 0) * SLOT_BYTES + off);
-    const uint64_t a1l = desc_sw64(sb + (ip.g1a * 2 + 1) * SLOT_BYTES + off);
-    const uint64_t b1h = desc_sw64(sb + (ip.g1b * 2 + 0) * SLOT_BYTES + ip.boff + off);
-    const uint64_t b1l = desc_sw64(sb + (ip.g1b * 2 + 1) * SLOT_BYTES + ip.boff + off);
+    const uint32_t off = sb + (uint32_t)((1 - k) * 32);
+    const uint64_t a1h = desc_sw64(off + o.a1), a1l = desc_sw64(off + o.a1 + SLOT_BYTES);
+    const uint64_t b1h = desc_sw64(off + o.b1), b1l = desc_sw64(off + o.b1 + SLOT_BYTES);
     const uint32_t acc0 = (kb > 0 || k > 0) ? 1u : 0u;
-    tc_mma<BF16>(dx, a1l, b1h, idesc, acc0);
-    tc_mma<BF16, 1>(dx, a1h, b1l, idesc, 1u);
-    tc_mma<BF16, 2>(dx, a1h, b1h, idesc, 1u);
-    if (ip.two) {
-      const uint64_t a2h = desc_sw64(sb + (ip.g2a * 2 + 0) * SLOT_BYTES + off);
-      const uint64_t a2l = desc_sw64(sb + (ip.g2a * 2 + 1) * SLOT_BYTES + off);
-      const uint64_t b2h = desc_sw64(sb + (ip.g2b * 2 + 0) * SLOT_BYTES + ip.boff + off);
-      const uint64_t b2l = desc_sw64(sb + (ip.g2b * 2 + 1) * SLOT_BYTES + ip.boff + off);
-      tc_mma<BF16>(dy, a2l, b2h, idesc, acc0);
-      tc_mma<BF16, 1>(dy, a2h, b2l, idesc, 1u);
-      tc_mma<BF16, 2>(dy, a2h, b2h, idesc, 1u);
+    tc_mma_if<BF16>(leader, dx, a1l, b1h, idesc, acc0);
+    tc_mma_if<BF16, 1>(leader, dx, a1h, b1l, idesc, 1u);
+    tc_mma_if<BF16, 2>(leader, dx, a1h, b1h, idesc, 1u);
+    if (two) {
+      const uint64_t a2h = desc_sw64(off + o.a2), a2l = desc_sw64(off + o.a2 + SLOT_BYTES);
+      const uint64_t b2h = desc_sw64(off + o.b2), b2l = desc_sw64(off + o.b2 + SLOT_BYTES);
+      tc_mma_if<BF16>(leader, dy, a2l, b2h, idesc, acc0);
+      tc_mma_if<BF16, 1>(leader, dy, a2h, b2l, idesc, 1u);
+      tc_mma_if<BF16, 2>(leader, dy, a2h, b2h, idesc, 1u);
     }
   }
 }
@@ -461,178 +462,155 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
+    const uint32_t leader = tc_elect();
+    if (leader) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_hi) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_lo) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_hi64) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&map_lo64) : "memory");
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      constexpr int KE = KB_BYTES / (BF16 ? 2 : 4);
-      for (int idx = it0; ok && idx < it1; ++idx) {
-        const MolDesc* md;
-        const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
-        const int kblocks = md->kblocks, row0 = md->row0, nVpad = md->nVpad;
-        if (a.prefetch == 0) {
-          // The common path. The producer thread is close to the critical path (8
-          // TMA issues per stage against 12 MMAs), so everything that does not
-          // change along K is set up once per item: rows, maps, shared-memory
-          // offsets, L2 policies of the loaded slots and the stage's bytes.
-          const int nl = ip.nload;
-          int srow[4];
-          uint32_t soff[4];
-          const CUtensorMap* mh[4];
-          const CUtensorMap* ml[4];
-          uint32_t bytes = 0;
+    }
+    __syncwarp();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    constexpr int KE = KB_BYTES / (BF16 ? 2 : 4);
+    for (int idx = it0; ok && idx < it1; ++idx) {
+      // Everything that does not change along K is set up once per item: rows, maps,
+      // shared-memory offsets of the loaded slots and the stage's bytes.
+      const MolDesc* md;
+      const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
+      const int kblocks = (int)tc_uniform((uint32_t)md->kblocks), nVpad = md->nVpad;
+      const int nl = (int)tc_uniform((uint32_t)ip.nload);
+      int srow[4];
+      uint32_t soff[4];
+      const CUtensorMap* mh[4];
+      const CUtensorMap* ml[4];
+      uint32_t bytes = 0;
 #pragma unroll
-          for (int l = 0; l < 4; ++l) {
-            const int sl = l < nl ? ip.load[l] : 0;
-            // B-only slots (odd ids) of a narrow tile: 64 rows
-            const bool half = ip.narrow && (sl & 1);
-            srow[l] = row0 + slot_row(ip, sl, nVpad);
-            soff[l] = (uint32_t)(sl * 2 * SLOT_BYTES);
-            mh[l] = half ? &map_hi64 : &map_hi;
-            ml[l] = half ? &map_lo64 : &map_lo;
-            if (l < nl) bytes += half ? SLOT_BYTES : 2 * SLOT_BYTES;
-          }
-          const int kq0 = md->kq0 + (kblocks - 1) * KE;
-          for (int kb = 0; kb < kblocks; ++kb) {
-            if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
-              ok = false;
-              break;
-            }
-            uint8_t* st = tiles + stage * STAGE_BYTES;
-            mbar_expect_tx(&full[stage], bytes);
-            const int kq = kq0 - kb * KE;
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-              if (l >= nl) break;
-              tma_load_2d(st + soff[l], mh[l], &full[stage], kq, srow[l]);
-              tma_load_2d(st + soff[l] + SLOT_BYTES, ml[l], &full[stage], kq, srow[l]);
-            }
-            if (++stage == STAGES) {
-              stage = 0;
-              phase ^= 1u;
-            }
-          }
-          continue;
+      for (int l = 0; l < 4; ++l) {
+        const int sl = (int)tc_uniform((uint32_t)(l < nl ? ip.load[l] : 0));
+        // B-only slots (odd ids) of a narrow tile: 64 rows
+        const bool half = __all_sync(0xffffffffu, ip.narrow && (sl & 1));
+        srow[l] = (int)tc_uniform((uint32_t)(md->row0 + slot_row(ip, sl, nVpad)));
+        soff[l] = (uint32_t)(sl * 2 * SLOT_BYTES);
+        mh[l] = half ? &map_hi64 : &map_hi;
+        ml[l] = half ? &map_lo64 : &map_lo;
+        if (l < nl) bytes += half ? SLOT_BYTES : 2 * SLOT_BYTES;
+      }
+      const int kq0 = (int)tc_uniform((uint32_t)md->kq0) + (kblocks - 1) * KE;
+      // L2 prefetch of later stages (a schedule option the autotuner has never kept)
+      const int pf = a.prefetch;
+      const MolDesc* mdn = md;
+      ItemPlan ipn = ip;
+      const bool has_next = pf > 0 && idx + 1 < it1;
+      if (has_next) ipn = plan_item<HALVES>(a, idx + 1, &mdn);
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!TC_WARP_WAIT(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
+          ok = false;
+          break;
         }
-        // with L2 prefetch (a schedule option the autotuner has never kept)
-        // the next item of this CTA, for prefetches that run past this one
-        const MolDesc* mdn = md;
-        ItemPlan ipn = ip;
-        const bool has_next = idx + 1 < it1;
-        if (has_next) ipn = plan_item<HALVES>(a, idx + 1, &mdn);
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = tiles + stage * STAGE_BYTES;
-          uint32_t bytes = 0;
-          for (int l = 0; l < ip.nload; ++l)
-            bytes += (ip.narrow && (ip.load[l] & 1)) ? SLOT_BYTES : 2 * SLOT_BYTES;
-          mbar_expect_tx(&full[stage], bytes);
-          const int kq = md->kq0 + (kblocks - 1 - kb) * KE;
-          for (int l = 0; l < ip.nload; ++l) {
-            const int sl = ip.load[l];
-            const int row = row0 + slot_row(ip, sl, nVpad);
-            // B-only slots (odd ids) of a narrow tile: 64 rows
-            const bool half = ip.narrow && (sl & 1);
-            tma_load_2d(st + (sl * 2 + 0) * SLOT_BYTES, half ? &map_hi64 : &map_hi, &full[stage], kq,
-                        row);
-            tma_load_2d(st + (sl * 2 + 1) * SLOT_BYTES, half ? &map_lo64 : &map_lo, &full[stage], kq,
-                        row);
-          }
-          if (a.prefetch > 0) {
-            // L2 prefetch of the stage `prefetch` ahead (in this item or the next)
-            const int kf = kb + a.prefetch;
-            if (kf < kblocks) {
-              const int kqf = md->kq0 + (kblocks - 1 - kf) * KE;
-              for (int l = 0; l < ip.nload; ++l) {
-                const int row = row0 + slot_row(ip, ip.load[l], nVpad);
-                tma_prefetch_2d(&map_hi, kqf, row);
-                tma_prefetch_2d(&map_lo, kqf, row);
-              }
-            } else if (has_next && kf - kblocks < mdn->kblocks) {
-              const int kqf = mdn->kq0 + (mdn->kblocks - 1 - (kf - kblocks)) * KE;
-              for (int l = 0; l < ipn.nload; ++l) {
-                const int row = mdn->row0 + slot_row(ipn, ipn.load[l], mdn->nVpad);
-                tma_prefetch_2d(&map_hi, kqf, row);
-                tma_prefetch_2d(&map_lo, kqf, row);
-              }
+        uint8_t* st = tiles + stage * STAGE_BYTES;
+        mbar_expect_tx_if(leader, &full[stage], bytes);
+        const int kq = kq0 - kb * KE;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          if (l >= nl) break;
+          tma_load_2d_if(leader, st + soff[l], mh[l], &full[stage], kq, srow[l]);
+          tma_load_2d_if(leader, st + soff[l] + SLOT_BYTES, ml[l], &full[stage], kq, srow[l]);
+        }
+        if (pf > 0 && leader) {
+          // the stage `prefetch` ahead (in this item or the next)
+          const int kf = kb + pf;
+          if (kf < kblocks) {
+            const int kqf = md->kq0 + (kblocks - 1 - kf) * KE;
+            for (int l = 0; l < ip.nload; ++l) {
+              const int row = md->row0 + slot_row(ip, ip.load[l], nVpad);
+              tma_prefetch_2d(&map_hi, kqf, row);
+              tma_prefetch_2d(&map_lo, kqf, row);
+            }
+          } else if (has_next && kf - kblocks < mdn->kblocks) {
+            const int kqf = mdn->kq0 + (mdn->kblocks - 1 - (kf - kblocks)) * KE;
+            for (int l = 0; l < ipn.nload; ++l) {
+              const int row = mdn->row0 + slot_row(ipn, ipn.load[l], mdn->nVpad);
+              tma_prefetch_2d(&map_hi, kqf, row);
+              tma_prefetch_2d(&map_lo, kqf, row);
             }
           }
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
+        }
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok) {
-        // drain: wait (bounded) until the copies of the stages still in flight have landed
-        int s = stage;
-        uint32_t ph = phase;
-        for (int k = 0; k < STAGES; ++k) {
-          if (--s < 0) {
-            s = STAGES - 1;
-            ph ^= 1u;
-          }
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
-          }
+    }
+    if (!ok && leader) {
+      // drain: wait (bounded) until the copies of the stages still in flight have landed
+      int s = stage;
+      uint32_t ph = phase;
+      for (int k = 0; k < STAGES; ++k) {
+        if (--s < 0) {
+          s = STAGES - 1;
+          ph ^= 1u;
+        }
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int tbuf = 0;
-      uint32_t tphase = 0;
-      bool ok = true;
-      bool issued = false;
-      for (int idx = it0; ok && idx < it1; ++idx) {
-        const MolDesc* md;
-        const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
-        const int kblocks = md->kblocks;
-        if (!mbar_wait(&tempty[tbuf], tphase ^ 1u, abort_flag, a.status)) {
+    const uint32_t leader = tc_elect(), tmem_u = tc_uniform(tmem_base);
+    int stage = 0;
+    uint32_t phase = 0;
+    int tbuf = 0;
+    uint32_t tphase = 0;
+    bool ok = true;
+    bool issued = false;
+    for (int idx = it0; ok && idx < it1; ++idx) {
+      const MolDesc* md;
+      const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
+      const int kblocks = (int)tc_uniform((uint32_t)md->kblocks);
+      MmaSlots o;
+      o.a1 = tc_uniform((uint32_t)(ip.g1a * 2 * SLOT_BYTES));
+      o.b1 = tc_uniform((uint32_t)(ip.g1b * 2 * SLOT_BYTES + ip.boff));
+      o.a2 = tc_uniform((uint32_t)(ip.g2a * 2 * SLOT_BYTES));
+      o.b2 = tc_uniform((uint32_t)(ip.g2b * 2 * SLOT_BYTES + ip.boff));
+      const uint32_t idesc = idesc_128xn<BF16>(tc_uniform((uint32_t)ip.nB));
+      const bool two = __all_sync(0xffffffffu, ip.two);
+      if (!TC_WARP_WAIT(&tempty[tbuf], tphase ^ 1u, abort_flag, a.status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t dx = tmem_u + (uint32_t)(tbuf * 256);
+      const uint32_t dy = dx + 128;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!TC_WARP_WAIT(&full[stage], phase, abort_flag, a.status)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t dx = tmem_base + (uint32_t)(tbuf * 256);
-        const uint32_t dy = dx + 128;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&full[stage], phase, abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sb = su32(tiles + stage * STAGE_BYTES);
-          ccvv_stage_mmas<BF16>(dx, dy, sb, ip, kb);
-          issued = true;
-          tc_commit(&empty[stage]);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-        if (!ok) break;
-        tc_commit(&tfull[tbuf]);
-        if (++tbuf == 2) {
-          tbuf = 0;
-          tphase ^= 1u;
+        ccvv_stage_mmas<BF16>(leader, dx, dy, su32(tiles) + (uint32_t)(stage * STAGE_BYTES), o, idesc,
+                              two, kb);
+        issued = true;
+        tc_commit_if(leader, &empty[stage]);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok && issued) {
-        // drain: every MMA issued so far completes before the TMEM is released
-        tc_commit(drain);
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
-        }
+      if (!ok) break;
+      tc_commit_if(leader, &tfull[tbuf]);
+      if (++tbuf == 2) {
+        tbuf = 0;
+        tphase ^= 1u;
+      }
+    }
+    if (!ok && issued && leader) {
+      // drain: every MMA issued so far completes before the TMEM is released
+      tc_commit(drain);
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
       }
     }
   } else {
