@@ -1299,10 +1299,11 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   }
   const int nA4 = z.nA * z.nA * z.nA * z.nA;
   {
+    const bool f32 = p->prec != DSRG_PREC_FP64;
     const size_t smg = (size_t)3 * z.nA * z.nA * ACTVV_CH * sizeof(double);
 #define ACTVV_GEN(NA_)                                                                       \
   case NA_:                                                                                  \
-    if (ints_ready) {                                                                        \
+    if (f32) {                                                                        \
       raise_smem_limit((const void*)actvv_gen_kernel<NA_, true>, smg);                       \
       actvv_gen_kernel<NA_, true><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     } else {                                                                                 \
@@ -1312,13 +1313,13 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     break;
     switch (z.nA) {
       case 1:
-        if (ints_ready)
+        if (f32)
           actvv_small_kernel<1, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         else
           actvv_small_kernel<1, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         break;
       case 2:
-        if (ints_ready)
+        if (f32)
           actvv_small_kernel<2, true><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);
         else
           actvv_small_kernel<2, false><<<ACTVV_BLOCKS, 256, 0, st>>>(eps, s, z, w.M, w.P12part);

@@ -117,6 +117,7 @@ static void free_all(dsrg_plan* p) {
   if (p->st_copy) cudaStreamDestroy(p->st_copy);
   p->st_copy = nullptr;
   if (p->split) split_free(p);
+  if (p->f64) fp64_tc_free(p);
   if (p->rest) rest_free(p);
   if (p->grad) grad_free(p);
   for (void* a : p->allocs) cudaFree(a);
@@ -234,6 +235,7 @@ dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precis
   if (ok && prec != DSRG_PREC_FP64)
     ok = share ? split_alloc_at(p, share->hi, share->lo, share->Qld, share->row_base, nullptr, nullptr)
                : split_alloc(p);
+  if (ok && prec == DSRG_PREC_FP64) ok = fp64_tc_alloc(p);
   if (ok && p->rest_tc) ok = rest_alloc(p, share ? share->y : nullptr);
   if (ok && (flags & DSRG_PLAN_GRAD)) ok = grad_alloc(p);
   if (ok && (flags & DSRG_PLAN_HOST_IO)) {
@@ -339,11 +341,13 @@ dsrg_status_t run_blocks(dsrg_plan* p, const double* B, const double* eps, const
   if (p->rest_tc) {
     // one tensor-core GEMM feeds CAVV, CCAV and the active-block integrals
     if ((e = launch_split_rest(p, B, eps, G, s)) != cudaSuccess) return cuda_fail(p, e, "cavv/ccav");
+  } else if (p->f64) {
+    if ((e = launch_rest_fp64_tc(p, B, eps, G, s)) != cudaSuccess) return cuda_fail(p, e, "cavv/ccav");
   } else {
     if ((e = launch_cavv_fp64(p, B, eps, G, s)) != cudaSuccess) return cuda_fail(p, e, "cavv");
     if ((e = launch_ccav_fp64(p, B, eps, G, s)) != cudaSuccess) return cuda_fail(p, e, "ccav");
   }
-  if ((e = launch_active(p, B, eps, G, L, L3, F1, s, p->rest_tc)) != cudaSuccess)
+  if ((e = launch_active(p, B, eps, G, L, L3, F1, s, p->rest_tc || p->f64)) != cudaSuccess)
     return cuda_fail(p, e, "active");
   return DSRG_OK;
 }
@@ -367,7 +371,7 @@ static dsrg_status_t run_energy(dsrg_plan* p, const double* B, const double* eps
                                 double* out) {
   cudaError_t e;
   if (p->prec == DSRG_PREC_FP64)
-    e = launch_ccvv_fp64(p, B, eps, s);
+    e = launch_ccvv_fp64_tc(p, B, eps, s);
   else
     e = launch_split_ccvv(p, B, eps, s);
   if (e != cudaSuccess) return cuda_fail(p, e, "ccvv");
@@ -405,7 +409,7 @@ dsrg_status_t dsrg_ccvv_pair_energies(dsrg_plan_t* p, const double* B, const dou
   p->launches = 0;
   cudaError_t e;
   if (p->prec == DSRG_PREC_FP64)
-    e = launch_ccvv_fp64(p, B, eps, s);
+    e = launch_ccvv_fp64_tc(p, B, eps, s);
   else
     e = launch_split_ccvv(p, B, eps, s);
   if (e != cudaSuccess) return cuda_fail(p, e, "ccvv");

@@ -438,7 +438,7 @@ dsrg_status_t dsrg_mrpt2_energy_batched(dsrg_batch_t* b, const double* const* B,
       dsrg_plan* p = b->plans[m];
       p->stream = K > 1 ? b->side[m % K] : b->cap_stream;
       p->launches = 0;
-      e = split ? dsrg::split_stage(p, B[m], eps[m], s[m]) : dsrg::launch_ccvv_fp64(p, B[m], eps[m], s[m]);
+      e = split ? dsrg::split_stage(p, B[m], eps[m], s[m]) : dsrg::launch_ccvv_fp64_tc(p, B[m], eps[m], s[m]);
       if (e != cudaSuccess) st = DSRG_ERR_CUDA;
     }
     if (st == DSRG_OK && split && K > 1) {

@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "oz_gemm.cuh"
 #include "regulators.cuh"
 
 namespace dsrg {
@@ -90,12 +91,14 @@ __global__ void __launch_bounds__(256) gemm_fp64_kernel(GemmArgs g) {
 
 // Gradient workspace (DSRG_PLAN_GRAD).
 struct GradWs {
+  OzWork oz;              // FP64 plans: workspace of the products on the tensor cores
   double* Wk = nullptr;   // [kgroup][nC][nVp][nVp]
   int nVp = 0;
   int kgroup = 1;         // core rows whose W^{kj} are formed before one batched GEMM
   size_t nB = 0;          // elements of B
   double* dX = nullptr;   // [nC][nA][nV][nV]
   double* dZ = nullptr;   // [nA][nC][nC][nV]
+  float* Z32 = nullptr;   // split plans: [nC nV][nC nA], (me|nu)
   double *dW1Vt = nullptr, *dW1T = nullptr, *dTi = nullptr, *dV1 = nullptr;
   double *dW2Vt = nullptr, *dW2T = nullptr, *dV2 = nullptr;
   double *dt1 = nullptr, *dft = nullptr, *dS = nullptr, *dP12 = nullptr;
@@ -112,9 +115,9 @@ cudaError_t launch_gemm_fp64(cudaStream_t st, const GemmArgs& g) {
 // The FP64 plans' GEMMs (split plans assemble dB on the tensor cores).
 static cudaError_t gemm(dsrg_plan* p, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, g.nb);
-  gemm_fp64_kernel<<<grid, 256, 0, p->stream>>>(g);
-  DSRG_LAUNCH_CHECK(p);
+  const cudaError_t e = launch_gemm(p->stream, g, p->grad->oz);
+  if (e != cudaSuccess) return e;
+  p->launches++;
   return cudaSuccess;
 }
 
@@ -233,7 +236,8 @@ template <int NA, typename T>
 __global__ void __launch_bounds__(256) cavv_adj_kernel(
     const double* __restrict__ B, const double* __restrict__ eps, const double* __restrict__ G,
     double s, Sizes z, const int2* __restrict__ tps, int n_tp, int nVp, double* __restrict__ dX,
-    double* __restrict__ deps, double* __restrict__ ds) {
+    double* __restrict__ deps, double* __restrict__ ds, const double* __restrict__ Y, long long ldy,
+    int nVpad) {
   __shared__ T sMA[8][32], sMB[8][32];
   __shared__ T sUA[NA][8][32], sUB[NA][8][32];
   __shared__ double sG[NA][NA];
@@ -255,7 +259,8 @@ __global__ void __launch_bounds__(256) cavv_adj_kernel(
   for (int u = 0; u < NA; ++u)
 #pragma unroll
     for (int r = 0; r < 4; ++r) Xa[u][r] = Xta[u][r] = (T)0;
-  for (int q0 = 0; q0 < z.Q; q0 += 8) {
+  // X from the energy call's Y, or by the FP64 pipe from B
+  for (int q0 = 0; !Y && q0 < z.Q; q0 += 8) {
     for (int e = threadIdx.x; e < 8 * 32; e += 256) {
       const int qq = e / 32, c = e % 32, q = q0 + qq;
       const bool qok = q < z.Q;
@@ -292,6 +297,11 @@ __global__ void __launch_bounds__(256) cavv_adj_kernel(
     for (int r = 0; r < 4; ++r) {
       X[u][r] = (double)Xa[u][r];
       Xt[u][r] = (double)Xta[u][r];
+      const int a = a0 + ty * 4 + r, bb = b0 + tx;
+      if (Y && a < z.nV && bb < z.nV) {
+        X[u][r] = Y[(size_t)(m * nVpad + a) * ldy + u * nVpad + bb];
+        Xt[u][r] = Y[(size_t)(m * nVpad + bb) * ldy + u * nVpad + a];
+      }
     }
   const bool mirror = ab.x < ab.y;
   const int b = b0 + tx;
@@ -376,12 +386,67 @@ __global__ void __launch_bounds__(256) cavv_adj_kernel(
 }
 
 // ---------------------------------------------------------------------------
+// Z_u[m,n,e] = (me|nu) of a split plan's F3 adjoint into Z[(m,e)][(n,u)], FP32 sums over
+// ascending Q: a 64 x 64 tile per CTA, 4 x 4 values per thread. In the adjoint kernel
+// itself, a CTA per e with two shared-memory loads per FMA, these sums took three
+// quarters of its 817 us at 24/2/372/1200; 200 us now for both kernels.
+// ---------------------------------------------------------------------------
+constexpr int ZT = 64, ZK = 16;
+__global__ void __launch_bounds__(256) ccav_z_kernel(const double* __restrict__ B, Sizes z,
+                                                     float* __restrict__ Z) {
+  __shared__ __align__(16) float sr[2][ZK][ZT], sc[2][ZK][ZT];
+  const int M = z.nC * z.nV, N = z.nC * z.nA, r0 = blockIdx.x * ZT, c0 = blockIdx.y * ZT;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  // the row and the column whose Q entries this thread stages: q = threadIdx.x / 64 + 4 k
+  const int lane = threadIdx.x & (ZT - 1), lq = threadIdx.x / ZT;
+  const int r = r0 + lane, c = c0 + lane;
+  const long long HP = (long long)z.nH * z.nP;
+  const double* pr = B + (long long)(r / z.nV) * z.nP + z.nA + r % z.nV;
+  const double* pc = B + (long long)(c / z.nA) * z.nP + c % z.nA;
+  float a[ZK / 4], b[ZK / 4], acc[4][4] = {};
+  auto fetch = [&](int q0) {
+#pragma unroll
+    for (int k = 0; k < ZK / 4; ++k) {
+      const int q = q0 + lq + 4 * k;
+      a[k] = (q < z.Q && r < M) ? (float)pr[q * HP] : 0.0f;
+      b[k] = (q < z.Q && c < N) ? (float)pc[q * HP] : 0.0f;
+    }
+  };
+  fetch(0);
+  for (int q0 = 0, s = 0; q0 < z.Q; q0 += ZK, s ^= 1) {
+#pragma unroll
+    for (int k = 0; k < ZK / 4; ++k) {
+      sr[s][lq + 4 * k][lane] = a[k];
+      sc[s][lq + 4 * k][lane] = b[k];
+    }
+    __syncthreads();  // also: the other buffer's readers are done (they are one chunk behind)
+    fetch(q0 + ZK);
+#pragma unroll
+    for (int k = 0; k < ZK; ++k) {
+      const float4 x = *(const float4*)&sr[s][k][ty * 4], y = *(const float4*)&sc[s][k][tx * 4];
+      const float xr[4] = {x.x, x.y, x.z, x.w}, yc[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xr[i], yc[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (r0 + ty * 4 + i < M && c0 + tx * 4 + j < N)
+        Z[(size_t)(r0 + ty * 4 + i) * N + c0 + tx * 4 + j] = acc[i][j];
+}
+
+// ---------------------------------------------------------------------------
 // F3 adjoint: one CTA per virtual e; writes dZ[w][m][n][e].
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) ccav_adj_kernel(
     const double* __restrict__ B, const double* __restrict__ eps, const double* __restrict__ G,
-    double s, Sizes z, double* __restrict__ dZ, double* __restrict__ deps, double* __restrict__ ds) {
+    double s, Sizes z, double* __restrict__ dZ, double* __restrict__ deps, double* __restrict__ ds,
+    const T* __restrict__ Y, long long ldy, int nVpad, long long xc) {
   extern __shared__ double smem[];
   const int nC = z.nC, nA = z.nA;
   double* accm = smem;                 // [nC]  deps of core orbitals
@@ -392,9 +457,16 @@ __global__ void __launch_bounds__(256) ccav_adj_kernel(
   __shared__ double red[8];
   const int e = blockIdx.x;
   const int nz = nA * nC * nC;
-  for (int k = threadIdx.x; k < nz; k += 256) Z[k] = (T)0;
+  // Z_u[m,n,e] = (me|nu) from Y (the energy call's, or ccav_z_kernel's), or from B
+  for (int k = threadIdx.x; k < nz; k += 256) {
+    const int mn = Y ? k / nA : 0, u = Y ? k % nA : 0;  // lanes along Y's columns (n, u)
+    if (Y)
+      Z[u * nC * nC + mn] = Y[(size_t)((mn / nC) * nVpad + e) * ldy + xc + (mn % nC) * nA + u];
+    else
+      Z[k] = (T)0;
+  }
   for (int k = threadIdx.x; k < nC + nA; k += 256) accm[k] = 0.0;
-  for (int q0 = 0; q0 < z.Q; q0 += 8) {
+  for (int q0 = 0; !Y && q0 < z.Q; q0 += 8) {
     __syncthreads();
     for (int k = threadIdx.x; k < 8 * nC * (1 + nA); k += 256) {
       const int qq = k / (nC * (1 + nA)), r = k % (nC * (1 + nA)), q = q0 + qq;
@@ -1196,6 +1268,10 @@ bool grad_alloc(dsrg_plan* p) {
     const size_t kmax = ((size_t)2 << 30) / per_w;
     g->kgroup = (int)(kmax < 1 ? 1 : (kmax > (size_t)z.nC ? (size_t)z.nC : kmax));
     ok = plan_alloc(p, (void**)&g->Wk, per_w * g->kgroup);
+    // the largest product: dB of a group of rows from W
+    g->oz.bytes = oz_work_bytes(z.Q, z.nV, (long long)z.nC * z.nV, g->kgroup, true, false);
+    ok = ok && plan_alloc(p, &g->oz.mem, g->oz.bytes);
+    g->oz.status = p->d_status;
   } else {
     // split plans: S and B^T planes of the tensor-core assembly (tc_adjoint.cu)
     ok = tc_adj_alloc(p);
@@ -1207,6 +1283,8 @@ bool grad_alloc(dsrg_plan* p) {
     const size_t nA4 = (size_t)z.nA * z.nA * z.nA * z.nA;
     ok = ok && plan_alloc(p, (void**)&g->dX, (size_t)z.nC * z.nA * z.nV * z.nV * 8) &&
          plan_alloc(p, (void**)&g->dZ, (size_t)z.nA * z.nC * z.nC * z.nV * 8) &&
+         (p->prec == DSRG_PREC_FP64 ||
+          plan_alloc(p, (void**)&g->Z32, (size_t)z.nA * z.nC * z.nC * z.nV * 4)) &&
          plan_alloc(p, (void**)&g->dW1Vt, w1n * 8) && plan_alloc(p, (void**)&g->dW1T, w1n * 8) &&
          plan_alloc(p, (void**)&g->dTi, w1n * 8) && plan_alloc(p, (void**)&g->dV1, w1n * 8) &&
          plan_alloc(p, (void**)&g->dW2Vt, w2n * 8) && plan_alloc(p, (void**)&g->dW2T, w2n * 8) &&
@@ -1324,7 +1402,12 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     const int kg = (z.nC - k0) < w->kgroup ? (z.nC - k0) : w->kgroup;
     // multi-GPU share: groups of core rows dealt round-robin (their dB rows are disjoint)
     if (!pair_in_shard(grp, p->shard_rank, p->shard_world)) continue;
-    for (int k = k0; k < k0 + kg; ++k) {
+    // all rows at once: the pairs i <= j on the tensor cores, W^{ji} = W^{ij T}
+    const bool pairwise = p->f64 && kg == z.nC && p->shard_world == 1;
+    if (pairwise &&
+        (e = launch_ccvv_adj_fp64_tc(p, B, eps, s, w->nVp, w->Wk, deps, ds)) != cudaSuccess)
+      return e;
+    for (int k = k0; !pairwise && k < k0 + kg; ++k) {
       ccvv_adj_kernel<double><<<z.nC * n_tp, 256, 0, st>>>(B, eps, s, z, k, p->d_tp_ccvv, n_tp,
                                                            w->nVp, w->Wk + (k - k0) * wstride,
                                                            deps, ds);
@@ -1345,6 +1428,10 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     return cudaSuccess;
   }
   const long long nV = z.nV, nV2 = nV * nV;
+  // the integrals with one or two active indices as the energy call formed them
+  long long ldy = 0, xc = 0;
+  int nVpad = 0;
+  const double* Yd = fp64 ? fp64_tc_y(p, &ldy, &nVpad, &xc) : nullptr;
 
   // ---- F2
   {
@@ -1352,10 +1439,10 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
   case NA_:                                                                                      \
     if (fp64)                                                                                    \
       cavv_adj_kernel<NA_, double><<<z.nC * p->n_tp_cavv, 256, 0, st>>>(                         \
-          B, eps, G, s, z, p->d_tp_cavv, p->n_tp_cavv, z.nV, w->dX, deps, ds);                   \
+          B, eps, G, s, z, p->d_tp_cavv, p->n_tp_cavv, z.nV, w->dX, deps, ds, Yd, ldy, nVpad);   \
     else                                                                                         \
       cavv_adj_kernel<NA_, float><<<z.nC * p->n_tp_cavv, 256, 0, st>>>(                          \
-          B, eps, G, s, z, p->d_tp_cavv, p->n_tp_cavv, z.nV, w->dX, deps, ds);                   \
+          B, eps, G, s, z, p->d_tp_cavv, p->n_tp_cavv, z.nV, w->dX, deps, ds, nullptr, 0, 0);    \
     break;
     if (!fp64 && p->rest_tc) {
       // X from the energy call's tensor-core GEMM output
@@ -1385,10 +1472,15 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     const size_t sm = ccav_adj_smem(z);
     if (fp64) {
       raise_smem_limit((const void*)ccav_adj_kernel<double>, sm);
-      ccav_adj_kernel<double><<<z.nV, 256, sm, st>>>(B, eps, G, s, z, w->dZ, deps, ds);
+      ccav_adj_kernel<double><<<z.nV, 256, sm, st>>>(B, eps, G, s, z, w->dZ, deps, ds, Yd, ldy, nVpad,
+                                                     xc);
     } else {
+      const dim3 gz((unsigned)(((long long)z.nC * z.nV + ZT - 1) / ZT), (unsigned)((z.nC * z.nA + ZT - 1) / ZT));
+      ccav_z_kernel<<<gz, 256, 0, st>>>(B, z, w->Z32);
+      DSRG_LAUNCH_CHECK(p);
       raise_smem_limit((const void*)ccav_adj_kernel<float>, sm);
-      ccav_adj_kernel<float><<<z.nV, 256, sm, st>>>(B, eps, G, s, z, w->dZ, deps, ds);
+      ccav_adj_kernel<float><<<z.nV, 256, sm, st>>>(B, eps, G, s, z, w->dZ, deps, ds, w->Z32,
+                                                    (long long)z.nC * z.nA, z.nV, 0);
     }
     DSRG_LAUNCH_CHECK(p);
   }

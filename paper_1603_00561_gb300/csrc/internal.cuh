@@ -54,6 +54,7 @@ struct ActiveWs {
   int actvv_blocks = 0;
 };
 
+struct Fp64Tc;     // FP64 plans on the tensor cores (fp64_tc.cu)
 struct SplitWs;    // tensor-core path workspace (tc_split.cu)
 struct RestState;  // tensor-core CAVV / CCAV / active integrals (tc_rest.cu)
 struct GradWs;   // gradient workspace (grad.cu)
@@ -95,6 +96,7 @@ struct dsrg_plan {
   double* d_pairbuf = nullptr;  // [nC*nC] pair energies (scratch for the pairs entry)
 
   dsrg::ActiveWs act;
+  dsrg::Fp64Tc* f64 = nullptr;
   dsrg::SplitWs* split = nullptr;
   dsrg::RestState* rest = nullptr;  // split CAVV / CCAV / active integrals (tc_rest.cu)
   dsrg::GradWs* grad = nullptr;  // gradient workspace (DSRG_PLAN_GRAD)
@@ -130,6 +132,18 @@ bool plan_alloc(dsrg_plan* p, void** ptr, size_t bytes);
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
 
 // Launchers (each returns cudaSuccess or the launch error; adds to p->launches).
+// FP64 plans: tensor-core products (fp64_tc.cu) when their workspace is a small enough
+// part of the device's memory (then p->f64 is set), else the CUDA-core kernels.
+bool fp64_tc_alloc(dsrg_plan* p);
+void fp64_tc_free(dsrg_plan* p);
+cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps, double s);
+cudaError_t launch_rest_fp64_tc(dsrg_plan* p, const double* B, const double* eps, const double* G,
+                                double s);
+cudaError_t launch_ccvv_adj_fp64_tc(dsrg_plan* p, const double* B, const double* eps, double s, int nVp,
+                                    double* W, double* deps, double* ds);
+// The FP64 integrals of the energy call just made: Y[(g,e)][u nVpad + f] = (ge|uf),
+// Y[(g,e)][xc + h nA + x] = (ge|hx) (null without p->f64).
+const double* fp64_tc_y(const dsrg_plan* p, long long* ldy, int* nVpad, long long* xc);
 cudaError_t launch_ccvv_fp64(dsrg_plan* p, const double* B, const double* eps, double s);
 cudaError_t launch_cavv_fp64(dsrg_plan* p, const double* B, const double* eps, const double* G,
                              double s);

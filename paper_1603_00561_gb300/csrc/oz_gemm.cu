@@ -1,0 +1,592 @@
+// FP64 products on the tensor cores: C = A . B^T from exact integer slices.
+//
+// The FP64 pipe of this GPU gives 1.1 TFLOP/s, its BF16 tensor cores 1900. The
+// scheme is that of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59 (2012) 95),
+// with fixed-point slices as in Ootomo, Ozaki and Yokota (IJHPCA 38 (2024) 297):
+// every row of an operand gets one power-of-two scale 2^E above its largest
+// magnitude and each value becomes a 56-bit fixed-point number, cut into seven
+// signed base-256 digits d_1 .. d_7 in [-128, 128], exact in BF16:
+//     x = 2^E sum_i d_i 2^{1 - 8i},   |error| <= 2^{E - 56}.
+// A product of two digits is at most 2^14, so sums of up to seven of them over 128
+// K values stay below 2^24 and the FP32 accumulator of the tensor cores holds them
+// exactly, whatever the order (its truncation never acts). Digit products with the
+// same weight i + j = g share an accumulator; g = 2 .. 9 are kept (34 products, the
+// first dropped weight is 2^-78 of the scales). After every 128 K values the
+// epilogue takes the eight integer sums out of TMEM and adds them into a 96-bit
+// integer per element; one conversion and one rounding to FP64 end the tile. The
+// result does not depend on the order of anything. Its error, set by the slicing
+// (2^-56 of the row scale per value) and that rounding, is below that of a chain of
+// FP64 FMAs (tests/test_gpu_oz_gemm.py).
+//
+// A row with a NaN gives NaN; a row with an infinity is multiplied by FP64 FMAs in the
+// epilogue, so that infinities propagate as in a plain FP64 product.
+//
+// Kernel (one CTA per SM, persistent, tiles 128 x 64):
+//   warp 0      producer: bulk copies of the seven slices of 128 A rows (56 KB, one
+//               copy) and of 64 B rows (28 KB, seven copies), 32 K values; 2 stages
+//   warp 1      TMEM allocator and MMA issuer: 2 x 34 MMAs (N = 64) per stage; the
+//               products of one A slice run back to back on the collector buffer
+//   warps 2-9   epilogue (32 columns each): TMEM -> integers -> FP64 stores
+// TMEM: 8 accumulators x 64 columns = all 512. Every wait is bounded (about 2 s).
+// The slices lie in memory as the MMAs want them in shared memory, [row / 128][K / 32]
+// [slice][row % 128][64 bytes, swizzled]: as K-major planes behind a tensor map a stage
+// was 1344 rows of 64 bytes and took 4400 clocks to arrive, twice what its MMAs take.
+#include <cuda_bf16.h>
+
+#include "internal.cuh"
+#include "oz_gemm.cuh"
+#include "tc_common.cuh"
+
+namespace dsrg {
+
+constexpr int OZ_BM = 128, OZ_BN = 64;
+constexpr int OZ_KB = 32;                     // K values per stage (64 bytes: one swizzle span)
+constexpr int OZ_CHUNK = 4;                   // stages per exact accumulation (128 K values)
+constexpr int OZ_STAGES = 2;
+constexpr int OZ_A_SLICE = OZ_BM * 64, OZ_B_SLICE = OZ_BN * 64;
+constexpr int OZ_A_BYTES = OZ_S * OZ_A_SLICE, OZ_B_BYTES = OZ_S * OZ_B_SLICE;
+constexpr int OZ_STAGE_BYTES = OZ_A_BYTES + OZ_B_BYTES;
+constexpr int OZ_THREADS = 320, OZ_EPI_WARPS = 8;
+constexpr int OZ_EXP_INF = 0x7ff;             // "exponent" of a row with an infinity
+constexpr int OZ_EXP_NAN = 0x800;             // ... with a NaN
+
+// ------------------------------- row scales -------------------------------
+// Biased exponent of the largest magnitude of every row, by atomicMax (rexp starts
+// at 0). One CTA: 64 rows x 64 K values; lanes run along the contiguous index.
+template <bool KCONT>
+__global__ void __launch_bounds__(256) oz_rowmax_kernel(OzRows s, int* __restrict__ rexp) {
+  __shared__ int mx[64];
+  const int r0 = blockIdx.x * 64, l0 = blockIdx.y * 64, K = s.L1 * s.L2;
+  if (threadIdx.x < 64) mx[threadIdx.x] = 0;
+  __syncthreads();
+  const int f = threadIdx.x & 63, g = threadIdx.x >> 6;
+  int m = 0;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int rr = KCONT ? g + 4 * k : f, l = l0 + (KCONT ? f : g + 4 * k);
+    long long off;
+    int e = 0;
+    if (oz_row(s, r0 + rr, off) && l < K) {
+      const double x = s.p[off + oz_k(s, l)];
+      e = (__double2hiint(x) >> 20) & 0x7ff;
+      if (x != x) e = OZ_EXP_NAN;
+    }
+    if (KCONT) {
+      for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+      if ((threadIdx.x & 31) == 0) atomicMax(&mx[rr], e);
+    } else {
+      m = max(m, e);
+    }
+  }
+  if (!KCONT) atomicMax(&mx[f], m);
+  __syncthreads();
+  if (threadIdx.x < 64 && r0 + threadIdx.x < s.total) atomicMax(&rexp[r0 + threadIdx.x], mx[threadIdx.x]);
+}
+
+// ------------------------------- slices -------------------------------
+// x as a fixed-point integer of the row scale: round(x 2^{55 - E}), |.| <= 2^55.
+__device__ __forceinline__ long long oz_fixed(double x, int rowexp) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(u >> 52) & 0x7ff;
+  if (e == 0 || rowexp >= OZ_EXP_INF) return 0;  // zeros and values below 2^-1022; see the epilogue
+  unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int sh = rowexp - e - 2;  // right shift of the 53-bit significand
+  if (sh <= 0)
+    m <<= -sh;  // 0, 1 or 2 places (e <= rowexp)
+  else if (sh < 64)
+    m = (m + (1ull << (sh - 1))) >> sh;
+  else
+    m = 0;
+  return (u >> 63) ? -(long long)m : (long long)m;
+}
+
+// Byte offset of the 8 values (16 bytes) from K index l (a multiple of 8) of a slice of a
+// plane row: 64-byte rows with the 64-byte swizzle (16-byte chunk ^= row bits 1-2).
+__device__ __forceinline__ size_t oz_off(int row, int l, int sl, int nkb) {
+  const int r = row & 127;
+  const size_t blk = ((size_t)(row >> 7) * nkb + (l >> 5)) * OZ_S + sl;
+  return (blk * 128 + r) * 64 + (size_t)((((l >> 3) & 3) ^ ((r >> 1) & 3)) * 16);
+}
+
+// 64 rows x 64 K values per CTA through shared memory.
+template <bool KCONT>
+__global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __restrict__ rexp,
+                                                       __nv_bfloat16* __restrict__ planes, int Kp) {
+  __shared__ long long t[64][65];
+  const int r0 = blockIdx.x * 64, l0 = blockIdx.y * 64, K = s.L1 * s.L2;
+  const int f = threadIdx.x & 63, g = threadIdx.x >> 6;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int rr = KCONT ? g + 4 * k : f, ll = KCONT ? f : g + 4 * k;
+    long long off, v = 0;
+    if (oz_row(s, r0 + rr, off) && l0 + ll < K) v = oz_fixed(s.p[off + oz_k(s, l0 + ll)], rexp[r0 + rr]);
+    t[rr][ll] = v;
+  }
+  __syncthreads();
+  const int rr = threadIdx.x >> 2, c0 = (threadIdx.x & 3) * 16;
+  if (r0 + rr >= s.total || l0 + c0 >= Kp) return;
+  const int nkb = Kp / OZ_KB;
+  long long v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = t[rr][c0 + k];
+#pragma unroll
+  for (int sl = OZ_S - 1; sl >= 0; --sl) {
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      const int d0 = sl ? (int)(signed char)v[k] : (int)v[k];
+      const int d1 = sl ? (int)(signed char)v[k + 1] : (int)v[k + 1];
+      v[k] = (v[k] - d0) >> 8;
+      v[k + 1] = (v[k + 1] - d1) >> 8;
+      const __nv_bfloat162 h = __floats2bfloat162_rn((float)d0, (float)d1);
+      w[k / 2] = *(const uint32_t*)&h;
+    }
+    uint8_t* o = (uint8_t*)planes;
+    *(uint4*)(o + oz_off(r0 + rr, l0 + c0, sl, nkb)) = make_uint4(w[0], w[1], w[2], w[3]);
+    *(uint4*)(o + oz_off(r0 + rr, l0 + c0 + 8, sl, nkb)) = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
+// ------------------------------- the product -------------------------------
+__device__ __forceinline__ void oz_bulk(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          su32(dst)),
+      "l"(src), "r"(bytes), "r"(su32(bar))
+      : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void oz_mma(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                       uint32_t acc) {
+#define OZ_MMA(CU)                                                                               \
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"         \
+               " @q tcgen05.mma.cta_group::1.kind::f16" CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
+               "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(leader)                                 \
+               : "memory")
+  if (N == 0) OZ_MMA(".collector::a::fill");
+  else if (N == 1) OZ_MMA(".collector::a::use");
+  else OZ_MMA(".collector::a::lastuse");
+#undef OZ_MMA
+}
+
+// One K step (16 values): digit pairs (i, j), i + j <= 9, the j of one i back to back.
+__device__ __forceinline__ void oz_kstep(uint32_t leader, uint32_t d, uint32_t sa, uint32_t sb, bool first) {
+  constexpr uint32_t idesc = idesc_128xn<true>(OZ_BN);
+#pragma unroll
+  for (int i = 1; i <= OZ_S; ++i) {
+    const uint64_t a = desc_sw64(sa + (i - 1) * OZ_A_SLICE);
+    const int jn = (OZ_G + 1 - i) < OZ_S ? (OZ_G + 1 - i) : OZ_S;  // j <= 9 - i and <= 7
+#pragma unroll
+    for (int j = 1; j <= jn; ++j) {
+      const int g = i + j;
+      const uint64_t b = desc_sw64(sb + (j - 1) * OZ_B_SLICE);
+      // the first product of a weight starts its accumulator
+      const int i0 = g - OZ_S > 1 ? g - OZ_S : 1;
+      const uint32_t acc = (first && i == i0) ? 0u : 1u;
+      const uint32_t dg = d + (uint32_t)((g - 2) * OZ_BN);
+      if (j == 1) oz_mma<0>(leader, dg, a, b, idesc, acc);
+      else if (j == jn) oz_mma<2>(leader, dg, a, b, idesc, acc);
+      else oz_mma<1>(leader, dg, a, b, idesc, acc);
+    }
+  }
+}
+
+__device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                 "=r"(r[7])
+               : "r"(taddr));
+}
+
+struct OzTile {
+  int arow, brow;       // first plane rows
+  int i0, j0;           // first row and column of C
+  long long coff;       // its problem's offset in C
+};
+__device__ __forceinline__ OzTile oz_tile(const OzArgs& a, int it) {
+  const int per = a.mt * a.nt, pr = it / per, r = it % per;
+  OzTile t;
+  // row blocks of `band` tiles with the columns inside: the CTAs running at one time
+  // share operand slabs in L2
+  const int mb = r / (a.band * a.nt), rem = r % (a.band * a.nt);
+  const int rows = min(a.band, a.mt - mb * a.band);
+  const int n = rem / rows, m = mb * a.band + rem % rows;
+  t.i0 = m * OZ_BM;
+  t.j0 = n * OZ_BN;
+  const int2 ij = a.pairs ? a.pairs[a.p0 + pr * a.pstep] : make_int2(pr, pr);
+  t.arow = a.arow0 + ij.x * a.astep + t.i0;
+  t.brow = a.brow0 + ij.y * a.bstep + t.j0;
+  t.coff = (long long)pr * a.sc;
+  return t;
+}
+
+// An element whose row of A or B is not finite.
+static __device__ __noinline__ double oz_not_finite(const OzArgs& a, int ra, int rb, int e) {
+  if (e >= OZ_EXP_NAN) return __longlong_as_double(0x7ff8000000000000ll);
+  long long oa, ob;
+  oz_row(a.a, ra, oa);
+  oz_row(a.b, rb, ob);
+  double d = 0.0;
+  for (int l = 0; l < a.a.L1 * a.a.L2; ++l) d = fma(a.a.p[oa + oz_k(a.a, l)], a.b.p[ob + oz_k(a.b, l)], d);
+  return d;
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 1)
+    oz_gemm_kernel(const uint8_t* __restrict__ pa, const uint8_t* __restrict__ pb,
+                   const __grid_constant__ OzArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + OZ_STAGES * OZ_STAGE_BYTES);
+  uint64_t* empty = full + OZ_STAGES;
+  uint64_t* tfull = empty + OZ_STAGES;
+  uint64_t* tempty = tfull + 1;
+  uint64_t* drain = tempty + 1;
+  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < OZ_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, OZ_EPI_WARPS);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     su32(tmem_slot)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    const uint32_t leader = tc_elect();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < a.n_items; it += gridDim.x) {
+      const OzTile t = oz_tile(a, it);
+      const uint8_t* ga = pa + (size_t)(t.arow >> 7) * a.kstages * OZ_A_BYTES;
+      const uint8_t* gb = pb + (size_t)(t.brow >> 7) * a.kstages * OZ_A_BYTES + (t.brow & 64) * 64;
+      for (int kb = 0; kb < a.kstages; ++kb) {
+        if (!TC_WARP_WAIT(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        uint8_t* st = smem + stage * OZ_STAGE_BYTES;
+        mbar_expect_tx_if(leader, &full[stage], (uint32_t)OZ_STAGE_BYTES);
+        if (leader) {
+          // A: a whole 128-row block; B: a 64-row half of every slice of its block
+          oz_bulk(st, ga + (size_t)kb * OZ_A_BYTES, OZ_A_BYTES, &full[stage]);
+#pragma unroll
+          for (int sl = 0; sl < OZ_S; ++sl)
+            oz_bulk(st + OZ_A_BYTES + sl * OZ_B_SLICE, gb + (size_t)kb * OZ_A_BYTES + sl * OZ_A_SLICE,
+                    OZ_B_SLICE, &full[stage]);
+        }
+        __syncwarp();
+        if (++stage == OZ_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    if (!ok && leader) {
+      int s = stage;
+      uint32_t ph = phase;
+      for (int k = 0; k < OZ_STAGES; ++k) {
+        if (--s < 0) {
+          s = OZ_STAGES - 1;
+          ph ^= 1u;
+        }
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    const uint32_t leader = tc_elect();
+    const uint32_t tm = tc_uniform(tmem);
+    int stage = 0;
+    uint32_t phase = 0, tphase = 0;
+    bool ok = true, issued = false;
+    for (int it = blockIdx.x; ok && it < a.n_items; it += gridDim.x) {
+      for (int kb = 0; kb < a.kstages; ++kb) {
+        if (kb % OZ_CHUNK == 0) {
+          if (!TC_WARP_WAIT(tempty, tphase ^ 1u, abort_flag, a.status)) {
+            ok = false;
+            break;
+          }
+          tphase ^= 1u;
+        }
+        if (!TC_WARP_WAIT(&full[stage], phase, abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t sa = su32(smem) + stage * OZ_STAGE_BYTES, sb = sa + OZ_A_BYTES;
+        oz_kstep(leader, tm, sa, sb, kb % OZ_CHUNK == 0);
+        oz_kstep(leader, tm, sa + 32, sb + 32, false);
+        issued = true;
+        tc_commit_if(leader, &empty[stage]);
+        if (++stage == OZ_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+        if (kb % OZ_CHUNK == OZ_CHUNK - 1 || kb == a.kstages - 1) tc_commit_if(leader, tfull);
+      }
+    }
+    if (!ok && issued && leader) {
+      tc_commit(drain);
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
+      }
+    }
+  } else {
+    const int quarter = warp & 3, ch = (warp - 2) >> 2;  // TMEM lanes and column half
+    const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ch * 32);
+    uint32_t tphase = 0;
+    const int nchunks = (a.kstages + OZ_CHUNK - 1) / OZ_CHUNK;
+    for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
+      const OzTile t = oz_tile(a, it);
+      // 96-bit sums in units of 2^-70 of the scales: hi 2^32 + lo
+      long long hi[32];
+      uint32_t lo[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        hi[c] = 0;
+        lo[c] = 0;
+      }
+      bool ok = true;
+      for (int ck = 0; ck < nchunks; ++ck) {
+        ok = mbar_wait(tfull, tphase, abort_flag, a.status) && ok;
+        tphase ^= 1u;
+        tc_fence_after();
+        if (ok) {
+#pragma unroll
+          for (int c8 = 0; c8 < 4; ++c8) {
+            uint32_t r[4][8];
+            // weights 6 .. 9 (2^-70 units: 2^24, 2^16, 2^8, 1)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) oz_tmem_ld8(tb + (uint32_t)((4 + g) * OZ_BN + 8 * c8), r[g]);
+            tmem_ld_wait();
+            int carry[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const int k = 8 * c8 + c;
+              long long v = (long long)lo[k] + __float2int_rn(__uint_as_float(r[3][c]));
+              v += (long long)__float2int_rn(__uint_as_float(r[2][c])) << 8;
+              v += (long long)__float2int_rn(__uint_as_float(r[1][c])) << 16;
+              v += (long long)__float2int_rn(__uint_as_float(r[0][c])) << 24;
+              lo[k] = (uint32_t)v;
+              carry[c] = (int)(v >> 32);
+            }
+            // weights 2 .. 5 (2^-38 units)
+#pragma unroll
+            for (int g = 0; g < 4; ++g) oz_tmem_ld8(tb + (uint32_t)(g * OZ_BN + 8 * c8), r[g]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const int k = 8 * c8 + c;
+              long long v = hi[k] + carry[c] + __float2int_rn(__uint_as_float(r[3][c]));
+              v += (long long)__float2int_rn(__uint_as_float(r[2][c])) << 8;
+              v += (long long)__float2int_rn(__uint_as_float(r[1][c])) << 16;
+              v += (long long)__float2int_rn(__uint_as_float(r[0][c])) << 24;
+              hi[k] = v;
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+      if (!ok) continue;
+      const int i = t.i0 + quarter * 32 + lane;
+      if (i < a.M) {
+        // value = (hi + lo 2^-32) 2^-38 2^{Ea + Eb}, E = exponent field - 1022
+        const int ra = t.arow + quarter * 32 + lane, ea = a.aexp[ra];
+        double* crow = a.C + t.coff + (long long)i * a.ci;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const int j = t.j0 + ch * 32 + c;
+          if (j < a.N) {
+            double d = fma((double)lo[c], 2.3283064365386962890625e-10, (double)hi[c]);
+            const int rb = t.brow + ch * 32 + c, eb = a.bexp[rb];
+            const int e = ea + eb - 2 * 1022 - 38;
+            const int hw = __double2hiint(d), ef = (hw >> 20) & 0x7ff;
+            if (max(ea, eb) >= OZ_EXP_INF) {
+              d = oz_not_finite(a, ra, rb, max(ea, eb));
+            } else if (ef != 0) {
+              if (ef + e > 0 && ef + e < 0x7ff)
+                d = __hiloint2double(hw + (e << 20), __double2loint(d));
+              else
+                d = scalbn(d, e);
+            }
+            if (a.alpha != 1.0) d *= a.alpha;
+            double* p = crow + (long long)j * a.cj;
+            *p = a.accumulate ? *p + d : d;
+          }
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+  }
+}
+
+// ------------------------------- host side -------------------------------
+cudaError_t oz_pack(cudaStream_t st, const OzRows& s, __nv_bfloat16* planes, int* rexp) {
+  const int Kp = oz_kpad((long long)s.L1 * s.L2);
+  const dim3 grid((unsigned)((s.total + 63) / 64), (unsigned)((Kp + 63) / 64));
+  cudaError_t e = cudaMemsetAsync(rexp, 0, (size_t)s.total * sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  // lanes along K when K is the unit-stride index, else along the rows
+  if ((s.L2 == 1 ? s.k1 : s.k2) == 1 && s.ri != 1) {
+    oz_rowmax_kernel<true><<<grid, 256, 0, st>>>(s, rexp);
+    oz_slice_kernel<true><<<grid, 256, 0, st>>>(s, rexp, planes, Kp);
+  } else {
+    oz_rowmax_kernel<false><<<grid, 256, 0, st>>>(s, rexp);
+    oz_slice_kernel<false><<<grid, 256, 0, st>>>(s, rexp, planes, Kp);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t oz_multiply(cudaStream_t st, const __nv_bfloat16* pa, const __nv_bfloat16* pb, OzArgs a,
+                        int n_prob) {
+  const int Kp = oz_kpad((long long)a.a.L1 * a.a.L2);
+  a.mt = (a.M + OZ_BM - 1) / OZ_BM;
+  a.nt = (a.N + OZ_BN - 1) / OZ_BN;
+  a.band = 12;
+  a.kstages = Kp / OZ_KB;
+  const long long items = (long long)a.mt * a.nt * n_prob;
+  if (items <= 0 || items > 0x7fffffff) return cudaErrorInvalidValue;
+  a.n_items = (int)items;
+  int dev = 0, nsm = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t sm = (size_t)OZ_STAGES * OZ_STAGE_BYTES + 1024 + 256;
+  raise_smem_limit((const void*)oz_gemm_kernel, sm);
+  oz_gemm_kernel<<<(unsigned)(items < nsm ? items : nsm), OZ_THREADS, sm, st>>>(
+      (const uint8_t*)pa, (const uint8_t*)pb, a);
+  return cudaGetLastError();
+}
+
+// ------------------------------- generic GEMM -------------------------------
+static long long oz_up(long long x, long long m) { return (x + m - 1) / m * m; }
+static size_t oz_row_bytes(long long K) { return (size_t)OZ_S * oz_kpad(K) * 2 + sizeof(int); }
+
+size_t oz_work_bytes(long long M, long long N, long long K, long long nb, bool shared_a, bool shared_b) {
+  const long long mp = oz_up(M, OZ_ROW_PAD), np = oz_up(N, OZ_ROW_PAD);
+  const size_t need = ((shared_a ? mp : mp * nb) + (shared_b ? np : np * nb)) * oz_row_bytes(K);
+  const size_t one = (mp + np) * oz_row_bytes(K);
+  const size_t cap = need < OZ_WS_CAP ? need : OZ_WS_CAP;
+  return (cap > one ? cap : (one < 4 * OZ_WS_CAP ? one : 4 * OZ_WS_CAP)) + 4096;
+}
+
+// The tensor-core form costs about six launches and the slicing; the FP64 pipe does
+// 1.1 TFLOP/s on whole 64 x 64 tiles. At 5e7 operations both take about 60 us.
+static bool oz_worthwhile(double flops) { return flops >= 5e7; }
+
+cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
+  GemmArgs g = g0;
+  if (g.M <= 0 || g.N <= 0 || g.nb <= 0) return cudaSuccess;
+  // batches that are one matrix: the shared operand's problems follow one another
+  if (g.nb > 1 && g.sb == 0 && g.sa == (long long)g.M * g.ai && g.sc == (long long)g.M * g.ci &&
+      (long long)g.M * g.nb < (1ll << 30)) {
+    g.M *= g.nb;
+    g.nb = 1;
+  } else if (g.nb > 1 && g.sa == 0 && g.sb == (long long)g.N * g.bj && g.sc == (long long)g.N * g.cj &&
+             (long long)g.N * g.nb < (1ll << 30)) {
+    g.N *= g.nb;
+    g.nb = 1;
+  }
+  const long long K = (long long)g.L1 * g.L2;
+  const double flops = 2.0 * g.M * g.N * (double)K * g.nb;
+  if (!w.mem || !oz_worthwhile(flops) || K > (1 << 21)) return launch_gemm_fp64(st, g0);
+  // the operand on the 128-row side: the one that wastes less of the tiles
+  auto tiles = [](long long m, long long n) {
+    return oz_up(m, OZ_BM) * oz_up(n, OZ_BN);
+  };
+  const bool swap = tiles(g.N, g.M) < tiles(g.M, g.N);
+  const int m = swap ? g.N : g.M, n = swap ? g.M : g.N;
+  const double *pm = swap ? g.Bm : g.A, *pn = swap ? g.A : g.Bm;
+  const long long rm = swap ? g.bj : g.ai, m1 = swap ? g.b1 : g.a1, m2 = swap ? g.b2 : g.a2,
+                  zm = swap ? g.sb : g.sa;
+  const long long rn = swap ? g.ai : g.bj, n1 = swap ? g.a1 : g.b1, n2 = swap ? g.a2 : g.b2,
+                  zn = swap ? g.sa : g.sb;
+  const long long cm = swap ? g.cj : g.ci, cn = swap ? g.ci : g.cj;
+  const bool share_m = g.nb > 1 && zm == 0, share_n = g.nb > 1 && zn == 0;
+  const size_t rb = oz_row_bytes(K);
+  const size_t avail = w.bytes > 2048 ? w.bytes - 2048 : 0;
+  const long long np = oz_up(n, OZ_ROW_PAD);
+  long long mb = oz_up(m, OZ_ROW_PAD);  // rows of the 128-row side at a time
+  // problems at a time
+  const size_t fixed = ((share_m ? mb : 0) + (share_n ? np : 0)) * rb;
+  const size_t per = ((share_m ? 0 : mb) + (share_n ? 0 : np)) * rb;
+  long long zb = fixed + per <= avail ? (long long)((avail - fixed) / per) : 0;
+  if (zb > g.nb) zb = g.nb;
+  if (zb < 1) {
+    // not even one problem: a problem's rows in blocks
+    const long long rows = avail / rb > (size_t)np ? (long long)(avail / rb) - np : 0;
+    mb = rows / OZ_ROW_PAD * OZ_ROW_PAD;
+    if (mb < OZ_ROW_PAD) return launch_gemm_fp64(st, g0);
+    zb = 1;
+  }
+  uint8_t* base = (uint8_t*)w.mem;
+  const long long m_rows = mb * (share_m ? 1 : zb), n_rows = np * (share_n ? 1 : zb);
+  __nv_bfloat16* plm = (__nv_bfloat16*)base;
+  __nv_bfloat16* pln = (__nv_bfloat16*)(base + oz_up(oz_plane_bytes(m_rows, K), 256));
+  int* xm = (int*)((uint8_t*)pln + oz_up(oz_plane_bytes(n_rows, K), 256));
+  int* xn = xm + m_rows;
+  cudaError_t e;
+  for (long long z0 = 0; z0 < g.nb; z0 += zb) {
+    const int nz = (int)(g.nb - z0 < zb ? g.nb - z0 : zb);
+    OzArgs a;
+    a.b = oz_rows(pn + z0 * zn, share_n ? 1 : nz, n, (int)np, rn, zn, g.L1, g.L2, n1, n2);
+    if (z0 == 0 || !share_n)
+      if ((e = oz_pack(st, a.b, pln, xn)) != cudaSuccess) return e;
+    for (long long r0 = 0; r0 < m; r0 += mb) {
+      const int mr = (int)(m - r0 < mb ? m - r0 : mb);
+      a.a = oz_rows(pm + z0 * zm + r0 * rm, share_m ? 1 : nz, mr, (int)(mb < m ? oz_up(mr, OZ_ROW_PAD) : mb),
+                    rm, zm, g.L1, g.L2, m1, m2);
+      if (z0 == 0 || !share_m || mb < m)
+        if ((e = oz_pack(st, a.a, plm, xm)) != cudaSuccess) return e;
+      a.aexp = xm;
+      a.bexp = xn;
+      a.status = w.status;
+      a.C = g.C + z0 * g.sc + r0 * cm;
+      a.ci = cm;
+      a.cj = cn;
+      a.sc = g.sc;
+      a.M = mr;
+      a.N = n;
+      a.pairs = nullptr;
+      a.p0 = 0;
+      a.pstep = 1;
+      a.arow0 = a.brow0 = 0;
+      a.astep = share_m ? 0 : a.a.rpad;
+      a.bstep = share_n ? 0 : a.b.rpad;
+      a.alpha = g.alpha;
+      a.accumulate = g.accumulate;
+      if ((e = oz_multiply(st, plm, pln, a, nz)) != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
+}  // namespace dsrg
