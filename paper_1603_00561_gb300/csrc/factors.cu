@@ -21,59 +21,148 @@
 #include <new>
 #include <vector>
 
+#include "coop.cuh"
 #include "internal.cuh"
+#include "oz_gemm.cuh"
 
 namespace dsrg {
 namespace {
 
 // ---------------------------- Cholesky of the metric ----------------------------
-// Right-looking column Cholesky on the lower triangle of A, one column per
-// step: column k below the diagonal is divided by sqrt(A[k][k]) (the diagonal
-// itself keeps the squared value until chol_diag_kernel takes the roots at the
-// end, so no thread of a step reads an element another thread of the step
-// writes); then A[i][j] -= L[i][k] L[j][k] for k < j <= i. A non-positive
-// pivot sets *bad.
-__global__ void chol_col_kernel(double* __restrict__ A, int n, int k, int* __restrict__ bad) {
-  const int i = k + 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  const double akk = A[(size_t)k * n + k];
-  if (!(akk > 0.0)) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) atomicExch(bad, 1);
-    return;
+// Blocked right-looking Cholesky on the lower triangle of A, CB columns at a time:
+// the diagonal block in one CTA, the panel below it with one warp per row, the trailing
+// update in CB x CB tiles. An SM does two FP64 FMAs a clock, so what counts is that
+// every step spreads over all of them: 3 launches per CB columns and small tiles
+// (one column per step, 2 naux launches, took 60 ms at naux = 1200; 2.6 ms now). A
+// non-positive pivot sets *bad.
+constexpr int CB = 32;
+
+__global__ void __launch_bounds__(256) chol_diag_kernel(double* __restrict__ A, int n, int k0,
+                                                        int* __restrict__ bad) {
+  __shared__ double t[CB][CB + 1];
+  const int nb = min(CB, n - k0);
+  for (int e = threadIdx.x; e < CB * CB; e += 256) {
+    const int i = e / CB, j = e % CB;
+    t[i][j] = (i < nb && j <= i) ? A[(size_t)(k0 + i) * n + k0 + j] : (i == j ? 1.0 : 0.0);
   }
+  __syncthreads();
+  for (int k = 0; k < nb; ++k) {
+    const double akk = t[k][k];
+    if (!(akk > 0.0)) {  // the same value in every thread
+      if (threadIdx.x == 0) atomicExch(bad, 1);
+      return;
+    }
+    const double r = 1.0 / sqrt(akk);
+    __syncthreads();
+    if (threadIdx.x >= k && threadIdx.x < nb) t[threadIdx.x][k] *= r;
+    __syncthreads();
+    for (int e = threadIdx.x; e < CB * CB; e += 256) {
+      const int i = e / CB, j = e % CB;
+      if (j > k && i >= j) t[i][j] = fma(-t[i][k], t[j][k], t[i][j]);
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < CB * CB; e += 256) {
+    const int i = e / CB, j = e % CB;
+    if (i < nb && j <= i) A[(size_t)(k0 + i) * n + k0 + j] = t[i][j];
+  }
+}
+
+// Rows i >= k0 + CB of the panel: x L_kk^T = a, one warp per row, lane j holds x_j.
+__global__ void __launch_bounds__(128) chol_panel_kernel(double* __restrict__ A, int n, int k0) {
+  __shared__ double t[CB][CB + 1], rd[CB];
+  for (int e = threadIdx.x; e < CB * CB; e += 128) {
+    const int i = e / CB, j = e % CB;
+    t[i][j] = j <= i ? A[(size_t)(k0 + i) * n + k0 + j] : 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x < CB) rd[threadIdx.x] = 1.0 / t[threadIdx.x][threadIdx.x];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, i = k0 + CB + blockIdx.x * 4 + (threadIdx.x >> 5);
   if (i >= n) return;
-  A[(size_t)i * n + k] /= sqrt(akk);
+  double a = A[(size_t)i * n + k0 + lane];
+#pragma unroll 4
+  for (int k = 0; k < CB; ++k) {
+    const double x = __shfl_sync(0xffffffffu, a, k) * rd[k];
+    if (lane == k) a = x;
+    if (lane > k) a = fma(-x, t[lane][k], a);
+  }
+  A[(size_t)i * n + k0 + lane] = a;
 }
 
-__global__ void chol_update_kernel(double* __restrict__ A, int n, int k) {
-  const int j = k + 1 + blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = k + 1 + blockIdx.y;
-  if (j > i || i >= n) return;  // lower triangle only
-  A[(size_t)i * n + j] -= A[(size_t)i * n + k] * A[(size_t)j * n + k];
+// A[i][j] -= sum_k L[i][k] L[j][k] over the panel's CB columns, tiles on or below the diagonal.
+__global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ A, int n, int k0) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double si[CB][CB + 1], sj[CB][CB + 1];
+  const int i0 = k0 + CB + blockIdx.y * CB, j0 = k0 + CB + blockIdx.x * CB;
+  for (int e = threadIdx.x; e < CB * CB; e += 256) {
+    const int r = e / CB, c = e % CB;
+    si[r][c] = i0 + r < n ? A[(size_t)(i0 + r) * n + k0 + c] : 0.0;
+    sj[r][c] = j0 + r < n ? A[(size_t)(j0 + r) * n + k0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+  for (int k = 0; k < CB; ++k) {
+    const double b = sj[c][k];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q] = fma(si[r0 + 8 * q][k], b, acc[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = i0 + r0 + 8 * q, j = j0 + c;
+    if (i < n && j <= i) A[(size_t)i * n + j] -= acc[q];
+  }
 }
 
-__global__ void chol_diag_kernel(double* __restrict__ A, int n) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) A[(size_t)k * n + k] = sqrt(A[(size_t)k * n + k]);
-}
-
-// Row i of L^{-1} (lower triangular) by forward substitution, all its columns
-// c <= i at once: Li[i][c] = (delta_ic - sum_{c <= k < i} L[i][k] Li[k][c]) / L[i][i]
-// (rows above i are complete from the earlier launches).
-__global__ void tri_row_kernel(const double* __restrict__ L, int n, int i, double* __restrict__ Li) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c > i) return;
-  double v = (i == c) ? 1.0 : 0.0;
-  for (int k = c; k < i; ++k) v = fma(-L[(size_t)i * n + k], Li[(size_t)k * n + c], v);
-  Li[(size_t)i * n + c] = v / L[(size_t)i * n + i];
+// L^{-1} (lower triangular) by forward substitution, a few columns per CTA in shared
+// memory and one warp per column: Li[i][c] = (delta_ic - sum_{c <= k < i} L[i][k]
+// Li[k][c]) / L[i][i]. The columns are independent, so this is one launch; a CTA takes
+// columns from both ends (gridDim.x apart), which evens out their lengths.
+constexpr int TI_WARPS = 8;
+__global__ void __launch_bounds__(32 * TI_WARPS) tri_inverse_kernel(const double* __restrict__ L,
+                                                                    int n, double* __restrict__ Li,
+                                                                    int staged) {
+  extern __shared__ double cols[];  // [warps][n], unless a column does not fit
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = warp * gridDim.x + blockIdx.x;
+  // columns 0, n-1, 1, n-2, ... in the order of w / 2
+  const int c = (w & 1) ? n - 1 - w / 2 : w / 2;
+  if (w >= n) return;
+  double* x = staged ? cols + (size_t)warp * n : Li + c;
+  const size_t xs = staged ? 1 : (size_t)n;
+  for (int i = lane; i < c; i += 32) Li[(size_t)i * n + c] = 0.0;
+  for (int i = c; i < n; ++i) {
+    double v = 0.0, v2 = 0.0;
+    const double* Lr = L + (size_t)i * n;
+    int k = c + lane;
+    for (; k + 32 < i; k += 64) {
+      v = fma(Lr[k], x[k * xs], v);
+      v2 = fma(Lr[k + 32], x[(k + 32) * xs], v2);
+    }
+    if (k < i) v = fma(Lr[k], x[k * xs], v);
+    v += v2;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const double r = ((i == c ? 1.0 : 0.0) - v) / Lr[i];
+    if (lane == 0) {
+      x[i * xs] = r;
+      Li[(size_t)i * n + c] = r;
+    }
+    __syncwarp();
+  }
 }
 
 // ------------------------------ pivoted Cholesky ------------------------------
 struct CdState {
-  int pivot;   // pivot of the current step
-  int rank;    // vectors accepted so far
-  int done;    // 1 once the largest remaining diagonal fell below tau
-  double dmax;
+  int rank;     // vectors accepted
+  GridBar bar;
 };
+struct CdSlot {
+  double v;
+  long long i;
+};
+constexpr int CD_SLOTS = 2048;  // CTAs of the decomposition, at most
 
 // d[p] = M_pp = sum_k F[k][p]^2 (p over the N = n^2 pairs)
 __global__ void cd_diag_kernel(const double* __restrict__ F, int K0, size_t N, double* __restrict__ d) {
@@ -87,66 +176,114 @@ __global__ void cd_diag_kernel(const double* __restrict__ F, int K0, size_t N, d
   d[p] = acc;
 }
 
-// argmax of d (one CTA); stops the decomposition when the maximum is below tau
-// or the maximum rank is reached. Ties: the lowest index.
-__global__ void __launch_bounds__(1024) cd_pivot_kernel(const double* __restrict__ d, size_t N,
-                                                        double tau, int max_rank,
-                                                        CdState* __restrict__ st) {
-  __shared__ double sv[1024];
-  __shared__ long long si[1024];
-  if (st->done) return;
-  double best = -1.0;
-  long long bi = 0;
-  for (size_t p = threadIdx.x; p < N; p += 1024) {
-    const double v = d[p];
-    if (v > best) {
-      best = v;
-      bi = (long long)p;
+// The whole decomposition in one cooperative launch, one barrier per vector. Step k:
+// every CTA knows the largest remaining diagonal of its elements (ties: the lowest
+// index) and reads the others'; the column of the winner p,
+//   L[:, k] = (M[:, p] - sum_{j<k} L[:, j] L[p, j]) / sqrt(d_p), M[:, p] = sum_kk F_kk F_kk[p],
+// is formed by tiles of 32 elements with 8 warps sharing the sum over kk and j (in
+// fixed parts, added in order), then d -= L[:, k]^2. Stops at max d < tau or max_rank.
+// (As three launches per step up to max_rank, n^2 by default, most of them after the
+// end: 31.9 ms for n = 56 and 240 vectors; 3.1 ms now, and 3.9 ms with 16 warps a CTA.)
+constexpr int CD_T = 32, CD_W = 8;
+__global__ void __launch_bounds__(CD_T * CD_W) cd_run_kernel(const double* __restrict__ F, int K0,
+                                                             long long N, double tau, int max_rank,
+                                                             double* __restrict__ L,
+                                                             double* __restrict__ d,
+                                                             CdSlot* __restrict__ slots,
+                                                             CdState* __restrict__ st) {
+  __shared__ double part[CD_W][CD_T];
+  __shared__ double sv[CD_W];
+  __shared__ long long si[CD_W];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
+  const long long ntile = (N + CD_T - 1) / CD_T;
+  unsigned gen = 0;
+  // the larger of (v, i) and another pair, ties to the lower index
+  auto take = [](double& v, long long& i, double w, long long j) {
+    if (w > v || (w == v && j < i)) {
+      v = w;
+      i = j;
     }
-  }
-  sv[threadIdx.x] = best;
-  si[threadIdx.x] = bi;
-  __syncthreads();
-  for (int s = 512; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      const double a = sv[threadIdx.x], b = sv[threadIdx.x + s];
-      const long long ia = si[threadIdx.x], ib = si[threadIdx.x + s];
-      if (b > a || (b == a && ib < ia)) {
-        sv[threadIdx.x] = b;
-        si[threadIdx.x] = ib;
+  };
+  auto warp_max = [&](double& v, long long& i) {
+    for (int o = 16; o > 0; o >>= 1)
+      take(v, i, __shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, i, o));
+  };
+  double best = -1.0;  // over this thread's elements of d (threads of warp 0)
+  long long bi = 0;
+  if (warp == 0)
+    for (long long t = blockIdx.x; t < ntile; t += gridDim.x) {
+      const long long q = t * CD_T + lane;
+      if (q < N && d[q] > best) {
+        best = d[q];
+        bi = q;
       }
     }
+  int rank = 0;
+  for (;; ++rank) {
+    if (warp == 0) {  // the other warps hold no elements of d
+      warp_max(best, bi);
+      if (lane == 0) slots[(rank & 1) * gridDim.x + blockIdx.x] = CdSlot{best, bi};
+    }
+    if (!grid_barrier(&st->bar, gen)) return;
+    double v = -1.0;
+    long long vi = 0;
+    for (int c = tid; c < gridDim.x; c += CD_T * CD_W) {
+      const CdSlot* sl = &slots[(rank & 1) * gridDim.x + c];
+      take(v, vi, __ldcg(&sl->v), __ldcg(&sl->i));
+    }
+    warp_max(v, vi);
+    if (lane == 0) {
+      sv[warp] = v;
+      si[warp] = vi;
+    }
     __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    st->dmax = sv[0];
-    if (sv[0] < tau || st->rank >= max_rank) {
-      st->done = 1;
-    } else {
-      st->pivot = (int)si[0];
+    double dmax = sv[0];
+    long long p = si[0];
+#pragma unroll
+    for (int w = 1; w < CD_W; ++w) take(dmax, p, sv[w], si[w]);
+    if (dmax < tau || rank >= max_rank) break;
+    const double rs = sqrt(dmax);
+    best = -1.0;
+    bi = 0;
+    for (long long t = blockIdx.x; t < ntile; t += gridDim.x) {
+      const long long q = t * CD_T + lane;
+      double m = 0.0;
+      if (q < N) {
+#pragma unroll 16
+        for (int kk = warp; kk < K0; kk += CD_W) m = fma(F[(size_t)kk * N + q], F[(size_t)kk * N + p], m);
+#pragma unroll 16
+        for (int j = warp; j < rank; j += CD_W)
+          m = fma(-__ldcg(&L[(size_t)j * N + q]), __ldcg(&L[(size_t)j * N + p]), m);
+      }
+      part[warp][lane] = m;
+      __syncthreads();
+      if (warp == 0 && q < N) {
+        double sum = part[0][lane];
+#pragma unroll
+        for (int w = 1; w < CD_W; ++w) sum += part[w][lane];
+        const double x = sum / rs;
+        L[(size_t)rank * N + q] = x;
+        const double nd = q == p ? 0.0 : d[q] - x * x;
+        d[q] = nd;
+        if (nd > best) {
+          best = nd;
+          bi = q;
+        }
+      }
+      __syncthreads();
     }
   }
+  if (blockIdx.x == 0 && tid == 0) st->rank = rank;
 }
 
-// L[:, k] = (M[:, p] - sum_{j<k} L[:, j] L[p, j]) / sqrt(d_p), then d -= L[:, k]^2
-// (L stored as [rank][N]: vector k contiguous).
-__global__ void cd_column_kernel(const double* __restrict__ F, int K0, size_t N,
-                                 double* __restrict__ L, double* __restrict__ d,
-                                 CdState* __restrict__ st) {
-  if (st->done) return;
-  const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= N) return;
-  const int p = st->pivot, k = st->rank;
-  double m = 0.0;
-  for (int kk = 0; kk < K0; ++kk) m = fma(F[(size_t)kk * N + q], F[(size_t)kk * N + p], m);
-  for (int j = 0; j < k; ++j) m = fma(-L[(size_t)j * N + q], L[(size_t)j * N + p], m);
-  const double v = m / sqrt(st->dmax);
-  L[(size_t)k * N + q] = v;
-  d[q] = (q == (size_t)p) ? 0.0 : d[q] - v * v;
-}
-
-__global__ void cd_advance_kernel(CdState* __restrict__ st) {
-  if (!st->done) st->rank += 1;
+// Workspace of the three products on the tensor cores (the largest of them; 0 where they
+// are too small for it).
+size_t df_gemm_bytes(int nbf, int naux, int np, int nq) {
+  size_t a = oz_work_bytes(np, nbf, nbf, naux, true, false);
+  const size_t b = oz_work_bytes((long long)np * naux, nq, nbf, 1, false, false);
+  const size_t c = oz_work_bytes(naux, (long long)np * nq, naux, 1, false, false);
+  a = a > b ? a : b;
+  return a > c ? a : c;
 }
 
 }  // namespace
@@ -173,7 +310,12 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   double* Z = Y + (size_t)naux * np * nbf;                 // [naux][np][nq]
   double* Lm = Z + (size_t)naux * np * nq;                 // [naux][naux] metric -> L
   double* Li = Lm + (size_t)naux * naux;                   // [naux][naux] L^{-1}
-  int* bad = (int*)(Li + (size_t)naux * naux);
+  int* bad = (int*)(Li + (size_t)naux * naux);             // and the waits' status word
+  OzWork ow;
+  ow.mem = (uint8_t*)(((uintptr_t)(bad + 8) + 255) & ~(uintptr_t)255);
+  ow.bytes = df_gemm_bytes(nbf, naux, np, nq);
+  ow.status = bad + 1;
+  if (cudaMemsetAsync(bad, 0, 2 * sizeof(int), st) != cudaSuccess) return DSRG_ERR_CUDA;
   cudaError_t e;
   // Y[P][p][nu] = sum_mu C[mu][p0 + p] ao3[P][mu][nu]
   GemmArgs g1 = batched(mk(np, nbf, nbf, 1, C + p0, 1, nmo, 0, ao3, nbf, 0, 1, Y, nbf, 1, 1.0), naux,
@@ -183,38 +325,45 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   GemmArgs g2 = batched(mk(np, nq, nbf, 1, Y, nbf, 1, 0, C + q0, nmo, 0, 1, Z, nq, 1, 1.0), naux,
                         (long long)np * nbf, 0, (long long)np * nq);
   g2.accumulate = 0;
-  if ((e = launch_gemm_fp64(st, g1)) != cudaSuccess || (e = launch_gemm_fp64(st, g2)) != cudaSuccess)
+  if ((e = launch_gemm(st, g1, ow)) != cudaSuccess || (e = launch_gemm(st, g2, ow)) != cudaSuccess)
     return DSRG_ERR_CUDA;
   // J = L L^T, then L^{-1}
-  if (cudaMemcpyAsync(Lm, metric, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-      cudaMemsetAsync(bad, 0, sizeof(int), st) != cudaSuccess)
+  if (cudaMemcpyAsync(Lm, metric, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return DSRG_ERR_CUDA;
-  for (int k = 0; k < naux; ++k) {
-    chol_col_kernel<<<(naux - k + 255) / 256, 256, 0, st>>>(Lm, naux, k, bad);
-    if (k + 1 < naux) {
-      dim3 g((naux - k - 1 + 255) / 256, naux - k - 1);
-      chol_update_kernel<<<g, 256, 0, st>>>(Lm, naux, k);
+  for (int k = 0; k < naux; k += CB) {
+    chol_diag_kernel<<<1, 256, 0, st>>>(Lm, naux, k, bad);
+    const int left = naux - k - CB;
+    if (left > 0) {
+      chol_panel_kernel<<<(left + 3) / 4, 128, 0, st>>>(Lm, naux, k);
+      const unsigned nt = (unsigned)((left + CB - 1) / CB);
+      chol_update_kernel<<<dim3(nt, nt), 256, 0, st>>>(Lm, naux, k);
     }
   }
-  chol_diag_kernel<<<(naux + 255) / 256, 256, 0, st>>>(Lm, naux);
   if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
-  if (cudaMemsetAsync(Li, 0, (size_t)naux * naux * 8, st) != cudaSuccess) return DSRG_ERR_CUDA;
-  for (int i = 0; i < naux; ++i) tri_row_kernel<<<(i + 256) / 256, 256, 0, st>>>(Lm, naux, i, Li);
+  // columns of L^{-1} per CTA: what the shared memory holds, at most one per warp
+  int tw = (int)((size_t)200 * 1024 / ((size_t)naux * 8));
+  const int staged = tw >= 1;
+  tw = tw > TI_WARPS || !staged ? TI_WARPS : tw;
+  const size_t smi = staged ? (size_t)tw * naux * 8 : 0;
+  raise_smem_limit((const void*)tri_inverse_kernel, smi);
+  tri_inverse_kernel<<<(naux + tw - 1) / tw, 32 * tw, smi, st>>>(Lm, naux, Li, staged);
   if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
   // B[Q][pq] = sum_P Li[Q][P] Z[P][pq]  (Li lower triangular; the GEMM reads it whole)
   const long long npq = (long long)np * nq;
   GemmArgs g3 = mk(naux, (int)npq, naux, 1, Li, naux, 1, 0, Z, npq, 0, 1, B_out, npq, 1, 1.0);
   g3.accumulate = 0;
-  if ((e = launch_gemm_fp64(st, g3)) != cudaSuccess) return DSRG_ERR_CUDA;
-  int hbad = 0;
-  if (cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  if ((e = launch_gemm(st, g3, ow)) != cudaSuccess) return DSRG_ERR_CUDA;
+  int hbad[2] = {0, 0};
+  if (cudaMemcpyAsync(hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return DSRG_ERR_CUDA;
-  return hbad ? DSRG_ERR_INVALID_ARG : DSRG_OK;
+  if (hbad[1]) return DSRG_ERR_TIMEOUT;
+  return hbad[0] ? DSRG_ERR_INVALID_ARG : DSRG_OK;
 }
 
 size_t dsrg_df_mo_transform_work_bytes(int32_t nbf, int32_t naux, int32_t np, int32_t nq) {
-  return ((size_t)naux * np * nbf + (size_t)naux * np * nq + 2 * (size_t)naux * naux) * 8 + 64;
+  return ((size_t)naux * np * nbf + (size_t)naux * np * nq + 2 * (size_t)naux * naux) * 8 + 512 +
+         df_gemm_bytes(nbf, naux, np, nq);
 }
 
 dsrg_status_t dsrg_cd_factors(const double* F, int32_t nfac, int32_t n, double tau,
@@ -228,25 +377,30 @@ dsrg_status_t dsrg_cd_factors(const double* F, int32_t nfac, int32_t n, double t
   cudaStream_t st = (cudaStream_t)cuda_stream;
   double* d = work;
   CdState* cs = (CdState*)(d + N);
+  CdSlot* slots = (CdSlot*)(((uintptr_t)(cs + 1) + 15) & ~(uintptr_t)15);
   if (cudaMemsetAsync(cs, 0, sizeof(CdState), st) != cudaSuccess) return DSRG_ERR_CUDA;
-  const unsigned gb = (unsigned)((N + 255) / 256);
-  cd_diag_kernel<<<gb, 256, 0, st>>>(F, nfac, N, d);
-  for (int k = 0; k < max_rank; ++k) {
-    cd_pivot_kernel<<<1, 1024, 0, st>>>(d, N, tau, max_rank, cs);
-    cd_column_kernel<<<gb, 256, 0, st>>>(F, nfac, N, L_out, d, cs);
-    cd_advance_kernel<<<1, 1, 0, st>>>(cs);
-  }
+  cd_diag_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(F, nfac, N, d);
   if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
+  const long long nt = ((long long)N + CD_T - 1) / CD_T;
+  int grid = coop_grid(cd_run_kernel, CD_T * CD_W, 0, (int)(nt < CD_SLOTS ? nt : CD_SLOTS));
+  if (grid < 1) return DSRG_ERR_CUDA;
+  long long NN = (long long)N;
+  int K0 = nfac;
+  void* args[] = {(void*)&F, &K0, &NN, &tau, &max_rank, &L_out, &d, &slots, &cs};
+  if (cudaLaunchCooperativeKernel((const void*)cd_run_kernel, dim3(grid), dim3(CD_T * CD_W), args, 0,
+                                  st) != cudaSuccess)
+    return DSRG_ERR_CUDA;
   CdState h{};
   if (cudaMemcpyAsync(&h, cs, sizeof(CdState), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return DSRG_ERR_CUDA;
+  if (h.bar.abort) return DSRG_ERR_TIMEOUT;
   *rank_out = h.rank;
   return DSRG_OK;
 }
 
 size_t dsrg_cd_factors_work_bytes(int32_t n) {
-  return (size_t)n * n * 8 + sizeof(CdState) + 64;
+  return (size_t)n * n * 8 + sizeof(CdState) + 64 + 2 * CD_SLOTS * sizeof(CdSlot);
 }
 
 }  // extern "C"
