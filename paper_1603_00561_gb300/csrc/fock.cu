@@ -26,7 +26,17 @@
 #include <numeric>
 #include <vector>
 
+#include "coop.cuh"
 #include "internal.cuh"
+#include "oz_gemm.cuh"
+
+namespace dsrg {
+struct JacState {
+  GridBar bar;
+  int sweeps;  // of the slowest block so far
+  int wait;    // status word of the products' bounded waits
+};
+}  // namespace dsrg
 
 struct dsrg_sc_plan {
   dsrg::Sizes z{};
@@ -37,18 +47,21 @@ struct dsrg_sc_plan {
   size_t ws_bytes = 0;
   double *w = nullptr;      // [naux]
   double *J = nullptr;      // [n][n]
-  double *K = nullptr;      // [n][n]
+  double *K = nullptr;      // [nk][n][n]
   double *X = nullptr;      // [naux][n][nH]
   double *f = nullptr;      // [n][n]
   double *U = nullptr;      // [n][n]
   double *T = nullptr;      // [n][n]
   double *A = nullptr;      // [mmax][mmax] Jacobi work matrix
   double *V = nullptr;      // [mmax][mmax] Jacobi eigenvectors
-  double2 *cs = nullptr;    // [mmax/2 + 1] rotation (c, s) per pair
-  double *off = nullptr;    // [2] off-diagonal and total squared norms
+  double *A2 = nullptr;     // [mmax][mmax] its other copy
+  double *diag = nullptr;   // [mmax] eigenvalues in matrix order
+  double2 *slots = nullptr; // [JAC_SLOTS] partial norms
+  dsrg::JacState *jac = nullptr;
+  int nk = 1;               // partial exchange matrices (parts of the sum over Q)
+  dsrg::OzWork oz;          // workspace of the tensor-core products
   double *Bhp = nullptr;    // [naux][nH][nP] gathered hole x particle factors
   double *Bt = nullptr;     // [naux][nH][nP] after the particle rotation
-  int *perm = nullptr;      // [mmax]
   double *L3t = nullptr;    // [(2 nA)^6] intermediate of the lambda3 rotation
   int mmax = 0;
   int sweeps_last = 0;
@@ -118,15 +131,21 @@ __global__ void fock_x_kernel(const double* __restrict__ B, const double* __rest
   X[k] = v;
 }
 
-// f = h + J - K / 2, symmetrised (the two halves round differently only in K)
+// f = h + J - K / 2 (K in nk parts), symmetrised (the two halves round differently only in K)
 __global__ void fock_sum_kernel(const double* __restrict__ h, const double* __restrict__ J,
-                                const double* __restrict__ K, int n, double* __restrict__ f) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= (size_t)n * n) return;
+                                const double* __restrict__ K, int nk, int n,
+                                double* __restrict__ f) {
+  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nn = (size_t)n * n;
+  if (k >= nn) return;
   const int p = (int)(k / n), q = (int)(k % n);
   const size_t kt = (size_t)q * n + p;
-  const double a = fma(-0.5, K[k], h[k] + J[k]);
-  const double b = fma(-0.5, K[kt], h[kt] + J[kt]);
+  double ka = 0.0, kb = 0.0;
+  for (int z = 0; z < nk; ++z) {
+    ka += K[z * nn + k];
+    kb += K[z * nn + kt];
+  }
+  const double a = fma(-0.5, ka, h[k] + J[k]);
+  const double b = fma(-0.5, kb, h[kt] + J[kt]);
   f[k] = 0.5 * (a + b);
 }
 
@@ -146,106 +165,192 @@ __global__ void jac_copy_kernel(const double* __restrict__ f, int n, int lo, int
   V[k] = (i == j) ? 1.0 : 0.0;
 }
 
-// (c, s) of every pair of step t: the 2 x 2 symmetric Schur decomposition.
-__global__ void jac_params_kernel(const double* __restrict__ A, int m, int mp, int t,
-                                  double2* __restrict__ cs) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= mp / 2) return;
-  const int p = rr_slot(k, t, mp), q = rr_slot(mp - 1 - k, t, mp);
-  double c = 1.0, s = 0.0;
-  if (p < m && q < m) {
-    const double apq = A[(size_t)p * m + q];
-    if (apq != 0.0) {
-      const double app = A[(size_t)p * m + p], aqq = A[(size_t)q * m + q];
-      const double tau = (aqq - app) / (2.0 * apq);
-      const double tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-      c = 1.0 / sqrt(1.0 + tt * tt);
-      s = tt * c;
+// The whole diagonalisation in one cooperative launch, one barrier per step (a step is
+// 2 us of FP64 work at m = 372; as three launches per step, 11 000 in all, it was the
+// launches that took the 90 ms: 20.6 ms of it now). A tile is 16 x 16 pairs of pairs: with
+// the (c, s) of its 32 pairs, formed in the CTA from the current diagonal blocks, each
+// thread turns one 2 x 2 block A[P][R] -> J_P^T A[P][R] J_R from one copy of A into the
+// other, so no CTA waits for another within a step; the same CTA turns 32 rows of V by
+// its 16 column pairs in place.
+// The angle comes from FP32 and one Newton-Raphson step (46 bits: what it leaves of
+// A[p][q] is below the stopping threshold); c^2 + s^2 = 1 holds to FP64.
+constexpr int JT = 16;
+constexpr int JAC_SLOTS = 2048;  // CTAs, at most
+
+__device__ __forceinline__ double2 jac_rotation(double app, double aqq, double apq) {
+  if (apq == 0.0) return make_double2(1.0, 0.0);
+  // tan of the angle, |t| <= 1; scaled so that the FP32 quotient neither under- nor overflows
+  const double num = aqq - app, den = 2.0 * apq;
+  const double sc = fmax(fabs(num), fabs(den));
+  const int e = ((__double2hiint(sc) >> 20) & 0x7ff) - 1023;
+  const double f = __hiloint2double((1023 - (e < -1000 ? -1000 : (e > 1000 ? 1000 : e))) << 20, 0);
+  const double nf = num * f, df = den * f, h = 0.5 * df;
+  const float tau = (float)nf / (float)df;
+  float tf = 1.0f / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+  if (tau < 0.0f) tf = -tf;
+  // one Newton-Raphson step on h t^2 + nf t - h = 0 (slope |nf + df t| >= 1)
+  double t = (double)tf;
+  const float slope = (float)fma(df, t, nf);
+  t = fma(-fma(fma(h, t, nf), t, -h), (double)(1.0f / slope), t);
+  const double w = fma(t, t, 1.0);
+  double c = (double)rsqrtf((float)w);
+  c = c * fma(-0.5 * w * c, c, 1.5);
+  c = c * fma(-0.5 * w * c, c, 1.5);
+  return make_double2(c, t * c);
+}
+
+__global__ void __launch_bounds__(JT * JT) jac_run_kernel(double* __restrict__ A0,
+                                                          double* __restrict__ A1,
+                                                          double* __restrict__ V, int m, int mp,
+                                                          int max_sweeps, double2* __restrict__ slots,
+                                                          double* __restrict__ diag,
+                                                          JacState* __restrict__ st) {
+  __shared__ double2 rot[2][JT];
+  __shared__ double sh0[JT * JT], sh1[JT * JT];
+  const int K = mp / 2, nt = (K + JT - 1) / JT, tid = threadIdx.x;
+  const int tx = tid % JT, ty = tid / JT;
+  unsigned gen = 0;
+  double *Ac = A0, *An = A1;
+  int sweep = 0;
+  for (;; ++sweep) {
+    // off-diagonal and whole squared norm, in a fixed order
+    double o = 0.0, w = 0.0;
+    for (size_t k = (size_t)blockIdx.x * (JT * JT) + tid; k < (size_t)m * m; k += (size_t)gridDim.x * JT * JT) {
+      const double x = __ldcg(&Ac[k]);
+      w = fma(x, x, w);
+      if (k / m != k % m) o = fma(x, x, o);
     }
-  }
-  cs[k] = make_double2(c, s);
-}
-
-// rows p, q of A <- J^T A (all pairs of the step at once; they are disjoint)
-__global__ void jac_rows_kernel(double* __restrict__ A, int m, int mp, int t,
-                                const double2* __restrict__ cs) {
-  const int k = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
-  const int p = rr_slot(k, t, mp), q = rr_slot(mp - 1 - k, t, mp);
-  if (p >= m || q >= m) return;
-  const double c = cs[k].x, s = cs[k].y;
-  if (s == 0.0) return;
-  const double ap = A[(size_t)p * m + j], aq = A[(size_t)q * m + j];
-  A[(size_t)p * m + j] = c * ap - s * aq;
-  A[(size_t)q * m + j] = s * ap + c * aq;
-}
-
-// columns p, q of A and of V <- (.) J
-__global__ void jac_cols_kernel(double* __restrict__ A, double* __restrict__ V, int m, int mp,
-                                int t, const double2* __restrict__ cs) {
-  const int k = blockIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
-  const int p = rr_slot(k, t, mp), q = rr_slot(mp - 1 - k, t, mp);
-  if (p >= m || q >= m) return;
-  const double c = cs[k].x, s = cs[k].y;
-  if (s == 0.0) return;
-  double ap = A[(size_t)i * m + p], aq = A[(size_t)i * m + q];
-  A[(size_t)i * m + p] = c * ap - s * aq;
-  A[(size_t)i * m + q] = s * ap + c * aq;
-  ap = V[(size_t)i * m + p];
-  aq = V[(size_t)i * m + q];
-  V[(size_t)i * m + p] = c * ap - s * aq;
-  V[(size_t)i * m + q] = s * ap + c * aq;
-}
-
-// off[0] = sum_{i != j} A_ij^2, off[1] = sum A_ij^2 (one CTA)
-__global__ void __launch_bounds__(256) jac_norm_kernel(const double* __restrict__ A, int m,
-                                                       double* __restrict__ off) {
-  __shared__ double s0[256], s1[256];
-  double a = 0.0, b = 0.0;
-  for (size_t k = threadIdx.x; k < (size_t)m * m; k += 256) {
-    const double x = A[k];
-    b = fma(x, x, b);
-    if (k / m != k % m) a = fma(x, x, a);
-  }
-  s0[threadIdx.x] = a;
-  s1[threadIdx.x] = b;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      s0[threadIdx.x] += s0[threadIdx.x + st];
-      s1[threadIdx.x] += s1[threadIdx.x + st];
-    }
+    sh0[tid] = o;
+    sh1[tid] = w;
     __syncthreads();
+    for (int h = JT * JT / 2; h > 0; h >>= 1) {
+      if (tid < h) {
+        sh0[tid] += sh0[tid + h];
+        sh1[tid] += sh1[tid + h];
+      }
+      __syncthreads();
+    }
+    if (tid == 0) slots[blockIdx.x] = make_double2(sh0[0], sh1[0]);
+    if (!grid_barrier(&st->bar, gen)) return;
+    o = w = 0.0;
+    for (int c = tid; c < gridDim.x; c += JT * JT) {
+      const double2 x = __ldcg(&slots[c]);
+      o += x.x;
+      w += x.y;
+    }
+    sh0[tid] = o;
+    sh1[tid] = w;
+    __syncthreads();
+    for (int h = JT * JT / 2; h > 0; h >>= 1) {
+      if (tid < h) {
+        sh0[tid] += sh0[tid + h];
+        sh1[tid] += sh1[tid + h];
+      }
+      __syncthreads();
+    }
+    const double off = sh0[0], all = sh1[0];
+    __syncthreads();
+    if (off <= 1e-30 * all || off == 0.0 || sweep >= max_sweeps) break;
+    for (int t = 0; t < mp - 1; ++t) {
+      for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
+        const int tp = tile / nt, tr = tile % nt;
+        // this thread's pairs and, before the rotations are known, its elements: the loads
+        // and the rotations' arithmetic overlap
+        auto pair = [&](int k, int& i, int& j) {
+          i = k < K ? rr_slot(k, t, mp) : m;  // m: no such index
+          j = k < K ? rr_slot(mp - 1 - k, t, mp) : m;
+        };
+        int p, q, r, s;
+        pair(tp * JT + ty, p, q);
+        pair(tr * JT + tx, r, s);
+        auto get = [&](int i, int j) { return i < m && j < m ? __ldcg(&Ac[(size_t)i * m + j]) : 0.0; };
+        const double pr = get(p, r), ps = get(p, s), qr = get(q, r), qs = get(q, s);
+        double vx[2], vy[2];  // V rows 32 tp .. by the column pairs of this tile
+        const bool cols = r < m && s < m;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int i = 2 * JT * tp + ty + JT * h;
+          vx[h] = i < m && cols ? __ldcg(&V[(size_t)i * m + r]) : 0.0;
+          vy[h] = i < m && cols ? __ldcg(&V[(size_t)i * m + s]) : 0.0;
+        }
+        __syncthreads();  // the previous tile's reads of rot
+        if (tid < 2 * JT) {
+          int i, j;
+          pair((tid < JT ? tp : tr) * JT + tid % JT, i, j);
+          rot[tid / JT][tid % JT] = i < m && j < m ? jac_rotation(get(i, i), get(j, j), get(i, j))
+                                                   : make_double2(1.0, 0.0);
+        }
+        __syncthreads();
+        const double2 a = rot[0][ty], b = rot[1][tx];
+        const double pr1 = a.x * pr - a.y * qr, qr1 = a.y * pr + a.x * qr;
+        const double ps1 = a.x * ps - a.y * qs, qs1 = a.y * ps + a.x * qs;
+        auto put = [&](int i, int j, double v) {
+          if (i < m && j < m) An[(size_t)i * m + j] = v;
+        };
+        put(p, r, b.x * pr1 - b.y * ps1);
+        put(p, s, b.y * pr1 + b.x * ps1);
+        put(q, r, b.x * qr1 - b.y * qs1);
+        put(q, s, b.y * qr1 + b.x * qs1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int i = 2 * JT * tp + ty + JT * h;
+          if (i < m && cols) {
+            V[(size_t)i * m + r] = b.x * vx[h] - b.y * vy[h];
+            V[(size_t)i * m + s] = b.y * vx[h] + b.x * vy[h];
+          }
+        }
+      }
+      if (!grid_barrier(&st->bar, gen)) return;
+      double* x = Ac;
+      Ac = An;
+      An = x;
+    }
   }
-  if (threadIdx.x == 0) {
-    off[0] = s0[0];
-    off[1] = s1[0];
-  }
+  for (int k = blockIdx.x * (JT * JT) + tid; k < m; k += gridDim.x * JT * JT)
+    diag[k] = __ldcg(&Ac[(size_t)k * m + k]);
+  if (blockIdx.x == 0 && tid == 0) st->sweeps = max(st->sweeps, sweep);
 }
 
-// U block and eps from the converged A, V: column perm[k] of V becomes column
-// lo+k of U, with its largest-magnitude component made positive (first one on ties).
-__global__ void jac_store_kernel(const double* __restrict__ A, const double* __restrict__ V, int m,
-                                 const int* __restrict__ perm, int n, int lo,
-                                 double* __restrict__ U, double* __restrict__ eps) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= m) return;
-  const int c = perm[k];
-  int imax = 0;
+// U block and eps from the eigenvalues diag and V, one CTA per column: column c of V
+// becomes column lo + rank of U, rank = its place in ascending order (equal values in
+// index order), with its largest-magnitude component made positive (first one on ties).
+__global__ void __launch_bounds__(128) jac_store_kernel(const double* __restrict__ diag,
+                                                        const double* __restrict__ V, int m, int n,
+                                                        int lo, double* __restrict__ U,
+                                                        double* __restrict__ eps) {
+  __shared__ int cnt;
+  __shared__ double sv[128];
+  __shared__ int si[128];
+  const int c = blockIdx.x, tid = threadIdx.x;
+  const double dc = diag[c];
+  if (tid == 0) cnt = 0;
+  __syncthreads();
+  int below = 0, imax = 0;
   double vmax = -1.0;
-  for (int i = 0; i < m; ++i) {
+  for (int i = tid; i < m; i += 128) {
+    const double x = diag[i];
+    below += x < dc || (x == dc && i < c);
     const double a = fabs(V[(size_t)i * m + c]);
     if (a > vmax) {
       vmax = a;
       imax = i;
     }
   }
-  const double sg = V[(size_t)imax * m + c] < 0.0 ? -1.0 : 1.0;
-  for (int i = 0; i < m; ++i) U[(size_t)(lo + i) * n + lo + k] = sg * V[(size_t)i * m + c];
-  eps[lo + k] = A[(size_t)c * m + c];
+  atomicAdd(&cnt, below);
+  sv[tid] = vmax;
+  si[tid] = imax;
+  __syncthreads();
+  for (int o = 64; o > 0; o >>= 1) {
+    if (tid < o && (sv[tid + o] > sv[tid] || (sv[tid + o] == sv[tid] && si[tid + o] < si[tid]))) {
+      sv[tid] = sv[tid + o];
+      si[tid] = si[tid + o];
+    }
+    __syncthreads();
+  }
+  const int k = cnt;
+  const double sg = V[(size_t)si[0] * m + c] < 0.0 ? -1.0 : 1.0;
+  for (int i = tid; i < m; i += 128) U[(size_t)(lo + i) * n + lo + k] = sg * V[(size_t)i * m + c];
+  if (tid == 0) eps[lo + k] = dc;
 }
 
 // ------------------------------ transformations ------------------------------
@@ -328,49 +433,21 @@ cudaError_t jacobi_block(dsrg_sc_plan* p, int lo, int m, double* eps) {
   if (m == 0) return cudaSuccess;
   cudaStream_t st = p->stream;
   const int n = p->z.n;
-  const int mp = m + (m & 1);
   cudaError_t e;
   jac_copy_kernel<<<(m * m + 255) / 256, 256, 0, st>>>(p->f, n, lo, m, p->A, p->V);
   if ((e = sc_check(p)) != cudaSuccess) return e;
-  int sweeps = 0;
-  if (m > 1) {
-    for (; sweeps < 30; ++sweeps) {
-      jac_norm_kernel<<<1, 256, 0, st>>>(p->A, m, p->off);
-      if ((e = sc_check(p)) != cudaSuccess) return e;
-      double off[2] = {0.0, 0.0};
-      if ((e = cudaMemcpyAsync(off, p->off, 2 * sizeof(double), cudaMemcpyDeviceToHost, st)) !=
-          cudaSuccess)
-        return e;
-      if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-      if (off[0] <= 1e-30 * off[1] || off[0] == 0.0) break;
-      for (int t = 0; t < mp - 1; ++t) {
-        jac_params_kernel<<<(mp / 2 + 127) / 128, 128, 0, st>>>(p->A, m, mp, t, p->cs);
-        dim3 g((m + 127) / 128, mp / 2);
-        jac_rows_kernel<<<g, 128, 0, st>>>(p->A, m, mp, t, p->cs);
-        jac_cols_kernel<<<g, 128, 0, st>>>(p->A, p->V, m, mp, t, p->cs);
-      }
-      if ((e = sc_check(p)) != cudaSuccess) return e;
-    }
-  }
-  p->sweeps_last = std::max(p->sweeps_last, sweeps);
-  // sort the eigenvalues ascending (host: m values)
-  std::vector<double> diag(m);
-  std::vector<double> Ah((size_t)m * m);
-  if ((e = cudaMemcpyAsync(Ah.data(), p->A, (size_t)m * m * sizeof(double), cudaMemcpyDeviceToHost,
-                           st)) != cudaSuccess)
-    return e;
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-  for (int i = 0; i < m; ++i) diag[i] = Ah[(size_t)i * m + i];
-  std::vector<int> perm(m);
-  std::iota(perm.begin(), perm.end(), 0);
-  std::stable_sort(perm.begin(), perm.end(), [&](int a, int b) { return diag[a] < diag[b]; });
-  if ((e = cudaMemcpyAsync(p->perm, perm.data(), m * sizeof(int), cudaMemcpyHostToDevice, st)) !=
-      cudaSuccess)
-    return e;
-  jac_store_kernel<<<(m + 127) / 128, 128, 0, st>>>(p->A, p->V, m, p->perm, n, lo, p->U, eps);
-  if ((e = sc_check(p)) != cudaSuccess) return e;
-  // the host vectors above must outlive the copy
-  return cudaStreamSynchronize(st);
+  int mp = m + (m & 1);
+  const int nt = (mp / 2 + JT - 1) / JT;
+  int grid = coop_grid(jac_run_kernel, JT * JT, 0, nt * nt < JAC_SLOTS ? nt * nt : JAC_SLOTS);
+  if (grid < 1) return cudaErrorInvalidConfiguration;
+  int max_sweeps = m > 1 ? 30 : 0;
+  e = cudaMemsetAsync(&p->jac->bar.count, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&p->A, &p->A2, &p->V, &m, &mp, &max_sweeps, &p->slots, &p->diag, &p->jac};
+  e = cudaLaunchCooperativeKernel((const void*)jac_run_kernel, dim3(grid), dim3(JT * JT), args, 0, st);
+  if (e != cudaSuccess) return e;
+  jac_store_kernel<<<m, 128, 0, st>>>(p->diag, p->V, m, n, lo, p->U, eps);
+  return sc_check(p);
 }
 
 cudaError_t build_fock(dsrg_sc_plan* p, const double* h, const double* B, const double* G) {
@@ -386,11 +463,20 @@ cudaError_t build_fock(dsrg_sc_plan* p, const double* h, const double* B, const 
   fock_x_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, st>>>(B, G, z, p->X);
   if ((e = sc_check(p)) != cudaSuccess) return e;
   // K[p][q] = sum_{Q, r in H} X[Q][p][r] B[Q][r][q]
-  GemmArgs g = mk(z.n, z.n, z.Q, z.nH, p->X, z.nH, (long long)z.n * z.nH, 1, B,
-                  (long long)nn, z.n, 1, p->K, z.n, 1, 1.0);
-  g.accumulate = 0;
-  if ((e = launch_gemm_fp64(st, g)) != cudaSuccess) return e;
-  fock_sum_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(h, p->J, p->K, z.n, p->f);
+  const int qc = (z.Q + p->nk - 1) / p->nk, full = z.Q / qc, rest = z.Q - full * qc;
+  auto part = [&](int q0, int nq, double* K) {
+    GemmArgs g = mk(z.n, z.n, nq, z.nH, p->X + (size_t)q0 * z.n * z.nH, z.nH, (long long)z.n * z.nH, 1,
+                    B + (size_t)q0 * nn, (long long)nn, z.n, 1, K, z.n, 1, 1.0);
+    g.accumulate = 0;
+    return g;
+  };
+  if ((e = launch_gemm(st, batched(part(0, qc, p->K), full, (long long)qc * z.n * z.nH, (long long)qc * nn,
+                                   (long long)nn), p->oz)) != cudaSuccess)
+    return e;
+  if (rest && (e = launch_gemm(st, part(full * qc, rest, p->K + (size_t)full * nn), p->oz)) != cudaSuccess)
+    return e;
+  fock_sum_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(h, p->J, p->K, full + (rest ? 1 : 0), z.n,
+                                                               p->f);
   return sc_check(p);
 }
 
@@ -425,16 +511,33 @@ dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t** out, const dsrg_sizes_t* sz, 
   p->mmax = std::max(z.nC, std::max(z.nA, z.nV));
   const size_t nn = (size_t)z.n * z.n, mm = (size_t)p->mmax * p->mmax;
   const size_t nhp = (size_t)z.Q * z.nH * z.nP;
+  {
+    // the exchange matrix has few tiles and a long sum: parts of it over Q, so that about
+    // two tiles per SM run, each part at least 512 long
+    const long long tiles = ((z.n + 127) / 128) * (long long)((z.n + 63) / 64);
+    long long nk = 304 / tiles, most = (long long)z.Q * z.nH / 512;
+    nk = nk > 16 ? 16 : nk;
+    nk = nk > most ? most : nk;
+    p->nk = nk < 1 ? 1 : (int)(nk > z.Q ? z.Q : nk);
+    const long long qc = (z.Q + p->nk - 1) / p->nk;
+    size_t b = oz_work_bytes(z.n, z.n, qc * z.nH, p->nk, false, false);
+    b = std::max(b, oz_work_bytes(z.n, z.n, z.n, 1, false, false));
+    b = std::max(b, oz_work_bytes((long long)z.Q * z.nH, z.nP, z.nP, 1, false, false));
+    b = std::max(b, oz_work_bytes(z.nH, z.nP, z.nH, z.Q, true, false));
+    p->oz.bytes = b;
+  }
   bool ok = sc_alloc(p, (void**)&p->w, (size_t)z.Q * 8) && sc_alloc(p, (void**)&p->J, nn * 8) &&
-            sc_alloc(p, (void**)&p->K, nn * 8) &&
+            sc_alloc(p, (void**)&p->K, p->nk * nn * 8) &&
             sc_alloc(p, (void**)&p->X, (size_t)z.Q * z.n * z.nH * 8) &&
             sc_alloc(p, (void**)&p->f, nn * 8) && sc_alloc(p, (void**)&p->U, nn * 8) &&
             sc_alloc(p, (void**)&p->T, nn * 8) && sc_alloc(p, (void**)&p->A, mm * 8) &&
             sc_alloc(p, (void**)&p->V, mm * 8) &&
-            sc_alloc(p, (void**)&p->cs, ((size_t)p->mmax / 2 + 2) * sizeof(double2)) &&
-            sc_alloc(p, (void**)&p->off, 16) && sc_alloc(p, (void**)&p->Bhp, nhp * 8) &&
-            sc_alloc(p, (void**)&p->Bt, nhp * 8) &&
-            sc_alloc(p, (void**)&p->perm, ((size_t)p->mmax + 1) * sizeof(int));
+            sc_alloc(p, (void**)&p->A2, mm * 8) && sc_alloc(p, (void**)&p->diag, (size_t)p->mmax * 8) &&
+            sc_alloc(p, (void**)&p->slots, JAC_SLOTS * sizeof(double2)) &&
+            sc_alloc(p, (void**)&p->jac, sizeof(JacState)) && sc_alloc(p, (void**)&p->Bhp, nhp * 8) &&
+            sc_alloc(p, (void**)&p->Bt, nhp * 8) && sc_alloc(p, &p->oz.mem, p->oz.bytes);
+  ok = ok && cudaMemset(p->jac, 0, sizeof(JacState)) == cudaSuccess;
+  if (ok) p->oz.status = &p->jac->wait;
   size_t n3 = 1;
   for (int d = 0; d < 6; ++d) n3 *= (size_t)(2 * z.nA);
   ok = ok && (z.nA == 0 || sc_alloc(p, (void**)&p->L3t, n3 * 8));
@@ -488,6 +591,7 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
   cudaStream_t st = p->stream;
   const size_t nn = (size_t)z.n * z.n;
   p->sweeps_last = 0;
+  if (cudaMemsetAsync(p->jac, 0, sizeof(JacState), st) != cudaSuccess) return DSRG_ERR_CUDA;
   if (build_fock(p, h, Bfull, gamma1) != cudaSuccess) return DSRG_ERR_CUDA;
   if (cudaMemsetAsync(p->U, 0, nn * 8, st) != cudaSuccess) return DSRG_ERR_CUDA;
   if (jacobi_block(p, 0, z.nC, eps_out) != cudaSuccess ||
@@ -500,7 +604,7 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
   g1.accumulate = 0;
   GemmArgs g2 = mk(z.n, z.n, z.n, 1, p->U, 1, z.n, 0, p->T, z.n, 0, 1, p->K, z.n, 1, 1.0);
   g2.accumulate = 0;
-  if ((e = launch_gemm_fp64(st, g1)) != cudaSuccess || (e = launch_gemm_fp64(st, g2)) != cudaSuccess)
+  if ((e = launch_gemm(st, g1, p->oz)) != cudaSuccess || (e = launch_gemm(st, g2, p->oz)) != cudaSuccess)
     return DSRG_ERR_CUDA;
   f1_kernel<<<(z.nH * z.nP + 255) / 256, 256, 0, st>>>(p->K, z, f1_out);
   if (sc_check(p) != cudaSuccess) return DSRG_ERR_CUDA;
@@ -516,7 +620,7 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
                            1.0),
                         z.Q, 0, (long long)z.nH * z.nP, (long long)z.nH * z.nP);
   g4.accumulate = 0;
-  if ((e = launch_gemm_fp64(st, g3)) != cudaSuccess || (e = launch_gemm_fp64(st, g4)) != cudaSuccess)
+  if ((e = launch_gemm(st, g3, p->oz)) != cudaSuccess || (e = launch_gemm(st, g4, p->oz)) != cudaSuccess)
     return DSRG_ERR_CUDA;
   if (z.nA > 0) {
     const int n4 = z.nA * z.nA * z.nA * z.nA + z.nA * z.nA;
@@ -538,6 +642,15 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
   }
   if (U_out && cudaMemcpyAsync(U_out, p->U, nn * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return DSRG_ERR_CUDA;
+  JacState js{};
+  if (cudaMemcpyAsync(&js, p->jac, sizeof(js), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return DSRG_ERR_CUDA;
+  p->sweeps_last = js.sweeps;
+  if (js.bar.abort || js.wait) {
+    p->last_error = "a device-side wait ran out";
+    return DSRG_ERR_TIMEOUT;
+  }
   return DSRG_OK;
 }
 
