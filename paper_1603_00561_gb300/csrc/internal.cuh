@@ -49,6 +49,7 @@ struct ActiveWs {
   double* ft = nullptr;   // [2nH][2nP]
   double* M = nullptr;    // (xe|uf) [nA][nA][nV][nV]
   double* P12 = nullptr;  // P1, P2 [2][nA^4]
+  double* L3p = nullptr;  // [triples][triples] three-body cumulant of terms J and K
   double* P12part = nullptr;  // per-CTA partials of P1/P2 [nblk][2][nA^4]
   size_t w1n = 0, w2n = 0;
   int actvv_blocks = 0;
@@ -322,12 +323,8 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
 void* split_plane_ptr(const dsrg_plan* p, bool hi);
 const float* split_tail_ptr(const dsrg_plan* p);  // [plane rows + 256][32] fl32(B), Q < 32
 size_t split_tail_bytes(const Sizes& z);
-// Factor tables of exp(-s D^2) for the active pairs and the pair-independent
-// table, formed by launch_split_rest of the same call.
-__global__ void abs_max_kernel(const double* __restrict__ x, int n, double* __restrict__ out);
-double* rest_take_tau1(dsrg_plan* p);
-void rest_act_tables(const dsrg_plan* p, const double** alpha, const double** pinfo,
-                     const double** tau, int* ld);
+__global__ void pair_info_kernel(const double* __restrict__ eps, double c, Sizes z,
+                                 const int2* __restrict__ pairs, int n, double2* __restrict__ pinfo);
 int split_qld(const dsrg_plan* p);
 // Adjoint of F2 from the energy call's GEMM output and factor tables (split
 // plans with the tensor-core rest): dX [nC][nA][nV][nV], adds to deps, ds.

@@ -31,9 +31,9 @@ struct RegD {
   double v, dD, ds;
 };
 
-__device__ __forceinline__ RegD rt_d(double D, double s) {
+__device__ __forceinline__ RegD rt_d(double D, double s, double& g) {
   const double x = s * D * D;
-  const double g = exp(-x);
+  g = exp(-x);
   RegD r;
   if (x < 1e-4) {
     r.v = s * D * (1.0 - 0.5 * x + x * x / 6.0);
@@ -49,9 +49,21 @@ __device__ __forceinline__ RegD rt_d(double D, double s) {
   return r;
 }
 
+__device__ __forceinline__ RegD rt_d(double D, double s) {
+  double g;
+  return rt_d(D, s, g);
+}
+
 __device__ __forceinline__ RegD rv_d(double D, double s) {
   const double g = exp(-s * D * D);
   return RegD{1.0 + g, -2.0 * s * D * g, -D * D * g};
+}
+
+// Both, with one exponential.
+__device__ __forceinline__ void rtv_d(double D, double s, RegD& rt, RegD& rv) {
+  double g;
+  rt = rt_d(D, s, g);
+  rv = RegD{1.0 + g, -2.0 * s * D * g, -D * D * g};
 }
 
 __device__ __forceinline__ RegD rf1_d(double D, double s) {

@@ -341,44 +341,6 @@ __global__ void xx_gram_kernel(const double* __restrict__ Xq, int T, int Q, doub
   }
 }
 
-// Factors of exp(-s D_u^2), D_u = E_mu - e_a - e_b, E_mu = e_m + e_u, for the
-// pairs mu = (m core, u active) and then (x active, u active) (the active VV
-// sums of the active block).
-__global__ void cavv_tables_kernel(const double* __restrict__ eps, double s, Sizes z, int nVpad,
-                                   double* __restrict__ alpha, double* __restrict__ pinfo,
-                                   double* __restrict__ tau1, const double* __restrict__ vmaxp) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int ve = z.nC + z.nA;
-  const int nmu = (z.nC + z.nA) * z.nA;
-  const size_t na = (size_t)nmu * nVpad, nt = (size_t)nVpad * nVpad;
-  if (k < na) {
-    const int mu = (int)(k / nVpad), b = (int)(k % nVpad);
-    const int m = mu / z.nA, u = mu % z.nA;  // m < nC: core; m >= nC: active x = m - nC
-    const double E = eps[m] + eps[z.nC + u];
-    alpha[k] = (b < z.nV) ? exp(2.0 * s * E * eps[ve + b]) : 0.0;
-    if (b == 0) {
-      const double vmax = *vmaxp;  // max |e_v| over the virtual orbitals
-      // factors are multiplied left to right (pair, row, column, table); the partial
-      // products carry -sE^2 + 2sE e_e (+ 2sE e_f), bounded by the sum of magnitudes
-      const bool ok = (s * E * E + 4.0 * s * fabs(E) * vmax <= 700.0) &&
-                      (4.0 * s * vmax * vmax <= 700.0);
-      pinfo[4 * mu + 0] = E;
-      pinfo[4 * mu + 1] = exp(-s * E * E);
-      pinfo[4 * mu + 2] = ok ? 1.0 : 0.0;
-      pinfo[4 * mu + 3] = 0.0;
-    }
-  } else if (k < na + nt) {
-    const size_t r = k - na;
-    const int aa = (int)(r / nVpad), bb = (int)(r % nVpad);
-    double v = 0.0;
-    if (aa < z.nV && bb < z.nV) {
-      const double t = eps[ve + aa] + eps[ve + bb];
-      v = exp(-s * t * t);
-    }
-    tau1[r] = v;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // F2 (CAVV), spin-adapted (closed-shell spin sum of Table 2's F2):
 //   F2 = sum_m sum_{u,v} G_uv sum_ef X_u[e,f] (2 X_v[e,f] - X_v[f,e]) Rv_u Rt_v,
@@ -399,7 +361,7 @@ __global__ void __launch_bounds__(256) cavv_f2_kernel(const float* __restrict__ 
                                                       int nVpad, const double* __restrict__ eps,
                                                       const double* __restrict__ G, double s, Sizes z,
                                                       const int2* __restrict__ tps, int n_tp,
-                                                      const double* __restrict__ pinfo,
+                                                      const double2* __restrict__ pinfo,
                                                       double* __restrict__ partials,
                                                       unsigned long long* __restrict__ counts) {
   extern __shared__ float f2s[];
@@ -443,13 +405,13 @@ __global__ void __launch_bounds__(256) cavv_f2_kernel(const float* __restrict__ 
     if (t == 0) {
       int fact = 1, far = 1;
       for (int u = 0; u < NA; ++u) {
-        const double E = pinfo[4 * (m * z.nA + u)];
+        const double E = pinfo[m * z.nA + u].x;
         sE[u] = E;
         sEP[u] = ff_from(E);
         // a pair whose energies leave the range of the FP32 pairs counts as one
         // whose factors overflow
         const float dhi = (float)E - elo - flo, dlo = (float)E - ehi - fhi;
-        fact = fact && pinfo[4 * (m * z.nA + u) + 2] != 0.0 &&
+        fact = fact && pinfo[m * z.nA + u].y != 0.0 &&
                fmaxf(fabsf(dhi), fabsf(dlo)) < 1e15f;
         const float dn = dhi <= 0.0f ? dhi : (dlo >= 0.0f ? dlo : 0.0f);
         far = far && (dhi <= -0.25f || dlo >= 0.25f) && dn * dn > 46.0f / (float)s;
@@ -574,28 +536,40 @@ __global__ void __launch_bounds__(256) cavv_f2_kernel(const float* __restrict__ 
 // ---------------------------------------------------------------------------
 // Adjoint of F2 for the gradient of split plans: X_u from the GEMM output Y of
 // the energy call just made (its error, about 1e-8 relative, is far below the
-// gradient's), regulators from the same factor tables. Per position (e, f)
-// (and its mirror (f, e) for E < F), with P_v = 2 X_v[e,f] - X_v[f,e]:
+// gradient's). Per position (e, f) (and its mirror (f, e) for E < F), with
+// P_v = 2 X_v[e,f] - X_v[f,e]:
 //   dE/dX_u[e,f] = Rv_u s1_u + Rt_u s2_u,
 //   s1_u = sum_v G_uv Rt_v P_v,  s2_u = sum_v G_vu Rv_v P_v,
 // and the derivative of the summand with respect to D_u,
 //   X_u Rv_u' s1_u + (sum_w G_wu Rv_w X_w) P_u Rt_u',
 // goes to e_m and e_u (+) and to e_e, e_f (-); the s derivative likewise.
+// Away from D = 0 (the paths of the energy kernel) regulators and sums are pairs of
+// FP32 numbers (ff.cuh); near it RegD and FP64. In FP64 throughout, with the
+// exponentials from tables and an atomic per position for e_e, the kernel was bound by
+// the FP64 pipe: 682 us at 24/2/372/1200, 178 us now.
 // ---------------------------------------------------------------------------
+// a warp's sum of pairs, the same in every lane
+__device__ __forceinline__ ff ff_warp_sum(ff v) {
+  for (int o = 16; o > 0; o >>= 1)
+    v = ff_add(v, ff{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+  return v;
+}
+__device__ __forceinline__ ff ff_fma(ff a, ff b, ff c) { return ff_add(c, ff_mul(a, b)); }
+__device__ __forceinline__ ff ff_neg(ff a) { return ff{-a.h, -a.l}; }
+
 template <int NA>
 __global__ void __launch_bounds__(256) cavv_adj_tc_kernel(
     const float* __restrict__ Y, long long ldy, int nVpad, const double* __restrict__ eps,
     const double* __restrict__ G, double s, Sizes z, const int2* __restrict__ tps, int n_tp,
-    const double* __restrict__ alpha, const double* __restrict__ pinfo,
-    const double* __restrict__ tau1, double* __restrict__ dX, double* __restrict__ deps,
+    const double2* __restrict__ pinfo, double* __restrict__ dX, double* __restrict__ deps,
     double* __restrict__ ds) {
   extern __shared__ float f2s[];
   float* sX = f2s;                              // [NA][32][33]   X_u[e,f]
   float* sXt = sX + NA * F2_T * (F2_T + 1);     // [NA][32][33]   X_u[f,e]
-  __shared__ double sBAe[NA][F2_T], sAf[NA][F2_T], sEe[F2_T], sEf[F2_T], sG[NA * NA];
-  __shared__ double sE[NA];
+  __shared__ double sEe[F2_T], sEf[F2_T], sE[NA];
+  __shared__ ff sEeP[F2_T], sEfP[F2_T], sEP[NA], sG[NA * NA], sTab[8];
   __shared__ int sFact, sFar;
-  __shared__ double rowacc[F2_T], colacc[F2_T], uacc[NA];
+  __shared__ double rowacc[F2_T], colacc[F2_T];
   __shared__ double red[8];
   const int m = blockIdx.x / n_tp;
   const int2 ab = tps[blockIdx.x % n_tp];
@@ -607,153 +581,187 @@ __global__ void __launch_bounds__(256) cavv_adj_tc_kernel(
     sX[(u * F2_T + r) * (F2_T + 1) + c] = Ym[(size_t)(E0 + r) * ldy + u * nVpad + F0 + c];
     sXt[(u * F2_T + c) * (F2_T + 1) + r] = Ym[(size_t)(F0 + r) * ldy + u * nVpad + E0 + c];
   }
-  if (threadIdx.x < F2_T) {
+  if (threadIdx.x < F2_T) {  // warp 0: the paths of cavv_f2_kernel
     const int t = threadIdx.x;
     const int e = E0 + t, f = F0 + t;
-    sEe[t] = e < z.nV ? eps[ve + e] : 0.0;
-    sEf[t] = f < z.nV ? eps[ve + f] : 0.0;
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-      const double* al = alpha + (size_t)(m * z.nA + u) * nVpad;
-      sBAe[u][t] = pinfo[4 * (m * z.nA + u) + 1] * al[E0 + t];
-      sAf[u][t] = al[F0 + t];
-    }
-    rowacc[t] = 0.0;
+    const double xe = e < z.nV ? eps[ve + e] : 0.0, xf = f < z.nV ? eps[ve + f] : 0.0;
+    sEe[t] = xe;
+    sEf[t] = xf;
+    sEeP[t] = ff_from(xe);
+    sEfP[t] = ff_from(xf);
     colacc[t] = 0.0;
-  }
-  if (threadIdx.x < NA * NA) sG[threadIdx.x] = G[threadIdx.x];
-  if (threadIdx.x < NA) uacc[threadIdx.x] = 0.0;
-  if (threadIdx.x == 0) {
-    int fact = 1;
-    for (int u = 0; u < NA; ++u) {
-      sE[u] = pinfo[4 * (m * z.nA + u)];
-      fact = fact && (pinfo[4 * (m * z.nA + u) + 2] != 0.0);
+    float elo = e < z.nV ? (float)xe : 3.0e38f, ehi = e < z.nV ? (float)xe : -3.0e38f;
+    float flo = f < z.nV ? (float)xf : 3.0e38f, fhi = f < z.nV ? (float)xf : -3.0e38f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      elo = fminf(elo, __shfl_xor_sync(0xffffffffu, elo, o));
+      ehi = fmaxf(ehi, __shfl_xor_sync(0xffffffffu, ehi, o));
+      flo = fminf(flo, __shfl_xor_sync(0xffffffffu, flo, o));
+      fhi = fmaxf(fhi, __shfl_xor_sync(0xffffffffu, fhi, o));
     }
-    sFact = fact;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // every D_u of the tile pair so far from 0 that exp(-s D_u^2) < 2^-63
-    double elo = 1e300, flo = 1e300, ehi = -1e300, fhi = -1e300;
-    for (int t = 0; t < F2_T; ++t) {
-      if (E0 + t < z.nV) elo = fmin(elo, sEe[t]), ehi = fmax(ehi, sEe[t]);
-      if (F0 + t < z.nV) flo = fmin(flo, sEf[t]), fhi = fmax(fhi, sEf[t]);
+    if (t == 0) {
+      int fact = 1, far = 1;
+      for (int u = 0; u < NA; ++u) {
+        const double E = pinfo[m * z.nA + u].x;
+        sE[u] = E;
+        sEP[u] = ff_from(E);
+        const float dhi = (float)E - elo - flo, dlo = (float)E - ehi - fhi;
+        fact = fact && pinfo[m * z.nA + u].y != 0.0 && fmaxf(fabsf(dhi), fabsf(dlo)) < 1e15f;
+        const float dn = dhi <= 0.0f ? dhi : (dlo >= 0.0f ? dlo : 0.0f);
+        far = far && (dhi <= -0.25f || dlo >= 0.25f) && dn * dn > 46.0f / (float)s;
+      }
+      sFact = fact;
+      sFar = far && fact;
     }
-    int far = 1;
-    for (int u = 0; u < NA; ++u) {
-      const double dhi = sE[u] - elo - flo, dlo = sE[u] - ehi - fhi;
-      const double dn = dhi <= 0.0 ? dhi : (dlo >= 0.0 ? dlo : 0.0);
-      far = far && (dhi <= -0.25 || dlo >= 0.25) && s * dn * dn > 44.0;
-    }
-    sFar = far;
   }
+  if (threadIdx.x < NA * NA) sG[threadIdx.x] = ff_from(G[threadIdx.x]);
+  if (threadIdx.x >= 248) sTab[threadIdx.x - 248] = ff_exp_entry(threadIdx.x - 248);
   __syncthreads();
   const bool mirror = ab.x < ab.y;
   const bool fact = sFact != 0;
   const bool tile_far = sFar != 0;
   const int c = threadIdx.x & 31;
   const int f = F0 + c;
-  double dm = 0.0, dss = 0.0, cacc = 0.0;
-  double du[NA];
+  const ff kreg = ff_reg_scale(s), s2 = ff_from(2.0 * s);
+  const ff zero = {0.f, 0.f};
+  ff dss = zero, cacc = zero, du[NA];
 #pragma unroll
-  for (int u = 0; u < NA; ++u) du[u] = 0.0;
-  if (f < z.nV) {
-    for (int r = threadIdx.x >> 5; r < F2_T; r += 8) {
-      const int e = E0 + r;
-      if (e >= z.nV) break;
-      const double tau = (fact && !tile_far) ? tau1[(size_t)e * nVpad + f] : 0.0;
-      const double eef = sEe[r] + sEf[c];
-      RegD Rv[NA], Rt[NA];
-      double X[NA], Xt[NA], Dd[NA];
+  for (int u = 0; u < NA; ++u) du[u] = zero;
+  for (int r = threadIdx.x >> 5; r < F2_T; r += 8) {
+    const int e = E0 + r;
+    if (e >= z.nV) break;
+    ff gsum = zero;
+    if (f < z.nV) {
+      const ff eef = ff_add(sEeP[r], sEfP[c]);
+      float X[NA], Xt[NA];
       bool far = fact;
 #pragma unroll
       for (int u = 0; u < NA; ++u) {
         X[u] = sX[(u * F2_T + r) * (F2_T + 1) + c];
         Xt[u] = sXt[(u * F2_T + r) * (F2_T + 1) + c];
-        Dd[u] = sE[u] - eef;
-        far = far && fabs(Dd[u]) >= 0.25;
+        far = far && fabsf(sEP[u].h - eef.h) >= 0.25f;
       }
+      double* dxp = dX + ((size_t)m * NA * z.nV + e) * z.nV + f;        // (e, f), then (f, e)
       if (far || tile_far) {
+        // Rt = (1 - g)/D, Rt' = 2 s g - Rt/D, dRt/ds = D g; Rv = 1 + g, Rv' = -2 s D g,
+        // dRv/ds = -D^2 g
+        ff Rt[NA], Rd[NA], Rs[NA], Rv[NA];
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
-          const double D = Dd[u];
-          const double g = tile_far ? 0.0 : sBAe[u][r] * sAf[u][c] * tau;
-          float r0f;
-          asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0f) : "f"((float)D));
-          const double r0 = (double)r0f;
-          const double en = fma(-D, r0, 1.0);
-          const double inv = fma(r0, en, r0);
-          const double R0 = fma(-g, r0, r0);
-          const double x = s * D * D;
-          Rt[u].v = fma(R0, en, R0);                        // (1 - g) / D
-          Rt[u].dD = fma(2.0 * x, g, g - 1.0) * inv * inv;  // (2 x g + e^{-x} - 1) / D^2
-          Rt[u].ds = D * g;
-          Rv[u].v = 1.0 + g;
-          Rv[u].dD = -2.0 * s * D * g;
-          Rv[u].ds = -D * D * g;
+          const ff D = ff_diff(sEP[u], eef), inv = ff_inv(D);
+          Rt[u] = inv;
+          Rs[u] = zero;
+          Rv[u] = ff{1.f, 0.f};
+          if (!tile_far) {
+            const ff om = ff_one_minus_exp(D, kreg, sTab), g = ff_diff(ff{1.f, 0.f}, om);
+            Rt[u] = ff_mul(om, inv);
+            Rs[u] = ff_mul(D, g);
+            Rv[u] = ff_add(ff{1.f, 0.f}, g);
+            Rd[u] = ff_diff(ff_mul(g, s2), ff_mul(Rt[u], inv));
+          } else {
+            Rd[u] = ff_neg(ff_mul(inv, inv));
+          }
+        }
+        // one side per pass: (e, f) with X, then its mirror with X and Xt exchanged
+#pragma unroll 1
+        for (int side = 0; side < (mirror ? 2 : 1); ++side) {
+          ff b[NA], w[NA], x[NA];
+#pragma unroll
+          for (int v = 0; v < NA; ++v) {
+            const ff P = ff_two_sum(2.0f * X[v], -Xt[v]);
+            b[v] = ff_mul(Rt[v], P);
+            w[v] = ff_mul(Rv[v], P);
+            x[v] = ff_mul(X[v], Rv[v]);
+          }
+#pragma unroll
+          for (int u = 0; u < NA; ++u) {
+            ff s1 = zero, sw = zero, cw = zero;
+#pragma unroll
+            for (int v = 0; v < NA; ++v) {
+              // volatile: reloaded instead of held in 4 NA^2 registers
+              volatile const ff& g1 = sG[u * NA + v];
+              volatile const ff& g2 = sG[v * NA + u];
+              const ff guv = {g1.h, g1.l}, gvu = {g2.h, g2.l};
+              s1 = ff_fma(guv, b[v], s1);
+              sw = ff_fma(gvu, w[v], sw);
+              cw = ff_fma(gvu, x[v], cw);
+            }
+            dxp[(size_t)u * z.nV * z.nV] = ff_to(ff_fma(Rt[u], sw, ff_mul(Rv[u], s1)));
+            const ff xs = ff_mul(X[u], s1), cp = ff_mul(cw, ff_two_sum(2.0f * X[u], -Xt[u]));
+            // X Rv' s1 + cw P Rt' and the same by s: Rv' = -2 s Rs, dRv/ds = -D Rs
+            const ff gD = ff_diff(ff_mul(cp, Rd[u]), ff_mul(xs, ff_mul(s2, Rs[u])));
+            ff_acc(du[u], gD);
+            ff_acc(gsum, gD);
+            if (!tile_far) {
+              const ff D = ff_diff(sEP[u], eef);
+              ff_acc(dss, ff_mul(Rs[u], ff_diff(cp, ff_mul(D, xs))));
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < NA; ++v) {
+            const float t = X[v];
+            X[v] = Xt[v];
+            Xt[v] = t;
+          }
+          dxp = dX + ((size_t)m * NA * z.nV + f) * z.nV + e;
         }
       } else {
+        // a D_u near 0 (or a pair whose factors could overflow) in FP64
+        const double ee = sEe[r] + sEf[c];
+        RegD Rv[NA], Rt[NA];
 #pragma unroll
-        for (int u = 0; u < NA; ++u) {
-          Rt[u] = rt_d(Dd[u], s);
-          Rv[u] = rv_d(Dd[u], s);
+        for (int u = 0; u < NA; ++u) rtv_d(sE[u] - ee, s, Rt[u], Rv[u]);
+#pragma unroll 1
+        for (int side = 0; side < (mirror ? 2 : 1); ++side) {
+#pragma unroll
+          for (int u = 0; u < NA; ++u) {
+            double s1 = 0.0, sw = 0.0, cw = 0.0;
+#pragma unroll
+            for (int v = 0; v < NA; ++v) {
+              const double P = 2.0 * (double)X[v] - (double)Xt[v], gv = G[v * NA + u] * Rv[v].v;
+              s1 = fma(G[u * NA + v] * Rt[v].v, P, s1);
+              sw = fma(gv, P, sw);
+              cw = fma(gv, (double)X[v], cw);
+            }
+            const double P = 2.0 * (double)X[u] - (double)Xt[u], xs = (double)X[u] * s1, cp = cw * P;
+            dxp[(size_t)u * z.nV * z.nV] = Rv[u].v * s1 + Rt[u].v * sw;
+            const ff gD = ff_from(xs * Rv[u].dD + cp * Rt[u].dD);
+            ff_acc(du[u], gD);
+            ff_acc(gsum, gD);
+            ff_acc(dss, ff_from(xs * Rv[u].ds + cp * Rt[u].ds));
+          }
+#pragma unroll
+          for (int v = 0; v < NA; ++v) {
+            const float t = X[v];
+            X[v] = Xt[v];
+            Xt[v] = t;
+          }
+          dxp = dX + ((size_t)m * NA * z.nV + f) * z.nV + e;
         }
       }
-      double P[NA], Pt[NA];
-#pragma unroll
-      for (int u = 0; u < NA; ++u) {
-        P[u] = 2.0 * X[u] - Xt[u];
-        Pt[u] = 2.0 * Xt[u] - X[u];
-      }
-      double gsum = 0.0;
-#pragma unroll
-      for (int u = 0; u < NA; ++u) {
-        double s1 = 0.0, s2 = 0.0, s1t = 0.0, s2t = 0.0, cw = 0.0, cwt = 0.0;
-#pragma unroll
-        for (int v = 0; v < NA; ++v) {
-          const double gt = sG[u * NA + v] * Rt[v].v, gv = sG[v * NA + u] * Rv[v].v;
-          s1 = fma(gt, P[v], s1);
-          s2 = fma(gv, P[v], s2);
-          s1t = fma(gt, Pt[v], s1t);
-          s2t = fma(gv, Pt[v], s2t);
-          cw = fma(gv, X[v], cw);
-          cwt = fma(gv, Xt[v], cwt);
-        }
-        dX[(((size_t)m * NA + u) * z.nV + e) * z.nV + f] = Rv[u].v * s1 + Rt[u].v * s2;
-        if (mirror) dX[(((size_t)m * NA + u) * z.nV + f) * z.nV + e] = Rv[u].v * s1t + Rt[u].v * s2t;
-        double gD = X[u] * Rv[u].dD * s1 + cw * P[u] * Rt[u].dD;
-        double gs = X[u] * Rv[u].ds * s1 + cw * P[u] * Rt[u].ds;
-        if (mirror) {
-          gD += Xt[u] * Rv[u].dD * s1t + cwt * Pt[u] * Rt[u].dD;
-          gs += Xt[u] * Rv[u].ds * s1t + cwt * Pt[u] * Rt[u].ds;
-        }
-        du[u] += gD;
-        gsum += gD;
-        dss += gs;
-      }
-      dm += gsum;
-      atomicAdd(&rowacc[r], -gsum);
-      cacc -= gsum;
+      ff_acc(cacc, gsum);
     }
+    __syncwarp();
+    const ff t = ff_warp_sum(gsum);  // row r is this warp's alone
+    if (c == 0) rowacc[r] = ff_to(t);
   }
-  atomicAdd(&colacc[c], cacc);
-  const double tm = block_sum<256>(dm, red);
-  const double ts = block_sum<256>(dss, red);
+  atomicAdd(&colacc[c], ff_to(cacc));
+  double tm = 0.0;
+  const double ts = block_sum<256>(ff_to(dss), red);
 #pragma unroll
   for (int u = 0; u < NA; ++u) {
-    const double t = block_sum<256>(du[u], red);
-    if (threadIdx.x == 0) uacc[u] = t;
+    const double t = block_sum<256>(ff_to(du[u]), red);
+    tm += t;
+    if (threadIdx.x == 0) atomicAdd(&deps[z.nC + u], t);
   }
-  __syncthreads();
   if (threadIdx.x == 0) {
     atomicAdd(&deps[m], tm);
     atomicAdd(ds, ts);
-    for (int u = 0; u < NA; ++u) atomicAdd(&deps[z.nC + u], uacc[u]);
   }
   if (threadIdx.x < F2_T) {
-    const int e = E0 + threadIdx.x, ff = F0 + threadIdx.x;
-    if (e < z.nV) atomicAdd(&deps[ve + e], rowacc[threadIdx.x]);
-    if (ff < z.nV) atomicAdd(&deps[ve + ff], colacc[threadIdx.x]);
+    const int e = E0 + threadIdx.x, ff_ = F0 + threadIdx.x;
+    if (e < z.nV) atomicAdd(&deps[ve + e], -rowacc[threadIdx.x]);
+    if (ff_ < z.nV) atomicAdd(&deps[ve + ff_], -colacc[threadIdx.x]);
   }
 }
 
@@ -902,15 +910,9 @@ struct RestState {
   float* Y = nullptr;
   double* Xq = nullptr;
   double* Gxx = nullptr;
-  double* alpha = nullptr;
-  double* pinfo = nullptr;
-  double* tau1 = nullptr;
-  double* vmax = nullptr;  // max |e_v| over the virtual orbitals
+  double2* pinfo = nullptr;  // [nC nA]  E_m + E_u, factorisable flag (pair_info_kernel)
   int2* d_tp = nullptr;
   int n_tp = 0;
-  // tau1 was written by the pair tables of the CCVV kernel (split_stage_tables)
-  // queued before this call's CAVV tables: those skip it
-  bool tau1_staged = false;
 };
 
 int rest_xrows(const Sizes& z) {
@@ -972,10 +974,7 @@ bool rest_alloc(dsrg_plan* p, float* shared_y) {
     ok = plan_alloc(p, (void**)&st->Y, rest_y_bytes(z));
   ok = ok && plan_alloc(p, (void**)&st->Xq, (size_t)T * z.Q * 8) &&
        plan_alloc(p, (void**)&st->Gxx, (size_t)T * T * 8) &&
-       plan_alloc(p, (void**)&st->alpha, (size_t)z.nH * z.nA * st->nVpad * 8) &&
-       plan_alloc(p, (void**)&st->pinfo, (size_t)z.nH * z.nA * 4 * 8) &&
-       plan_alloc(p, (void**)&st->tau1, (size_t)st->nVpad * st->nVpad * 8) &&
-       plan_alloc(p, (void**)&st->vmax, 8) &&
+       plan_alloc(p, (void**)&st->pinfo, (size_t)z.nC * z.nA * sizeof(double2)) &&
        plan_alloc(p, (void**)&st->d_tp, (size_t)st->n_tp * sizeof(int2));
   if (!ok) return false;
   const int nt = (z.nV + F2_T - 1) / F2_T;
@@ -984,26 +983,6 @@ bool rest_alloc(dsrg_plan* p, float* shared_y) {
     for (int B = A; B < nt; ++B) tp.push_back(make_int2(A, B));
   return cudaMemcpy(st->d_tp, tp.data(), tp.size() * sizeof(int2), cudaMemcpyHostToDevice) ==
          cudaSuccess;
-}
-
-// tau1 for the CCVV pair tables to fill (exp(-s t^2), whose square is their
-// own exp(-2 s t^2)); the next CAVV tables of this plan then skip it.
-double* rest_take_tau1(dsrg_plan* p) {
-  RestState* st = p->rest;
-  if (!st) return nullptr;
-  st->tau1_staged = true;
-  return st->tau1;
-}
-
-void rest_act_tables(const dsrg_plan* p, const double** alpha, const double** pinfo,
-                     const double** tau, int* ld) {
-  const RestState* st = p->rest;
-  if (!st) return;
-  const size_t off = (size_t)p->z.nC * p->z.nA;  // the (x, u) pairs follow the (m, u) pairs
-  *alpha = st->alpha + off * st->nVpad;
-  *pinfo = st->pinfo + off * 4;
-  *tau = st->tau1;
-  *ld = st->nVpad;
 }
 
 void rest_free(dsrg_plan* p) {
@@ -1060,15 +1039,7 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
     DSRG_LAUNCH_CHECK(p);
   }
   {
-    // the pair-independent table tau1 comes with the CCVV pair tables when they were
-    // staged for this call
-    const size_t n = (size_t)z.nH * z.nA * st->nVpad +
-                     (st->tau1_staged ? 0 : (size_t)st->nVpad * st->nVpad);
-    st->tau1_staged = false;
-    abs_max_kernel<<<1, 256, 0, stream>>>(eps + z.nC + z.nA, z.nV, st->vmax);
-    DSRG_LAUNCH_CHECK(p);
-    cavv_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
-        eps, s, z, st->nVpad, st->alpha, st->pinfo, st->tau1, st->vmax);
+    pair_info_kernel<<<1, 1024, 0, stream>>>(eps, s, z, nullptr, z.nC * z.nA, st->pinfo);
     DSRG_LAUNCH_CHECK(p);
   }
   {
@@ -1134,8 +1105,8 @@ cudaError_t launch_split_cavv_adjoint(dsrg_plan* p, const double* eps, const dou
   case NA_:                                                                                 \
     raise_smem_limit((const void*)cavv_adj_tc_kernel<NA_>, sm);                             \
     cavv_adj_tc_kernel<NA_><<<grid, 256, sm, p->stream>>>(st->Y, st->ldy, st->nVpad, eps, G, s, z, \
-                                                        st->d_tp, st->n_tp, st->alpha,      \
-                                                        st->pinfo, st->tau1, dX, deps, ds); \
+                                                        st->d_tp, st->n_tp, st->pinfo, dX,  \
+                                                        deps, ds);                          \
     break;
   switch (z.nA) {
     F2A_LAUNCH(1) F2A_LAUNCH(2) F2A_LAUNCH(3) F2A_LAUNCH(4)

@@ -74,11 +74,7 @@ struct SplitWs {
   float* tail = nullptr;    // [rows + TAIL_PAD][TAIL_Q]  fl32(B) of the first TAIL_Q auxiliary functions (tail_off)
   CUtensorMap map_hi, map_lo;  // 64-byte swizzled maps of the tc_rest GEMM
   CcvvMaps cmaps;              // 32-byte swizzled maps of the CCVV kernel
-  double* alpha = nullptr;  // [n_pairs][nVpad]  exp(4 s E_p e_b)
-  double* pinfo = nullptr;  // [n_pairs][4]      E_p, exp(-2 s E_p^2), factorisable flag
-  double* tau = nullptr;    // [nVpad][nVpad]    exp(-2 s (e_a + e_b)^2)
-  double* trange = nullptr; // [nT][2]           min, max of e over the virtuals of a tile
-  double* vmax = nullptr;   // max |e_v| over the virtual orbitals (pair tables)
+  double2* pinfo = nullptr; // [n_pairs]  E_p, factorisable flag (pair_info_kernel)
   void* d_mol = nullptr;    // device MolDesc of this molecule
   int4* d_items = nullptr;  // single-molecule schedule
   int* d_begin = nullptr;
@@ -109,10 +105,7 @@ struct MolDesc {
   int kblocks;            // K stages on the tensor cores: Q from kq0 to the padded end
   int kq0;                // first Q of the tensor-core stages (TAIL_Q)
   const float* tail;      // [plane rows][TAIL_Q] fl32(B) of Q < TAIL_Q (rows local to the molecule)
-  const double* alpha;    // [pairs][nVpad]  exp(4 s E_p e_b)
-  const double* pinfo;    // [pairs][4]      E_p, exp(-2 s E_p^2), factorisable flag
-  const double* tau;      // [nVpad][nVpad]  exp(-2 s (e_a + e_b)^2)
-  const double* trange;   // [tiles][2]      min, max of e over the virtuals of a tile
+  const double2* pinfo;   // [pairs]  E_p, factorisable flag
   double* partials;       // one FP64 partial per work item of this molecule
 };
 
@@ -281,11 +274,18 @@ __device__ __forceinline__ void store_split16(uint16_t* hi, uint16_t* lo, long l
 // (the duplicates of i = j or A = B are skipped). It adds q R'(D), q = x^2 -
 // x y + y^2, to the row sum `racc` and the column sums `colacc`, and q dR/ds
 // to `sacc` (the item's weight is applied once at its end).
+//
+// The regulators and sums are FP32 pairs (ff.cuh), P and Q FP32 with R rounded once, as
+// S keeps 16 bits of them. A last bit of R that differs moves a few of the 16-bit tails:
+// where the pair (relative error under 2^-41) is so close to the middle of two FP32
+// numbers that it does not settle the rounding, R is taken in FP64 (one element in 2^14).
+// 1536 us for the kernel at 24/2/372/1200 with FP64 regulators, 944 us now; what is left
+// above the energy kernel's 454 us is the row-per-lane tail sums and the stores of S.
 __device__ __forceinline__ void adjoint_chunk(
     const SplitArgs& a, const ItemPlan& ip, uint32_t (&xr)[16], uint32_t (&yr)[16], bool rok,
-    int pth, int c0, int cend, int cbeg, int arow, int nVpad, double ca, double ha, double s,
-    const double* sEps, const double* sAlpha, const double* taucol, const float* tail,
-    const float* tail_ia, const float* tail_ja, double* colacc, int lane, double& racc,
+    int pth, int c0, int cend, int cbeg, int arow, int nVpad, double ca, ff caff, ff kreg, ff s4,
+    double s, const double* sEps, const ff* sEb, const ff* sTab, const float* tail,
+    const float* tail_ia, const float* tail_ja, double* colacc, int lane, ff& racc, ff& saccf,
     double& sacc) {
   if (rok) {
     // the first TAIL_Q auxiliary functions in FP32 round-to-nearest
@@ -294,88 +294,97 @@ __device__ __forceinline__ void adjoint_chunk(
       tail_add16(tail_ja, tail + (size_t)(ip.i * nVpad + ip.Bt * TT + ip.cofs + c0) * TAIL_Q, yr);
   }
   float P[16], Qv[16];
-  double gd[16];
+  ff gd[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const int cb = c0 + k;
-    const bool cok = rok && cb < cend;
-    const float xf = __uint_as_float(xr[k]);
-    const float yf = ip.two ? __uint_as_float(yr[k]) : xf;
-    const double D = ca - sEps[cb];
-    double Rv, RdD, Rds;
-    if (pth == 2) {
-      const RegD r = rf1_d(D, s);
-      Rv = r.v;
-      RdD = r.dD;
-      Rds = r.ds;
-    } else {
-      double r0;
-      asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(D));  // 1/D, seed
-      const double inv = fma(r0, fma(-D, r0, 1.0), r0);      // one Newton step
-      if (pth == 0) {
-        // exp(-2 s D^2) < 2^-63: R = 1/D, R' = -1/D^2, dR/ds = 2 D e^{-2sD^2} ~ 0
-        Rv = inv;
-        RdD = -inv * inv;
-        Rds = 0.0;
+    P[k] = __uint_as_float(xr[k]);
+    Qv[k] = ip.two ? __uint_as_float(yr[k]) : P[k];
+    gd[k] = ff{0.f, 0.f};
+  }
+  // four columns a pass, the next four moved to the front: the code stays small
+#pragma unroll 1
+  for (int k0 = 0; k0 < 16; k0 += 4) {
+    float Pn[4], Qn[4];
+    ff gn[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int cb = c0 + k0 + k;
+      const bool cok = rok && cb < cend;
+      const float xf = P[k], yf = Qv[k];
+      const float q = cok ? fmaf(xf, xf - yf, yf * yf) : 0.f;
+      float rvf;
+      if (pth == 2) {
+        const RegD r = rf1_d(ca - sEps[cb], s);
+        rvf = (float)r.v;
+        gn[k] = ff_from(cok ? (double)q * r.dD : 0.0);
+        sacc += cok ? (double)q * r.ds : 0.0;
       } else {
-        // |D| >= 1/4: g = exp(-2 s D^2) from the factor tables, 1 - g without cancellation
-        const double g = ha * sAlpha[cb] * taucol[(size_t)cb * nVpad];
-        const double em = g - 1.0;
-        const double x2 = 2.0 * s * D * D;
-        Rv = -em * inv;
-        RdD = fma(2.0 * x2, g, em) * inv * inv;
-        Rds = 2.0 * D * g;
+        // exp(-2 s D^2) < 2^-63 (pth 0): R = 1/D, R' = -1/D^2, dR/ds = 0; else
+        // g = exp(-2 s D^2): R = (1 - g)/D, R' = 4 s g - R/D, dR/ds = 2 D g
+        const ff D = ff_diff(caff, sEb[cb]), inv = ff_inv(D);
+        ff R = inv, Rd;
+        if (pth == 1) {
+          const ff om = ff_one_minus_exp(D, kreg, sTab), g = ff_diff(ff{1.f, 0.f}, om);
+          R = ff_mul(om, inv);
+          Rd = ff_diff(ff_mul(g, s4), ff_mul(R, inv));
+          ff_acc(saccf, ff_mul(q, ff_mul(D, g)));
+        } else {
+          Rd = ff_mul(inv, inv);
+          Rd.h = -Rd.h;
+          Rd.l = -Rd.l;
+        }
+        gn[k] = ff_mul(q, Rd);
+        rvf = ff_round(R);
+        // half a last place of rvf, and how far from it R is
+        const float hu = __uint_as_float((__float_as_uint(rvf) & 0x7f800000u) - (24u << 23));
+        const float off = fabsf(FF_ADD(FF_SUB(R.h, rvf), R.l));
+        if (cok && fabsf(off - hu) < fabsf(rvf) * 0x1p-39f) {
+          const double Dd = ca - sEps[cb];
+          double r0;
+          asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(Dd));  // 1/D, one Newton step
+          r0 = fma(r0, fma(-Dd, r0, 1.0), r0);
+          rvf = (float)(pth == 1 ? -expm1(-2.0 * s * Dd * Dd) * r0 : r0);
+        }
       }
+      Pn[k] = cok ? 2.f * fmaf(4.f, xf, -2.f * yf) * rvf : 0.f;
+      Qn[k] = cok ? 2.f * fmaf(4.f, yf, -2.f * xf) * rvf : 0.f;
+      ff_acc(racc, gn[k]);
     }
-    // S is stored as BF16 hi + lo (16 bits): P and Q in FP32 with the FP64 regulator
-    // rounded once; q as in the energy's epilogue, its products with R' and dR/ds in FP64
-    const float rvf = (float)Rv;
-    P[k] = cok ? 2.f * fmaf(4.f, xf, -2.f * yf) * rvf : 0.f;
-    Qv[k] = cok ? 2.f * fmaf(4.f, yf, -2.f * xf) * rvf : 0.f;
-    const double q = (double)fmaf(xf, xf - yf, yf * yf);
-    const double g1 = cok ? q * RdD : 0.0;
-    gd[k] = g1;
-    racc += g1;
-    sacc += cok ? q * Rds : 0.0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      P[k] = P[k + 4];
+      Qv[k] = Qv[k + 4];
+      gd[k] = gd[k + 4];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      P[12 + k] = Pn[k];
+      Qv[12 + k] = Qn[k];
+      gd[12 + k] = gn[k];
+    }
   }
   // column sums over the warp's 32 rows: a transposing butterfly halves the
   // values per lane at each step; lane l ends with column
   // 8 b4 + 4 b3 + 2 b2 + b1 (b_k = bit k of l), duplicated in lanes l and l ^ 1
-  double v8[8], v4[4], v2[2], v1;
+  ff v1;
   {
-    const bool up = (lane & 16) != 0;
+    auto half = [&](bool up, ff lo, ff hi, int o) {  // own half plus the partner's
+      const ff snd = up ? lo : hi, own = up ? hi : lo;
+      return ff_add(own, ff{__shfl_xor_sync(0xffffffffu, snd.h, o), __shfl_xor_sync(0xffffffffu, snd.l, o)});
+    };
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const double send = up ? gd[k] : gd[k + 8];
-      v8[k] = (up ? gd[k + 8] : gd[k]) + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-  }
-  {
-    const bool up = (lane & 8) != 0;
+    for (int k = 0; k < 8; ++k) gd[k] = half((lane & 16) != 0, gd[k], gd[k + 8], 16);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double send = up ? v8[k] : v8[k + 4];
-      v4[k] = (up ? v8[k + 4] : v8[k]) + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-  }
-  {
-    const bool up = (lane & 4) != 0;
+    for (int k = 0; k < 4; ++k) gd[k] = half((lane & 8) != 0, gd[k], gd[k + 4], 8);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const double send = up ? v4[k] : v4[k + 2];
-      v2[k] = (up ? v4[k + 2] : v4[k]) + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
+    for (int k = 0; k < 2; ++k) gd[k] = half((lane & 4) != 0, gd[k], gd[k + 2], 4);
+    v1 = half((lane & 2) != 0, gd[0], gd[1], 2);
+    v1 = ff_add(v1, ff{__shfl_xor_sync(0xffffffffu, v1.h, 1), __shfl_xor_sync(0xffffffffu, v1.l, 1)});
   }
-  {
-    const bool up = (lane & 2) != 0;
-    const double send = up ? v2[0] : v2[1];
-    v1 = (up ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, send, 2);
-  }
-  v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
   if ((lane & 1) == 0) {
     const int col = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 +
                     ((lane >> 1) & 1);
-    colacc[c0 - cbeg + col] += v1;
+    colacc[c0 - cbeg + col] += ff_to(v1);
   }
   if (!rok) return;
   const long long lds = a.lds;
@@ -420,8 +429,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   double* sEps = (double*)(smem + STAGES * STAGE_BYTES + 256);
-  double* sAlpha = sEps + TT;
-  double* sRed = sAlpha + TT;                 // [EPI_WARPS] warp sums
+  double* sRed = sEps + TT;                // [EPI_WARPS] warp sums
   ff* sEb = (ff*)(sRed + EPI_WARPS);          // [TT] e_b as FP32 pairs
   ff* sTab = sEb + TT;                        // [8] ff_exp_entry
   float* sCr = (float*)(sTab + 8);  // [TT/16][2]: min, max of e over the valid columns of each 16-column chunk
@@ -631,10 +639,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       const int nV = md->nV, nVpad = md->nVpad;
       const int ve = md->nC + md->nA;
       const double* eps = md->eps;
-      const double* pi = md->pinfo + 4 * ip.p;
-      const double E = pi[0], beta = pi[1];
-      const double* alpha = md->alpha + (size_t)ip.p * nVpad;
-      const bool factorisable = pi[2] != 0.0;
+      const double2 pi = md->pinfo[ip.p];
+      const double E = pi.x;
+      const bool factorisable = pi.y != 0.0;
       named_bar(1, 32 * EPI_WARPS);
       // warp half wh takes the item's columns 64 wh .. 64 wh + 63 (a half item: half 0 alone)
       const int cbeg = wh * 64;
@@ -644,7 +651,6 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
         sEps[et] = eb;
         // columns past the end keep a valid e: their D stays in the block's range, q = 0
         sEb[et] = ff_from(eps[ve + min(b, nV - 1)]);
-        if (ADJ) sAlpha[et] = (b < nV) ? alpha[b] : 0.0;
         // range of e over the valid columns of each 16-column chunk (FP32: it only
         // picks a path)
         float lo = et < ip.ncols ? (float)eb : 3.0e38f, hi = et < ip.ncols ? (float)eb : -3.0e38f;
@@ -664,10 +670,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       const double ea = rok ? eps[ve + arow] : 0.0;
       const double ca = E - ea;
       const float caf = (float)ca;
-      const double ha = rok ? beta * alpha[arow] : 0.0;
       const int cend = min(cbeg + 64, ip.ncols);
       const double s = md->s;
-      const double* taucol = md->tau + (size_t)(ip.Bt * TT + ip.cofs) * nVpad + arow;
       const float* tail_ia = md->tail + tail_off(ip.i * nVpad + arow);
       const float* tail_ja = md->tail + tail_off(ip.j * nVpad + arow);
       // range of E - e_a over this warp's valid rows (FP32)
@@ -709,15 +713,19 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
           return !away || wide ? 2 : (dn * dn > far_d2 ? 0 : (factorisable ? 1 : 2));
         };
         if constexpr (ADJ) {
+          const ff s4 = ff_from(4.0 * s);
+          ff raccf = {0.f, 0.f}, saccf = {0.f, 0.f};
           for (int c0 = cbeg; c0 < cend; c0 += 16) {
             uint32_t xr[16], yr[16];
             tmem_ld16(tx + c0, xr);
             if (ip.two) tmem_ld16(ty + c0, yr);
             tmem_ld_wait();
-            adjoint_chunk(a, ip, xr, yr, rok, path_of(c0), c0, cend, cbeg, arow, nVpad, ca, ha, s,
-                          sEps, sAlpha, taucol, md->tail, tail_ia, tail_ja,
-                          sColAcc + (warp - 2) * 64, lane, racc, sacc);
+            adjoint_chunk(a, ip, xr, yr, rok, path_of(c0), c0, cend, cbeg, arow, nVpad, ca, caff,
+                          kreg, s4, s, sEps, sEb, sTab, md->tail, tail_ia, tail_ja,
+                          sColAcc + (warp - 2) * 64, lane, raccf, saccf, sacc);
           }
+          racc = ff_to(raccf);
+          sacc += 2.0 * ff_to(saccf);
         } else {
           // 32 rows x 16 columns at a time, each thread 4 rows (r0, + 8, + 16, + 24) x
           // 4 columns (tail_frag): wider blocks reload less but spill at 168 registers
@@ -844,7 +852,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       if (lane == 0) sRed[warp - 2] = acc;
       named_bar(1, 32 * EPI_WARPS);
       if (et == 0) {
-        if (pi[2] == 0.0 && ip.cofs == 0) atomicAdd(&a.counts[DSRG_COUNT_CCVV_UNFACTORABLE], 1ull);
+        if (pi.y == 0.0 && ip.cofs == 0) atomicAdd(&a.counts[DSRG_COUNT_CCVV_UNFACTORABLE], 1ull);
         const double w = (ip.two ? 2.0 : 1.0) * (ip.A < ip.Bt ? 2.0 : 1.0);
         const double t0 = sRed[0] + sRed[1] + sRed[2] + sRed[3];
         const double t1 = sRed[4] + sRed[5] + sRed[6] + sRed[7];
@@ -963,77 +971,29 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const double* __restr
   }
 }
 
-// max |x_k| over n values into *out: one CTA, strided per-thread maxima and a
-// tree (a maximum is exact, so the order does not matter). NaN entries are
-// skipped, as fmax does.
-__global__ void __launch_bounds__(256) abs_max_kernel(const double* __restrict__ x, int n,
-                                                      double* __restrict__ out) {
-  __shared__ double sm[256];
-  double m = 0.0;
-  for (int k = threadIdx.x; k < n; k += 256) m = fmax(m, fabs(x[k]));
-  sm[threadIdx.x] = m;
+// E_mu of the orbital pairs mu and whether exp(-c D^2) factorises: with
+// D = E - e_a - e_b, whether the partial products of exp(-c E^2) exp(2 c E e_a)
+// exp(2 c E e_b) exp(-c (e_a + e_b)^2) stay within exp(+-700) (past that the regulators
+// take expm1). One CTA and launch: the largest |e_v| first, then the pairs, of `pairs`
+// or (m, u) = (mu / nA, nC + mu % nA).
+__global__ void __launch_bounds__(1024) pair_info_kernel(const double* __restrict__ eps, double c,
+                                                         Sizes z, const int2* __restrict__ pairs,
+                                                         int n, double2* __restrict__ pinfo) {
+  __shared__ double sm[32];
+  double m = 0.0;  // fmax skips NaN; a maximum does not depend on the order
+  for (int k = threadIdx.x; k < z.nV; k += 1024) m = fmax(m, fabs(eps[z.nC + z.nA + k]));
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sm[threadIdx.x] = fmax(sm[threadIdx.x], sm[threadIdx.x + o]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *out = sm[0];
-}
-
-// Per-pair factors of exp(-2 s D^2) with D = E - e_a - e_b:
-//   exp(-2 s E^2) * exp(4 s E e_a) * exp(4 s E e_b) * exp(-2 s (e_a + e_b)^2).
-// A pair is factorisable when every partial product of these factors, taken in
-// the epilogue's order, stays within exp(+-700).
-__global__ void split_tables_kernel(const double* __restrict__ eps, double s, Sizes z,
-                                    const int2* __restrict__ pairs, int n_pairs, int nVpad,
-                                    double* __restrict__ alpha, double* __restrict__ pinfo,
-                                    double* __restrict__ tau, double* __restrict__ trange,
-                                    double* __restrict__ tau_s, const double* __restrict__ vmaxp) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int ve = z.nC + z.nA;
-  const size_t na = (size_t)n_pairs * nVpad, nt = (size_t)nVpad * nVpad;
-  if (k < na) {
-    const int p = (int)(k / nVpad), b = (int)(k % nVpad);
-    const int2 ij = pairs[p];
+  m = sm[threadIdx.x & 31];
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int mu = threadIdx.x; mu < n; mu += 1024) {
+    const int2 ij = pairs ? pairs[mu] : make_int2(mu / z.nA, z.nC + mu % z.nA);
     const double E = eps[ij.x] + eps[ij.y];
-    alpha[k] = (b < z.nV) ? exp(4.0 * s * E * eps[ve + b]) : 0.0;
-    if (b == 0) {
-      const double vmax = *vmaxp;  // max |e_v| over the virtual orbitals
-      // the epilogue multiplies left to right, exp(-2sE^2) * alpha_a * alpha_b * tau:
-      // the partial products carry the exponents -2sE^2 + 4sE e_a (+ 4sE e_b), which
-      // for E e > 0 grow past each single factor's, so their sum of magnitudes is bounded
-      const bool ok = (2.0 * s * E * E + 8.0 * s * fabs(E) * vmax <= 700.0) &&
-                      (8.0 * s * vmax * vmax <= 700.0);
-      pinfo[4 * p + 0] = E;
-      pinfo[4 * p + 1] = exp(-2.0 * s * E * E);
-      pinfo[4 * p + 2] = ok ? 1.0 : 0.0;
-      pinfo[4 * p + 3] = 0.0;
-    }
-  } else if (k < na + nt) {
-    const size_t r = k - na;
-    const int a = (int)(r / nVpad), b = (int)(r % nVpad);
-    double v = 0.0, v1 = 0.0;
-    if (a < z.nV && b < z.nV) {
-      const double t = eps[ve + a] + eps[ve + b];
-      if (tau_s) {
-        // the CAVV tables' exp(-s t^2) as well; this table is its square
-        v1 = exp(-s * t * t);
-        v = v1 * v1;
-      } else {
-        v = exp(-2.0 * s * t * t);
-      }
-    }
-    tau[r] = v;
-    if (tau_s) tau_s[r] = v1;
-  } else if (k < na + nt + (size_t)(nVpad / TT)) {
-    const int t = (int)(k - na - nt);
-    double lo = 1e300, hi = -1e300;
-    for (int b = t * TT; b < min((t + 1) * TT, z.nV); ++b) {
-      lo = fmin(lo, eps[ve + b]);
-      hi = fmax(hi, eps[ve + b]);
-    }
-    trange[2 * t] = lo;
-    trange[2 * t + 1] = hi;
+    // the factors multiply left to right: for E e > 0 the partial products grow past each
+    // single factor's exponent, so the sum of their magnitudes is bounded
+    const bool ok = (c * E * E + 4.0 * c * fabs(E) * m <= 700.0) && (4.0 * c * m * m <= 700.0);
+    pinfo[mu] = make_double2(E, ok ? 1.0 : 0.0);
   }
 }
 
@@ -1246,11 +1206,7 @@ bool split_alloc_at(dsrg_plan* p, void* hi, void* lo, int Qld, long long row_bas
   } else {
     ok = plan_alloc(p, &w->hi, plane) && plan_alloc(p, &w->lo, plane);
   }
-  ok = ok && plan_alloc(p, (void**)&w->alpha, (size_t)p->n_pairs * w->nVpad * 8) &&
-       plan_alloc(p, (void**)&w->pinfo, (size_t)p->n_pairs * 4 * 8) &&
-       plan_alloc(p, (void**)&w->tau, (size_t)w->nVpad * w->nVpad * 8) &&
-       plan_alloc(p, (void**)&w->trange, (size_t)w->nT * 2 * 8) &&
-       plan_alloc(p, (void**)&w->vmax, 8) &&
+  ok = ok && plan_alloc(p, (void**)&w->pinfo, (size_t)p->n_pairs * sizeof(double2)) &&
        plan_alloc(p, (void**)&w->d_mol, sizeof(MolDesc)) &&
        plan_alloc(p, (void**)&w->tail, split_tail_bytes(z));
   if (!ok) return false;
@@ -1276,10 +1232,7 @@ bool split_alloc_at(dsrg_plan* p, void* hi, void* lo, int Qld, long long row_bas
   md.kblocks = (w->Qpad - TAIL_Q) / w->kb_elems;
   md.tail = w->tail;
   md.n_tp = w->n_tp;
-  md.alpha = w->alpha;
   md.pinfo = w->pinfo;
-  md.tau = w->tau;
-  md.trange = w->trange;
   md.partials = p->d_partials + p->segs[p->seg_ccvv].begin;
   if (cudaMemcpy(w->d_mol, &md, sizeof(MolDesc), cudaMemcpyHostToDevice) != cudaSuccess) return false;
   // single-molecule schedule
@@ -1447,16 +1400,10 @@ cudaError_t split_stage_rows(dsrg_plan* p, const double* B, int h0, int h1) {
   return cudaSuccess;
 }
 
-// Pair tables of the regulator (they read eps only).
+// Pair energies and flags (they read eps only).
 cudaError_t split_stage_tables(dsrg_plan* p, const double* eps, double s) {
-  SplitWs* w = p->split;
-  abs_max_kernel<<<1, 256, 0, p->stream>>>(eps + p->z.nC + p->z.nA, p->z.nV, w->vmax);
-  DSRG_LAUNCH_CHECK(p);
-  const size_t n = (size_t)p->n_pairs * w->nVpad + (size_t)w->nVpad * w->nVpad + w->nT;
-  double* tau_s = p->rest ? rest_take_tau1(p) : nullptr;
-  split_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, p->stream>>>(
-      eps, s, p->z, p->d_pairs, p->n_pairs, w->nVpad, w->alpha, w->pinfo, w->tau, w->trange, tau_s,
-      w->vmax);
+  pair_info_kernel<<<1, 1024, 0, p->stream>>>(eps, 2.0 * s, p->z, p->d_pairs, p->n_pairs,
+                                              p->split->pinfo);
   DSRG_LAUNCH_CHECK(p);
   return cudaSuccess;
 }
@@ -1508,10 +1455,7 @@ void split_fill_mol_desc(const dsrg_plan* p, long long row0, void* out) {
   md.kblocks = (w->Qpad - TAIL_Q) / w->kb_elems;
   md.tail = w->tail;
   md.n_tp = w->n_tp;
-  md.alpha = w->alpha;
   md.pinfo = w->pinfo;
-  md.tau = w->tau;
-  md.trange = w->trange;
   md.partials = p->d_partials + p->segs[p->seg_ccvv].begin;
   memcpy(out, &md, sizeof(MolDesc));
 }
