@@ -31,24 +31,28 @@ namespace dsrg {
 // ---------------------------------------------------------------------------
 // Generic FP64 GEMM with composite K index:
 //   C[i*ci + j*cj] (+)= alpha * sum_{l1<L1, l2<L2} A[i*ai + l1*a1 + l2*a2] * Bm[l1*b1 + l2*b2 + j*bj]
-// 64 x 64 tiles, 256 threads, K chunks of 16 over l = l1*L2 + l2.
+// Tiles of 16 R x 16 R, 256 threads with R x R values each, K chunks of 16 over
+// l = l1*L2 + l2. An SM does 2 FP64 FMAs a clock whatever the tile, so small tiles cost
+// little and a product too small for 64 x 64 tiles to fill the chip takes smaller ones.
 // ---------------------------------------------------------------------------
+template <int R>
 __global__ void __launch_bounds__(256) gemm_fp64_kernel(GemmArgs g) {
-  __shared__ double sA[16][65], sB[16][65];
+  constexpr int T = 16 * R;
+  __shared__ double sA[16][T + 1], sB[16][T + 1];
   g.A += blockIdx.z * g.sa;
   g.Bm += blockIdx.z * g.sb;
   g.C += blockIdx.z * g.sc;
-  const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+  const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const long long L = (long long)g.L1 * g.L2;
-  double acc[4][4];
+  double acc[R][R];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.0;
+    for (int c = 0; c < R; ++c) acc[r][c] = 0.0;
   for (long long l0 = 0; l0 < L; l0 += 16) {
-    for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-      const int ll = e / 64, c = e % 64;
+    for (int e = threadIdx.x; e < 16 * T; e += 256) {
+      const int ll = e / T, c = e % T;
       const long long l = l0 + ll;
       double va = 0.0, vb = 0.0;
       if (l < L) {
@@ -62,26 +66,26 @@ __global__ void __launch_bounds__(256) gemm_fp64_kernel(GemmArgs g) {
     __syncthreads();
 #pragma unroll 4
     for (int ll = 0; ll < 16; ++ll) {
-      double ra[4], rb[4];
+      double ra[R], rb[R];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        ra[r] = sA[ll][ty * 4 + r];
-        rb[r] = sB[ll][tx * 4 + r];
+      for (int r = 0; r < R; ++r) {
+        ra[r] = sA[ll][ty * R + r];
+        rb[r] = sB[ll][tx * R + r];
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fma(ra[r], rb[c], acc[r][c]);
+        for (int c = 0; c < R; ++c) acc[r][c] = fma(ra[r], rb[c], acc[r][c]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = i0 + ty * 4 + r;
+  for (int r = 0; r < R; ++r) {
+    const int i = i0 + ty * R + r;
     if (i >= g.M) continue;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int j = j0 + tx * 4 + c;
+    for (int c = 0; c < R; ++c) {
+      const int j = j0 + tx * R + c;
       if (j >= g.N) continue;
       double* p = g.C + (long long)i * g.ci + (long long)j * g.cj;
       *p = g.accumulate ? fma(g.alpha, acc[r][c], *p) : g.alpha * acc[r][c];
@@ -105,10 +109,20 @@ struct GradWs {
   double *dK1 = nullptr, *dK2 = nullptr, *dK3 = nullptr, *dM = nullptr;
 };
 
+// The largest tile of which every SM gets two, else the smallest: the adjoints' products
+// at 10/4/60/200 (M = 200, N = 10 to 60, K = 40 to 600, 1 to 10 problems) took 338 us each
+// with 64 x 64 tiles on 16 to 40 SMs, 57 us with 16 x 16 ones.
 cudaError_t launch_gemm_fp64(cudaStream_t st, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, g.nb);
-  gemm_fp64_kernel<<<grid, 256, 0, st>>>(g);
+  auto grid = [&](int t) { return dim3((g.N + t - 1) / t, (g.M + t - 1) / t, g.nb); };
+  auto ctas = [&](int t) { const dim3 d = grid(t); return (double)d.x * d.y * d.z; };
+  constexpr double FILL = 2.0 * 152;
+  if (ctas(64) >= FILL || (g.M + 15) / 16 > 65535)
+    gemm_fp64_kernel<4><<<grid(64), 256, 0, st>>>(g);
+  else if (ctas(32) >= FILL)
+    gemm_fp64_kernel<2><<<grid(32), 256, 0, st>>>(g);
+  else
+    gemm_fp64_kernel<1><<<grid(16), 256, 0, st>>>(g);
   return cudaGetLastError();
 }
 
@@ -318,8 +332,7 @@ __global__ void __launch_bounds__(256) cavv_adj_kernel(
 #pragma unroll
     for (int u = 0; u < NA; ++u) {
       const double D = base + eps[z.nC + u];
-      Rv[u] = rv_d(D, s);
-      Rt[u] = rt_d(D, s);
+      rtv_d(D, s, Rt[u], Rv[u]);
     }
     double P[NA], Pt[NA];  // 2 X - X^T at (a,b) and at (b,a)
 #pragma unroll
@@ -499,8 +512,7 @@ __global__ void __launch_bounds__(256) ccav_adj_kernel(
     double P[NA_MAX];
     for (int u = 0; u < nA; ++u) {
       const double D = base - eps[nC + u];
-      Rv[u] = rv_d(D, s);
-      Rt[u] = rt_d(D, s);
+      rtv_d(D, s, Rt[u], Rv[u]);
       P[u] = 2.0 * (double)Z[(u * nC + m) * nC + n] - (double)Z[(u * nC + n) * nC + m];
     }
     double gsum = 0.0;
@@ -593,92 +605,121 @@ __device__ __forceinline__ size_t L3I(int n2, int U, int V, int W, int X, int Y,
   return (((((size_t)U * n2 + V) * n2 + W) * n2 + X) * n2 + Y) * n2 + Z;
 }
 
-// (A1) term adjoints landing on W1-shaped tables: d(vt), d(t) direct, d(Ti).
+// (A1) term adjoints landing on W1-shaped tables: d(vt), d(t) direct, d(Ti). Every
+// factor conserves spin (W1[I,U,A,X] = 0 unless s_I + s_U = s_A + s_X, the cumulant
+// unless s_U + s_V = s_X + s_Y, gamma and eta between different spins), so only the
+// spin-allowed elements are formed, and only spin-allowed terms of their sums. A thread
+// is one (I, U, A, spatial X), the spin of A outermost: a warp's sums have one shape.
+// (All elements and terms: 656 us at 10/4/60/200, 108 us now.)
 __global__ void adj_w1_terms_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.w1n) return;
-  const int X = (int)(k % d.nA2);
-  const int A = (int)((k / d.nA2) % d.nP2);
-  const int U = (int)((k / ((size_t)d.nA2 * d.nP2)) % d.nA2);
-  const int I = (int)(k / ((size_t)d.nA2 * d.nP2 * d.nA2));
+  const size_t k0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (2 * k0 >= a.w1n) return;
+  const int nA = d.nA2 / 2, nP = d.nP2 / 2, sA = (int)((k0 / ((size_t)nA * nP)) & 1);
+  const int A = 2 * (int)((k0 / nA) % nP) + sA;
+  const int U = (int)((k0 / ((size_t)nA * d.nP2)) % d.nA2);
+  const int I = (int)(k0 / ((size_t)nA * d.nP2 * d.nA2));
+  const int sI = I & 1, sU = U & 1, sX = sI + sU - sA;
+  const int X = 2 * (int)(k0 % nA) + (sX == 1);
+  const size_t k = W1(d, I, U, A, X);
+  a.dW1Vt[k ^ 1] = 0.0;  // X of the other spin
+  a.dW1T[k ^ 1] = 0.0;
+  a.dTi[k ^ 1] = 0.0;
+  if (sX < 0 || sX > 1) {
+    a.dW1Vt[k] = 0.0;
+    a.dW1T[k] = 0.0;
+    a.dTi[k] = 0.0;
+    return;
+  }
   const bool Iact = I >= d.nC2, Avir = A >= d.nA2;
   const double* lam = a.lam;
   const double* gA = a.gA;
   double dvt = 0.0, dt = 0.0, dti = 0.0;
   // term I (all elements): vt_{jx}^{bu} at (J=I, x=U, b=A, u=X); Ti at (J=I, V=U, B=A, Y=X)
-  for (int V = 0; V < d.nA2; ++V)
-    for (int Y = 0; Y < d.nA2; ++Y) dvt = fma(a.Ti[W1(d, I, V, A, Y)], lam[LM(d, X, V, U, Y)], dvt);
-  for (int Uu = 0; Uu < d.nA2; ++Uu)
-    for (int Xx = 0; Xx < d.nA2; ++Xx)
+  for (int V = 0; V < d.nA2; ++V) {
+    const int sy = sI + (V & 1) - sA;
+    if (sy < 0 || sy > 1) continue;
+    for (int Y = sy; Y < d.nA2; Y += 2) dvt = fma(a.Ti[W1(d, I, V, A, Y)], lam[LM(d, X, V, U, Y)], dvt);
+  }
+  for (int Uu = 0; Uu < d.nA2; ++Uu) {
+    const int sx = sA + (Uu & 1) - sI;
+    if (sx < 0 || sx > 1) continue;
+    for (int Xx = sx; Xx < d.nA2; Xx += 2)
       dti = fma(a.W1Vt[W1(d, I, Xx, A, Uu)], lam[LM(d, Uu, U, Xx, X)], dti);
+  }
   if (Iact && Avir) {
-    const int Xa = I - d.nC2;  // the active hole of the first slot
+    const int Xa = I - d.nC2;  // the active hole of the first slot (same spin as I)
     // B: 1/2 vt[Xa,Y=U,e,V=X] t1[U',e] lam[U',V,Xa,Y]
-    for (int Uu = 0; Uu < d.nA2; ++Uu)
+    for (int Uu = sA; Uu < d.nA2; Uu += 2)
       dvt = fma(0.5 * a.t1[(size_t)(d.nC2 + Uu) * d.nP2 + A], lam[LM(d, Uu, X, Xa, U)], dvt);
     // GVA: 1/4 sum lam[U',V',Xa,Y] W1Vt[Xa,Y,e,C] tg[U',V',C], tg = sum_A' eta[C][A'] W1T[U',V',e,A']
-    for (int Uu = 0; Uu < d.nA2; ++Uu)
-      for (int Vv = 0; Vv < d.nA2; ++Vv) {
+    for (int Uu = 0; Uu < d.nA2; ++Uu) {
+      const int sv = sI + sU - (Uu & 1);
+      if (sv < 0 || sv > 1) continue;
+      for (int Vv = sv; Vv < d.nA2; Vv += 2) {
         double tg = 0.0;
-        for (int Ap = 0; Ap < d.nA2; ++Ap)
+        for (int Ap = sX; Ap < d.nA2; Ap += 2)
           tg = fma(eAA(d, gA, X, Ap), a.W1T[W1(d, d.nC2 + Uu, Vv, A, Ap)], tg);
         dvt = fma(0.25 * lam[LM(d, Uu, Vv, Xa, U)], tg, dvt);
       }
+    }
     // D: 1/2 ft[Xx,e] t[Ua=Xa, V=U, e, Y=X] lam[Ua,V,Xx,Y]  -> d(t)
-    for (int Xx = 0; Xx < d.nA2; ++Xx)
+    for (int Xx = sA; Xx < d.nA2; Xx += 2)
       dt = fma(0.5 * a.ft[(size_t)(d.nC2 + Xx) * d.nP2 + A], lam[LM(d, Xa, U, Xx, X)], dt);
     // GVA -> d(t) at (Ua=Xa, Vv=U, e, A'=X): sum_C eta[C][A'] dtg[Ua,Vv,C]
-    for (int C = 0; C < d.nA2; ++C) {
+    for (int C = sX; C < d.nA2; C += 2) {
       const double ec = eAA(d, gA, C, X);
       if (ec == 0.0) continue;
       double dtg = 0.0;
-      for (int Xx = 0; Xx < d.nA2; ++Xx)
-        for (int Y = 0; Y < d.nA2; ++Y)
+      for (int Xx = 0; Xx < d.nA2; ++Xx) {
+        const int sy = sI + sU - (Xx & 1);
+        if (sy < 0 || sy > 1) continue;
+        for (int Y = sy; Y < d.nA2; Y += 2)
           dtg = fma(lam[LM(d, Xa, U, Xx, Y)], a.W1Vt[W1(d, d.nC2 + Xx, Y, A, C)], dtg);
+      }
       dt = fma(0.25 * ec, dtg, dt);
     }
     // F7: vt[Ya, Z=U, e, V=X]: 1/2 sum gA[Ya,W] gA[Z,X'] eta[U',V] W1T[W, X', e, U']
-    for (int W = 0; W < d.nA2; ++W) {
+    for (int W = sI; W < d.nA2; W += 2) {
       const double g1 = gAA(d, gA, Xa, W);
       if (g1 == 0.0) continue;
-      for (int Xx = 0; Xx < d.nA2; ++Xx) {
+      for (int Xx = sU; Xx < d.nA2; Xx += 2) {
         const double g2 = gAA(d, gA, U, Xx);
         if (g2 == 0.0) continue;
-        for (int Uu = 0; Uu < d.nA2; ++Uu)
+        for (int Uu = sX; Uu < d.nA2; Uu += 2)
           dvt = fma(0.5 * g1 * g2 * eAA(d, gA, Uu, X), a.W1T[W1(d, d.nC2 + W, Xx, A, Uu)], dvt);
       }
     }
     // F7 -> d(t) at (Wa=Xa, X'=U, e, U'=X): 1/2 sum gA[Y,Wa] gA[Z,X'] eta[U',V] W1Vt[Y, Z, e, V]
-    for (int Y = 0; Y < d.nA2; ++Y) {
+    for (int Y = sI; Y < d.nA2; Y += 2) {
       const double g1 = gAA(d, gA, Y, Xa);
       if (g1 == 0.0) continue;
-      for (int Z = 0; Z < d.nA2; ++Z) {
+      for (int Z = sU; Z < d.nA2; Z += 2) {
         const double g2 = gAA(d, gA, Z, U);
         if (g2 == 0.0) continue;
-        for (int V = 0; V < d.nA2; ++V)
+        for (int V = sX; V < d.nA2; V += 2)
           dt = fma(0.5 * g1 * g2 * eAA(d, gA, X, V), a.W1Vt[W1(d, d.nC2 + Y, Z, A, V)], dt);
       }
     }
   }
   if (!Iact && !Avir) {
     // C: -1/2 vt[M, Y=U, U'=A, V=X] t1[M, X'] lam[A, X, X', U]
-    for (int Xx = 0; Xx < d.nA2; ++Xx)
+    for (int Xx = sI; Xx < d.nA2; Xx += 2)
       dvt = fma(-0.5 * a.t1[(size_t)I * d.nP2 + Xx], lam[LM(d, A, X, Xx, U)], dvt);
     // F8: vt[M, W=U, V'=A, Y=X]: 1/2 sum gA[W,Z] eta[U',V'] eta[X',Y] W1T[M, Z, U', X']
-    for (int Z = 0; Z < d.nA2; ++Z) {
+    for (int Z = sU; Z < d.nA2; Z += 2) {
       const double g = gAA(d, gA, U, Z);
       if (g == 0.0) continue;
-      for (int Uu = 0; Uu < d.nA2; ++Uu)
-        for (int Xx = 0; Xx < d.nA2; ++Xx)
+      for (int Uu = sA; Uu < d.nA2; Uu += 2)
+        for (int Xx = sX; Xx < d.nA2; Xx += 2)
           dvt = fma(0.5 * g * eAA(d, gA, Uu, A) * eAA(d, gA, Xx, X), a.W1T[W1(d, I, Z, Uu, Xx)], dvt);
     }
     // F8 -> d(t) at (M, Z=U, U'=A, X'=X): 1/2 sum gA[W,Z] eta[U',V'] eta[X',Y] W1Vt[M, W, V', Y]
-    for (int W = 0; W < d.nA2; ++W) {
+    for (int W = sU; W < d.nA2; W += 2) {
       const double g = gAA(d, gA, W, U);
       if (g == 0.0) continue;
-      for (int V = 0; V < d.nA2; ++V)
-        for (int Y = 0; Y < d.nA2; ++Y)
+      for (int V = sA; V < d.nA2; V += 2)
+        for (int Y = sX; Y < d.nA2; Y += 2)
           dt = fma(0.5 * g * eAA(d, gA, A, V) * eAA(d, gA, X, Y), a.W1Vt[W1(d, I, W, V, Y)], dt);
     }
   }
@@ -732,17 +773,17 @@ __global__ void adj_w1_terms_kernel(ActAdjArgs a) {
   }
   if (!Iact && Avir) {
     // F6: vt[M, X'=U, e, V'=X]: sum gA[X',Y] eta[U',V'] W1T[M, Y, e, U']
-    for (int Y = 0; Y < d.nA2; ++Y) {
+    for (int Y = sU; Y < d.nA2; Y += 2) {
       const double g = gAA(d, gA, U, Y);
       if (g == 0.0) continue;
-      for (int Uu = 0; Uu < d.nA2; ++Uu)
+      for (int Uu = sX; Uu < d.nA2; Uu += 2)
         dvt = fma(g * eAA(d, gA, Uu, X), a.W1T[W1(d, I, Y, A, Uu)], dvt);
     }
     // F6 -> d(t) at (M, Y=U, e, U'=X): sum gA[X',Y] eta[U',V'] W1Vt[M, X', e, V']
-    for (int Xx = 0; Xx < d.nA2; ++Xx) {
+    for (int Xx = sU; Xx < d.nA2; Xx += 2) {
       const double g = gAA(d, gA, Xx, U);
       if (g == 0.0) continue;
-      for (int V = 0; V < d.nA2; ++V) dt = fma(g * eAA(d, gA, X, V), a.W1Vt[W1(d, I, Xx, A, V)], dt);
+      for (int V = sX; V < d.nA2; V += 2) dt = fma(g * eAA(d, gA, X, V), a.W1Vt[W1(d, I, Xx, A, V)], dt);
     }
   }
   a.dW1Vt[k] = dvt;
@@ -753,35 +794,52 @@ __global__ void adj_w1_terms_kernel(ActAdjArgs a) {
 // (A2) term adjoints on W2-shaped tables (E, H, F5).
 __global__ void adj_w2_terms_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.w2n) return;
-  const int Y = (int)(k % d.nA2);
-  const int X = (int)((k / d.nA2) % d.nA2);
-  const int J = (int)((k / ((size_t)d.nA2 * d.nA2)) % d.nH2);
-  const int I = (int)(k / ((size_t)d.nA2 * d.nA2 * d.nH2));
+  const size_t k0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (2 * k0 >= a.w2n) return;
+  const int nA = d.nA2 / 2, sX = (int)((k0 / (nA * nA)) & 1);
+  const int X = 2 * (int)((k0 / nA) % nA) + sX;
+  const int J = (int)((k0 / ((size_t)nA * d.nA2)) % d.nH2);
+  const int I = (int)(k0 / ((size_t)nA * d.nA2 * d.nH2));
+  const int sI = I & 1, sJ = J & 1, sY = sI + sJ - sX;
+  const int Y = 2 * (int)(k0 % nA) + (sY == 1);
+  const size_t k = W2(d, I, J, X, Y);
+  a.dW2Vt[k ^ 1] = 0.0;  // as in adj_w1_terms_kernel: the spin-allowed elements and terms
+  a.dW2T[k ^ 1] = 0.0;
+  if (sY < 0 || sY > 1) {
+    a.dW2Vt[k] = 0.0;
+    a.dW2T[k] = 0.0;
+    return;
+  }
   const double* lam = a.lam;
   const double* gA = a.gA;
   double dvt = 0.0, dt = 0.0;
   // H: vt[K=I, L=J, U=X, V=Y] * Th[K,L,X',Y'] lam[U,V,X',Y'] / 8
   {
-    const int i0 = (I < d.nC2) ? I : d.nC2, i1 = (I < d.nC2) ? I + 1 : d.nH2;
-    const int j0 = (J < d.nC2) ? J : d.nC2, j1 = (J < d.nC2) ? J + 1 : d.nH2;
-    for (int Xx = 0; Xx < d.nA2; ++Xx)
-      for (int Yy = 0; Yy < d.nA2; ++Yy) {
+    // gamma couples core orbitals to themselves, active ones to the same spin
+    const int i0 = (I < d.nC2) ? I : d.nC2 + sI, i1 = (I < d.nC2) ? I + 1 : d.nH2;
+    const int j0 = (J < d.nC2) ? J : d.nC2 + sJ, j1 = (J < d.nC2) ? J + 1 : d.nH2;
+    for (int Xx = 0; Xx < d.nA2; ++Xx) {
+      const int sy = sI + sJ - (Xx & 1);
+      if (sy < 0 || sy > 1) continue;
+      for (int Yy = sy; Yy < d.nA2; Yy += 2) {
         double th = 0.0;
-        for (int I2 = i0; I2 < i1; ++I2)
-          for (int J2 = j0; J2 < j1; ++J2)
+        for (int I2 = i0; I2 < i1; I2 += 2)
+          for (int J2 = j0; J2 < j1; J2 += 2)
             th = fma(gH(d, gA, I, I2) * gH(d, gA, J, J2), a.W2T[W2(d, I2, J2, Xx, Yy)], th);
         dvt = fma(0.125 * th, lam[LM(d, X, Y, Xx, Yy)], dvt);
       }
+    }
     // H -> d(t) at (I'=I, J'=J, X'=X, Y'=Y): sum_{K,L} gamma[K,I] gamma[L,J] dTh[K,L,X,Y]
-    for (int K = i0; K < i1; ++K)
-      for (int L = j0; L < j1; ++L) {
+    for (int K = i0; K < i1; K += 2)
+      for (int L = j0; L < j1; L += 2) {
         const double gg = gH(d, gA, K, I) * gH(d, gA, L, J);
         if (gg == 0.0) continue;
         double dth = 0.0;
-        for (int U = 0; U < d.nA2; ++U)
-          for (int V = 0; V < d.nA2; ++V) dth = fma(a.W2Vt[W2(d, K, L, U, V)], lam[LM(d, U, V, X, Y)], dth);
+        for (int U = 0; U < d.nA2; ++U) {
+          const int sv = sX + sY - (U & 1);
+          if (sv < 0 || sv > 1) continue;
+          for (int V = sv; V < d.nA2; V += 2) dth = fma(a.W2Vt[W2(d, K, L, U, V)], lam[LM(d, U, V, X, Y)], dth);
+        }
         dt = fma(0.125 * gg, dth, dt);
       }
   }
@@ -793,76 +851,87 @@ __global__ void adj_w2_terms_kernel(ActAdjArgs a) {
   }
   // F5: 1/4 vt[M,N,V,Y] t[M,N,U,X] eta[U,V] eta[X,Y] (both core)
   if (I < d.nC2 && J < d.nC2) {
-    for (int U = 0; U < d.nA2; ++U)
-      for (int Xx = 0; Xx < d.nA2; ++Xx)
+    for (int U = sX; U < d.nA2; U += 2)
+      for (int Xx = sY; Xx < d.nA2; Xx += 2)
         dvt = fma(0.25 * eAA(d, gA, U, X) * eAA(d, gA, Xx, Y), a.W2T[W2(d, I, J, U, Xx)], dvt);
-    for (int V = 0; V < d.nA2; ++V)
-      for (int Yy = 0; Yy < d.nA2; ++Yy)
+    for (int V = sX; V < d.nA2; V += 2)
+      for (int Yy = sY; Yy < d.nA2; Yy += 2)
         dt = fma(0.25 * eAA(d, gA, X, V) * eAA(d, gA, Y, Yy), a.W2Vt[W2(d, I, J, V, Yy)], dt);
   }
   a.dW2Vt[k] = dvt;
   a.dW2T[k] = dt;
 }
 
-// (A3) term adjoints on t1 and ft ([2nH][2nP]) from terms A-E.
-__global__ void adj_t1ft_terms_kernel(ActAdjArgs a) {
+// (A3) term adjoints on t1 and ft ([2nH][2nP]) from terms A-E, one warp per element
+// (spin-conserving ones; the others stay zero). With one thread, up to 500 products in a
+// row: 188 us at 10/4/60/200, 9 us now.
+__global__ void __launch_bounds__(256) adj_t1ft_terms_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= d.nH2 * d.nP2) return;
-  const int I = k / d.nP2, A = k % d.nP2;
+  const int w = (int)(((size_t)blockIdx.x * 256 + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (w >= d.nH2 * (d.nP2 / 2)) return;
+  const int I = w / (d.nP2 / 2), sp = I & 1, A = 2 * (w % (d.nP2 / 2)) + sp, nA = d.nA2 / 2;
   const double* lam = a.lam;
   const double* gA = a.gA;
   double dt1 = 0.0, dft = 0.0;
   // A: dft[I,A] = sum_J gamma[J,I] te[J,A], te[J,A] = sum_A' eta[A',A] t1[J,A']
   //    dt1[I,A] = sum_B eta[A,B] gf[I,B], gf[I,B] = sum_K gamma[I,K] ft[K,B]
   {
-    const int j0 = (I < d.nC2) ? I : d.nC2, j1 = (I < d.nC2) ? I + 1 : d.nH2;
-    const int b0 = (A < d.nA2) ? 0 : A, b1 = (A < d.nA2) ? d.nA2 : A + 1;
-    for (int J = j0; J < j1; ++J) {
-      const double g = gH(d, gA, J, I);
-      if (g == 0.0) continue;
-      double te = 0.0;
-      for (int Ap = b0; Ap < b1; ++Ap) te = fma(eP(d, gA, Ap, A), a.t1[(size_t)J * d.nP2 + Ap], te);
-      dft = fma(g, te, dft);
-    }
-    for (int Bp = b0; Bp < b1; ++Bp) {
-      const double e = eP(d, gA, A, Bp);
-      if (e == 0.0) continue;
-      double gf = 0.0;
-      for (int K = j0; K < j1; ++K) gf = fma(gH(d, gA, I, K), a.ft[(size_t)K * d.nP2 + Bp], gf);
-      dt1 = fma(e, gf, dt1);
+    const bool ic = I < d.nC2, av = A >= d.nA2;
+    const int nj = ic ? 1 : nA, nb = av ? 1 : nA;
+    for (int e = lane; e < nj * nb; e += 32) {
+      const int J = ic ? I : d.nC2 + 2 * (e / nb) + sp, Bp = av ? A : 2 * (e % nb) + sp;
+      const size_t o = (size_t)J * d.nP2 + Bp;
+      dft = fma(gH(d, gA, J, I) * eP(d, gA, Bp, A), a.t1[o], dft);
+      dt1 = fma(gH(d, gA, I, J) * eP(d, gA, A, Bp), a.ft[o], dt1);
     }
   }
   if (I >= d.nC2 && A >= d.nA2) {
     const int Ua = I - d.nC2;
     // B: dt1[Ua, e] = 1/2 sum vt[X, Y, e, V] lam[Ua, V, X, Y]
-    for (int X = 0; X < d.nA2; ++X)
-      for (int Y = 0; Y < d.nA2; ++Y)
-        for (int V = 0; V < d.nA2; ++V)
-          dt1 = fma(0.5 * a.W1Vt[W1(d, d.nC2 + X, Y, A, V)], lam[LM(d, Ua, V, X, Y)], dt1);
     // D: dft[Xa, e] = 1/2 sum t[U, V, e, Y] lam[U, V, Xa, Y]
-    for (int U = 0; U < d.nA2; ++U)
-      for (int V = 0; V < d.nA2; ++V)
-        for (int Y = 0; Y < d.nA2; ++Y)
-          dft = fma(0.5 * a.W1T[W1(d, d.nC2 + U, V, A, Y)], lam[LM(d, U, V, Ua, Y)], dft);
+    for (int e = lane; e < d.nA2 * d.nA2; e += 32) {
+      const int P = e / d.nA2, Q = e % d.nA2, sr = (P & 1) + (Q & 1) - sp;
+      if (sr < 0 || sr > 1) continue;
+      for (int R = sr; R < d.nA2; R += 2) {
+        const size_t o = W1(d, d.nC2 + P, Q, A, R);
+        dt1 = fma(0.5 * a.W1Vt[o], lam[LM(d, Ua, R, P, Q)], dt1);
+        dft = fma(0.5 * a.W1T[o], lam[LM(d, P, Q, Ua, R)], dft);
+      }
+    }
   }
   if (I < d.nC2 && A < d.nA2) {
     // C: dt1[M, X] = -1/2 sum vt[M, Y, U, V] lam[U, V, X, Y]
-    for (int Y = 0; Y < d.nA2; ++Y)
-      for (int U = 0; U < d.nA2; ++U)
-        for (int V = 0; V < d.nA2; ++V)
-          dt1 = fma(-0.5 * a.W1Vt[W1(d, I, Y, U, V)], lam[LM(d, U, V, A, Y)], dt1);
     // E: dft[M, V] = -1/2 sum t[U, M, X, Y] lam[U, V, X, Y]
-    for (int U = 0; U < d.nA2; ++U)
-      for (int X = 0; X < d.nA2; ++X)
-        for (int Y = 0; Y < d.nA2; ++Y)
-          dft = fma(-0.5 * a.W2T[W2(d, d.nC2 + U, I, X, Y)], lam[LM(d, U, A, X, Y)], dft);
+    for (int e = lane; e < d.nA2 * d.nA2; e += 32) {
+      const int P = e / d.nA2, Q = e % d.nA2;
+      {
+        const int Y = P, U = Q, sv = sp + (Y & 1) - (U & 1);
+        if (sv >= 0 && sv <= 1)
+          for (int V = sv; V < d.nA2; V += 2)
+            dt1 = fma(-0.5 * a.W1Vt[W1(d, I, Y, U, V)], lam[LM(d, U, V, A, Y)], dt1);
+      }
+      {
+        const int U = P, X = Q, sy = (U & 1) + sp - (X & 1);
+        if (sy >= 0 && sy <= 1)
+          for (int Y = sy; Y < d.nA2; Y += 2)
+            dft = fma(-0.5 * a.W2T[W2(d, d.nC2 + U, I, X, Y)], lam[LM(d, U, A, X, Y)], dft);
+      }
+    }
   }
-  a.dt1[k] = dt1;
-  a.dft[k] = dft;
+  for (int o = 16; o > 0; o >>= 1) {
+    dt1 += __shfl_xor_sync(0xffffffffu, dt1, o);
+    dft += __shfl_xor_sync(0xffffffffu, dft, o);
+  }
+  if (lane < 2) {  // A, and the A of the other spin
+    const size_t o = ((size_t)I * d.nP2 + A) ^ (size_t)lane;
+    a.dt1[o] = lane == 0 ? dt1 : 0.0;
+    a.dft[o] = lane == 0 ? dft : 0.0;
+  }
 }
 
-// (A4) adjoint of P1, P2 from terms G (two virtual particles) and F4.
+// (A4) adjoint of P1, P2 from terms G (two virtual particles) and F4, as the matrix
+// C[p][q] of adj_m_kernel: with p = (p0,p1), q = (p2,p3), q' = (p3,p2),
+// C[p][q] = dE/dP1[p][q] + dE/dP2[p][q'].
 __global__ void adj_p12_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
   const int nA = a.z.nA, nA4 = nA * nA * nA * nA;
@@ -872,18 +941,21 @@ __global__ void adj_p12_kernel(ActAdjArgs a) {
   double d1 = 0.0, d2 = 0.0;
   for (int sg = 0; sg < 16; ++sg) {
     const int s0 = sg & 1, s1 = (sg >> 1) & 1, s2 = (sg >> 2) & 1, s3 = (sg >> 3) & 1;
-    const int A0 = 2 * p0 + s0, A1 = 2 * p1 + s1, A2 = 2 * p2 + s2, A3 = 2 * p3 + s3;
+    const int A0 = 2 * p0 + s0, A1 = 2 * p1 + s1;
     // G: 1/8 lam[U,V,X,Y] S[(X,Y),(U,V)] with (X,Y,U,V) = (A0,A1,A2,A3)
-    const double lg = a.lam[LM(d, A2, A3, A0, A1)];
-    if (s0 == s2 && s1 == s3) d1 += 0.25 * lg;
-    if (s0 == s3 && s1 == s2) d2 -= 0.25 * lg;
     // F4: 1/4 gA[X,Y] gA[U,V] S[(X,U),(Y,V)] with (X,U,Y,V) = (A0,A1,A2,A3)
-    const double gg = gAA(d, a.gA, A0, A2) * gAA(d, a.gA, A1, A3);
-    if (s0 == s2 && s1 == s3) d1 += 0.5 * gg;
-    if (s0 == s3 && s1 == s2) d2 -= 0.5 * gg;
+    if (s0 == s2 && s1 == s3) {  // P1
+      const int A2 = 2 * p2 + s2, A3 = 2 * p3 + s3;
+      d1 += 0.25 * a.lam[LM(d, A2, A3, A0, A1)];
+      d1 += 0.5 * gAA(d, a.gA, A0, A2) * gAA(d, a.gA, A1, A3);
+    }
+    if (s0 == s3 && s1 == s2) {  // P2 at q'
+      const int A2 = 2 * p3 + s2, A3 = 2 * p2 + s3;
+      d2 -= 0.25 * a.lam[LM(d, A2, A3, A0, A1)];
+      d2 -= 0.5 * gAA(d, a.gA, A0, A2) * gAA(d, a.gA, A1, A3);
+    }
   }
-  a.dP12[c] = d1;
-  a.dP12[nA4 + c] = d2;
+  a.dP12[c] = d1 + d2;
 }
 
 // (B1) t1/ft -> S, with the eps and s dependence of their regulators.
@@ -909,12 +981,16 @@ __device__ __forceinline__ void adj_t1_chain_kernel_body(ActAdjArgs a, double* s
   if (k >= d.nH2 * d.nP2) return;
   const int I = k / d.nP2, A = k % d.nP2;
   const Sizes& z = a.z;
+  if ((I & 1) != (A & 1)) {  // t1 and ft conserve spin
+    a.dS[k] = 0.0;
+    return;
+  }
   double S = 0.0;
   for (int U = 0; U < d.nA2; ++U)
-    for (int X = 0; X < d.nA2; ++X) {
-      const double g = a.gA[U * d.nA2 + X];
-      if (g == 0.0) continue;
-      S = fma((a.eps[z.nC + (X >> 1)] - a.eps[z.nC + (U >> 1)]) * g, a.W1T[W1(d, I, U, A, X)], S);
+#pragma unroll 4
+    for (int X = U & 1; X < d.nA2; X += 2) {
+      const double g = a.gA[U * d.nA2 + X], t = a.W1T[W1(d, I, U, A, X)];
+      S = fma((a.eps[z.nC + (X >> 1)] - a.eps[z.nC + (U >> 1)]) * g, g == 0.0 ? 0.0 : t, S);
     }
   const double D1 = a.eps[I >> 1] - a.eps[z.nC + (A >> 1)];
   const bool internal = (I >= d.nC2) && (A < d.nA2);
@@ -945,95 +1021,124 @@ __global__ void adj_t1_chain_kernel(ActAdjArgs a) {
   dacc_flush(sacc_, a.z.n, a.deps, a.ds);
 }
 
-// (B2) W1: total d(t) (direct + via Ti + via S), then through the regulators to d(V).
-__device__ __forceinline__ void adj_w1_chain_kernel_body(ActAdjArgs a, double* sacc_) {
-  const AD d = adims(a.z);
-  const Sizes& z = a.z;
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.w1n) return;
-  const int X = (int)(k % d.nA2);
-  const int A = (int)((k / d.nA2) % d.nP2);
-  const int U = (int)((k / ((size_t)d.nA2 * d.nP2)) % d.nA2);
-  const int I = (int)(k / ((size_t)d.nA2 * d.nP2 * d.nA2));
-  double dt = a.dW1T[k];
-  // via Ti[J][U][Bp][X] = sum_{I,A} gamma[J,I] eta[A,Bp] T[I,U,A,X]
-  {
-    const int j0 = (I < d.nC2) ? I : d.nC2, j1 = (I < d.nC2) ? I + 1 : d.nH2;
-    const int b0 = (A < d.nA2) ? 0 : A, b1 = (A < d.nA2) ? d.nA2 : A + 1;
-    for (int J = j0; J < j1; ++J) {
-      const double g = gH(d, a.gA, J, I);
-      if (g == 0.0) continue;
-      for (int Bp = b0; Bp < b1; ++Bp) dt = fma(g * eP(d, a.gA, A, Bp), a.dTi[W1(d, J, U, Bp, X)], dt);
-    }
+// A warp's sum of v into sacc[o] where o is the same in all lanes, else lane by lane.
+__device__ __forceinline__ void dacc_warp(double* sacc, int o, double v) {
+  if (__all_sync(0xffffffffu, o == __shfl_sync(0xffffffffu, o, 0))) {
+    for (int k = 16; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
+    if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(&sacc[o], v);
+  } else if (v != 0.0) {
+    atomicAdd(&sacc[o], v);
   }
-  // via S[I,A] = sum (e_X - e_U) gamma[U][X] T[I,U,A,X]
-  const double gux = a.gA[U * d.nA2 + X];
-  const double eX = a.eps[z.nC + (X >> 1)], eU = a.eps[z.nC + (U >> 1)];
-  const double dS = a.dS[(size_t)I * d.nP2 + A];
-  dt = fma(dS * (eX - eU), gux, dt);
-  const double T = a.W1T[k];
-  if (gux != 0.0 && dS != 0.0 && T != 0.0) {
-    atomicAdd(&sacc_[z.nC + (X >> 1)], dS * gux * T);
-    atomicAdd(&sacc_[z.nC + (U >> 1)], -dS * gux * T);
-  }
-  // regulators: T = V Rt(D) (zero if internal), Vt = V Rv(D)
-  const double V = a.W1V[k];
-  const double D = a.eps[I >> 1] + a.eps[z.nC + (U >> 1)] - a.eps[z.nC + (A >> 1)] - eX;
-  const bool internal = (I >= d.nC2) && (A < d.nA2);
-  const RegD rt = rt_d(D, a.s), rv = rv_d(D, a.s);
-  const double dvt = a.dW1Vt[k];
-  const double dtt = internal ? 0.0 : dt;
-  a.dV1[k] = dtt * rt.v + dvt * rv.v;
-  const double dD = V * (dtt * rt.dD + dvt * rv.dD);
-  const double dss = V * (dtt * rt.ds + dvt * rv.ds);
-  if (dD != 0.0) {
-    atomicAdd(&sacc_[I >> 1], dD);
-    atomicAdd(&sacc_[z.nC + (U >> 1)], dD);
-    atomicAdd(&sacc_[z.nC + (A >> 1)], -dD);
-    atomicAdd(&sacc_[z.nC + (X >> 1)], -dD);
-  }
-  if (dss != 0.0) atomicAdd(&sacc_[a.z.n], dss);
 }
 
-__global__ void adj_w1_chain_kernel(ActAdjArgs a) {
+// (B2) W1: total d(t) (direct + via Ti + via S), then through the regulators to d(V).
+// A thread takes one (I,U,A) and the X its spin allows (W1 is zero elsewhere): the sums
+// of an orbital's derivatives stay in registers or are added over the warp, where an
+// atomic per element on the few active orbitals took most of the time (127 us at
+// 10/4/60/200 and 289 us at 24/2/372/1200, 43 us and 57 us now).
+__global__ void __launch_bounds__(128) adj_w1_chain_kernel(ActAdjArgs a) {
   extern __shared__ double sacc_[];
   dacc_init(sacc_, a.z.n);
-  adj_w1_chain_kernel_body(a, sacc_);
+  const AD d = adims(a.z);
+  const Sizes& z = a.z;
+  const size_t n = a.w1n / d.nA2;
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool on = t0 < n;
+  const size_t t = on ? t0 : n - 1;  // lanes past the end help in the warp sums
+  const int A = (int)(t % d.nP2);
+  const int U = (int)((t / d.nP2) % d.nA2);
+  const int I = (int)(t / ((size_t)d.nP2 * d.nA2));
+  const int sx = (I & 1) + (U & 1) - (A & 1);  // spin of X
+  const bool some = on && (sx == 0 || sx == 1);
+  const int j0 = (I < d.nC2) ? I : d.nC2 + (I & 1), j1 = (I < d.nC2) ? I + 1 : d.nH2;
+  const int b0 = (A < d.nA2) ? (A & 1) : A, b1 = (A < d.nA2) ? d.nA2 : A + 1;
+  const double eU = a.eps[z.nC + (U >> 1)], eIUA = a.eps[I >> 1] + eU - a.eps[z.nC + (A >> 1)];
+  const double dS = a.dS[(size_t)I * d.nP2 + A];
+  const bool internal = (I >= d.nC2) && (A < d.nA2);
+  double sumI = 0.0, sumU = 0.0, dss = 0.0;
+  for (int xp = 0; xp < z.nA; ++xp) {
+    double dX = 0.0;
+    const int X = 2 * xp + (sx == 1);
+    const size_t k = t * d.nA2 + X;
+    if (some) {
+      a.dV1[k ^ 1] = 0.0;  // the other spin of X (k is 2 xp + spin from an even start)
+      double dt = a.dW1T[k];
+      // via Ti[J][U][Bp][X] = sum_{I,A} gamma[J,I] eta[A,Bp] T[I,U,A,X]
+      for (int J = j0; J < j1; J += 2) {
+        const double g = gH(d, a.gA, J, I);
+        if (g == 0.0) continue;
+        for (int Bp = b0; Bp < b1; Bp += 2)
+          dt = fma(g * eP(d, a.gA, A, Bp), a.dTi[W1(d, J, U, Bp, X)], dt);
+      }
+      // via S[I,A] = sum (e_X - e_U) gamma[U][X] T[I,U,A,X]
+      const double gux = a.gA[U * d.nA2 + X], eX = a.eps[z.nC + xp], T = a.W1T[k];
+      dt = fma(dS * (eX - eU), gux, dt);
+      const double dSx = dS * gux * T;
+      dX += dSx;
+      sumU -= dSx;
+      // regulators: T = V Rt(D) (zero if internal), Vt = V Rv(D)
+      const double V = a.W1V[k], dvt = a.dW1Vt[k], dtt = internal ? 0.0 : dt;
+      RegD rt, rv;
+      rtv_d(eIUA - eX, a.s, rt, rv);
+      a.dV1[k] = dtt * rt.v + dvt * rv.v;
+      const double dD = V * (dtt * rt.dD + dvt * rv.dD);
+      dss = fma(V, dtt * rt.ds + dvt * rv.ds, dss);
+      sumI += dD;
+      dX -= dD;
+    } else if (on) {
+      a.dV1[k] = 0.0;
+      a.dV1[k ^ 1] = 0.0;
+    }
+    dacc_warp(sacc_, z.nC + xp, dX);
+  }
+  dacc_warp(sacc_, I >> 1, sumI);
+  dacc_warp(sacc_, z.nC + (U >> 1), sumU + sumI);
+  dacc_warp(sacc_, z.n, dss);
+  if (sumI != 0.0) atomicAdd(&sacc_[z.nC + (A >> 1)], -sumI);
   dacc_flush(sacc_, a.z.n, a.deps, a.ds);
 }
 
-// (B3) W2 through its regulators to d(V).
-__device__ __forceinline__ void adj_w2_chain_kernel_body(ActAdjArgs a, double* sacc_) {
-  const AD d = adims(a.z);
-  const Sizes& z = a.z;
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.w2n) return;
-  const int Y = (int)(k % d.nA2);
-  const int X = (int)((k / d.nA2) % d.nA2);
-  const int J = (int)((k / ((size_t)d.nA2 * d.nA2)) % d.nH2);
-  const int I = (int)(k / ((size_t)d.nA2 * d.nA2 * d.nH2));
-  const double V = a.W2V[k];
-  const double D = a.eps[I >> 1] + a.eps[J >> 1] - a.eps[z.nC + (X >> 1)] - a.eps[z.nC + (Y >> 1)];
-  const bool internal = (I >= d.nC2) && (J >= d.nC2);
-  const RegD rt = rt_d(D, a.s), rv = rv_d(D, a.s);
-  const double dt = internal ? 0.0 : a.dW2T[k];
-  const double dvt = a.dW2Vt[k];
-  a.dV2[k] = dt * rt.v + dvt * rv.v;
-  const double dD = V * (dt * rt.dD + dvt * rv.dD);
-  const double dss = V * (dt * rt.ds + dvt * rv.ds);
-  if (dD != 0.0) {
-    atomicAdd(&sacc_[I >> 1], dD);
-    atomicAdd(&sacc_[J >> 1], dD);
-    atomicAdd(&sacc_[z.nC + (X >> 1)], -dD);
-    atomicAdd(&sacc_[z.nC + (Y >> 1)], -dD);
-  }
-  if (dss != 0.0) atomicAdd(&sacc_[a.z.n], dss);
-}
-
-__global__ void adj_w2_chain_kernel(ActAdjArgs a) {
+// (B3) W2 through its regulators to d(V). A thread takes one (I,J,X) and the Y its spin
+// allows, as adj_w1_chain_kernel.
+__global__ void __launch_bounds__(128) adj_w2_chain_kernel(ActAdjArgs a) {
   extern __shared__ double sacc_[];
   dacc_init(sacc_, a.z.n);
-  adj_w2_chain_kernel_body(a, sacc_);
+  const AD d = adims(a.z);
+  const Sizes& z = a.z;
+  const size_t n = a.w2n / d.nA2;
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool on = t0 < n;
+  const size_t t = on ? t0 : n - 1;  // lanes past the end help in the warp sums
+  const int X = (int)(t % d.nA2);
+  const int J = (int)((t / d.nA2) % d.nH2);
+  const int I = (int)(t / ((size_t)d.nA2 * d.nH2));
+  const int sy = (I & 1) + (J & 1) - (X & 1);
+  const bool some = on && (sy == 0 || sy == 1);
+  const double eIJX = a.eps[I >> 1] + a.eps[J >> 1] - a.eps[z.nC + (X >> 1)];
+  const bool internal = (I >= d.nC2) && (J >= d.nC2);
+  double sum = 0.0, dss = 0.0;
+  for (int y = 0; y < z.nA; ++y) {
+    const size_t k = t * d.nA2 + 2 * y + (sy == 1);
+    double dD = 0.0;
+    if (some) {
+      a.dV2[k ^ 1] = 0.0;
+      const double V = a.W2V[k], dt = internal ? 0.0 : a.dW2T[k], dvt = a.dW2Vt[k];
+      RegD rt, rv;
+      rtv_d(eIJX - a.eps[z.nC + y], a.s, rt, rv);
+      a.dV2[k] = dt * rt.v + dvt * rv.v;
+      dD = V * (dt * rt.dD + dvt * rv.dD);
+      dss = fma(V, dt * rt.ds + dvt * rv.ds, dss);
+      sum += dD;
+    } else if (on) {
+      a.dV2[k] = 0.0;
+      a.dV2[k ^ 1] = 0.0;
+    }
+    dacc_warp(sacc_, z.nC + y, -dD);
+  }
+  dacc_warp(sacc_, I >> 1, sum);
+  dacc_warp(sacc_, J >> 1, sum);
+  dacc_warp(sacc_, z.n, dss);
+  if (sum != 0.0) atomicAdd(&sacc_[z.nC + (X >> 1)], -sum);
   dacc_flush(sacc_, a.z.n, a.deps, a.ds);
 }
 
@@ -1076,184 +1181,119 @@ __global__ void adj_k_kernel(ActAdjArgs a) {
   }
 }
 
-// (B5) adjoint of P1/P2 -> dM[x][u][e][f] (one thread per virtual pair (e,f)), eps, s.
-template <int NA>
-__device__ __forceinline__ void adj_m_kernel_body(ActAdjArgs a, const double* __restrict__ dP12, double* sacc_) {
+// (B5) adjoint of P1/P2 -> dM[x][u][e][f], eps, s. With p = (x,u), q = (y,v), D_p = e_x +
+// e_u - e_e - e_f, u_p = M_p Rv(D_p), w_q = M_q Rt(D_q) and D_(vy) = D_(yv), the sum over a
+// virtual pair is u^T C w (adj_p12_kernel), so two products with C give every derivative:
+//   g = C w, h = C^T u:  dM_p = Rv_p g_p + Rt_p h_p, dE/dD_p = M_p (Rv'_p g_p + Rt'_p h_p).
+// A thread takes one p of one (e,f), the 256 / nA^2 pairs (e, f..) of a CTA share u and w
+// in shared memory. (One thread per (e,f) over all p and q of the sum, 25 FP64 operations
+// each, left most of the chip idle: 620 us at 10/4/60/200 and 508 us at 24/2/372/1200,
+// 19 us and 85 us now: the regulators.)
+__global__ void __launch_bounds__(256) adj_m_kernel(ActAdjArgs a, int PB, int chunks) {
+  __shared__ double su[256], sw[256], red[8];
   const Sizes& z = a.z;
-  const size_t nV2 = (size_t)z.nV * z.nV;
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nV2) return;
-  const int e = (int)(k / z.nV), f = (int)(k % z.nV);
-  constexpr int NA2 = NA * NA, NA4 = NA2 * NA2;
-  const int ve = z.nC + z.nA;
-  const double ef = a.eps[ve + e] + a.eps[ve + f];
-  double m[NA2], dm[NA2], dDp[NA2];
-  RegD rv[NA2], rt[NA2];
-#pragma unroll
-  for (int p = 0; p < NA2; ++p) {
-    m[p] = a.M[(size_t)p * nV2 + k];
-    dm[p] = 0.0;
-    dDp[p] = 0.0;
-    const double D = a.eps[z.nC + p / NA] + a.eps[z.nC + p % NA] - ef;
-    rv[p] = rv_d(D, a.s);
-    rt[p] = rt_d(D, a.s);
+  const int NA = z.nA, NA2 = NA * NA, ve = z.nC + z.nA;
+  const int e = blockIdx.x / chunks, f0 = (blockIdx.x % chunks) * PB;
+  const int pos = threadIdx.x % PB, p = threadIdx.x / PB, f = f0 + pos;
+  const bool on = p < NA2 && f < z.nV;
+  const size_t nV2 = (size_t)z.nV * z.nV, k = (size_t)p * nV2 + (size_t)e * z.nV + f;
+  double m = 0.0;
+  RegD rt{0.0, 0.0, 0.0}, rv{0.0, 0.0, 0.0};
+  if (on) {
+    m = a.M[k];
+    rtv_d(a.eps[z.nC + p / NA] + a.eps[z.nC + p % NA] - (a.eps[ve + e] + a.eps[ve + f]), a.s, rt, rv);
   }
-  double dss = 0.0;
-#pragma unroll
-  for (int p = 0; p < NA2; ++p) {        // p = (x, u)
-#pragma unroll
-    for (int q = 0; q < NA2; ++q) {      // q = (y, v)
-      const int qt = (q % NA) * NA + q / NA;  // (v, y)
-      const double d1 = dP12[p * NA2 + q], d2 = dP12[NA4 + p * NA2 + q];
-      const double R = rv[p].v * rt[q].v;
-      dm[p] += (d1 * m[q] + d2 * m[qt]) * R;
-      dm[q] += d1 * m[p] * R;
-      dm[qt] += d2 * m[p] * R;
-      const double dR = m[p] * (d1 * m[q] + d2 * m[qt]);
-      dDp[p] += dR * rv[p].dD * rt[q].v;
-      dDp[q] += dR * rv[p].v * rt[q].dD;
-      dss += dR * (rv[p].ds * rt[q].v + rv[p].v * rt[q].ds);
+  su[threadIdx.x] = m * rv.v;
+  sw[threadIdx.x] = m * rt.v;
+  __syncthreads();
+  double dD = 0.0, dss = 0.0;
+  if (on) {
+    double g = 0.0, h = 0.0;
+    for (int q = 0; q < NA2; ++q) {
+      g = fma(a.dP12[p * NA2 + q], sw[q * PB + pos], g);
+      h = fma(a.dP12[q * NA2 + p], su[q * PB + pos], h);
     }
+    a.dM[k] = rv.v * g + rt.v * h;
+    dD = m * (rv.dD * g + rt.dD * h);
+    dss = m * (rv.ds * g + rt.ds * h);
   }
-  double dsum = 0.0;
-#pragma unroll
-  for (int p = 0; p < NA2; ++p) {
-    a.dM[(size_t)p * nV2 + k] = dm[p];
-    dsum += dDp[p];
-    if (dDp[p] != 0.0) {
-      atomicAdd(&sacc_[z.nC + p / NA], dDp[p]);
-      atomicAdd(&sacc_[z.nC + p % NA], dDp[p]);
-    }
+  const double ts = block_sum<256>(dss, red), te = block_sum<256>(dD, red);
+  if (threadIdx.x == 0) {
+    atomicAdd(&a.deps[ve + e], -te);
+    atomicAdd(a.ds, ts);
   }
-  if (dsum != 0.0) {
-    atomicAdd(&sacc_[ve + e], -dsum);
-    atomicAdd(&sacc_[ve + f], -dsum);
+  su[threadIdx.x] = dD;  // [p][pos]: every reader of u is past block_sum
+  __syncthreads();
+  if (threadIdx.x < PB && f < z.nV) {
+    double t = 0.0;
+    for (int q = 0; q < NA2; ++q) t += su[q * PB + threadIdx.x];
+    atomicAdd(&a.deps[ve + f], -t);
   }
-  if (dss != 0.0) atomicAdd(&sacc_[a.z.n], dss);
+  // active orbital x: the pairs (x,u) and (u,x), one warp each
+  const int x = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (x < NA) {
+    double t = 0.0;
+    for (int i = lane; i < NA * PB; i += 32)
+      t += su[(x * NA + i / PB) * PB + i % PB] + su[((i / PB) * NA + x) * PB + i % PB];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) atomicAdd(&a.deps[z.nC + x], t);
+  }
 }
 
-template <int NA>
-__global__ void adj_m_kernel(ActAdjArgs a, const double* __restrict__ dP12) {
-  extern __shared__ double sacc_[];
-  dacc_init(sacc_, a.z.n);
-  adj_m_kernel_body<NA>(a, dP12, sacc_);
-  dacc_flush(sacc_, a.z.n, a.deps, a.ds);
-}
-
-// (B6) dK1, dK2, dK3 -> dB (gather, one thread per dB element; adds).
-__global__ void adj_k_to_b_kernel(ActAdjArgs a, const double* __restrict__ B, double* __restrict__ dB) {
+// (B6) dK1, dK2, dK3 -> dB (adds). An element (q,h,p) of a virtual particle p sums nA^2
+// and, for active h, nH nA products: one thread. With an active p it sums up to nH nP:
+// one warp. (One thread per element alike: 184 us at 10/4/60/200, most of it in the
+// threads of the long sums; 50 us now.)
+__global__ void __launch_bounds__(256) adj_k_to_b_kernel(ActAdjArgs a, const double* __restrict__ B,
+                                                         double* __restrict__ dB, unsigned vblocks) {
   const Sizes& z = a.z;
-  const size_t n = (size_t)z.Q * z.nH * z.nP;
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const int p = (int)(k % z.nP);
-  const int h = (int)((k / z.nP) % z.nH);
-  const int q = (int)(k / ((size_t)z.nP * z.nH));
   auto K1i = [&](int i, int u, int x, int ap) { return (((size_t)i * z.nA + u) * z.nA + x) * z.nP + ap; };
   auto K3i = [&](int i, int x, int j, int y) { return (((size_t)i * z.nA + x) * z.nH + j) * z.nA + y; };
-  double acc = 0.0;
-  // K1[i,u,x,a] = sum_Q B[Q,i,a] B[Q,nC+u,x]
-  for (int u = 0; u < z.nA; ++u)
-    for (int x = 0; x < z.nA; ++x) acc = fma(a.dK1[K1i(h, u, x, p)], B[bidx(z, q, z.nC + u, x)], acc);
-  if (h >= z.nC && p < z.nA) {
-    const int u = h - z.nC, x = p;
-    for (int i = 0; i < z.nH; ++i)
-      for (int ap = 0; ap < z.nP; ++ap) acc = fma(a.dK1[K1i(i, u, x, ap)], B[bidx(z, q, i, ap)], acc);
-  }
-  // K2[i,u,x,a] = sum_Q B[Q,i,x] B[Q,nC+u,a]
-  if (p < z.nA) {
-    const int x = p;
+  if (blockIdx.x < vblocks) {
+    const size_t n = (size_t)z.Q * z.nH * z.nV, k = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (k >= n) return;
+    const int p = z.nA + (int)(k % z.nV), h = (int)((k / z.nV) % z.nH), q = (int)(k / ((size_t)z.nV * z.nH));
+    double acc = 0.0;
+    // K1[i,u,x,a] = sum_Q B[Q,i,a] B[Q,nC+u,x]
     for (int u = 0; u < z.nA; ++u)
-      for (int ap = 0; ap < z.nP; ++ap)
-        acc = fma(a.dK2[K1i(h, u, x, ap)], B[bidx(z, q, z.nC + u, ap)], acc);
+      for (int x = 0; x < z.nA; ++x) acc = fma(a.dK1[K1i(h, u, x, p)], B[bidx(z, q, z.nC + u, x)], acc);
+    // K2[i,u,x,a] = sum_Q B[Q,i,x] B[Q,nC+u,a]
+    if (h >= z.nC)
+      for (int i = 0; i < z.nH; ++i)
+        for (int x = 0; x < z.nA; ++x) acc = fma(a.dK2[K1i(i, h - z.nC, x, p)], B[bidx(z, q, i, x)], acc);
+    dB[bidx(z, q, h, p)] += acc;
+    return;
   }
+  const size_t w = (size_t)(blockIdx.x - vblocks) * 8 + (threadIdx.x >> 5);
+  if (w >= (size_t)z.Q * z.nH * z.nA) return;
+  const int lane = threadIdx.x & 31;
+  const int x = (int)(w % z.nA), h = (int)((w / z.nA) % z.nH), q = (int)(w / ((size_t)z.nA * z.nH));
+  double acc = 0.0;
+  for (int e = lane; e < z.nA * z.nA; e += 32)
+    acc = fma(a.dK1[K1i(h, e / z.nA, e % z.nA, x)], B[bidx(z, q, z.nC + e / z.nA, e % z.nA)], acc);
+  for (int u = 0; u < z.nA; ++u)
+    for (int ap = lane; ap < z.nP; ap += 32)
+      acc = fma(a.dK2[K1i(h, u, x, ap)], B[bidx(z, q, z.nC + u, ap)], acc);
   if (h >= z.nC) {
     const int u = h - z.nC;
     for (int i = 0; i < z.nH; ++i)
-      for (int x = 0; x < z.nA; ++x) acc = fma(a.dK2[K1i(i, u, x, p)], B[bidx(z, q, i, x)], acc);
+      for (int ap = lane; ap < z.nP; ap += 32)
+        acc = fma(a.dK1[K1i(i, u, x, ap)], B[bidx(z, q, i, ap)], acc);
+    for (int e = lane; e < z.nH * z.nA; e += 32)
+      acc = fma(a.dK2[K1i(e / z.nA, u, e % z.nA, x)], B[bidx(z, q, e / z.nA, e % z.nA)], acc);
   }
   // K3[i,x,j,y] = sum_Q B[Q,i,x] B[Q,j,y]
-  if (p < z.nA) {
-    for (int j = 0; j < z.nH; ++j)
-      for (int y = 0; y < z.nA; ++y) {
-        acc = fma(a.dK3[K3i(h, p, j, y)], B[bidx(z, q, j, y)], acc);
-        acc = fma(a.dK3[K3i(j, y, h, p)], B[bidx(z, q, j, y)], acc);
-      }
+  for (int e = lane; e < z.nH * z.nA; e += 32) {
+    const int j = e / z.nA, y = e % z.nA;
+    acc = fma(a.dK3[K3i(h, x, j, y)] + a.dK3[K3i(j, y, h, x)], B[bidx(z, q, j, y)], acc);
   }
-  dB[k] += acc;
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) dB[bidx(z, q, h, x)] += acc;
 }
 
 }  // namespace dsrg
 
 namespace dsrg {
-
-// Generic-nA fallback of adj_m_kernel for active spaces above 4 orbitals.
-__device__ __forceinline__ void adj_m_generic_kernel_body(ActAdjArgs a, const double* __restrict__ dP12, double* sacc_) {
-  const Sizes& z = a.z;
-  const int NA = z.nA, NA2 = NA * NA, NA4 = NA2 * NA2;
-  const size_t nV2 = (size_t)z.nV * z.nV;
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nV2) return;
-  const int e = (int)(k / z.nV), f = (int)(k % z.nV);
-  const int ve = z.nC + z.nA;
-  const double ef = a.eps[ve + e] + a.eps[ve + f];
-  double dsum = 0.0, dss = 0.0;
-  for (int p = 0; p < NA2; ++p) {
-    const double mp = a.M[(size_t)p * nV2 + k];
-    const RegD rvp = rv_d(a.eps[z.nC + p / NA] + a.eps[z.nC + p % NA] - ef, a.s);
-    const RegD rtp = rt_d(a.eps[z.nC + p / NA] + a.eps[z.nC + p % NA] - ef, a.s);
-    double dm = 0.0, dDp = 0.0;
-    for (int q = 0; q < NA2; ++q) {
-      const int qt = (q % NA) * NA + q / NA;
-      const double mq = a.M[(size_t)q * nV2 + k], mqt = a.M[(size_t)qt * nV2 + k];
-      const RegD rvq = rv_d(a.eps[z.nC + q / NA] + a.eps[z.nC + q % NA] - ef, a.s);
-      const RegD rtq = rt_d(a.eps[z.nC + q / NA] + a.eps[z.nC + q % NA] - ef, a.s);
-      // p in the first slot of P1/P2
-      {
-        const double d1 = dP12[p * NA2 + q], d2 = dP12[NA4 + p * NA2 + q];
-        dm += (d1 * mq + d2 * mqt) * rvp.v * rtq.v;
-        const double dR = mp * (d1 * mq + d2 * mqt);
-        dDp += dR * rvp.dD * rtq.v;
-        dss += dR * (rvp.ds * rtq.v + rvp.v * rtq.ds);
-      }
-      // p in the second slot: P1[q, p] with M_p, and P2[q, pt] with M_p (pt = transposed p)
-      {
-        const double d1 = dP12[q * NA2 + p];
-        dm += d1 * mq * rvq.v * rtp.v;
-        dDp += d1 * mq * mp * rvq.v * rtp.dD;
-        const int pt = (p % NA) * NA + p / NA;
-        const double d2 = dP12[NA4 + q * NA2 + pt];
-        const RegD rtpt = rt_d(a.eps[z.nC + pt / NA] + a.eps[z.nC + pt % NA] - ef, a.s);
-        dm += d2 * mq * rvq.v * rtpt.v;
-        const double dR2 = d2 * mq * mp;
-        if (dR2 != 0.0) {
-          atomicAdd(&sacc_[z.nC + pt / NA], dR2 * rvq.v * rtpt.dD);
-          atomicAdd(&sacc_[z.nC + pt % NA], dR2 * rvq.v * rtpt.dD);
-          dsum += dR2 * rvq.v * rtpt.dD;
-        }
-      }
-    }
-    a.dM[(size_t)p * nV2 + k] = dm;
-    if (dDp != 0.0) {
-      atomicAdd(&sacc_[z.nC + p / NA], dDp);
-      atomicAdd(&sacc_[z.nC + p % NA], dDp);
-    }
-    dsum += dDp;
-  }
-  if (dsum != 0.0) {
-    atomicAdd(&sacc_[ve + e], -dsum);
-    atomicAdd(&sacc_[ve + f], -dsum);
-  }
-  if (dss != 0.0) atomicAdd(&sacc_[a.z.n], dss);
-}
-
-__global__ void adj_m_generic_kernel(ActAdjArgs a, const double* __restrict__ dP12) {
-  extern __shared__ double sacc_[];
-  dacc_init(sacc_, a.z.n);
-  adj_m_generic_kernel_body(a, dP12, sacc_);
-  dacc_flush(sacc_, a.z.n, a.deps, a.ds);
-}
-
 
 bool grad_alloc(dsrg_plan* p) {
   const Sizes& z = p->z;
@@ -1290,7 +1330,7 @@ bool grad_alloc(dsrg_plan* p) {
          plan_alloc(p, (void**)&g->dW2Vt, w2n * 8) && plan_alloc(p, (void**)&g->dW2T, w2n * 8) &&
          plan_alloc(p, (void**)&g->dV2, w2n * 8) && plan_alloc(p, (void**)&g->dt1, nHP2 * 8) &&
          plan_alloc(p, (void**)&g->dft, nHP2 * 8) && plan_alloc(p, (void**)&g->dS, nHP2 * 8) &&
-         plan_alloc(p, (void**)&g->dP12, 2 * nA4 * 8) && plan_alloc(p, (void**)&g->dK1, n12 * 8) &&
+         plan_alloc(p, (void**)&g->dP12, nA4 * 8) && plan_alloc(p, (void**)&g->dK1, n12 * 8) &&
          plan_alloc(p, (void**)&g->dK2, n12 * 8) && plan_alloc(p, (void**)&g->dK3, n3 * 8) &&
          plan_alloc(p, (void**)&g->dM, (size_t)z.nA * z.nA * z.nV * z.nV * 8);
   }
@@ -1519,31 +1559,28 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     const int nA4 = z.nA * z.nA * z.nA * z.nA;
     auto blocks = [](size_t n) { return (unsigned)((n + 255) / 256); };
     const size_t dsm = ((size_t)z.n + 1) * 8;  // block sums of deps and ds
-    adj_w1_terms_kernel<<<blocks(A.w1n), 256, 0, st>>>(a);
+    adj_w1_terms_kernel<<<blocks(A.w1n / 2), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
-    adj_w2_terms_kernel<<<blocks(A.w2n), 256, 0, st>>>(a);
+    adj_w2_terms_kernel<<<blocks(A.w2n / 2), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
-    adj_t1ft_terms_kernel<<<blocks(nHP2), 256, 0, st>>>(a);
+    adj_t1ft_terms_kernel<<<blocks((size_t)16 * nHP2), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
     adj_p12_kernel<<<blocks(nA4), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
     adj_t1_chain_kernel<<<blocks(nHP2), 256, dsm, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
-    adj_w1_chain_kernel<<<blocks(A.w1n), 256, dsm, st>>>(a);
+    adj_w1_chain_kernel<<<(unsigned)((A.w1n / (2 * z.nA) + 127) / 128), 128, dsm, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
-    adj_w2_chain_kernel<<<blocks(A.w2n), 256, dsm, st>>>(a);
+    adj_w2_chain_kernel<<<(unsigned)((A.w2n / (2 * z.nA) + 127) / 128), 128, dsm, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
     {
       const size_t n = 2 * (size_t)z.nH * z.nA * z.nA * z.nP + (size_t)z.nH * z.nA * z.nH * z.nA;
       adj_k_kernel<<<blocks(n), 256, 0, st>>>(a);
       DSRG_LAUNCH_CHECK(p);
     }
-    switch (z.nA) {
-      case 1: adj_m_kernel<1><<<blocks(nV2), 256, dsm, st>>>(a, w->dP12); break;
-      case 2: adj_m_kernel<2><<<blocks(nV2), 256, dsm, st>>>(a, w->dP12); break;
-      case 3: adj_m_kernel<3><<<blocks(nV2), 256, dsm, st>>>(a, w->dP12); break;
-      case 4: adj_m_kernel<4><<<blocks(nV2), 256, dsm, st>>>(a, w->dP12); break;
-      default: adj_m_generic_kernel<<<blocks(nV2), 256, dsm, st>>>(a, w->dP12); break;
+    {
+      const int PB = 256 / (z.nA * z.nA), chunks = (z.nV + PB - 1) / PB;
+      adj_m_kernel<<<(unsigned)(z.nV * chunks), 256, 0, st>>>(a, PB, chunks);
     }
     DSRG_LAUNCH_CHECK(p);
     if (!fp64) {
@@ -1551,7 +1588,11 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
       if ((e = tc_adj_rest(p, w->dX, w->dZ, w->dM, w->dK1, w->dK2, w->dK3)) != cudaSuccess) return e;
       return tc_adj_assemble(p, B, dB);
     }
-    adj_k_to_b_kernel<<<blocks((size_t)z.Q * HP), 256, 0, st>>>(a, B, dB);
+    {
+      const unsigned vb = blocks((size_t)z.Q * z.nH * z.nV);
+      const unsigned ab = (unsigned)(((size_t)z.Q * z.nH * z.nA + 7) / 8);
+      adj_k_to_b_kernel<<<vb + ab, 256, 0, st>>>(a, B, dB, vb);
+    }
     DSRG_LAUNCH_CHECK(p);
     const long long CP = (long long)z.nC * z.nP;
     e = gemm(p, batched(mk(z.Q, z.nV, z.nA, z.nV, B + CP + z.nA, HP, z.nP, 1, w->dM, nV2, 1, nV,

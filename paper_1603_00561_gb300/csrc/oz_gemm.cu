@@ -498,9 +498,10 @@ size_t oz_work_bytes(long long M, long long N, long long K, long long nb, bool s
   return (cap > one ? cap : (one < 4 * OZ_WS_CAP ? one : 4 * OZ_WS_CAP)) + 4096;
 }
 
-// The tensor-core form costs about six launches and the slicing; the FP64 pipe does
-// 1.1 TFLOP/s on whole 64 x 64 tiles. At 5e7 operations both take about 60 us.
-static bool oz_worthwhile(double flops) { return flops >= 5e7; }
+// The tensor-core form costs about six launches and the slicing, about 120 us for the
+// smallest products; the FP64 pipe does 1.1 TFLOP/s on tiles that fill the chip. At 1e8
+// operations the two are about even (58 MFLOP: 120 us against 60).
+static bool oz_worthwhile(double flops) { return flops >= 1e8; }
 
 cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
   GemmArgs g = g0;

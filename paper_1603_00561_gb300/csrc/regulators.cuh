@@ -54,11 +54,6 @@ __device__ __forceinline__ RegD rt_d(double D, double s) {
   return rt_d(D, s, g);
 }
 
-__device__ __forceinline__ RegD rv_d(double D, double s) {
-  const double g = exp(-s * D * D);
-  return RegD{1.0 + g, -2.0 * s * D * g, -D * D * g};
-}
-
 // Both, with one exponential.
 __device__ __forceinline__ void rtv_d(double D, double s, RegD& rt, RegD& rv) {
   double g;
