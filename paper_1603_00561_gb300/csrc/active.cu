@@ -21,7 +21,8 @@
 // eta = 1 - gamma on particles (1 on virtuals). Cumulant from the opposite-
 // spin input L: same spin L[u,v,x,y] - L[u,v,y,x]; (alpha beta|alpha beta)
 // L[u,v,x,y]; (beta alpha|beta alpha) L[v,u,y,x]; (alpha beta|beta alpha)
-// -L[u,v,y,x]; (beta alpha|alpha beta) -L[v,u,x,y].
+// -L[u,v,y,x]; (beta alpha|alpha beta) -L[v,u,x,y]; of the last four the mean over the
+// two spin orders is kept (build_tables_kernel).
 #include <type_traits>
 
 #include "ff.cuh"
@@ -176,13 +177,14 @@ __global__ void small_ints_kernel(const double* __restrict__ B, Sizes z, double*
 
 // Spin-orbital W1, W2 (V, T, Vt), cumulant and active gamma. One thread per
 // spatial quadruple of W1 / W2: the regulators depend on the spatial orbitals
-// only, so they are evaluated once and the 16 spin combinations written.
+// only, so they are evaluated once and the 16 spin combinations written (V itself, a
+// third of the bytes, only for plans whose adjoint reads it).
 __global__ void build_tables_kernel(const double* __restrict__ eps, const double* __restrict__ G,
                                     const double* __restrict__ L, double s, Sizes z,
                                     const double* __restrict__ K1, const double* __restrict__ K2,
                                     const double* __restrict__ K3, double* __restrict__ W1,
                                     double* __restrict__ W2, double* __restrict__ lam,
-                                    double* __restrict__ gA, size_t w1n, size_t w2n) {
+                                    double* __restrict__ gA, size_t w1n, size_t w2n, bool with_v) {
   const ActDims d = act_dims(z);
   const size_t n1 = (size_t)z.nH * z.nA * z.nP * z.nA;   // spatial (i, u, a, x)
   const size_t n2 = (size_t)z.nH * z.nH * z.nA * z.nA;   // spatial (i, j, x, y)
@@ -205,7 +207,7 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
       if (si == sa && su == sx) V += k1;
       if (si == sx && su == sa) V -= k2;
       const size_t o = w1i(d, 2 * i + si, 2 * u + su, 2 * a + sa, 2 * x + sx);
-      W1[o] = V;
+      if (with_v) W1[o] = V;
       W1[w1n + o] = internal ? 0.0 : V * rt;
       W1[2 * w1n + o] = V * rv;
     }
@@ -226,7 +228,7 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
       if (si == sx && sj == sy) V += kxy;
       if (si == sy && sj == sx) V -= kyx;
       const size_t o = w2i(d, 2 * i + si, 2 * j + sj, 2 * x + sx, 2 * y + sy);
-      W2[o] = V;
+      if (with_v) W2[o] = V;
       W2[w2n + o] = internal ? 0.0 : V * rt;
       W2[2 * w2n + o] = V * rv;
     }
@@ -242,9 +244,12 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
     if (su == sv && sv == sx && sx == sy) {
       val = Lf(u, v, x, y) - Lf(u, v, y, x);
     } else if (su == sx && sv == sy) {
-      val = (su == 0) ? Lf(u, v, x, y) : Lf(v, u, y, x);
+      // the mean of both spin orders, equal for a cumulant with L[u,v,x,y] = L[v,u,y,x]:
+      // integrals and densities do not change when all spins flip, so only the mean
+      // contributes, and the terms sum one spin of their first orbital (twice)
+      val = 0.5 * (Lf(u, v, x, y) + Lf(v, u, y, x));
     } else if (su == sy && sv == sx) {
-      val = (su == 0) ? -Lf(u, v, y, x) : -Lf(v, u, x, y);
+      val = -0.5 * (Lf(u, v, y, x) + Lf(v, u, x, y));
     }
     lam[r] = val;
   } else if (k < n1 + n2 + nl + ng) {
@@ -256,30 +261,39 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
 
 // T1 amplitudes and modified Fock elements over spin orbitals [2nH][2nP]
 // (Eqs. (12), (14)); f1 is the optional off-diagonal Fock block [nH][nP]
-// (spatial, spin-diagonal; its active x active entries are not read).
-__global__ void t1_kernel(const double* __restrict__ eps, double s, Sizes z,
-                          const double* __restrict__ W1T, const double* __restrict__ gA,
-                          const double* __restrict__ f1, double* __restrict__ t1,
-                          double* __restrict__ ft) {
+// (spatial, spin-diagonal; its active x active entries are not read). One thread per
+// (I, a) with A of I's spin: both conserve spin, so the others are zero. The sum over
+// (U, X) of one spin has its loads in flight together (skipping zero gammas by branches,
+// over both spins, took 26 us at 10/4/60/200, 12 us now).
+template <int NA>
+__global__ void __launch_bounds__(128) t1_kernel(const double* __restrict__ eps, double s, Sizes z,
+                                                 const double* __restrict__ W1T,
+                                                 const double* __restrict__ gA,
+                                                 const double* __restrict__ f1,
+                                                 double* __restrict__ t1, double* __restrict__ ft) {
   const ActDims d = act_dims(z);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= d.nH2 * d.nP2) return;
-  const int I = k / d.nP2, A = k % d.nP2;
+  if (k >= d.nH2 * z.nP) return;
+  const int I = k / z.nP, a = k % z.nP, A = 2 * a + (I & 1);
   double S = 0.0;
-  for (int U = 0; U < d.nA2; ++U)
-    for (int X = 0; X < d.nA2; ++X) {
-      const double g = gA[U * d.nA2 + X];
-      if (g == 0.0) continue;
-      const double Dux = eps[z.nC + (X >> 1)] - eps[z.nC + (U >> 1)];
-      S = fma(Dux * g, W1T[w1i(d, I, U, A, X)], S);
+#pragma unroll
+  for (int u = 0; u < 2 * NA; ++u)
+#pragma unroll
+    for (int x = 0; x < NA; ++x) {
+      const int U = u, X = 2 * x + (u & 1);
+      const double g = gA[U * d.nA2 + X], t = W1T[w1i(d, I, U, A, X)];
+      const double Dux = eps[z.nC + x] - eps[z.nC + (u >> 1)];
+      S = fma(Dux * g, g == 0.0 ? 0.0 : t, S);
     }
-  const double D1 = eps[I >> 1] - eps[z.nC + (A >> 1)];
-  const bool internal = (I >= d.nC2) && (A < d.nA2);
-  const double F = (f1 && !internal && (I & 1) == (A & 1)) ? f1[(size_t)(I >> 1) * z.nP + (A >> 1)]
-                                                           : 0.0;
+  const double D1 = eps[I >> 1] - eps[z.nC + a];
+  const bool internal = (I >= d.nC2) && (a < z.nA);
+  const double F = (f1 && !internal) ? f1[(size_t)(I >> 1) * z.nP + a] : 0.0;
   const double g = exp(-s * D1 * D1);
-  t1[k] = internal ? 0.0 : (F + S) * reg_t(D1, s);
-  ft[k] = fma(F, 1.0 + g, S * g);
+  const size_t o = (size_t)I * d.nP2 + A;
+  t1[o] = internal ? 0.0 : (F + S) * reg_t(D1, s);
+  ft[o] = fma(F, 1.0 + g, S * g);
+  t1[o ^ 1] = 0.0;
+  ft[o ^ 1] = 0.0;
 }
 
 // Term A with no active orbitals (the only term then, from f^(1)): per core
@@ -322,13 +336,17 @@ __global__ void ti_kernel(Sizes z, const double* __restrict__ W1T, const double*
   const int Bp = (int)((k / d.nA2) % d.nP2);
   const int V = (int)((k / ((size_t)d.nA2 * d.nP2)) % d.nA2);
   const int J = (int)(k / ((size_t)d.nA2 * d.nP2 * d.nA2));
-  const int i0 = (J < d.nC2) ? J : d.nC2, i1 = (J < d.nC2) ? J + 1 : d.nH2;
-  const int a0 = (Bp < d.nA2) ? 0 : Bp, a1 = (Bp < d.nA2) ? d.nA2 : Bp + 1;
+  if ((J & 1) + (V & 1) != (Bp & 1) + (Y & 1)) {  // gamma, eta and t conserve spin
+    Ti[k] = 0.0;
+    return;
+  }
+  const int i0 = (J < d.nC2) ? J : d.nC2 + (J & 1), i1 = (J < d.nC2) ? J + 1 : d.nH2;
+  const int a0 = (Bp < d.nA2) ? (Bp & 1) : Bp, a1 = (Bp < d.nA2) ? d.nA2 : Bp + 1;
   double acc = 0.0;
-  for (int I = i0; I < i1; ++I) {
+  for (int I = i0; I < i1; I += 2) {
     const double g = gam_h(d, gA, J, I);
     if (g == 0.0) continue;
-    for (int A = a0; A < a1; ++A) acc = fma(g * eta_p(d, gA, A, Bp), W1T[w1i(d, I, V, A, Y)], acc);
+    for (int A = a0; A < a1; A += 2) acc = fma(g * eta_p(d, gA, A, Bp), W1T[w1i(d, I, V, A, Y)], acc);
   }
   Ti[k] = acc;
 }
@@ -385,8 +403,9 @@ __global__ void __launch_bounds__(256) gram_aavv_kernel(const double* __restrict
 
 // P1[xu][yv] = sum_ef M_xu[ef] M_yv[ef] R, P2[xu][yv] = sum_ef M_xu[ef] M_vy[ef] R
 // (M_vy[e,f] = M_yv[f,e]) with R = (1 + exp(-s D_xu^2)) (1 - exp(-s D_yv^2))/D_yv.
-constexpr int ACTVV_BLOCKS = 152;
-constexpr int ACTVV_CH = 64;      // positions (e, f) per chunk of the active VV sums
+constexpr int ACTVV_BLOCKS = 304;  // two CTAs per SM
+constexpr int ACTVV_CH = 64;       // positions (e, f) per chunk of the active VV sums
+constexpr int ACTVV_LD = ACTVV_CH + 1;  // their pitch in shared memory: a warp reads 32 rows at once
 
 // Rv = 1 + exp(-s D^2) and Rt = (1 - exp(-s D^2)) / D as FP32 pairs (split-precision
 // plans; 7 FP64 instructions less per pair and position): true if |D| >= 1/4 and in
@@ -548,8 +567,9 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
 // p' = (u,x), a_p = M_p Rv_p, b_p = M_p Rt_p and c_p = M_p' Rt_p in shared memory
 // (nA^2 regulator pairs per position; D_p' = D_p), then accumulates
 // P1[p][q] += a_p b_q and P2[p][q] += a_p c_q (M_vy = M_(yv)') over the chunk,
-// each thread holding a fixed set of (p, q).
-
+// each thread holding a fixed set of (p, q). (With a pitch of 64 the lanes' rows all lay
+// in one bank: 390 us at 31/5/467/1609, 158 us now.)
+//
 // F32 (split-precision plans): the regulated factors are rounded to FP32 and each
 // 64-term chunk of the sum over (e, f) runs in FP32 on CUDA cores (round to
 // nearest), the chunk sums in FP64; the regulators themselves stay FP64.
@@ -561,9 +581,9 @@ __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict
   constexpr int NA2 = NA * NA, NA4 = NA2 * NA2;
   constexpr int PER = (NA4 + 255) / 256;  // (p,q) outputs per thread
   extern __shared__ double avs[];
-  T* sa = (T*)avs;                         // [NA2][CH]
-  T* sb = sa + NA2 * ACTVV_CH;             // [NA2][CH]
-  T* sc = sb + NA2 * ACTVV_CH;             // [NA2][CH]
+  T* sa = (T*)avs;                         // [NA2][LD]
+  T* sb = sa + NA2 * ACTVV_LD;             // [NA2][LD]
+  T* sc = sb + NA2 * ACTVV_LD;             // [NA2][LD]
   __shared__ double red[8];
   const size_t nV2 = (size_t)z.nV * z.nV;
   const int ve = z.nC + z.nA;
@@ -601,18 +621,19 @@ __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict
           c = (T)(mt * rt);
         }
       }
-      sa[it] = a;
-      sb[it] = b;
-      sc[it] = c;
+      const int o = pidx * ACTVV_LD + kk;
+      sa[o] = a;
+      sb[o] = b;
+      sc[o] = c;
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
       const int o = threadIdx.x + 256 * r;
       if (o < NA4) {
-        const T* ap = sa + (o / NA2) * ACTVV_CH;
-        const T* bq = sb + (o % NA2) * ACTVV_CH;
-        const T* cq = sc + (o % NA2) * ACTVV_CH;
+        const T* ap = sa + (o / NA2) * ACTVV_LD;
+        const T* bq = sb + (o % NA2) * ACTVV_LD;
+        const T* cq = sc + (o % NA2) * ACTVV_LD;
         if constexpr (F32) {
           float t1 = 0.f, t2 = 0.f;
 #pragma unroll 8
@@ -700,25 +721,34 @@ __device__ __forceinline__ double s_vv(const ActDims& d, int nA, const double* P
 // over the rest. gamma and eta are spin-diagonal, the cumulant is non-zero
 // only for {s_u, s_v} = {s_x, s_y} and t1, ft conserve spin, so the inner loops
 // run over spatial orbitals of the one spin that can give a non-zero product.
+// Flipping all spins changes nothing (build_tables_kernel), so the first orbital of
+// every term takes spin 0 and the sum counts twice.
+// The integrals and amplitudes are antisymmetric in a pair of holes or of active
+// particles, so the long terms (GVA, H, F5, F8) sum over unordered pairs, with the
+// cumulant antisymmetrised over (u,v) as it is over (x,y): a quarter of the products
+// (all terms but I, F6, F7, J, K at 31/5/467/1609: 420 us with full sums over both spins, 108 us now).
+// Unordered pair U < V of n: index p in [0, n (n - 1) / 2).
+__device__ __forceinline__ void pair_of(int n, int p, int& U, int& V) {
+  int u = 0;
+  while (p >= n - 1 - u) p -= n - 1 - u++;
+  U = u;
+  V = u + 1 + p;
+}
 __device__ __forceinline__ long term_count(int term, const ActDims& d) {
-  const long a2 = (long)d.nA2 * d.nA2;
+  const long a2 = (long)d.nA2 * d.nA2, ap = (long)d.nA2 * (d.nA2 - 1) / 2;
   switch (term) {
-    case T_A: return (long)d.nH2 * d.nP2;
-    case T_B: return (long)d.nV2 * a2;
-    case T_C: return (long)d.nC2 * a2;
-    case T_D: return (long)d.nV2 * a2;
-    case T_E: return (long)d.nC2 * a2;
-    case T_GVA: return (long)d.nV2 * a2;
-    case T_GVV: return a2 * a2;
-    case T_H: return (long)d.nH2 * d.nH2 * a2;
-    case T_I: return (long)d.nH2 * d.nP2 * a2;
-    case T_F4: return a2 * a2;
-    case T_F5: return (long)d.nC2 * d.nC2 * a2;
-    case T_F6: return (long)d.nC2 * d.nV2 * a2;
-    case T_F7: return (long)d.nV2 * a2 * d.nA2;
-    case T_F8: return (long)d.nC2 * a2 * d.nA2;
-    case T_J: return (long)d.nC2 * a2 * d.nA2;
-    case T_K: return (long)d.nV2 * a2 * d.nA2;
+    case T_A: return (long)d.nH2 / 2 * d.nP2;
+    case T_B: return (long)d.nV2 / 2 * a2;
+    case T_C: return (long)d.nC2 / 2 * a2;
+    case T_D: return (long)d.nV2 / 2 * a2;
+    case T_E: return (long)d.nC2 / 2 * a2;
+    case T_GVA: return (long)d.nV2 / 2 * ap;
+    case T_GVV: return a2 * a2 / 2;
+    case T_H: return (long)d.nH2 / 2 * d.nH2 * ap;
+    case T_I: return (long)d.nH2 / 2 * d.nP2 * a2;
+    case T_F4: return a2 * a2 / 2;
+    case T_F5: return (long)d.nC2 / 2 * d.nC2 * ap;
+    case T_F8: return (long)d.nC2 / 2 * ap * d.nA2;
   }
   return 0;
 }
@@ -730,7 +760,7 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
   double acc = 0.0;
   switch (term) {
     case T_A: {  // ft_j^b t_a^i gamma_i^j eta_b^a, outer (J, Bp)
-      const int J = (int)(o / d.nP2), Bp = (int)(o % d.nP2);
+      const int J = 2 * (int)(o / d.nP2), Bp = (int)(o % d.nP2);
       double gf = 0.0, te = 0.0;
       const int k0 = (J < C2) ? J : C2, k1 = (J < C2) ? J + 1 : d.nH2;
       for (int K = k0; K < k1; ++K) gf = fma(gam_h(d, t.gA, J, K), t.ft[(size_t)K * d.nP2 + Bp], gf);
@@ -740,7 +770,7 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
     }
     case T_B: {  // 1/2 vt_{xy}^{ev} t_e^u lambda_{uv}^{xy}, outer (E, X, Y)
       const int Y = (int)(o % nA2), X = (int)((o / nA2) % nA2);
-      const int Ap = nA2 + (int)(o / ((long)nA2 * nA2));
+      const int Ap = nA2 + 2 * (int)(o / ((long)nA2 * nA2));
       const int su = Ap & 1;  // t_e^u conserves spin
       for (int V = 0; V < nA2; ++V) {
         const double vt = t.W1Vt[w1i(d, C2 + X, Y, Ap, V)];
@@ -753,7 +783,7 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
       return 0.5 * acc;
     }
     case T_C: {  // -1/2 vt_{my}^{uv} t_x^m lambda_{uv}^{xy}, outer (M, Y, U)
-      const int U = (int)(o % nA2), Y = (int)((o / nA2) % nA2), M = (int)(o / ((long)nA2 * nA2));
+      const int U = (int)(o % nA2), Y = (int)((o / nA2) % nA2), M = 2 * (int)(o / ((long)nA2 * nA2));
       const int sx = M & 1;
       for (int V = 0; V < nA2; ++V) {
         const double vt = t.W1Vt[w1i(d, M, Y, U, V)];
@@ -767,7 +797,7 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
     }
     case T_D: {  // 1/2 ft_x^e t_{ey}^{uv} lambda_{uv}^{xy}, outer (E, U, V)
       const int V = (int)(o % nA2), U = (int)((o / nA2) % nA2);
-      const int Ap = nA2 + (int)(o / ((long)nA2 * nA2));
+      const int Ap = nA2 + 2 * (int)(o / ((long)nA2 * nA2));
       const int sx = Ap & 1;
       for (int Y = 0; Y < nA2; ++Y) {
         const double tt = t.W1T[w1i(d, C2 + U, V, Ap, Y)];
@@ -780,7 +810,7 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
       return 0.5 * acc;
     }
     case T_E: {  // -1/2 ft_m^v t_{xy}^{um} lambda_{uv}^{xy}, outer (M, U, X)
-      const int X = (int)(o % nA2), U = (int)((o / nA2) % nA2), M = (int)(o / ((long)nA2 * nA2));
+      const int X = (int)(o % nA2), U = (int)((o / nA2) % nA2), M = 2 * (int)(o / ((long)nA2 * nA2));
       const int sv = M & 1;
       for (int Y = 0; Y < nA2; ++Y) {
         const double tt = t.W2T[w2i(d, C2 + U, M, X, Y)];
@@ -792,36 +822,45 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
       }
       return -0.5 * acc;
     }
-    case T_GVA: {  // G with one virtual and one active particle, outer (E, U, V)
-      const int V = (int)(o % nA2), U = (int)((o / nA2) % nA2);
-      const int Ap = nA2 + (int)(o / ((long)nA2 * nA2));
-      for (int Cc = 0; Cc < nA2; ++Cc) {
+    case T_GVA: {  // G with one virtual and one active particle, outer (E, U < V)
+      const int np = nA2 * (nA2 - 1) / 2, Ap = nA2 + 2 * (int)(o / np);
+      int U, V;
+      pair_of(nA2, (int)(o % np), U, V);
+      const int sc = (U & 1) + (V & 1) - (Ap & 1);  // t_{e c}^{uv} conserves spin
+      if (sc < 0 || sc > 1) return 0.0;
+      for (int Cc = sc; Cc < nA2; Cc += 2) {
         double tg = 0.0;  // sum_a eta_c^a t_{a e}^{uv}, with the particle pair reversed
         for (int a = 0; a < nA; ++a) {
-          const int A = 2 * a + (Cc & 1);
+          const int A = 2 * a + sc;
           tg = fma(ea(d, t.gA, Cc, A), t.W1T[w1i(d, C2 + U, V, Ap, A)], tg);
         }
         if (tg == 0.0) continue;
+        double v = 0.0;
         for (int X = 0; X < nA2; ++X) {
           const int sy = (U & 1) + (V & 1) - (X & 1);  // cumulant spin rule
           if (sy < 0 || sy > 1) continue;
-          for (int y = 0; y < nA; ++y) {
-            const int Y = 2 * y + sy;
-            acc = fma(t.W1Vt[w1i(d, C2 + X, Y, Ap, Cc)] * tg, t.lam[lami(d, U, V, X, Y)], acc);
-          }
+          for (int Y = X + 1 + ((X + 1 + sy) & 1); Y < nA2; Y += 2)
+            v = fma(t.W1Vt[w1i(d, C2 + X, Y, Ap, Cc)],
+                    t.lam[lami(d, U, V, X, Y)] - t.lam[lami(d, V, U, X, Y)], v);
         }
+        acc = fma(v, tg, acc);
       }
-      return 0.25 * acc;
+      return 0.5 * acc;  // 1/4, both orders of (x, y)
     }
     case T_GVV: {  // G with two virtual particles, outer (X, Y, U, V)
       const int V = (int)(o % nA2), U = (int)((o / nA2) % nA2), Y = (int)((o / (nA2 * nA2)) % nA2),
-                X = (int)(o / (nA2 * nA2 * nA2));
+                X = 2 * (int)(o / (nA2 * nA2 * nA2));
       return 0.125 * t.lam[lami(d, U, V, X, Y)] * s_vv(d, z.nA, t.P12, X, Y, U, V);
     }
-    case T_H: {  // 1/8 vt_{kl}^{uv} t_{xy}^{ij} gamma_i^k gamma_j^l lambda_{uv}^{xy}, outer (K, L, X, Y)
-      const int Y = (int)(o % nA2), X = (int)((o / nA2) % nA2);
-      const long kl = o / ((long)nA2 * nA2);
-      const int K = (int)(kl / d.nH2), L = (int)(kl % d.nH2);
+    case T_H: {  // 1/8 vt_{kl}^{uv} t_{xy}^{ij} gamma_i^k gamma_j^l lambda_{uv}^{xy}, outer (K, L, X < Y)
+      const int np = nA2 * (nA2 - 1) / 2;
+      const long kl = o / np;
+      const int K = 2 * (int)(kl / d.nH2), L = (int)(kl % d.nH2);
+      const bool same = (L & 1) == 0;  // K's spin: each pair once
+      if (same && K >= L) return 0.0;
+      int X, Y;
+      pair_of(nA2, (int)(o % np), X, Y);
+      if ((K & 1) + (L & 1) != (X & 1) + (Y & 1)) return 0.0;
       double th = 0.0;
       const int ni = (K < C2) ? 1 : nA, nj = (L < C2) ? 1 : nA;
       for (int ii = 0; ii < ni; ++ii) {
@@ -837,17 +876,16 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
       for (int U = 0; U < nA2; ++U) {
         const int sv = (X & 1) + (Y & 1) - (U & 1);
         if (sv < 0 || sv > 1) continue;
-        for (int v = 0; v < nA; ++v) {
-          const int V = 2 * v + sv;
-          acc = fma(t.W2Vt[w2i(d, K, L, U, V)] * th, t.lam[lami(d, U, V, X, Y)], acc);
-        }
+        for (int V = U + 1 + ((U + 1 + sv) & 1); V < nA2; V += 2)
+          acc = fma(t.W2Vt[w2i(d, K, L, U, V)],
+                    t.lam[lami(d, U, V, X, Y)] - t.lam[lami(d, V, U, X, Y)], acc);
       }
-      return 0.125 * acc;
+      return (same ? 0.5 : 0.25) * th * acc;  // 1/8, both orders of (x, y) and of (k, l) if same
     }
     case T_I: {  // vt_{jx}^{bu} t_{ay}^{iv} gamma_i^j eta_b^a lambda_{uv}^{xy}, outer (J, Bp, U, X)
       const int X = (int)(o % nA2), U = (int)((o / nA2) % nA2);
       const long jb = o / ((long)nA2 * nA2);
-      const int J = (int)(jb / d.nP2), Bp = (int)(jb % d.nP2);
+      const int J = 2 * (int)(jb / d.nP2), Bp = (int)(jb % d.nP2);
       const double vt = t.W1Vt[w1i(d, J, X, Bp, U)];
       if (vt == 0.0) return 0.0;
       double c = 0.0;
@@ -861,55 +899,19 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
       }
       return vt * c;
     }
-    case T_J: {  // 1/4 vt_{mz}^{uv} t_{xy}^{mw} lambda_{uvw}^{xyz}, outer (M, W, X, Y)
-      if (!t.lam3) return 0.0;
-      const int Y = (int)(o % nA2), X = (int)((o / nA2) % nA2), W = (int)((o / (nA2 * nA2)) % nA2);
-      const int M = (int)(o / ((long)nA2 * nA2 * nA2));
-      const double tt = t.W1T[w1i(d, M, W, X, Y)];
-      if (tt == 0.0) return 0.0;
-      for (int Z = 0; Z < nA2; ++Z)
-        for (int U = 0; U < nA2; ++U) {
-          // <M Z||U V> conserves spin: s_V = s_M + s_Z - s_U
-          const int sv = (M & 1) + (Z & 1) - (U & 1);
-          if (sv < 0 || sv > 1) continue;
-          // the cumulant conserves spin: s_U + s_V + s_W = s_X + s_Y + s_Z
-          if ((U & 1) + sv + (W & 1) != (X & 1) + (Y & 1) + (Z & 1)) continue;
-          for (int v = 0; v < nA; ++v) {
-            const int V = 2 * v + sv;
-            acc = fma(t.W1Vt[w1i(d, M, Z, U, V)], t.lam3[lam3i(nA2, U, V, W, X, Y, Z)], acc);
-          }
-        }
-      return 0.25 * tt * acc;
-    }
-    case T_K: {  // 1/4 vt_{xy}^{we} t_{ez}^{uv} lambda_{uvw}^{xyz}, outer (E, U, V, Z)
-      // vt_{xy}^{we} = <xy||we> = -<xy||ew> = -W1Vt[x, y, e, w]; t_{ez}^{uv} = W1T[u, v, e, z]
-      if (!t.lam3) return 0.0;
-      const int Z = (int)(o % nA2), V = (int)((o / nA2) % nA2), U = (int)((o / (nA2 * nA2)) % nA2);
-      const int Ap = nA2 + (int)(o / ((long)nA2 * nA2 * nA2));
-      const double tt = t.W1T[w1i(d, C2 + U, V, Ap, Z)];
-      if (tt == 0.0) return 0.0;
-      for (int X = 0; X < nA2; ++X)
-        for (int Y = 0; Y < nA2; ++Y) {
-          // <X Y||E W> conserves spin: s_W = s_X + s_Y - s_E
-          const int sw = (X & 1) + (Y & 1) - (Ap & 1);
-          if (sw < 0 || sw > 1) continue;
-          if ((U & 1) + (V & 1) + sw != (X & 1) + (Y & 1) + (Z & 1)) continue;
-          for (int w = 0; w < nA; ++w) {
-            const int W = 2 * w + sw;
-            acc = fma(t.W1Vt[w1i(d, C2 + X, Y, Ap, W)], t.lam3[lam3i(nA2, U, V, W, X, Y, Z)], acc);
-          }
-        }
-      return -0.25 * tt * acc;
-    }
     case T_F4: {  // 1/4 vt_{xu}^{ef} t_{ef}^{yv} gamma_y^x gamma_v^u, outer (X, U, Y, V)
       const int V = (int)(o % nA2), Y = (int)((o / nA2) % nA2), U = (int)((o / (nA2 * nA2)) % nA2),
-                X = (int)(o / (nA2 * nA2 * nA2));
+                X = 2 * (int)(o / (nA2 * nA2 * nA2));
       return 0.25 * ga(d, t.gA, X, Y) * ga(d, t.gA, U, V) * s_vv(d, z.nA, t.P12, X, U, Y, V);
     }
-    case T_F5: {  // 1/4 vt_{mn}^{vy} t_{ux}^{mn} eta_v^u eta_y^x, outer (M, N, V, Y)
-      const int Y = (int)(o % nA2), V = (int)((o / nA2) % nA2);
-      const long mn = o / ((long)nA2 * nA2);
-      const int M = (int)(mn / C2), N = (int)(mn % C2);
+    case T_F5: {  // 1/4 vt_{mn}^{vy} t_{ux}^{mn} eta_v^u eta_y^x, outer (M, N, V < Y)
+      const int np = nA2 * (nA2 - 1) / 2;
+      const long mn = o / np;
+      const int M = 2 * (int)(mn / C2), N = (int)(mn % C2);
+      const bool same = (N & 1) == 0;  // M's spin: each pair once
+      if (same && M >= N) return 0.0;
+      int V, Y;
+      pair_of(nA2, (int)(o % np), V, Y);
       const double vt = t.W2Vt[w2i(d, M, N, V, Y)];
       if (vt == 0.0) return 0.0;
       for (int u = 0; u < nA; ++u) {
@@ -920,47 +922,13 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
           acc = fma(eu * ea(d, t.gA, X, Y), t.W2T[w2i(d, M, N, U, X)], acc);
         }
       }
-      return 0.25 * vt * acc;
+      return (same ? 1.0 : 0.5) * vt * acc;  // 1/4, both orders of (v, y) and of (m, n) if same
     }
-    case T_F6: {  // vt_{mx}^{ve} t_{ue}^{my} gamma_y^x eta_v^u, outer (M, E, X, V)
-      const int V = (int)(o % nA2), X = (int)((o / nA2) % nA2);
-      const long me = o / ((long)nA2 * nA2);
-      const int M = (int)(me / d.nV2), Ap = nA2 + (int)(me % d.nV2);
-      const double vt = t.W1Vt[w1i(d, M, X, Ap, V)];
-      if (vt == 0.0) return 0.0;
-      for (int y = 0; y < nA; ++y) {
-        const int Y = 2 * y + (X & 1);
-        const double gy = ga(d, t.gA, X, Y);
-        for (int u = 0; u < nA; ++u) {
-          const int U = 2 * u + (V & 1);
-          acc = fma(gy * ea(d, t.gA, U, V), t.W1T[w1i(d, M, Y, Ap, U)], acc);
-        }
-      }
-      return vt * acc;
-    }
-    case T_F7: {  // 1/2 vt_{yz}^{ve} t_{ue}^{wx} gamma_w^y gamma_x^z eta_v^u, outer (E, Y, Z, V)
-      const int V = (int)(o % nA2), Z = (int)((o / nA2) % nA2), Y = (int)((o / (nA2 * nA2)) % nA2);
-      const int Ap = nA2 + (int)(o / ((long)nA2 * nA2 * nA2));
-      const double vt = t.W1Vt[w1i(d, C2 + Y, Z, Ap, V)];
-      if (vt == 0.0) return 0.0;
-      for (int w = 0; w < nA; ++w) {
-        const int W = 2 * w + (Y & 1);
-        const double gw = ga(d, t.gA, Y, W);
-        for (int x = 0; x < nA; ++x) {
-          const int X = 2 * x + (Z & 1);
-          const double gg = gw * ga(d, t.gA, Z, X);
-          if (gg == 0.0) continue;
-          for (int u = 0; u < nA; ++u) {
-            const int U = 2 * u + (V & 1);
-            acc = fma(gg * ea(d, t.gA, U, V), t.W1T[w1i(d, C2 + W, X, Ap, U)], acc);
-          }
-        }
-      }
-      return 0.5 * vt * acc;
-    }
-    case T_F8: {  // 1/2 vt_{mw}^{vy} t_{ux}^{mz} gamma_z^w eta_v^u eta_y^x, outer (M, W, V, Y)
-      const int Y = (int)(o % nA2), V = (int)((o / nA2) % nA2), W = (int)((o / (nA2 * nA2)) % nA2);
-      const int M = (int)(o / ((long)nA2 * nA2 * nA2));
+    case T_F8: {  // 1/2 vt_{mw}^{vy} t_{ux}^{mz} gamma_z^w eta_v^u eta_y^x, outer (M, W, V < Y)
+      const int np = nA2 * (nA2 - 1) / 2;
+      int V, Y;
+      pair_of(nA2, (int)(o % np), V, Y);
+      const int W = (int)((o / np) % nA2), M = 2 * (int)(o / ((long)np * nA2));
       const double vt = t.W1Vt[w1i(d, M, W, V, Y)];
       if (vt == 0.0) return 0.0;
       for (int zz = 0; zz < nA; ++zz) {
@@ -976,10 +944,101 @@ __device__ double term_value(int term, long o, const Sizes& z, const ActDims& d,
           }
         }
       }
-      return 0.5 * vt * acc;
+      return vt * acc;  // 1/2, both orders of (v, y)
     }
   }
   return 0.0;
+}
+
+// Terms J and K, the ones with the three-body cumulant:
+//   K = -1/4 sum_E sum T[U,V,E,Z] lam3_{uvw}^{xyz} Vt[X,Y,E,W],
+//   J =  1/4 sum_M sum Vt[M,Z,U,V] lam3_{uvw}^{xyz} T[M,W,X,Y].
+// Vt and T are antisymmetric in the pairs (U,V) and (X,Y) and conserve spin, so for an
+// orbital e (or m) of spin s both are r^T L c with the triples (U < V, Z) and (X < Y, W),
+// s_U + s_V - s_Z = s, and L the cumulant antisymmetrised over both pairs: 175 triples at
+// nA = 5 where the full sums of a term ran over 375 x 375, each product from the L2. The
+// orbitals of spin 1 have the same r and c with all spins flipped, so L adds both.
+// l3_pack_kernel forms L once, term_jk_kernel the tiles of L c and their products with r.
+// (31/5/467/1609: the terms of term_value took 1343 us with J and K among them, 420 us without,
+// and J and K 54 us here; the FP64 pipe bounds it.)
+__host__ __device__ __forceinline__ int jk_triples(int nA) { return (nA * (nA - 1) / 2 + nA * nA) * nA; }
+// Triple r of spin 0: U | V << 8 | third << 16 (spin orbitals; with every spin flipped it
+// is a triple of spin 1).
+__device__ __forceinline__ int jk_triple(int nA, int r) {
+  const int n0 = nA * (nA - 1) / 2 * nA;
+  if (r < n0) {  // U and V of spin 0: the third too
+    int u, v;
+    pair_of(nA, r / nA, u, v);
+    return 2 * u | 2 * v << 8 | 2 * (r % nA) << 16;
+  }
+  r -= n0;  // one of each: the third of spin 1
+  const int p = r / nA;
+  return 2 * (p / nA) | (2 * (p % nA) + 1) << 8 | (2 * (r % nA) + 1) << 16;
+}
+
+__global__ void __launch_bounds__(256) l3_pack_kernel(Sizes z, const double* __restrict__ L3,
+                                                      double* __restrict__ Lp) {
+  const int R = jk_triples(z.nA), n2 = 2 * z.nA;
+  const int k = blockIdx.x * 256 + threadIdx.x;
+  if (k >= R * R) return;
+  const int a = jk_triple(z.nA, k / R), b = jk_triple(z.nA, k % R);
+  double v = 0.0;
+  for (int f = 0; f < 2; ++f) {
+    const int U = (a & 255) ^ f, V = ((a >> 8) & 255) ^ f, Z = (a >> 16) ^ f;
+    const int X = (b & 255) ^ f, Y = ((b >> 8) & 255) ^ f, W = (b >> 16) ^ f;
+    v += (L3[lam3i(n2, U, V, W, X, Y, Z)] - L3[lam3i(n2, V, U, W, X, Y, Z)]) -
+         (L3[lam3i(n2, U, V, W, Y, X, Z)] - L3[lam3i(n2, V, U, W, Y, X, Z)]);
+  }
+  Lp[k] = v;
+}
+
+constexpr int JK_T = 16;  // tile edge (triples x orbitals) and K chunk
+// blockIdx.y = 0: term K (orbitals e), 1: term J (orbitals m); the slots of terms_kernel.
+__global__ void __launch_bounds__(JK_T * JK_T) term_jk_kernel(Sizes z, TermArgs t,
+                                                              const double* __restrict__ Lp,
+                                                              double* __restrict__ partials) {
+  __shared__ double sL[JK_T][JK_T + 1], sC[JK_T][JK_T + 1], red[JK_T * JK_T / 32];
+  extern __shared__ int tri[];  // [R]
+  const ActDims d = act_dims(z);
+  const int nA = z.nA, R = jk_triples(nA), C2 = d.nC2;
+  const bool isK = blockIdx.y == 0;
+  const int n = isK ? z.nV : z.nC, nt = (n + JK_T - 1) / JK_T, rt = (R + JK_T - 1) / JK_T;
+  const int tx = threadIdx.x % JK_T, ty = threadIdx.x / JK_T;
+  double acc = 0.0;
+  if (blockIdx.x < nt * rt) {
+    for (int k = threadIdx.x; k < R; k += JK_T * JK_T) tri[k] = jk_triple(nA, k);
+    __syncthreads();
+  }
+  for (int tile = blockIdx.x; tile < nt * rt; tile += gridDim.x) {
+    const int r0 = tile / nt * JK_T, o0 = tile % nt * JK_T;
+    const int o = o0 + ty;  // the staged column's orbital
+    const int O = 2 * o;
+    double v = 0.0;
+    for (int c0 = 0; c0 < R; c0 += JK_T) {
+      const int c = c0 + tx;
+      double l = 0.0, x = 0.0;
+      if (c < R) {
+        if (r0 + ty < R) l = Lp[(size_t)(r0 + ty) * R + c];
+        if (o < n) {
+          const int b = tri[c], X = b & 255, Y = (b >> 8) & 255, W = b >> 16;
+          x = isK ? t.W1Vt[w1i(d, C2 + X, Y, d.nA2 + O, W)] : t.W1T[w1i(d, O, W, X, Y)];
+        }
+      }
+      __syncthreads();  // the previous chunk is read
+      sL[ty][tx] = l;
+      sC[ty][tx] = x;
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < JK_T; ++k) v = fma(sL[ty][k], sC[tx][k], v);
+    }
+    // element (triple r0 + ty, orbital o0 + tx)
+    if (r0 + ty < R && o0 + tx < n) {
+      const int a = tri[r0 + ty], U = a & 255, V = (a >> 8) & 255, Z = a >> 16, Q = 2 * (o0 + tx);
+      acc = fma(isK ? -t.W1T[w1i(d, C2 + U, V, d.nA2 + Q, Z)] : t.W1Vt[w1i(d, Q, Z, U, V)], v, acc);
+    }
+  }
+  const double tot = block_sum<JK_T * JK_T>(0.25 * acc, red);
+  if (threadIdx.x == 0) partials[(size_t)(isK ? T_K : T_J) * gridDim.x + blockIdx.x] = tot;
 }
 
 constexpr int TERM_NT = 128;
@@ -992,8 +1051,9 @@ __global__ void __launch_bounds__(TERM_NT) terms_kernel(Sizes z, TermArgs t,
   const int term = blockIdx.y;
   if (term == T_F6 || term == T_F7) return;  // term_f6_kernel, term_f7_kernel
   if (term == T_I && z.nA <= 6) return;      // term_i_kernel
+  if ((term == T_J || term == T_K) && t.lam3) return;  // term_jk_kernel
   const long n = term_count(term, d);
-  if ((long)blockIdx.x * TERM_NT >= n || ((term == T_J || term == T_K) && !t.lam3)) {
+  if ((long)blockIdx.x * TERM_NT >= n) {
     // nothing for this CTA: no block sum (its FP64 adds are what most CTAs of a small
     // system would spend their time on)
     if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = 0.0;
@@ -1002,7 +1062,7 @@ __global__ void __launch_bounds__(TERM_NT) terms_kernel(Sizes z, TermArgs t,
   double v = 0.0;
   for (long o = (long)blockIdx.x * TERM_NT + threadIdx.x; o < n; o += (long)gridDim.x * TERM_NT)
     v += term_value(term, o, z, d, t);
-  const double tot = block_sum<TERM_NT>(v, red);
+  const double tot = block_sum<TERM_NT>(2.0 * v, red);
   if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
 }
 
@@ -1035,8 +1095,8 @@ __global__ void __launch_bounds__(TERM_NT) term_f7_kernel(Sizes z, TermArgs t,
     se[k] = ((k / A2) == (k % A2) ? 1.0 : 0.0) - t.gA[k];
   }
   double acc = 0.0;
-  for (int e = blockIdx.x; e < d.nV2; e += gridDim.x) {
-    const int Ap = A2 + e;
+  for (int e = blockIdx.x; e < z.nV; e += gridDim.x) {
+    const int Ap = A2 + 2 * e;  // spin 0, twice
     __syncthreads();
     for (int k = threadIdx.x; k < A3; k += TERM_NT) {  // t[W,X,U], U fastest
       const int U = k % A2, X = (k / A2) % A2, W = k / (A2 * A2);
@@ -1076,7 +1136,7 @@ __global__ void __launch_bounds__(TERM_NT) term_f7_kernel(Sizes z, TermArgs t,
       acc = fma(t.W1Vt[w1i(d, C2 + Y, Z, Ap, V)], v, acc);
     }
   }
-  const double tot = block_sum<TERM_NT>(0.5 * acc, red);
+  const double tot = block_sum<TERM_NT>(acc, red);
   if (threadIdx.x == 0) partials[(size_t)T_F7 * gridDim.x + blockIdx.x] = tot;
 }
 
@@ -1094,9 +1154,9 @@ __global__ void __launch_bounds__(TERM_NT) term_f6_kernel(Sizes z, TermArgs t,
   }
   __syncthreads();
   double acc = 0.0;
-  const long n = (long)d.nC2 * d.nV2;
+  const long n = (long)z.nC * d.nV2;  // M of spin 0, twice
   for (long me = (long)blockIdx.x * NW + warp; me < n; me += (long)gridDim.x * NW) {
-    const int M = (int)(me / d.nV2), Ap = A2 + (int)(me % d.nV2);
+    const int M = 2 * (int)(me / d.nV2), Ap = A2 + (int)(me % d.nV2);
     for (int k = lane; k < A2 * A2; k += 32)  // T[Y,U] = T_{my}^{ue}
       sT[warp][k] = t.W1T[w1i(d, M, k / A2, Ap, k % A2)];
     __syncwarp();
@@ -1123,7 +1183,7 @@ __global__ void __launch_bounds__(TERM_NT) term_f6_kernel(Sizes z, TermArgs t,
     }
     __syncwarp();
   }
-  const double tot = block_sum<TERM_NT>(acc, red);
+  const double tot = block_sum<TERM_NT>(2.0 * acc, red);
   if (threadIdx.x == 0) partials[(size_t)T_F6 * gridDim.x + blockIdx.x] = tot;
 }
 
@@ -1146,14 +1206,14 @@ __global__ void __launch_bounds__(TI_NT) term_i_kernel(Sizes z, TermArgs t,
     lamT[k] = t.lam[lami(d, U, V, X, Y)];
   }
   double acc = 0.0;
-  const long n = (long)d.nH2 * d.nP2;
+  const long n = (long)z.nH * d.nP2;  // J of spin 0, twice
   for (long r0 = (long)blockIdx.x * TI_ROWS; r0 < n; r0 += (long)gridDim.x * TI_ROWS) {
     __syncthreads();  // the previous rows' reads are done (and the cumulant is staged)
     for (int k = threadIdx.x; k < TI_ROWS * AA; k += TI_NT) {
       const long r = r0 + k / AA;
       double v = 0.0;
       if (r < n) {
-        const int J = (int)(r / d.nP2), Bp = (int)(r % d.nP2), V = (k % AA) / A2, Y = k % A2;
+        const int J = 2 * (int)(r / d.nP2), Bp = (int)(r % d.nP2), V = (k % AA) / A2, Y = k % A2;
         v = t.Ti[w1i(d, J, V, Bp, Y)];
       }
       sTi[k] = v;
@@ -1166,7 +1226,7 @@ __global__ void __launch_bounds__(TI_NT) term_i_kernel(Sizes z, TermArgs t,
     for (int k = threadIdx.x; k < TI_ROWS * NUX; k += TI_NT) {
       const long r = r0 + k / NUX;
       if (r >= n) break;
-      const int J = (int)(r / d.nP2), Bp = (int)(r % d.nP2);
+      const int J = 2 * (int)(r / d.nP2), Bp = (int)(r % d.nP2);
       const int sJ = J & 1, sB = Bp & 1, m = k % NUX;
       int U, X;
       if (sJ == sB) {
@@ -1195,7 +1255,7 @@ __global__ void __launch_bounds__(TI_NT) term_i_kernel(Sizes z, TermArgs t,
       acc = fma(vt, c, acc);
     }
   }
-  const double tot = block_sum<TI_NT>(acc, red);
+  const double tot = block_sum<TI_NT>(2.0 * acc, red);
   if (threadIdx.x == 0) partials[(size_t)T_I * gridDim.x + blockIdx.x] = tot;
 }
 
@@ -1233,6 +1293,8 @@ bool active_alloc(dsrg_plan* p) {
   ok = ok && plan_alloc(p, (void**)&w.ft, (size_t)d.nH2 * d.nP2 * 8);
   ok = ok && plan_alloc(p, (void**)&w.M, (size_t)z.nA * z.nA * z.nV * z.nV * 8);
   ok = ok && plan_alloc(p, (void**)&w.P12, 2 * nA4 * 8);
+  const size_t R = jk_triples(z.nA);
+  ok = ok && plan_alloc(p, (void**)&w.L3p, R * R * 8);
   ok = ok && plan_alloc(p, (void**)&w.P12part, (size_t)ACTVV_BLOCKS * 2 * nA4 * 8);
   return ok;
 }
@@ -1281,12 +1343,21 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     const size_t n = w.w1n / 16 + w.w2n / 16 + (size_t)d.nA2 * d.nA2 * d.nA2 * d.nA2 +
                      (size_t)d.nA2 * d.nA2;
     build_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        eps, G, L, s, z, w.K1, w.K2, w.K3, w.W1, w.W2, w.lam, w.gA, w.w1n, w.w2n);
+        eps, G, L, s, z, w.K1, w.K2, w.K3, w.W1, w.W2, w.lam, w.gA, w.w1n, w.w2n,
+        p->grad != nullptr);
     DSRG_LAUNCH_CHECK(p);
   }
   {
-    const int n = d.nH2 * d.nP2;
-    t1_kernel<<<(n + 255) / 256, 256, 0, st>>>(eps, s, z, w.W1 + w.w1n, w.gA, F1, w.t1, w.ft);
+    const int n = d.nH2 * z.nP;
+#define T1_CASE(NA_)                                                                             \
+  case NA_:                                                                                      \
+    t1_kernel<NA_><<<(n + 127) / 128, 128, 0, st>>>(eps, s, z, w.W1 + w.w1n, w.gA, F1, w.t1, w.ft); \
+    break;
+    switch (z.nA) {
+      T1_CASE(1) T1_CASE(2) T1_CASE(3) T1_CASE(4) T1_CASE(5) T1_CASE(6) T1_CASE(7) T1_CASE(8)
+      default: return cudaErrorInvalidValue;
+    }
+#undef T1_CASE
     DSRG_LAUNCH_CHECK(p);
   }
   {
@@ -1300,7 +1371,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   const int nA4 = z.nA * z.nA * z.nA * z.nA;
   {
     const bool f32 = p->prec != DSRG_PREC_FP64;
-    const size_t smg = (size_t)3 * z.nA * z.nA * ACTVV_CH * sizeof(double);
+    const size_t smg = (size_t)3 * z.nA * z.nA * ACTVV_LD * sizeof(double);
 #define ACTVV_GEN(NA_)                                                                       \
   case NA_:                                                                                  \
     if (f32) {                                                                        \
@@ -1354,6 +1425,14 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     dim3 grid(term_blocks(z), N_TERMS);
     terms_kernel<<<grid, TERM_NT, 0, st>>>(z, ta, p->d_partials + sg.begin);
     DSRG_LAUNCH_CHECK(p);
+    if (L3) {
+      const int R = jk_triples(z.nA);
+      l3_pack_kernel<<<(R * R + 255) / 256, 256, 0, st>>>(z, L3, w.L3p);
+      DSRG_LAUNCH_CHECK(p);
+      term_jk_kernel<<<dim3(term_blocks(z), 2), JK_T * JK_T, R * sizeof(int), st>>>(
+          z, ta, w.L3p, p->d_partials + sg.begin);
+      DSRG_LAUNCH_CHECK(p);
+    }
     const size_t smf7 = f7_smem_bytes(z.nA), smti = ti_smem_bytes(z.nA);
 #define F67_LAUNCH(NA_)                                                                        \
   case NA_:                                                                                    \
