@@ -156,40 +156,166 @@ __device__ __forceinline__ void oz_bulk(void* dst, const void* src, uint32_t byt
       : "memory");
 }
 
-template <int N>
-__device__ __forceinline__ void oz_mma(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                       uint32_t acc) {
-#define OZ_MMA(CU)                                                                               \
-  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"         \
-               " @q tcgen05.mma.cta_group::1.kind::f16" CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
-               "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(leader)                                 \
-               : "memory")
-  if (N == 0) OZ_MMA(".collector::a::fill");
-  else if (N == 1) OZ_MMA(".collector::a::use");
-  else OZ_MMA(".collector::a::lastuse");
-#undef OZ_MMA
+// The products of digit i of A (descriptor low word a) with the digits 1 .. JN of B (from
+// b), into the accumulators from d on; the leader lane of a converged warp issues. MODE 0:
+// `acc` is for all of them, 1: for the last, the others accumulate, 2: all accumulate. A
+// stays in the collector buffer. One block per digit: see tc_mma3_if.
+template <int JN, int MODE>
+__device__ __forceinline__ void oz_row(uint32_t leader, uint32_t d, uint32_t a, uint32_t b, uint32_t acc) {
+  constexpr uint32_t idesc = idesc_128xn<true>(OZ_BN);
+  static_assert((MODE == 2 && JN >= 2 && JN <= 6) || (MODE < 2 && JN == 7), "the rows of oz_kstep");
+  if constexpr (JN == 7 && MODE == 0) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2, b3, b4, b5, b6;\n"
+        " setp.ne.b32 p, %16, 0;\n setp.ne.b32 q, %17, 0;\n mov.b64 a, {%14, %18};\n"
+        " mov.b64 b0, {%7, %18};\n"
+        " mov.b64 b1, {%8, %18};\n"
+        " mov.b64 b2, {%9, %18};\n"
+        " mov.b64 b3, {%10, %18};\n"
+        " mov.b64 b4, {%11, %18};\n"
+        " mov.b64 b5, {%12, %18};\n"
+        " mov.b64 b6, {%13, %18};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%2], a, b2, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%3], a, b3, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%4], a, b4, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%5], a, b5, %15, p;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%6], a, b6, %15, p;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN), "r"(d + 3 * OZ_BN),
+        "r"(d + 4 * OZ_BN), "r"(d + 5 * OZ_BN), "r"(d + 6 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(b + 3 * OZ_B_SLICE / 16), "r"(b + 4 * OZ_B_SLICE / 16), "r"(b + 5 * OZ_B_SLICE / 16),
+        "r"(b + 6 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 7 && MODE == 1) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2, b3, b4, b5, b6;\n"
+        " setp.ne.b32 p, %16, 0;\n setp.ne.b32 q, %17, 0;\n mov.b64 a, {%14, %18};\n"
+        " mov.b64 b0, {%7, %18};\n"
+        " mov.b64 b1, {%8, %18};\n"
+        " mov.b64 b2, {%9, %18};\n"
+        " mov.b64 b3, {%10, %18};\n"
+        " mov.b64 b4, {%11, %18};\n"
+        " mov.b64 b5, {%12, %18};\n"
+        " mov.b64 b6, {%13, %18};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%2], a, b2, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%3], a, b3, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%4], a, b4, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%5], a, b5, %15, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%6], a, b6, %15, p;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN), "r"(d + 3 * OZ_BN),
+        "r"(d + 4 * OZ_BN), "r"(d + 5 * OZ_BN), "r"(d + 6 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(b + 3 * OZ_B_SLICE / 16), "r"(b + 4 * OZ_B_SLICE / 16), "r"(b + 5 * OZ_B_SLICE / 16),
+        "r"(b + 6 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 6 && MODE == 2) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2, b3, b4, b5;\n"
+        " setp.ne.b32 p, %14, 0;\n setp.ne.b32 q, %15, 0;\n mov.b64 a, {%12, %16};\n"
+        " mov.b64 b0, {%6, %16};\n"
+        " mov.b64 b1, {%7, %16};\n"
+        " mov.b64 b2, {%8, %16};\n"
+        " mov.b64 b3, {%9, %16};\n"
+        " mov.b64 b4, {%10, %16};\n"
+        " mov.b64 b5, {%11, %16};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %13, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %13, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%2], a, b2, %13, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%3], a, b3, %13, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%4], a, b4, %13, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%5], a, b5, %13, q;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN), "r"(d + 3 * OZ_BN),
+        "r"(d + 4 * OZ_BN), "r"(d + 5 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(b + 3 * OZ_B_SLICE / 16), "r"(b + 4 * OZ_B_SLICE / 16), "r"(b + 5 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 5 && MODE == 2) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2, b3, b4;\n"
+        " setp.ne.b32 p, %12, 0;\n setp.ne.b32 q, %13, 0;\n mov.b64 a, {%10, %14};\n"
+        " mov.b64 b0, {%5, %14};\n"
+        " mov.b64 b1, {%6, %14};\n"
+        " mov.b64 b2, {%7, %14};\n"
+        " mov.b64 b3, {%8, %14};\n"
+        " mov.b64 b4, {%9, %14};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %11, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %11, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%2], a, b2, %11, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%3], a, b3, %11, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%4], a, b4, %11, q;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN), "r"(d + 3 * OZ_BN),
+        "r"(d + 4 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(b + 3 * OZ_B_SLICE / 16), "r"(b + 4 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 4 && MODE == 2) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2, b3;\n"
+        " setp.ne.b32 p, %10, 0;\n setp.ne.b32 q, %11, 0;\n mov.b64 a, {%8, %12};\n"
+        " mov.b64 b0, {%4, %12};\n"
+        " mov.b64 b1, {%5, %12};\n"
+        " mov.b64 b2, {%6, %12};\n"
+        " mov.b64 b3, {%7, %12};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %9, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %9, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%2], a, b2, %9, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%3], a, b3, %9, q;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN), "r"(d + 3 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(b + 3 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 3 && MODE == 2) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1, b2;\n"
+        " setp.ne.b32 p, %8, 0;\n setp.ne.b32 q, %9, 0;\n mov.b64 a, {%6, %10};\n"
+        " mov.b64 b0, {%3, %10};\n"
+        " mov.b64 b1, {%4, %10};\n"
+        " mov.b64 b2, {%5, %10};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %7, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], a, b1, %7, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%2], a, b2, %7, q;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN), "r"(d + 2 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16), "r"(b + 2 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  } else if constexpr (JN == 2 && MODE == 2) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n .reg .b64 a, b0, b1;\n"
+        " setp.ne.b32 p, %6, 0;\n setp.ne.b32 q, %7, 0;\n mov.b64 a, {%4, %8};\n"
+        " mov.b64 b0, {%2, %8};\n"
+        " mov.b64 b1, {%3, %8};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], a, b0, %5, q;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], a, b1, %5, q;\n"
+        "}\n" ::"r"(d + 0 * OZ_BN), "r"(d + 1 * OZ_BN),
+        "r"(b + 0 * OZ_B_SLICE / 16), "r"(b + 1 * OZ_B_SLICE / 16),
+        "r"(a), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)
+        : "memory");
+  }
 }
 
-// One K step (16 values): digit pairs (i, j), i + j <= 9, the j of one i back to back.
-__device__ __forceinline__ void oz_kstep(uint32_t leader, uint32_t d, uint32_t sa, uint32_t sb, bool first) {
-  constexpr uint32_t idesc = idesc_128xn<true>(OZ_BN);
-#pragma unroll
-  for (int i = 1; i <= OZ_S; ++i) {
-    const uint64_t a = desc_sw64(sa + (i - 1) * OZ_A_SLICE);
-    const int jn = (OZ_G + 1 - i) < OZ_S ? (OZ_G + 1 - i) : OZ_S;  // j <= 9 - i and <= 7
-#pragma unroll
-    for (int j = 1; j <= jn; ++j) {
-      const int g = i + j;
-      const uint64_t b = desc_sw64(sb + (j - 1) * OZ_B_SLICE);
-      // the first product of a weight starts its accumulator
-      const int i0 = g - OZ_S > 1 ? g - OZ_S : 1;
-      const uint32_t acc = (first && i == i0) ? 0u : 1u;
-      const uint32_t dg = d + (uint32_t)((g - 2) * OZ_BN);
-      if (j == 1) oz_mma<0>(leader, dg, a, b, idesc, acc);
-      else if (j == jn) oz_mma<2>(leader, dg, a, b, idesc, acc);
-      else oz_mma<1>(leader, dg, a, b, idesc, acc);
-    }
-  }
+// One K step (16 values) from the descriptor low words of the first slices: digit pairs
+// (i, j), i + j <= 9 (accumulator i + j - 2), the j of one i back to back. The first product
+// of a weight starts its accumulator: those of i = 1, and (2, 7).
+__device__ __forceinline__ void oz_kstep(uint32_t leader, uint32_t d, uint32_t a, uint32_t b, bool first) {
+  static_assert(OZ_S == 7 && OZ_G == 8, "the rows below");
+  constexpr uint32_t A = OZ_A_SLICE / 16;
+  const uint32_t acc = first ? 0u : 1u;
+  oz_row<7, 0>(leader, d, a, b, acc);
+  oz_row<7, 1>(leader, d + OZ_BN, a + A, b, acc);
+  oz_row<6, 2>(leader, d + 2 * OZ_BN, a + 2 * A, b, 1u);
+  oz_row<5, 2>(leader, d + 3 * OZ_BN, a + 3 * A, b, 1u);
+  oz_row<4, 2>(leader, d + 4 * OZ_BN, a + 4 * A, b, 1u);
+  oz_row<3, 2>(leader, d + 5 * OZ_BN, a + 5 * A, b, 1u);
+  oz_row<2, 2>(leader, d + 6 * OZ_BN, a + 6 * A, b, 1u);
 }
 
 __device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -315,7 +441,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
   } else if (warp == 1) {
     const uint32_t leader = tc_elect();
-    const uint32_t tm = tc_uniform(tmem);
+    const uint32_t tm = tc_uniform(tmem), base_lo = tc_uniform(desc_sw64_lo(su32(smem)));
     int stage = 0;
     uint32_t phase = 0, tphase = 0;
     bool ok = true, issued = false;
@@ -333,9 +459,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t sa = su32(smem) + stage * OZ_STAGE_BYTES, sb = sa + OZ_A_BYTES;
+        const uint32_t sa = base_lo + (uint32_t)(stage * (OZ_STAGE_BYTES / 16)), sb = sa + OZ_A_BYTES / 16;
         oz_kstep(leader, tm, sa, sb, kb % OZ_CHUNK == 0);
-        oz_kstep(leader, tm, sa + 32, sb + 32, false);
+        oz_kstep(leader, tm, sa + 32 / 16, sb + 32 / 16, false);
         issued = true;
         tc_commit_if(leader, &empty[stage]);
         if (++stage == OZ_STAGES) {

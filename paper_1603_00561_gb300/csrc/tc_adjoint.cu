@@ -17,14 +17,17 @@
 // must not carry the whole sum: every K stage (32 values) is its own
 // accumulation in TMEM every AG_CH = 2 stages (64 values, 12 MMAs), which the
 // epilogue adds in FP32 round-to-nearest into registers; every AG_L1 of those
-// the register sums go into a second FP32 sum in shared memory, and the two
-// are added in FP64 at the end.
+// the register sums go into a second FP32 sum in TMEM, and the two are added in
+// FP64 at the end.
 //
 // Roles (one CTA per SM, persistent): warp 0 TMA producer, warp 1 TMEM
 // allocator and MMA issuer, warps 2-9 epilogue (two warps per TMEM lane
-// quarter, 64 columns each). Shared memory: 4 stages x (S tile, B^T tile) x
-// (hi, lo) x 128 rows x 64 bytes, 64-byte swizzle; 64 KB of second-level sums.
-// TMEM: 4 buffers x 128 columns. Every wait is bounded (about 2 s).
+// quarter, 64 columns each). Shared memory: 6 stages x (S tile, B^T tile) x
+// (hi, lo) x 128 rows x 64 bytes, 64-byte swizzle. TMEM: 3 buffers x 128 columns and
+// the second-level sums. Every wait is bounded (about 2 s).
+// What bounds it is the warp that issues the MMAs (loads, drains and the tensor pipe, 45 %
+// busy, all have room): 24/2/372/1200 in 1130 us with one lane issuing, 950 us with a
+// converged warp, 660 us with the MMAs of a K step in one block (tc_mma3_if).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -35,15 +38,15 @@ namespace dsrg {
 
 constexpr int AG_BM = 128, AG_BN = 128;
 constexpr int AG_KB = 64;                     // K bytes per row per stage: 32 BF16, two MMA K steps
-constexpr int AG_STAGES = 4;
+constexpr int AG_STAGES = 6;
 constexpr int AG_TILE = AG_BM * AG_KB;        // 8 KB: one operand tile of one plane
 constexpr int AG_STAGE_BYTES = 4 * AG_TILE;   // S hi, S lo, B^T hi, B^T lo
 constexpr int AG_THREADS = 320;
 constexpr int AG_EPI = 8;
-constexpr int AG_NBUF = 4;                    // TMEM accumulators
+constexpr int AG_NBUF = 3;                    // TMEM accumulators, and one more of second-level sums
 constexpr int AG_CH = 2;                      // K stages per TMEM accumulation (12 MMAs)
-constexpr int AG_L1 = 16;                     // accumulations summed in registers before the shared-memory sum
-constexpr uint32_t AG_TMEM_COLS = AG_NBUF * AG_BN;
+constexpr int AG_L1 = 16;                     // accumulations summed in registers before the second-level sum
+constexpr uint32_t AG_TMEM_COLS = (AG_NBUF + 1) * AG_BN;
 constexpr int AG_BAND = 12;                   // m tiles per band of the item order
 
 struct TcAdjWs {
@@ -208,8 +211,7 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* tiles = smem;
-  float* sL2 = (float*)(smem + AG_STAGES * AG_STAGE_BYTES);  // [64][256] second-level sums
-  uint64_t* full = (uint64_t*)(sL2 + 64 * 256);
+  uint64_t* full = (uint64_t*)(smem + AG_STAGES * AG_STAGE_BYTES);
   uint64_t* empty = full + AG_STAGES;
   uint64_t* tfull = empty + AG_STAGES;
   uint64_t* tempty = tfull + AG_NBUF;
@@ -294,6 +296,7 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
   } else if (warp == 1) {
     constexpr uint32_t idesc = idesc_128x128<true>();
     const uint32_t leader = tc_elect(), tmem_u = tc_uniform(tmem_base);
+    const uint32_t tiles_lo = tc_uniform(desc_sw64_lo(su32(tiles)));
     int stage = 0, tb = 0;
     uint32_t phase = 0, tphase = 0;
     bool ok = true, issued = false;
@@ -307,18 +310,12 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
         }
         tc_fence_after();
         const uint32_t d = tmem_u + (uint32_t)(tb * AG_BN);
-        const uint32_t sa = su32(tiles) + (uint32_t)(stage * AG_STAGE_BYTES);
+        const uint32_t sa = tiles_lo + (uint32_t)(stage * (AG_STAGE_BYTES / 16));
+        constexpr uint32_t T = AG_TILE / 16;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const uint32_t off = (uint32_t)(k * 32);
-          const uint64_t ah = desc_sw64(sa + off), al = desc_sw64(sa + AG_TILE + off);
-          const uint64_t bh = desc_sw64(sa + 2 * AG_TILE + off);
-          const uint64_t bl = desc_sw64(sa + 3 * AG_TILE + off);
-          // a fresh accumulation every AG_CH stages: lo.hi, hi.lo (keeps A), hi.hi (reuses it)
-          tc_mma_if<true>(leader, d, al, bh, idesc, (sub > 0 || k > 0) ? 1u : 0u);
-          tc_mma_if<true, 1>(leader, d, ah, bl, idesc, 1u);
-          tc_mma_if<true, 2>(leader, d, ah, bh, idesc, 1u);
-        }
+        for (int k = 0; k < 2; ++k)  // a fresh accumulation every AG_CH stages
+          tc_mma3_if<true, false>(leader, d, sa + 2 * k + T, sa + 2 * k, sa + 2 * k + 3 * T,
+                                  sa + 2 * k + 2 * T, idesc, (sub > 0 || k > 0) ? 1u : 0u);
         issued = true;
         tc_commit_if(leader, &empty[stage]);
         if (++stage == AG_STAGES) {
@@ -341,7 +338,6 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
       }
     }
   } else {
-    const int et = threadIdx.x - 64;        // 0..255
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
     const int half = (warp - 2) >> 2;       // columns 64*half ..
@@ -353,10 +349,11 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
       ag_item(it, g.m_tiles, g.n_tiles, &mt, &nt);
       float l1[64];
 #pragma unroll
-      for (int c = 0; c < 64; ++c) {
-        l1[c] = 0.f;
-        sL2[c * 256 + et] = 0.f;
-      }
+      for (int c = 0; c < 64; ++c) l1[c] = 0.f;
+      // this warp's second-level sums (nothing in them yet)
+      const uint32_t l2 = tmem_base + ((uint32_t)(quarter * 32) << 16) +
+                          (uint32_t)(AG_NBUF * AG_BN + half * 64);
+      bool any = false;
       int nl1 = 0;
       for (int kc = 0; kc < g.kblocks / AG_CH; ++kc) {
         if (ok) ok = mbar_wait(&tfull[tb], tphase, abort_flag, g.status);
@@ -379,10 +376,23 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
             for (int c = 0; c < 16; ++c) l1[16 * j + c] += __uint_as_float(r[j][c]);
           if (++nl1 == AG_L1) {
 #pragma unroll
-            for (int c = 0; c < 64; ++c) {
-              sL2[c * 256 + et] += l1[c];
-              l1[c] = 0.f;
+            for (int j = 0; j < 4; ++j) {
+              uint32_t q[16];
+#pragma unroll
+              for (int c = 0; c < 16; ++c) q[c] = 0u;
+              if (any) {
+                tmem_ld16(l2 + 16 * j, q);
+                tmem_ld_wait();
+              }
+#pragma unroll
+              for (int c = 0; c < 16; ++c) {
+                q[c] = __float_as_uint(__uint_as_float(q[c]) + l1[16 * j + c]);
+                l1[16 * j + c] = 0.f;
+              }
+              tmem_st16(l2 + 16 * j, q);
             }
+            tmem_st_wait();
+            any = true;
             nl1 = 0;
           }
         }
@@ -393,14 +403,24 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
       }
       if (!ok) continue;
       // the row of dB this thread holds: (h, p) of plane row mt*128 + row
-      int h, p;
-      if (row_hp(mt * AG_BM + row, g.nH, g.nA, g.nV, g.nVpad, g.xr0, &h, &p) != 0) continue;
+      int h = 0, p = 0;
+      const bool live = row_hp(mt * AG_BM + row, g.nH, g.nA, g.nV, g.nVpad, g.xr0, &h, &p) == 0;
       double* out = g.dB + (size_t)h * g.nP + p;
       const int q0 = nt * AG_BN + half * 64;
 #pragma unroll
-      for (int c = 0; c < 64; ++c) {
-        const int q = q0 + c;
-        if (q < g.Q) out[(size_t)q * g.HP] = (double)sL2[c * 256 + et] + (double)l1[c];
+      for (int j = 0; j < 4; ++j) {
+        uint32_t s2[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) s2[c] = 0u;
+        if (any) {
+          tmem_ld16(l2 + 16 * j, s2);
+          tmem_ld_wait();
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const int q = q0 + 16 * j + c;
+          if (live && q < g.Q) out[(size_t)q * g.HP] = (double)__uint_as_float(s2[c]) + (double)l1[16 * j + c];
+        }
       }
     }
   }
@@ -416,7 +436,7 @@ __global__ void __launch_bounds__(AG_THREADS, 1)
 }
 
 static size_t ag_smem_bytes() {
-  return 1024 + (size_t)AG_STAGES * AG_STAGE_BYTES + 64 * 256 * 4 +
+  return 1024 + (size_t)AG_STAGES * AG_STAGE_BYTES +
          (2 * AG_STAGES + 2 * AG_NBUF + 1) * 8 + 16;
 }
 

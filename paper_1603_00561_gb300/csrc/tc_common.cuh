@@ -109,8 +109,11 @@ __device__ __forceinline__ uint32_t tc_elect() {
 }
 // A value that is the same in every lane, as a warp-uniform one.
 __device__ __forceinline__ uint32_t tc_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
-// Bounded wait of a whole warp (uniform result).
-#define TC_WARP_WAIT(...) __all_sync(0xffffffffu, mbar_wait(__VA_ARGS__))
+// Bounded wait of a whole warp (uniform result): one test in line, the rest in a call.
+#define TC_WARP_WAIT(bar, ...)                     \
+  (__all_sync(0xffffffffu, mbar_try(bar, FIRST_ARG(__VA_ARGS__))) || \
+   __all_sync(0xffffffffu, mbar_wait(bar, __VA_ARGS__)))
+#define FIRST_ARG(x, ...) (x)
 __device__ __forceinline__ void tc_commit_if(uint32_t leader, uint64_t* bar) {
   asm volatile(
       "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
@@ -124,49 +127,40 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                    su32(bar))
                : "memory");
 }
-// One MMA D (+)= A·B. COL selects the A-operand collector buffer: 0 reads A from
-// shared memory and keeps nothing, 1 reads it and keeps it (fill), 2 takes the
-// A kept by the previous MMA of this thread, which must have had the same
-// descriptor, and releases it (lastuse). Reusing A saves one shared-memory
-// read of the A tile.
-template <bool BF16, int COL = 0>
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                       uint32_t acc) {
-#define DSRG_MMA(KIND, CU)                                                                   \
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"                               \
-               " tcgen05.mma.cta_group::1.kind::" KIND CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
-               "l"(a), "l"(b), "r"(idesc), "r"(acc)                                          \
+// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows at a 64-byte
+// pitch. Low word: address / 16 (offsets add as offset / 16: shared memory ends below
+// 2^18 bytes) and the leading byte offset (unused for swizzled K-major); high word: stride
+// byte offset of 8 rows x 64 B, the descriptor version of tcgen05, the swizzle.
+constexpr uint32_t DESC_SW64_HI = (512u >> 4) | 1u << 14 | 4u << 29;
+__device__ __forceinline__ uint32_t desc_sw64_lo(uint32_t saddr) { return (saddr >> 4) | 1u << 16; }
+// The products of a split K step, D (+)= [A_lo B_lo +] A_lo B_hi + A_hi B_lo + A_hi B_hi, by
+// the leader lane (tc_elect) of a whole converged warp; descriptors by their low words
+// (desc_sw64_lo). `acc` 0: D starts at the first product. A_hi stays in the collector
+// buffer between its products. One block for all of them: an MMA takes 64 clocks, and the
+// issuing warp, at 4 to 6 clocks an instruction, is what limits short stages (every MMA
+// with its own predicates and 64-bit descriptors: 65 clocks each and 575 a stage).
+template <bool BF16, bool LOLO>
+__device__ __forceinline__ void tc_mma3_if(uint32_t leader, uint32_t d, uint32_t al, uint32_t ah,
+                                           uint32_t bl, uint32_t bh, uint32_t idesc, uint32_t acc) {
+#define DSRG_MMA3(KIND, FIRST, P2)                                                              \
+  asm volatile("{\n .reg .pred p, q;\n .reg .b64 xl, xh, yl, yh;\n"                            \
+               " setp.ne.b32 p, %6, 0;\n setp.ne.b32 q, %7, 0;\n"                              \
+               " mov.b64 xl, {%1, %8};\n mov.b64 xh, {%2, %8};\n"                              \
+               " mov.b64 yl, {%3, %8};\n mov.b64 yh, {%4, %8};\n" FIRST                        \
+               " @q tcgen05.mma.cta_group::1.kind::" KIND " [%0], xl, yh, %5, " P2 ";\n"        \
+               " @q tcgen05.mma.cta_group::1.kind::" KIND ".collector::a::fill [%0], xh, yl, %5, q;\n"    \
+               " @q tcgen05.mma.cta_group::1.kind::" KIND ".collector::a::lastuse [%0], xh, yh, %5, q;\n" \
+               "}\n" ::"r"(d),                                                                  \
+               "r"(al), "r"(ah), "r"(bl), "r"(bh), "r"(idesc), "r"(acc), "r"(leader),           \
+               "r"(DESC_SW64_HI)                                                                \
                : "memory")
-  if (BF16) {
-    if (COL == 1) DSRG_MMA("f16", ".collector::a::fill");
-    else if (COL == 2) DSRG_MMA("f16", ".collector::a::lastuse");
-    else DSRG_MMA("f16", "");
-  } else {
-    if (COL == 1) DSRG_MMA("tf32", ".collector::a::fill");
-    else if (COL == 2) DSRG_MMA("tf32", ".collector::a::lastuse");
-    else DSRG_MMA("tf32", "");
-  }
-#undef DSRG_MMA
-}
-// tc_mma of a whole converged warp, issued by its leader lane (tc_elect).
-template <bool BF16, int COL = 0>
-__device__ __forceinline__ void tc_mma_if(uint32_t leader, uint32_t d, uint64_t a, uint64_t b,
-                                          uint32_t idesc, uint32_t acc) {
-#define DSRG_MMA(KIND, CU)                                                                      \
-  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"        \
-               " @q tcgen05.mma.cta_group::1.kind::" KIND CU " [%0], %1, %2, %3, p;\n}\n" ::"r"(d), \
-               "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(leader)                                 \
-               : "memory")
-  if (BF16) {
-    if (COL == 1) DSRG_MMA("f16", ".collector::a::fill");
-    else if (COL == 2) DSRG_MMA("f16", ".collector::a::lastuse");
-    else DSRG_MMA("f16", "");
-  } else {
-    if (COL == 1) DSRG_MMA("tf32", ".collector::a::fill");
-    else if (COL == 2) DSRG_MMA("tf32", ".collector::a::lastuse");
-    else DSRG_MMA("tf32", "");
-  }
-#undef DSRG_MMA
+#define DSRG_LL(KIND) " @q tcgen05.mma.cta_group::1.kind::" KIND " [%0], xl, yl, %5, p;\n"
+  if (BF16 && LOLO) DSRG_MMA3("f16", DSRG_LL("f16"), "q");
+  else if (BF16) DSRG_MMA3("f16", "", "p");
+  else if (LOLO) DSRG_MMA3("tf32", DSRG_LL("tf32"), "q");
+  else DSRG_MMA3("tf32", "", "p");
+#undef DSRG_LL
+#undef DSRG_MMA3
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -186,6 +180,18 @@ __device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, uint32_t (&r)[16]
                  : "=r"(r[8 * h]), "=r"(r[8 * h + 1]), "=r"(r[8 * h + 2]), "=r"(r[8 * h + 3]),
                    "=r"(r[8 * h + 4]), "=r"(r[8 * h + 5]), "=r"(r[8 * h + 6]), "=r"(r[8 * h + 7])
                  : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+}
+// 16 columns of the warp's 32 lanes, one register per column
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+      "%12, %13, %14, %15, %16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+      "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() {
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -273,26 +279,6 @@ __device__ __forceinline__ void tmem_add_frag(uint32_t taddr, float (&t)[NC][16]
   }
 }
 
-// Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, rows at a
-// 64-byte pitch (8-row groups 512 bytes apart).
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;           // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(512 >> 4) << 32;  // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1 << 46;           // descriptor version of tcgen05
-  d |= (uint64_t)4 << 61;           // 64-byte swizzle
-  return d;
-}
-// Shared-memory matrix descriptor: K-major operand, 32-byte swizzle, rows at a
-// 32-byte pitch (8-row groups 256 bytes apart); one MMA K step per row.
-__device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;           // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(256 >> 4) << 32;  // stride byte offset: 8 rows x 32 B
-  d |= (uint64_t)1 << 46;           // descriptor version of tcgen05
-  d |= (uint64_t)6 << 61;           // 32-byte swizzle
-  return d;
-}
 // Instruction descriptor: D = F32, A/B = TF32 (2) or BF16 (1), both K-major, M = 128, N given
 // (a multiple of 16, 16..256).
 template <bool BF16>

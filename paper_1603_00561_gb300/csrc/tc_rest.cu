@@ -78,18 +78,10 @@ __device__ __forceinline__ void gemm_stage_mmas(uint32_t leader, uint32_t d, uin
   constexpr uint32_t idesc = idesc_mn(BF16, G_BM, G_BN);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const uint32_t off = (uint32_t)((1 - k) * 32);
-    const uint64_t ah = desc_sw64(sa + off), al = desc_sw64(sa + G_A_BYTES + off);
-    const uint64_t bh = desc_sw64(sb + off), bl = desc_sw64(sb + G_B_BYTES + off);
+    const uint32_t off = (1 - k) * 32 / 16;
     const uint32_t acc0 = (kb > 0 || k > 0) ? 1u : 0u;
-    if (GRAM) {
-      tc_mma_if<BF16>(leader, d, al, bl, idesc, acc0);
-      tc_mma_if<BF16>(leader, d, al, bh, idesc, 1u);
-    } else {
-      tc_mma_if<BF16>(leader, d, al, bh, idesc, acc0);
-    }
-    tc_mma_if<BF16, 1>(leader, d, ah, bl, idesc, 1u);
-    tc_mma_if<BF16, 2>(leader, d, ah, bh, idesc, 1u);
+    tc_mma3_if<BF16, GRAM>(leader, d, sa + off + G_A_BYTES / 16, sa + off, sb + off + G_B_BYTES / 16,
+                           sb + off, idesc, acc0);
   }
 }
 
@@ -186,6 +178,7 @@ __global__ void __launch_bounds__(G_THREADS, 1)
     }
   } else if (warp == 1) {
     const uint32_t leader = tc_elect(), tmem_u = tc_uniform(tmem_base);
+    const uint32_t tiles_lo = tc_uniform(desc_sw64_lo(su32(tiles)));
     int stage = 0;
     uint32_t phase = 0;
     int tbuf = 0;
@@ -207,8 +200,8 @@ __global__ void __launch_bounds__(G_THREADS, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t sa = su32(tiles) + (uint32_t)(stage * G_STAGE_BYTES);
-        const uint32_t sb = sa + 2 * G_A_BYTES;
+        const uint32_t sa = tiles_lo + (uint32_t)(stage * (G_STAGE_BYTES / 16));
+        const uint32_t sb = sa + 2 * G_A_BYTES / 16;
         if (gram)
           gemm_stage_mmas<BF16, true>(leader, d, sa, sb, kb);
         else

@@ -25,7 +25,8 @@
 // Measured on one GB300 (this kernel alone, BF16x3): cc-pVTZ size (24/2/372/1200)
 // 855 us with the FP64 regulator and row-per-lane tail sums, 475 us with FP32 pairs,
 // 454 us with the MMAs and copies issued from a converged warp (tc_elect); cc-pV5Z
-// size (24/2/1214/3400) 8.45 ms, 8.2 ms, 6.88 ms; TF32x3 at 31/5/467/1609
+// size (24/2/1214/3400) 8.45 ms, 8.2 ms, 6.88 ms, and 448 us and 6.5 ms with the MMAs of
+// a K step in one block (tc_mma3_if); TF32x3 at 31/5/467/1609
 // 2.41 ms to 1.83 ms by that last change. Without the epilogue the MMAs
 // took 297 us and 7.3 ms before it: what the epilogue adds is mostly the
 // tail rows' loads, which use the same shared-memory path.
@@ -209,29 +210,23 @@ __device__ __forceinline__ int slot_row(const ItemPlan& ip, int slot, int nVpad)
 // the accumulator small until the largest terms arrive, so few truncations act
 // on the full-size sum. hi*lo and hi*hi share their A operand, which the second
 // takes from the collector buffer. N is the item's tile width (nB).
-// shared-memory offsets of the A and B operand slots of both products.
+// Descriptor low words of the A and B operand slots of both products, in stage 0 (sb: the
+// stage's offset / 16).
 struct MmaSlots {
   uint32_t a1, b1, a2, b2;
 };
 template <bool BF16>
 __device__ __forceinline__ void ccvv_stage_mmas(uint32_t leader, uint32_t dx, uint32_t dy, uint32_t sb,
                                                 const MmaSlots& o, uint32_t idesc, bool two, int kb) {
+  constexpr uint32_t LO = SLOT_BYTES / 16;  // from the hi to the lo plane of a slot
+  const uint32_t a1 = o.a1 + sb, b1 = o.b1 + sb, a2 = o.a2 + sb, b2 = o.b2 + sb;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const uint32_t off = sb + (uint32_t)((1 - k) * 32);
-    const uint64_t a1h = desc_sw64(off + o.a1), a1l = desc_sw64(off + o.a1 + SLOT_BYTES);
-    const uint64_t b1h = desc_sw64(off + o.b1), b1l = desc_sw64(off + o.b1 + SLOT_BYTES);
+    const uint32_t off = (1 - k) * 32 / 16;
     const uint32_t acc0 = (kb > 0 || k > 0) ? 1u : 0u;
-    tc_mma_if<BF16>(leader, dx, a1l, b1h, idesc, acc0);
-    tc_mma_if<BF16, 1>(leader, dx, a1h, b1l, idesc, 1u);
-    tc_mma_if<BF16, 2>(leader, dx, a1h, b1h, idesc, 1u);
-    if (two) {
-      const uint64_t a2h = desc_sw64(off + o.a2), a2l = desc_sw64(off + o.a2 + SLOT_BYTES);
-      const uint64_t b2h = desc_sw64(off + o.b2), b2l = desc_sw64(off + o.b2 + SLOT_BYTES);
-      tc_mma_if<BF16>(leader, dy, a2l, b2h, idesc, acc0);
-      tc_mma_if<BF16, 1>(leader, dy, a2h, b2l, idesc, 1u);
-      tc_mma_if<BF16, 2>(leader, dy, a2h, b2h, idesc, 1u);
-    }
+    tc_mma3_if<BF16, false>(leader, dx, a1 + off + LO, a1 + off, b1 + off + LO, b1 + off, idesc, acc0);
+    if (two)
+      tc_mma3_if<BF16, false>(leader, dy, a2 + off + LO, a2 + off, b2 + off + LO, b2 + off, idesc, acc0);
   }
 }
 
@@ -579,10 +574,11 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
       const ItemPlan ip = plan_item<HALVES>(a, idx, &md);
       const int kblocks = (int)tc_uniform((uint32_t)md->kblocks);
       MmaSlots o;
-      o.a1 = tc_uniform((uint32_t)(ip.g1a * 2 * SLOT_BYTES));
-      o.b1 = tc_uniform((uint32_t)(ip.g1b * 2 * SLOT_BYTES + ip.boff));
-      o.a2 = tc_uniform((uint32_t)(ip.g2a * 2 * SLOT_BYTES));
-      o.b2 = tc_uniform((uint32_t)(ip.g2b * 2 * SLOT_BYTES + ip.boff));
+      const uint32_t t0 = su32(tiles);
+      o.a1 = tc_uniform(desc_sw64_lo(t0 + (uint32_t)(ip.g1a * 2 * SLOT_BYTES)));
+      o.b1 = tc_uniform(desc_sw64_lo(t0 + (uint32_t)(ip.g1b * 2 * SLOT_BYTES + ip.boff)));
+      o.a2 = tc_uniform(desc_sw64_lo(t0 + (uint32_t)(ip.g2a * 2 * SLOT_BYTES)));
+      o.b2 = tc_uniform(desc_sw64_lo(t0 + (uint32_t)(ip.g2b * 2 * SLOT_BYTES + ip.boff)));
       const uint32_t idesc = idesc_128xn<BF16>(tc_uniform((uint32_t)ip.nB));
       const bool two = __all_sync(0xffffffffu, ip.two);
       if (!TC_WARP_WAIT(&tempty[tbuf], tphase ^ 1u, abort_flag, a.status)) {
@@ -598,8 +594,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
           break;
         }
         tc_fence_after();
-        ccvv_stage_mmas<BF16>(leader, dx, dy, su32(tiles) + (uint32_t)(stage * STAGE_BYTES), o, idesc,
-                              two, kb);
+        ccvv_stage_mmas<BF16>(leader, dx, dy, (uint32_t)(stage * (STAGE_BYTES / 16)), o, idesc, two, kb);
         issued = true;
         tc_commit_if(leader, &empty[stage]);
         if (++stage == STAGES) {
