@@ -1333,7 +1333,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   }
   ActiveWs& w = p->act;
   const ActDims d = act_dims(z);
-  cudaStream_t st = p->stream;
+  cudaStream_t st = p->stream, sd = side_stream(p);
   if (!ints_ready) {
     const size_t n = 2 * (size_t)z.nH * z.nA * z.nA * z.nP + (size_t)z.nH * z.nA * z.nH * z.nA;
     small_ints_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(B, z, w.K1, w.K2, w.K3);
@@ -1379,6 +1379,11 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
       actvv_gen_kernel<NA_, true><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     } else {                                                                                 \
       raise_smem_limit((const void*)actvv_gen_kernel<NA_, false>, smg);                      \
+    // F6 and F7 read these tables only
+    if (p->forked) {
+      const cudaError_t e = plan_link(st, p->ev_tab, p->side);
+      if (e != cudaSuccess) return e;
+    }
       actvv_gen_kernel<NA_, false><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     }                                                                                        \
     break;
@@ -1437,9 +1442,9 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
 #define F67_LAUNCH(NA_)                                                                        \
   case NA_:                                                                                    \
     raise_smem_limit((const void*)term_f7_kernel<NA_>, smf7);                                  \
-    term_f7_kernel<NA_><<<term_blocks(z), TERM_NT, smf7, st>>>(z, ta, p->d_partials + sg.begin); \
+    term_f7_kernel<NA_><<<term_blocks(z), TERM_NT, smf7, sd>>>(z, ta, p->d_partials + sg.begin); \
     DSRG_LAUNCH_CHECK(p);                                                                      \
-    term_f6_kernel<NA_><<<term_blocks(z), TERM_NT, 0, st>>>(z, ta, p->d_partials + sg.begin);   \
+    term_f6_kernel<NA_><<<term_blocks(z), TERM_NT, 0, sd>>>(z, ta, p->d_partials + sg.begin);   \
     if (NA_ <= 6) {                                                                            \
       DSRG_LAUNCH_CHECK(p);                                                                    \
       raise_smem_limit((const void*)term_i_kernel<(NA_ <= 6 ? NA_ : 6)>, smti);                \

@@ -112,6 +112,10 @@ static std::vector<int> host_io_bounds(const Sizes& z) {
 }
 
 static void free_all(dsrg_plan* p) {
+  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_side})
+    if (*ev) cudaEventDestroy(*ev);
+  if (p->side) cudaStreamDestroy(p->side);
+  p->side = nullptr;
   for (cudaEvent_t ev : p->st_ev) cudaEventDestroy(ev);
   p->st_ev.clear();
   if (p->st_copy) cudaStreamDestroy(p->st_copy);
@@ -238,6 +242,7 @@ dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precis
   if (ok && prec == DSRG_PREC_FP64) ok = fp64_tc_alloc(p);
   if (ok && p->rest_tc) ok = rest_alloc(p, share ? share->y : nullptr);
   if (ok && (flags & DSRG_PLAN_GRAD)) ok = grad_alloc(p);
+  if (ok && !share) ok = plan_fork_alloc(p);
   if (ok && (flags & DSRG_PLAN_HOST_IO)) {
     const size_t nb = (size_t)z.Q * z.nH * z.nP;
     const size_t ne = (size_t)z.n, ng = (size_t)z.nA * z.nA, nl = ng * ng;
@@ -330,6 +335,25 @@ static dsrg_status_t check_common(dsrg_plan* p, const double* B, const double* e
 }  // extern "C"
 
 namespace dsrg {
+// The blocks of an energy call that do not wait for one another (CCVV, F2, F3, F6 and F7
+// against the active block's chain) run beside each other when the CCVV items are fewer
+// than the SMs: those kernels then leave SMs free, and one after another their latencies
+// add up (247 us at 10/4/60/200, 166 us beside each other). With more items CCVV holds every SM.
+bool plan_fork_alloc(dsrg_plan* p) {
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
+  if (!p->split || !p->rest_tc || p->z.nA == 0 || split_ccvv_grid(p) >= nsm) return true;
+  if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess) return false;
+  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_side})
+    if (cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess) return false;
+  return true;
+}
+
+cudaError_t plan_link(cudaStream_t from, cudaEvent_t ev, cudaStream_t to) {
+  const cudaError_t e = cudaEventRecord(ev, from);
+  return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ev, 0);
+}
+
 // The blocks besides CCVV: CAVV, CCAV and the active block (they do not read
 // the CCVV partials, so they may run beside the CCVV launch).
 dsrg_status_t run_blocks(dsrg_plan* p, const double* B, const double* eps, const double* G,
@@ -370,12 +394,22 @@ static dsrg_status_t run_energy(dsrg_plan* p, const double* B, const double* eps
                                 const double* L, const double* L3, const double* F1, double s,
                                 double* out) {
   cudaError_t e;
+  p->forked = p->side != nullptr && p->shard_rank == 0;
   if (p->prec == DSRG_PREC_FP64)
     e = launch_ccvv_fp64_tc(p, B, eps, s);
   else
     e = launch_split_ccvv(p, B, eps, s);
-  if (e != cudaSuccess) return cuda_fail(p, e, "ccvv");
-  return run_rest(p, B, eps, G, L, L3, F1, s, out);
+  dsrg_status_t st = DSRG_OK;
+  if (e != cudaSuccess)
+    st = cuda_fail(p, e, "ccvv");
+  else
+    st = run_blocks(p, B, eps, G, L, L3, F1, s);
+  if (p->forked) {  // also after a failure, so that a capture of the caller's ends
+    p->forked = false;
+    e = plan_link(p->side, p->ev_side, p->stream);
+    if (e != cudaSuccess && st == DSRG_OK) st = cuda_fail(p, e, "join");
+  }
+  return st != DSRG_OK ? st : run_reduce(p, out);
 }
 
 extern "C" {

@@ -990,7 +990,7 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
   RestState* st = p->rest;
   const Sizes& z = p->z;
   const bool bf16 = p->prec == DSRG_PREC_BF16X3;
-  cudaStream_t stream = p->stream;
+  cudaStream_t stream = p->stream, side = side_stream(p);
   const int T = z.nH * z.nA;
   const long long xrow0 = (long long)z.nH * st->nVpad;
   {
@@ -1032,7 +1032,12 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
     DSRG_LAUNCH_CHECK(p);
   }
   {
-    pair_info_kernel<<<1, 1024, 0, stream>>>(eps, s, z, nullptr, z.nC * z.nA, st->pinfo);
+    // F2 and F3 read Y only: beside the active block where the call has forked
+    if (p->forked) {
+      const cudaError_t e = plan_link(stream, p->ev_gemm, p->side);
+      if (e != cudaSuccess) return e;
+    }
+    pair_info_kernel<<<1, 1024, 0, side>>>(eps, s, z, nullptr, z.nC * z.nA, st->pinfo);
     DSRG_LAUNCH_CHECK(p);
   }
   {
@@ -1041,7 +1046,7 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
 #define F2_LAUNCH(NA_)                                                                             \
   case NA_:                                                                                        \
     raise_smem_limit((const void*)cavv_f2_kernel<NA_>, sm); \
-    cavv_f2_kernel<NA_><<<sg.count, 256, sm, stream>>>(st->Y, st->ldy, st->nVpad, eps, G, s, z,       \
+    cavv_f2_kernel<NA_><<<sg.count, 256, sm, side>>>(st->Y, st->ldy, st->nVpad, eps, G, s, z,       \
                                                       st->d_tp, st->n_tp, st->pinfo,              \
                                                       p->d_partials + sg.begin, p->d_counts);     \
     break;
@@ -1059,7 +1064,7 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
 #define F3_LAUNCH(NA_)                                                                             \
   case NA_:                                                                                        \
     raise_smem_limit((const void*)ccav_f3_kernel<NA_>, sm); \
-    ccav_f3_kernel<NA_><<<sg.count, 256, sm, stream>>>(st->Y, st->ldy, st->nVpad, st->xc, eps, G, s, \
+    ccav_f3_kernel<NA_><<<sg.count, 256, sm, side>>>(st->Y, st->ldy, st->nVpad, st->xc, eps, G, s, \
                                                       z, p->d_partials + sg.begin);              \
     break;
     switch (z.nA) {
