@@ -116,42 +116,79 @@ __global__ void __launch_bounds__(256) chol_update_kernel(double* __restrict__ A
   }
 }
 
-// L^{-1} (lower triangular) by forward substitution, a few columns per CTA in shared
-// memory and one warp per column: Li[i][c] = (delta_ic - sum_{c <= k < i} L[i][k]
-// Li[k][c]) / L[i][i]. The columns are independent, so this is one launch; a CTA takes
-// columns from both ends (gridDim.x apart), which evens out their lengths.
-constexpr int TI_WARPS = 8;
-__global__ void __launch_bounds__(32 * TI_WARPS) tri_inverse_kernel(const double* __restrict__ L,
-                                                                    int n, double* __restrict__ Li,
-                                                                    int staged) {
-  extern __shared__ double cols[];  // [warps][n], unless a column does not fit
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int w = warp * gridDim.x + blockIdx.x;
-  // columns 0, n-1, 1, n-2, ... in the order of w / 2
-  const int c = (w & 1) ? n - 1 - w / 2 : w / 2;
-  if (w >= n) return;
-  double* x = staged ? cols + (size_t)warp * n : Li + c;
-  const size_t xs = staged ? 1 : (size_t)n;
-  for (int i = lane; i < c; i += 32) Li[(size_t)i * n + c] = 0.0;
-  for (int i = c; i < n; ++i) {
-    double v = 0.0, v2 = 0.0;
-    const double* Lr = L + (size_t)i * n;
-    int k = c + lane;
-    for (; k + 32 < i; k += 64) {
-      v = fma(Lr[k], x[k * xs], v);
-      v2 = fma(Lr[k + 32], x[(k + 32) * xs], v2);
-    }
-    if (k < i) v = fma(Lr[k], x[k * xs], v);
-    v += v2;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const double r = ((i == c ? 1.0 : 0.0) - v) / Lr[i];
-    if (lane == 0) {
-      x[i * xs] = r;
-      Li[(size_t)i * n + c] = r;
-    }
-    __syncwarp();
+// L^{-1} (lower triangular, Li zeroed before), the diagonal blocks of CB columns: one warp
+// per block, lane c its column c, Li[i][c] = (delta_ic - sum_{k<i} L[i][k] Li[k][c]) / L[i][i].
+__global__ void __launch_bounds__(32) tri_diag_kernel(const double* __restrict__ L, int n,
+                                                      double* __restrict__ Li) {
+  __shared__ double t[CB][CB + 1], rd[CB];
+  const int lane = threadIdx.x, k0 = blockIdx.x * CB, nb = min(CB, n - k0);
+  for (int i = 0; i < CB; ++i)
+    t[i][lane] = (i < nb && lane <= i) ? L[(size_t)(k0 + i) * n + k0 + lane] : (i == lane ? 1.0 : 0.0);
+  __syncwarp();
+  rd[lane] = 1.0 / t[lane][lane];
+  __syncwarp();
+  double x[CB];
+#pragma unroll
+  for (int i = 0; i < CB; ++i) {
+    double v = i == lane ? 1.0 : 0.0;
+#pragma unroll
+    for (int k = 0; k < i; ++k) v = fma(-t[i][k], x[k], v);
+    x[i] = v * rd[i];
+    if (i < nb && lane <= i) Li[(size_t)(k0 + i) * n + k0 + lane] = x[i];
   }
 }
+
+// ... and the rest by doubling: with the inverses of two neighbouring diagonal blocks of
+// sizes w and w2 <= w, the block below the first is -Li_22 (L_21 Li_11), all pairs of a
+// size at once. L_21 Li_11 waits, transposed, in the upper triangle of L, which nothing
+// reads. (By forward substitution, a warp per column: 3.9 ms at naux = 1200, 0.9 ms now.)
+cudaError_t tri_inverse(cudaStream_t st, double* L, int n, double* Li, const OzWork& ow) {
+  cudaError_t e = cudaMemsetAsync(Li, 0, (size_t)n * n * 8, st);
+  if (e != cudaSuccess) return e;
+  tri_diag_kernel<<<(n + CB - 1) / CB, 32, 0, st>>>(L, n, Li);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  for (long long w = CB; w < n; w *= 2) {
+    const int full = (int)(n / (2 * w));                 // pairs of two whole blocks
+    const long long at = 2 * w * full, last = n - at - w;  // and one with a shorter second
+    for (int ragged = 0; ragged < 2; ++ragged) {
+      const int nb = ragged ? (last > 0 ? 1 : 0) : full;
+      if (nb == 0) continue;
+      const long long o = ragged ? at : 0, step = 2 * w * (n + 1);
+      const int w1 = (int)w, w2 = (int)(ragged ? last : w);
+      const double* L21 = L + (o + w) * n + o;
+      double* T = L + o * n + o + w;  // T[i][j] at [j][i]
+      double *L11 = Li + o * (n + 1), *L22 = Li + (o + w) * (n + 1), *X = Li + (o + w) * n + o;
+      GemmArgs g = batched(mk(w2, w1, w1, 1, L21, n, 1, 0, L11, n, 0, 1, T, 1, n, 1.0), nb, step, step, step);
+      g.accumulate = 0;
+      if ((e = launch_gemm(st, g, ow)) != cudaSuccess) return e;
+      g = batched(mk(w2, w1, w2, 1, L22, n, 1, 0, T, 1, 0, n, X, n, 1, -1.0), nb, step, step, step);
+      g.accumulate = 0;
+      if ((e = launch_gemm(st, g, ow)) != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
+// A second stream beside st for the scope: work queued on it starts after st's so far.
+struct SideStream {
+  cudaStream_t s = nullptr;
+  cudaEvent_t ev = nullptr;
+  bool open(cudaStream_t st) {
+    int lo = 0, hi = 0;
+    return cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+           cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, hi) == cudaSuccess &&
+           cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventRecord(ev, st) == cudaSuccess && cudaStreamWaitEvent(s, ev, 0) == cudaSuccess;
+  }
+  bool join(cudaStream_t st) {
+    return cudaEventRecord(ev, s) == cudaSuccess && cudaStreamWaitEvent(st, ev, 0) == cudaSuccess;
+  }
+  ~SideStream() {
+    if (s) cudaStreamSynchronize(s);  // (an error left it unjoined)
+    if (ev) cudaEventDestroy(ev);
+    if (s) cudaStreamDestroy(s);
+  }
+};
 
 // ------------------------------ pivoted Cholesky ------------------------------
 struct CdState {
@@ -276,14 +313,20 @@ __global__ void __launch_bounds__(CD_T * CD_W) cd_run_kernel(const double* __res
   if (blockIdx.x == 0 && tid == 0) st->rank = rank;
 }
 
-// Workspace of the three products on the tensor cores (the largest of them; 0 where they
+// Workspace of the products on the tensor cores (the largest of them; 0 where they
 // are too small for it).
 size_t df_gemm_bytes(int nbf, int naux, int np, int nq) {
   size_t a = oz_work_bytes(np, nbf, nbf, naux, true, false);
   const size_t b = oz_work_bytes((long long)np * naux, nq, nbf, 1, false, false);
   const size_t c = oz_work_bytes(naux, (long long)np * nq, naux, 1, false, false);
   a = a > b ? a : b;
-  return a > c ? a : c;
+  a = a > c ? a : c;
+  for (long long w = CB; w < naux; w *= 2) {  // tri_inverse
+    const long long nb = naux / (2 * w) > 0 ? naux / (2 * w) : 1;
+    const size_t t = oz_work_bytes(w, w, w, nb, false, false);
+    a = a > t ? a : t;
+  }
+  return a;
 }
 
 }  // namespace
@@ -317,6 +360,21 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   ow.status = bad + 1;
   if (cudaMemsetAsync(bad, 0, 2 * sizeof(int), st) != cudaSuccess) return DSRG_ERR_CUDA;
   cudaError_t e;
+  // J = L L^T: a chain of short launches, beside the two products that do not need it
+  SideStream side;
+  if (!side.open(st)) return DSRG_ERR_CUDA;
+  if (cudaMemcpyAsync(Lm, metric, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice, side.s) != cudaSuccess)
+    return DSRG_ERR_CUDA;
+  for (int k = 0; k < naux; k += CB) {
+    chol_diag_kernel<<<1, 256, 0, side.s>>>(Lm, naux, k, bad);
+    const int left = naux - k - CB;
+    if (left > 0) {
+      chol_panel_kernel<<<(left + 3) / 4, 128, 0, side.s>>>(Lm, naux, k);
+      const unsigned nt = (unsigned)((left + CB - 1) / CB);
+      chol_update_kernel<<<dim3(nt, nt), 256, 0, side.s>>>(Lm, naux, k);
+    }
+  }
+  if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
   // Y[P][p][nu] = sum_mu C[mu][p0 + p] ao3[P][mu][nu]
   GemmArgs g1 = batched(mk(np, nbf, nbf, 1, C + p0, 1, nmo, 0, ao3, nbf, 0, 1, Y, nbf, 1, 1.0), naux,
                         0, (long long)nbf * nbf, (long long)np * nbf);
@@ -327,27 +385,7 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   g2.accumulate = 0;
   if ((e = launch_gemm(st, g1, ow)) != cudaSuccess || (e = launch_gemm(st, g2, ow)) != cudaSuccess)
     return DSRG_ERR_CUDA;
-  // J = L L^T, then L^{-1}
-  if (cudaMemcpyAsync(Lm, metric, (size_t)naux * naux * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return DSRG_ERR_CUDA;
-  for (int k = 0; k < naux; k += CB) {
-    chol_diag_kernel<<<1, 256, 0, st>>>(Lm, naux, k, bad);
-    const int left = naux - k - CB;
-    if (left > 0) {
-      chol_panel_kernel<<<(left + 3) / 4, 128, 0, st>>>(Lm, naux, k);
-      const unsigned nt = (unsigned)((left + CB - 1) / CB);
-      chol_update_kernel<<<dim3(nt, nt), 256, 0, st>>>(Lm, naux, k);
-    }
-  }
-  if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
-  // columns of L^{-1} per CTA: what the shared memory holds, at most one per warp
-  int tw = (int)((size_t)200 * 1024 / ((size_t)naux * 8));
-  const int staged = tw >= 1;
-  tw = tw > TI_WARPS || !staged ? TI_WARPS : tw;
-  const size_t smi = staged ? (size_t)tw * naux * 8 : 0;
-  raise_smem_limit((const void*)tri_inverse_kernel, smi);
-  tri_inverse_kernel<<<(naux + tw - 1) / tw, 32 * tw, smi, st>>>(Lm, naux, Li, staged);
-  if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;
+  if (!side.join(st) || tri_inverse(st, Lm, naux, Li, ow) != cudaSuccess) return DSRG_ERR_CUDA;
   // B[Q][pq] = sum_P Li[Q][P] Z[P][pq]  (Li lower triangular; the GEMM reads it whole)
   const long long npq = (long long)np * nq;
   GemmArgs g3 = mk(naux, (int)npq, naux, 1, Li, naux, 1, 0, Z, npq, 0, 1, B_out, npq, 1, 1.0);
