@@ -172,8 +172,7 @@ __global__ void jac_copy_kernel(const double* __restrict__ f, int n, int lo, int
 // thread turns one 2 x 2 block A[P][R] -> J_P^T A[P][R] J_R from one copy of A into the
 // other, so no CTA waits for another within a step; the same CTA turns 32 rows of V by
 // its 16 column pairs in place.
-// The angle comes from FP32 and one Newton-Raphson step (46 bits: what it leaves of
-// A[p][q] is below the stopping threshold); c^2 + s^2 = 1 holds to FP64.
+// The angle comes from FP32 and two Newton-Raphson steps; c^2 + s^2 = 1 holds to FP64.
 constexpr int JT = 16;
 constexpr int JAC_SLOTS = 2048;  // CTAs, at most
 
@@ -188,15 +187,22 @@ __device__ __forceinline__ double2 jac_rotation(double app, double aqq, double a
   const float tau = (float)nf / (float)df;
   float tf = 1.0f / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
   if (tau < 0.0f) tf = -tf;
-  // one Newton-Raphson step on h t^2 + nf t - h = 0 (slope |nf + df t| >= 1)
+  // two Newton-Raphson steps on h t^2 + nf t - h = 0 (slope |nf + df t| >= 1)
   double t = (double)tf;
   const float slope = (float)fma(df, t, nf);
-  t = fma(-fma(fma(h, t, nf), t, -h), (double)(1.0f / slope), t);
+  const double is = (double)(1.0f / slope);
+  t = fma(-fma(fma(h, t, nf), t, -h), is, t);
+  t = fma(-fma(fma(h, t, nf), t, -h), is, t);
   const double w = fma(t, t, 1.0);
   double c = (double)rsqrtf((float)w);
   c = c * fma(-0.5 * w * c, c, 1.5);
-  c = c * fma(-0.5 * w * c, c, 1.5);
-  return make_double2(c, t * c);
+  // both by what is left of c^2 + s^2 = 1: one rounding each, so that thousands of
+  // rotations do not shrink or stretch a vector
+  double s = t * c;
+  const double u = 0.5 * fma(-s, s, fma(-c, c, 1.0));
+  c = fma(u, c, c);
+  s = fma(u, s, s);
+  return make_double2(c, s);
 }
 
 __global__ void __launch_bounds__(JT * JT) jac_run_kernel(double* __restrict__ A0,
