@@ -192,10 +192,12 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
   const size_t ng = (size_t)d.nA2 * d.nA2;
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n1) {
-    const int x = (int)(k % z.nA);
-    const int a = (int)((k / z.nA) % z.nP);
-    const int u = (int)((k / ((size_t)z.nA * z.nP)) % z.nA);
-    const int i = (int)(k / ((size_t)z.nA * z.nP * z.nA));
+    // (nH nA^2 nP and nH^2 nA^2 are below 2^31: 16 times fewer than the spin tables' elements)
+    const unsigned k32 = (unsigned)k;
+    const int x = (int)(k32 % z.nA);
+    const int a = (int)((k32 / z.nA) % z.nP);
+    const int u = (int)((k32 / (unsigned)(z.nA * z.nP)) % z.nA);
+    const int i = (int)(k32 / (unsigned)(z.nA * z.nP * z.nA));
     const size_t kk = (((size_t)i * z.nA + u) * z.nA + x) * z.nP + a;
     const double k1 = K1[kk], k2 = K2[kk];
     const double D = eps[i] + eps[z.nC + u] - eps[z.nC + a] - eps[z.nC + x];
@@ -212,11 +214,11 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
       W1[2 * w1n + o] = V * rv;
     }
   } else if (k < n1 + n2) {
-    const size_t r = k - n1;
+    const unsigned r = (unsigned)(k - n1);
     const int y = (int)(r % z.nA);
     const int x = (int)((r / z.nA) % z.nA);
-    const int j = (int)((r / ((size_t)z.nA * z.nA)) % z.nH);
-    const int i = (int)(r / ((size_t)z.nA * z.nA * z.nH));
+    const int j = (int)((r / (unsigned)(z.nA * z.nA)) % z.nH);
+    const int i = (int)(r / (unsigned)(z.nA * z.nA * z.nH));
     const double kxy = K3[(((size_t)i * z.nA + x) * z.nH + j) * z.nA + y];
     const double kyx = K3[(((size_t)i * z.nA + y) * z.nH + j) * z.nA + x];
     const double D = eps[i] + eps[j] - eps[z.nC + x] - eps[z.nC + y];
@@ -327,15 +329,15 @@ __device__ __forceinline__ double eta_p(const ActDims& d, const double* gA, int 
 }
 
 // Ti[J][V][B][Y] = sum_{I,A} gamma_I^J eta_B^A t_{AY}^{IV}  (the dressed T of term I).
+// blockIdx.y is (J, V), so that the index arithmetic is 32-bit (with 64-bit divisions per
+// element, for 16 bytes of traffic, 97 us at 31/5/467/1609, 91 us now).
 __global__ void ti_kernel(Sizes z, const double* __restrict__ W1T, const double* __restrict__ gA,
-                          double* __restrict__ Ti, size_t w1n) {
+                          double* __restrict__ Ti) {
   const ActDims d = act_dims(z);
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= w1n) return;
-  const int Y = (int)(k % d.nA2);
-  const int Bp = (int)((k / d.nA2) % d.nP2);
-  const int V = (int)((k / ((size_t)d.nA2 * d.nP2)) % d.nA2);
-  const int J = (int)(k / ((size_t)d.nA2 * d.nP2 * d.nA2));
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= d.nP2 * d.nA2) return;
+  const int Y = r % d.nA2, Bp = r / d.nA2, V = blockIdx.y % d.nA2, J = blockIdx.y / d.nA2;
+  const size_t k = (size_t)blockIdx.y * d.nP2 * d.nA2 + r;
   if ((J & 1) + (V & 1) != (Bp & 1) + (Y & 1)) {  // gamma, eta and t conserve spin
     Ti[k] = 0.0;
     return;
@@ -551,13 +553,44 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
       acc2[o] += (double)f2[o];
     }
   }
+  if constexpr (NA == 2) {
+    // 32 sums: a transposing butterfly halves a lane's values at each step, lane l ends
+    // with the warp's sum l (31 FP64 additions a lane; a block sum each took 20 us)
+    static_assert(2 * NA4 == 32, "one sum per lane");
+    __shared__ double sw[8][32];
+    const int lane = threadIdx.x & 31;
+    double v[32];
 #pragma unroll
-  for (int c = 0; c < NA4; ++c) {
-    const double t1 = block_sum<256>(acc1[c], red);
-    const double t2 = block_sum<256>(acc2[c], red);
-    if (threadIdx.x == 0) {
-      part[((size_t)blockIdx.x * 2 + 0) * NA4 + c] = t1;
-      part[((size_t)blockIdx.x * 2 + 1) * NA4 + c] = t2;
+    for (int c = 0; c < NA4; ++c) {
+      v[c] = acc1[c];
+      v[NA4 + c] = acc2[c];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const double snd = up ? v[k] : v[k + o];
+        v[k] = (up ? v[k + o] : v[k]) + __shfl_xor_sync(0xffffffffu, snd, o);
+      }
+    }
+    sw[threadIdx.x >> 5][lane] = v[0];
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t += sw[w][lane];
+      part[(size_t)blockIdx.x * 32 + lane] = t;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < NA4; ++c) {
+      const double t1 = block_sum<256>(acc1[c], red);
+      const double t2 = block_sum<256>(acc2[c], red);
+      if (threadIdx.x == 0) {
+        part[((size_t)blockIdx.x * 2 + 0) * NA4 + c] = t1;
+        part[((size_t)blockIdx.x * 2 + 1) * NA4 + c] = t2;
+      }
     }
   }
 }
@@ -1346,6 +1379,11 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
         eps, G, L, s, z, w.K1, w.K2, w.K3, w.W1, w.W2, w.lam, w.gA, w.w1n, w.w2n,
         p->grad != nullptr);
     DSRG_LAUNCH_CHECK(p);
+    // F6 and F7 read these tables only
+    if (p->forked) {
+      const cudaError_t e = plan_link(st, p->ev_tab, p->side);
+      if (e != cudaSuccess) return e;
+    }
   }
   {
     const int n = d.nH2 * z.nP;
@@ -1361,7 +1399,8 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     DSRG_LAUNCH_CHECK(p);
   }
   {
-    ti_kernel<<<(unsigned)((w.w1n + 255) / 256), 256, 0, st>>>(z, w.W1 + w.w1n, w.gA, w.Ti, w.w1n);
+    const dim3 grid((unsigned)((d.nP2 * d.nA2 + 255) / 256), (unsigned)(d.nH2 * d.nA2));
+    ti_kernel<<<grid, 256, 0, st>>>(z, w.W1 + w.w1n, w.gA, w.Ti);
     DSRG_LAUNCH_CHECK(p);
   }
   if (!ints_ready) {
@@ -1379,11 +1418,6 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
       actvv_gen_kernel<NA_, true><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     } else {                                                                                 \
       raise_smem_limit((const void*)actvv_gen_kernel<NA_, false>, smg);                      \
-    // F6 and F7 read these tables only
-    if (p->forked) {
-      const cudaError_t e = plan_link(st, p->ev_tab, p->side);
-      if (e != cudaSuccess) return e;
-    }
       actvv_gen_kernel<NA_, false><<<ACTVV_BLOCKS, 256, smg, st>>>(eps, s, z, w.M, w.P12part); \
     }                                                                                        \
     break;

@@ -104,7 +104,7 @@ struct GradWs {
   double* dZ = nullptr;   // [nA][nC][nC][nV]
   float* Z32 = nullptr;   // split plans: [nC nV][nC nA], (me|nu)
   double *dW1Vt = nullptr, *dW1T = nullptr, *dTi = nullptr, *dV1 = nullptr;
-  double *dW2Vt = nullptr, *dW2T = nullptr, *dV2 = nullptr;
+  double *dW2Vt = nullptr, *dW2T = nullptr, *dV2 = nullptr, *dw2 = nullptr;
   double *dt1 = nullptr, *dft = nullptr, *dS = nullptr, *dP12 = nullptr;
   double *dK1 = nullptr, *dK2 = nullptr, *dK3 = nullptr, *dM = nullptr;
 };
@@ -593,6 +593,7 @@ struct ActAdjArgs {
   double s;
   const double* eps;
   const double *K1, *K2, *K3, *W1V, *W1T, *W1Vt, *W2V, *W2T, *W2Vt, *Ti, *lam, *gA, *t1, *ft, *M;
+  double *thw2, *dw2;  // Th and D of term H (adj_w2_mid_kernel)
   double *dW1Vt, *dW1T, *dTi, *dW2Vt, *dW2T, *dt1, *dft, *dP12, *dS, *dV1, *dV2, *dK1, *dK2, *dK3,
       *dM;
   double *deps, *ds;
@@ -613,14 +614,13 @@ __device__ __forceinline__ size_t L3I(int n2, int U, int V, int W, int X, int Y,
 // (All elements and terms: 656 us at 10/4/60/200, 108 us now.)
 __global__ void adj_w1_terms_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
-  const size_t k0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (2 * k0 >= a.w1n) return;
-  const int nA = d.nA2 / 2, nP = d.nP2 / 2, sA = (int)((k0 / ((size_t)nA * nP)) & 1);
-  const int A = 2 * (int)((k0 / nA) % nP) + sA;
-  const int U = (int)((k0 / ((size_t)nA * d.nP2)) % d.nA2);
-  const int I = (int)(k0 / ((size_t)nA * d.nP2 * d.nA2));
+  const int nA = d.nA2 / 2, nP = d.nP2 / 2;
+  const int k0 = blockIdx.x * blockDim.x + threadIdx.x;  // (spin of A, a, x); blockIdx.y: (I, U)
+  if (k0 >= nA * d.nP2) return;
+  const int sA = k0 / (nA * nP), A = 2 * ((k0 / nA) % nP) + sA;
+  const int U = blockIdx.y % d.nA2, I = blockIdx.y / d.nA2;
   const int sI = I & 1, sU = U & 1, sX = sI + sU - sA;
-  const int X = 2 * (int)(k0 % nA) + (sX == 1);
+  const int X = 2 * (k0 % nA) + (sX == 1);
   const size_t k = W1(d, I, U, A, X);
   a.dW1Vt[k ^ 1] = 0.0;  // X of the other spin
   a.dW1T[k ^ 1] = 0.0;
@@ -791,6 +791,44 @@ __global__ void adj_w1_terms_kernel(ActAdjArgs a) {
   a.dTi[k] = dti;
 }
 
+// Sum over the orbitals K, L that gamma couples to I, J (core: themselves; active: the
+// same spin) of gamma[K,I] gamma[L,J] S[K,L,X,Y].
+__device__ __forceinline__ double gg_w2(const AD& d, const double* gA, const double* S, int I, int J,
+                                        int X, int Y) {
+  const int i0 = (I < d.nC2) ? I : d.nC2 + (I & 1), i1 = (I < d.nC2) ? I + 1 : d.nH2;
+  const int j0 = (J < d.nC2) ? J : d.nC2 + (J & 1), j1 = (J < d.nC2) ? J + 1 : d.nH2;
+  double v = 0.0;
+  for (int K = i0; K < i1; K += 2)
+    for (int L = j0; L < j1; L += 2) v = fma(gH(d, gA, K, I) * gH(d, gA, L, J), S[W2(d, K, L, X, Y)], v);
+  return v;
+}
+
+// The inner sums of term H once per element, Th = gamma gamma T and D = Vt lam (spin-allowed
+// elements): the outer sums of adj_w2_terms_kernel then have nA^2 products each where
+// the nested ones had nA^4, all in the few active-active elements (184 us at 10/4/60/200,
+// 50 us now).
+__global__ void adj_w2_mid_kernel(ActAdjArgs a) {
+  const AD d = adims(a.z);
+  const size_t k0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (2 * k0 >= a.w2n) return;
+  const int nA = d.nA2 / 2, sX = (int)((k0 / (nA * nA)) & 1);
+  const int X = 2 * (int)((k0 / nA) % nA) + sX;
+  const int J = (int)((k0 / ((size_t)nA * d.nA2)) % d.nH2);
+  const int I = (int)(k0 / ((size_t)nA * d.nA2 * d.nH2));
+  const int sY = (I & 1) + (J & 1) - sX;
+  if (sY < 0 || sY > 1) return;
+  const int Y = 2 * (int)(k0 % nA) + sY;
+  const size_t k = W2(d, I, J, X, Y);
+  double v = 0.0;
+  for (int U = 0; U < d.nA2; ++U) {
+    const int sv = sX + sY - (U & 1);
+    if (sv < 0 || sv > 1) continue;
+    for (int V = sv; V < d.nA2; V += 2) v = fma(a.W2Vt[W2(d, I, J, U, V)], a.lam[LM(d, U, V, X, Y)], v);
+  }
+  a.dw2[k] = v;
+  a.thw2[k] = gg_w2(d, a.gA, a.W2T, I, J, X, Y);
+}
+
 // (A2) term adjoints on W2-shaped tables (E, H, F5).
 __global__ void adj_w2_terms_kernel(ActAdjArgs a) {
   const AD d = adims(a.z);
@@ -813,35 +851,15 @@ __global__ void adj_w2_terms_kernel(ActAdjArgs a) {
   const double* lam = a.lam;
   const double* gA = a.gA;
   double dvt = 0.0, dt = 0.0;
-  // H: vt[K=I, L=J, U=X, V=Y] * Th[K,L,X',Y'] lam[U,V,X',Y'] / 8
+  // H: vt[I,J,X,Y] * Th[I,J,X',Y'] lam[X,Y,X',Y'] / 8, and d(t) = gamma gamma D / 8
   {
-    // gamma couples core orbitals to themselves, active ones to the same spin
-    const int i0 = (I < d.nC2) ? I : d.nC2 + sI, i1 = (I < d.nC2) ? I + 1 : d.nH2;
-    const int j0 = (J < d.nC2) ? J : d.nC2 + sJ, j1 = (J < d.nC2) ? J + 1 : d.nH2;
     for (int Xx = 0; Xx < d.nA2; ++Xx) {
       const int sy = sI + sJ - (Xx & 1);
       if (sy < 0 || sy > 1) continue;
-      for (int Yy = sy; Yy < d.nA2; Yy += 2) {
-        double th = 0.0;
-        for (int I2 = i0; I2 < i1; I2 += 2)
-          for (int J2 = j0; J2 < j1; J2 += 2)
-            th = fma(gH(d, gA, I, I2) * gH(d, gA, J, J2), a.W2T[W2(d, I2, J2, Xx, Yy)], th);
-        dvt = fma(0.125 * th, lam[LM(d, X, Y, Xx, Yy)], dvt);
-      }
+      for (int Yy = sy; Yy < d.nA2; Yy += 2)
+        dvt = fma(0.125 * a.thw2[W2(d, I, J, Xx, Yy)], lam[LM(d, X, Y, Xx, Yy)], dvt);
     }
-    // H -> d(t) at (I'=I, J'=J, X'=X, Y'=Y): sum_{K,L} gamma[K,I] gamma[L,J] dTh[K,L,X,Y]
-    for (int K = i0; K < i1; K += 2)
-      for (int L = j0; L < j1; L += 2) {
-        const double gg = gH(d, gA, K, I) * gH(d, gA, L, J);
-        if (gg == 0.0) continue;
-        double dth = 0.0;
-        for (int U = 0; U < d.nA2; ++U) {
-          const int sv = sX + sY - (U & 1);
-          if (sv < 0 || sv > 1) continue;
-          for (int V = sv; V < d.nA2; V += 2) dth = fma(a.W2Vt[W2(d, K, L, U, V)], lam[LM(d, U, V, X, Y)], dth);
-        }
-        dt = fma(0.125 * gg, dth, dt);
-      }
+    dt = 0.125 * gg_w2(d, gA, a.dw2, I, J, X, Y);
   }
   // E: -1/2 ft[M, V] t[U, M, X, Y] lam[U,V,X,Y]  (I active hole U, J core M)
   if (I >= d.nC2 && J < d.nC2) {
@@ -1041,13 +1059,11 @@ __global__ void __launch_bounds__(128) adj_w1_chain_kernel(ActAdjArgs a) {
   dacc_init(sacc_, a.z.n);
   const AD d = adims(a.z);
   const Sizes& z = a.z;
-  const size_t n = a.w1n / d.nA2;
-  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool on = t0 < n;
-  const size_t t = on ? t0 : n - 1;  // lanes past the end help in the warp sums
-  const int A = (int)(t % d.nP2);
-  const int U = (int)((t / d.nP2) % d.nA2);
-  const int I = (int)(t / ((size_t)d.nP2 * d.nA2));
+  const int a0 = blockIdx.x * blockDim.x + threadIdx.x;  // blockIdx.y: (I, U)
+  const bool on = a0 < d.nP2;
+  const int A = on ? a0 : d.nP2 - 1;  // lanes past the end help in the warp sums
+  const int U = blockIdx.y % d.nA2, I = blockIdx.y / d.nA2;
+  const size_t t = (size_t)blockIdx.y * d.nP2 + A;
   const int sx = (I & 1) + (U & 1) - (A & 1);  // spin of X
   const bool some = on && (sx == 0 || sx == 1);
   const int j0 = (I < d.nC2) ? I : d.nC2 + (I & 1), j1 = (I < d.nC2) ? I + 1 : d.nH2;
@@ -1328,7 +1344,7 @@ bool grad_alloc(dsrg_plan* p) {
          plan_alloc(p, (void**)&g->dW1Vt, w1n * 8) && plan_alloc(p, (void**)&g->dW1T, w1n * 8) &&
          plan_alloc(p, (void**)&g->dTi, w1n * 8) && plan_alloc(p, (void**)&g->dV1, w1n * 8) &&
          plan_alloc(p, (void**)&g->dW2Vt, w2n * 8) && plan_alloc(p, (void**)&g->dW2T, w2n * 8) &&
-         plan_alloc(p, (void**)&g->dV2, w2n * 8) && plan_alloc(p, (void**)&g->dt1, nHP2 * 8) &&
+         plan_alloc(p, (void**)&g->dV2, w2n * 8) && plan_alloc(p, (void**)&g->dw2, w2n * 8) && plan_alloc(p, (void**)&g->dt1, nHP2 * 8) &&
          plan_alloc(p, (void**)&g->dft, nHP2 * 8) && plan_alloc(p, (void**)&g->dS, nHP2 * 8) &&
          plan_alloc(p, (void**)&g->dP12, nA4 * 8) && plan_alloc(p, (void**)&g->dK1, n12 * 8) &&
          plan_alloc(p, (void**)&g->dK2, n12 * 8) && plan_alloc(p, (void**)&g->dK3, n3 * 8) &&
@@ -1559,7 +1575,14 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     const int nA4 = z.nA * z.nA * z.nA * z.nA;
     auto blocks = [](size_t n) { return (unsigned)((n + 255) / 256); };
     const size_t dsm = ((size_t)z.n + 1) * 8;  // block sums of deps and ds
-    adj_w1_terms_kernel<<<blocks(A.w1n / 2), 256, 0, st>>>(a);
+    {
+      const dim3 grid((unsigned)((2 * z.nP * z.nA + 127) / 128), (unsigned)(4 * z.nH * z.nA));
+      adj_w1_terms_kernel<<<grid, 128, 0, st>>>(a);
+    }
+    DSRG_LAUNCH_CHECK(p);
+    a.thw2 = w->dV2;  // (written by adj_w2_chain_kernel after its last reader)
+    a.dw2 = w->dw2;
+    adj_w2_mid_kernel<<<blocks(A.w2n / 2), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
     adj_w2_terms_kernel<<<blocks(A.w2n / 2), 256, 0, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
@@ -1569,7 +1592,10 @@ cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const 
     DSRG_LAUNCH_CHECK(p);
     adj_t1_chain_kernel<<<blocks(nHP2), 256, dsm, st>>>(a);
     DSRG_LAUNCH_CHECK(p);
-    adj_w1_chain_kernel<<<(unsigned)((A.w1n / (2 * z.nA) + 127) / 128), 128, dsm, st>>>(a);
+    {
+      const dim3 grid((unsigned)((2 * z.nP + 127) / 128), (unsigned)(4 * z.nH * z.nA));
+      adj_w1_chain_kernel<<<grid, 128, dsm, st>>>(a);
+    }
     DSRG_LAUNCH_CHECK(p);
     adj_w2_chain_kernel<<<(unsigned)((A.w2n / (2 * z.nA) + 127) / 128), 128, dsm, st>>>(a);
     DSRG_LAUNCH_CHECK(p);

@@ -869,10 +869,11 @@ __global__ void act_gather_kernel(const float* __restrict__ Y, long long ldy, in
   if (k < 2 * n12) {
     const bool second = k >= n12;
     const size_t r = second ? k - n12 : k;
-    const int a = (int)(r % z.nP);
-    const int x = (int)((r / z.nP) % nA);
-    const int u = (int)((r / ((size_t)z.nP * nA)) % nA);
-    const int i = (int)(r / ((size_t)z.nP * nA * nA));
+    const unsigned r32 = (unsigned)r;  // nH nA^2 nP < 2^31
+    const int a = (int)(r32 % z.nP);
+    const int x = (int)((r32 / z.nP) % nA);
+    const int u = (int)((r32 / (unsigned)(z.nP * nA)) % nA);
+    const int i = (int)(r32 / (unsigned)(z.nP * nA * nA));
     double v;
     if (!second) {  // (ia|ux)
       v = (a < nA) ? Gxx[(size_t)(i * nA + a) * T + (nC + u) * nA + x]
@@ -888,10 +889,9 @@ __global__ void act_gather_kernel(const float* __restrict__ Y, long long ldy, in
     K3[r] = Gxx[r];
   } else if (k < 2 * n12 + n3 + nm) {
     const size_t r = k - 2 * n12 - n3;
-    const int f = (int)(r % z.nV);
-    const int e = (int)((r / z.nV) % z.nV);
-    const int u = (int)((r / ((size_t)z.nV * z.nV)) % nA);
-    const int x = (int)(r / ((size_t)z.nV * z.nV * nA));
+    const size_t xu = r / ((size_t)z.nV * z.nV);
+    const unsigned ef = (unsigned)(r - xu * z.nV * z.nV);
+    const int f = (int)(ef % z.nV), e = (int)(ef / z.nV), u = (int)xu % nA, x = (int)xu / nA;
     M[r] = (double)Y[(size_t)((nC + x) * nVpad + e) * ldy + (size_t)u * nVpad + f];
   }
 }
