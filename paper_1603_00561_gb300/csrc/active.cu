@@ -1381,7 +1381,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     DSRG_LAUNCH_CHECK(p);
     // F6 and F7 read these tables only
     if (p->forked) {
-      const cudaError_t e = plan_link(st, p->ev_tab, p->side);
+      const cudaError_t e = plan_link(st, p->ev_tab, p->caller);
       if (e != cudaSuccess) return e;
     }
   }

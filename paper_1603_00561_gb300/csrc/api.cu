@@ -112,10 +112,10 @@ static std::vector<int> host_io_bounds(const Sizes& z) {
 }
 
 static void free_all(dsrg_plan* p) {
-  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_side})
+  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_join})
     if (*ev) cudaEventDestroy(*ev);
-  if (p->side) cudaStreamDestroy(p->side);
-  p->side = nullptr;
+  if (p->chain) cudaStreamDestroy(p->chain);
+  p->chain = nullptr;
   for (cudaEvent_t ev : p->st_ev) cudaEventDestroy(ev);
   p->st_ev.clear();
   if (p->st_copy) cudaStreamDestroy(p->st_copy);
@@ -335,16 +335,21 @@ static dsrg_status_t check_common(dsrg_plan* p, const double* B, const double* e
 }  // extern "C"
 
 namespace dsrg {
-// The blocks of an energy call that do not wait for one another (CCVV, F2, F3, F6 and F7
-// against the active block's chain) run beside each other when the CCVV items are fewer
-// than the SMs: those kernels then leave SMs free, and one after another their latencies
-// add up (247 us at 10/4/60/200, 166 us beside each other). With more items CCVV holds every SM.
+// The blocks of an energy call that do not wait for one another run beside each other: the
+// GEMM of the active integrals and the active block's chain of short launches on a stream
+// of high priority, so that they take the SMs as CCVV starts and the ones it leaves, CCVV,
+// F2, F3, F6 and F7 on the caller's. One after another their latencies add up: 247 us at
+// 10/4/60/200 and 161 us so, 807 and 730 us at 24/2/372/1200, 3.65 and 3.45 ms with all
+// terms at 31/5/467/1609; no difference at 24/2/1214/3400, where CCVV is most of it. (At
+// the caller's priority: 164, 740 us and 3.58 ms; all but CCVV on the chain: 207, 787 us
+// and 3.62 ms.)
 bool plan_fork_alloc(dsrg_plan* p) {
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
-  if (!p->split || !p->rest_tc || p->z.nA == 0 || split_ccvv_grid(p) >= nsm) return true;
-  if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess) return false;
-  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_side})
+  if (!p->split || !p->rest_tc || p->z.nA == 0) return true;
+  int lo = 0, hi = 0;
+  if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&p->chain, cudaStreamNonBlocking, hi) != cudaSuccess)
+    return false;
+  for (cudaEvent_t* ev : {&p->ev_fork, &p->ev_gemm, &p->ev_tab, &p->ev_join})
     if (cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess) return false;
   return true;
 }
@@ -394,19 +399,23 @@ static dsrg_status_t run_energy(dsrg_plan* p, const double* B, const double* eps
                                 const double* L, const double* L3, const double* F1, double s,
                                 double* out) {
   cudaError_t e;
-  p->forked = p->side != nullptr && p->shard_rank == 0;
+  p->forked = p->chain != nullptr && p->shard_rank == 0;
+  p->caller = p->stream;
   if (p->prec == DSRG_PREC_FP64)
     e = launch_ccvv_fp64_tc(p, B, eps, s);
   else
     e = launch_split_ccvv(p, B, eps, s);
   dsrg_status_t st = DSRG_OK;
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
     st = cuda_fail(p, e, "ccvv");
-  else
+  } else {
+    if (p->forked) p->stream = p->chain;
     st = run_blocks(p, B, eps, G, L, L3, F1, s);
+    p->stream = p->caller;
+  }
   if (p->forked) {  // also after a failure, so that a capture of the caller's ends
     p->forked = false;
-    e = plan_link(p->side, p->ev_side, p->stream);
+    e = plan_link(p->chain, p->ev_join, p->stream);
     if (e != cudaSuccess && st == DSRG_OK) st = cuda_fail(p, e, "join");
   }
   return st != DSRG_OK ? st : run_reduce(p, out);

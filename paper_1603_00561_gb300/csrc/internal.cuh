@@ -104,11 +104,11 @@ struct dsrg_plan {
   dsrg::TcAdjWs* tcadj = nullptr;  // split plans' S and B^T planes of the gradient
   bool rest_tc = false;        // CAVV, CCAV and the active integrals from the tensor-core GEMM
 
-  // Split plans whose CCVV items leave SMs free (plan_fork_alloc): a second stream for
-  // the parts of an energy call that do not depend on each other. `forked` is set while
-  // a call has work on it.
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_gemm = nullptr, ev_tab = nullptr, ev_side = nullptr;
+  // Split plans with active orbitals (plan_fork_alloc): a stream for the active block's
+  // chain of launches, beside the rest on the caller's. While a call is forked, `stream`
+  // is `chain` and `caller` the caller's in run_blocks.
+  cudaStream_t chain = nullptr, caller = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_gemm = nullptr, ev_tab = nullptr, ev_join = nullptr;
   bool forked = false;
 
   // device staging of dsrg_mrpt2_energy_host (DSRG_PLAN_HOST_IO)
@@ -139,11 +139,11 @@ bool plan_alloc(dsrg_plan* p, void** ptr, size_t bytes);
 // limit afterwards for a smaller problem would invalidate that launch.
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
 
-// The second stream where it helps (false: out of resources), an event from one of the
-// plan's two streams to the other, and the side stream while forked (else the plan's).
+// The plan's chain stream and events (false: out of resources), a wait of stream `to` for
+// what `from` holds, and the stream of the kernels beside the chain.
 bool plan_fork_alloc(dsrg_plan* p);
 cudaError_t plan_link(cudaStream_t from, cudaEvent_t ev, cudaStream_t to);
-inline cudaStream_t side_stream(const dsrg_plan* p) { return p->forked ? p->side : p->stream; }
+inline cudaStream_t side_stream(const dsrg_plan* p) { return p->forked ? p->caller : p->stream; }
 
 // Launchers (each returns cudaSuccess or the launch error; adds to p->launches).
 // FP64 plans: tensor-core products (fp64_tc.cu) when their workspace is a small enough
@@ -225,7 +225,6 @@ int split_kb_elems(bool bf16);
 size_t split_mol_desc_bytes();
 void split_fill_mol_desc(const dsrg_plan* p, long long row0, void* out);
 cudaError_t split_stage(dsrg_plan* p, const double* B, const double* eps, double s);
-int split_ccvv_grid(const dsrg_plan* p);  // CTAs of the plan's CCVV launch
 // one bounded wait that runs out (about 2 s) and records DSRG_ERR_TIMEOUT's status word
 cudaError_t launch_wait_selftest(dsrg_plan* p);
 cudaError_t split_stage_rows(dsrg_plan* p, const double* B, int h0, int h1);

@@ -1034,7 +1034,7 @@ cudaError_t launch_split_rest(dsrg_plan* p, const double* B, const double* eps, 
   {
     // F2 and F3 read Y only: beside the active block where the call has forked
     if (p->forked) {
-      const cudaError_t e = plan_link(stream, p->ev_gemm, p->side);
+      const cudaError_t e = plan_link(stream, p->ev_gemm, p->caller);
       if (e != cudaSuccess) return e;
     }
     pair_info_kernel<<<1, 1024, 0, side>>>(eps, s, z, nullptr, z.nC * z.nA, st->pinfo);

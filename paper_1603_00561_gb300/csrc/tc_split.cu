@@ -1585,18 +1585,11 @@ cudaError_t launch_split_ccvv(dsrg_plan* p, const double* B, const double* eps, 
   SplitWs* w = p->split;
   cudaError_t e = split_stage(p, B, eps, s);
   if (e != cudaSuccess) return e;
-  const cudaStream_t main = p->stream;
-  if (p->forked) {
-    if ((e = plan_link(main, p->ev_fork, p->side)) != cudaSuccess) return e;
-    p->stream = p->side;
-  }
-  if ((e = split_prepare_single(p, eps, s)) == cudaSuccess)
-    e = split_launch_ccvv(p, w->cmaps, w->d_mol, w->d_items,
-                          w->d_begin, w->grid, p->prec == DSRG_PREC_BF16X3, w->order);
-  p->stream = main;
-  return e;
+  // the chain needs the staged planes
+  if (p->forked && (e = plan_link(p->stream, p->ev_fork, p->chain)) != cudaSuccess) return e;
+  if ((e = split_prepare_single(p, eps, s)) != cudaSuccess) return e;
+  return split_launch_ccvv(p, w->cmaps, w->d_mol, w->d_items,
+                           w->d_begin, w->grid, p->prec == DSRG_PREC_BF16X3, w->order);
 }
-
-int split_ccvv_grid(const dsrg_plan* p) { return p->split->grid; }
 
 }  // namespace dsrg
