@@ -177,14 +177,15 @@ __global__ void small_ints_kernel(const double* __restrict__ B, Sizes z, double*
 
 // Spin-orbital W1, W2 (V, T, Vt), cumulant and active gamma. One thread per
 // spatial quadruple of W1 / W2: the regulators depend on the spatial orbitals
-// only, so they are evaluated once and the 16 spin combinations written (V itself, a
-// third of the bytes, only for plans whose adjoint reads it).
+// only, so they are evaluated once and the 16 spin combinations written. Without the
+// adjoint (`all` false) nothing reads V itself, nor rows whose first hole is a core orbital
+// of spin 1 (the terms sum one spin of their first orbital): a third of the bytes is left.
 __global__ void build_tables_kernel(const double* __restrict__ eps, const double* __restrict__ G,
                                     const double* __restrict__ L, double s, Sizes z,
                                     const double* __restrict__ K1, const double* __restrict__ K2,
                                     const double* __restrict__ K3, double* __restrict__ W1,
                                     double* __restrict__ W2, double* __restrict__ lam,
-                                    double* __restrict__ gA, size_t w1n, size_t w2n, bool with_v) {
+                                    double* __restrict__ gA, size_t w1n, size_t w2n, bool all) {
   const ActDims d = act_dims(z);
   const size_t n1 = (size_t)z.nH * z.nA * z.nP * z.nA;   // spatial (i, u, a, x)
   const size_t n2 = (size_t)z.nH * z.nH * z.nA * z.nA;   // spatial (i, j, x, y)
@@ -205,11 +206,12 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
     const bool internal = (i >= z.nC) && (a < z.nA);
     for (int sp = 0; sp < 16; ++sp) {
       const int si = sp >> 3, su = (sp >> 2) & 1, sa = (sp >> 1) & 1, sx = sp & 1;
+      if (si == 1 && i < z.nC && !all) break;
       double V = 0.0;
       if (si == sa && su == sx) V += k1;
       if (si == sx && su == sa) V -= k2;
       const size_t o = w1i(d, 2 * i + si, 2 * u + su, 2 * a + sa, 2 * x + sx);
-      if (with_v) W1[o] = V;
+      if (all) W1[o] = V;
       W1[w1n + o] = internal ? 0.0 : V * rt;
       W1[2 * w1n + o] = V * rv;
     }
@@ -226,11 +228,12 @@ __global__ void build_tables_kernel(const double* __restrict__ eps, const double
     const bool internal = (i >= z.nC) && (j >= z.nC);
     for (int sp = 0; sp < 16; ++sp) {
       const int si = sp >> 3, sj = (sp >> 2) & 1, sx = (sp >> 1) & 1, sy = sp & 1;
+      if (si == 1 && i < z.nC && !all) break;
       double V = 0.0;
       if (si == sx && sj == sy) V += kxy;
       if (si == sy && sj == sx) V -= kyx;
       const size_t o = w2i(d, 2 * i + si, 2 * j + sj, 2 * x + sx, 2 * y + sy);
-      if (with_v) W2[o] = V;
+      if (all) W2[o] = V;
       W2[w2n + o] = internal ? 0.0 : V * rt;
       W2[2 * w2n + o] = V * rv;
     }
@@ -272,11 +275,13 @@ __global__ void __launch_bounds__(128) t1_kernel(const double* __restrict__ eps,
                                                  const double* __restrict__ W1T,
                                                  const double* __restrict__ gA,
                                                  const double* __restrict__ f1,
-                                                 double* __restrict__ t1, double* __restrict__ ft) {
+                                                 double* __restrict__ t1, double* __restrict__ ft,
+                                                 bool all) {
   const ActDims d = act_dims(z);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= d.nH2 * z.nP) return;
   const int I = k / z.nP, a = k % z.nP, A = 2 * a + (I & 1);
+  if ((I & 1) && I < d.nC2 && !all) return;  // as in build_tables_kernel
   double S = 0.0;
 #pragma unroll
   for (int u = 0; u < 2 * NA; ++u)
@@ -332,12 +337,13 @@ __device__ __forceinline__ double eta_p(const ActDims& d, const double* gA, int 
 // blockIdx.y is (J, V), so that the index arithmetic is 32-bit (with 64-bit divisions per
 // element, for 16 bytes of traffic, 97 us at 31/5/467/1609, 91 us now).
 __global__ void ti_kernel(Sizes z, const double* __restrict__ W1T, const double* __restrict__ gA,
-                          double* __restrict__ Ti) {
+                          double* __restrict__ Ti, bool all) {
   const ActDims d = act_dims(z);
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= d.nP2 * d.nA2) return;
   const int Y = r % d.nA2, Bp = r / d.nA2, V = blockIdx.y % d.nA2, J = blockIdx.y / d.nA2;
   const size_t k = (size_t)blockIdx.y * d.nP2 * d.nA2 + r;
+  if ((J & 1) && J < d.nC2 && !all) return;  // as in build_tables_kernel
   if ((J & 1) + (V & 1) != (Bp & 1) + (Y & 1)) {  // gamma, eta and t conserve spin
     Ti[k] = 0.0;
     return;
@@ -1367,6 +1373,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   ActiveWs& w = p->act;
   const ActDims d = act_dims(z);
   cudaStream_t st = p->stream, sd = side_stream(p);
+  const bool all = p->grad != nullptr;  // the adjoint reads every spin of the tables
   if (!ints_ready) {
     const size_t n = 2 * (size_t)z.nH * z.nA * z.nA * z.nP + (size_t)z.nH * z.nA * z.nH * z.nA;
     small_ints_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(B, z, w.K1, w.K2, w.K3);
@@ -1376,8 +1383,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     const size_t n = w.w1n / 16 + w.w2n / 16 + (size_t)d.nA2 * d.nA2 * d.nA2 * d.nA2 +
                      (size_t)d.nA2 * d.nA2;
     build_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        eps, G, L, s, z, w.K1, w.K2, w.K3, w.W1, w.W2, w.lam, w.gA, w.w1n, w.w2n,
-        p->grad != nullptr);
+        eps, G, L, s, z, w.K1, w.K2, w.K3, w.W1, w.W2, w.lam, w.gA, w.w1n, w.w2n, all);
     DSRG_LAUNCH_CHECK(p);
     // F6 and F7 read these tables only
     if (p->forked) {
@@ -1389,7 +1395,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
     const int n = d.nH2 * z.nP;
 #define T1_CASE(NA_)                                                                             \
   case NA_:                                                                                      \
-    t1_kernel<NA_><<<(n + 127) / 128, 128, 0, st>>>(eps, s, z, w.W1 + w.w1n, w.gA, F1, w.t1, w.ft); \
+    t1_kernel<NA_><<<(n + 127) / 128, 128, 0, st>>>(eps, s, z, w.W1 + w.w1n, w.gA, F1, w.t1, w.ft, all); \
     break;
     switch (z.nA) {
       T1_CASE(1) T1_CASE(2) T1_CASE(3) T1_CASE(4) T1_CASE(5) T1_CASE(6) T1_CASE(7) T1_CASE(8)
@@ -1400,7 +1406,7 @@ cudaError_t launch_active(dsrg_plan* p, const double* B, const double* eps, cons
   }
   {
     const dim3 grid((unsigned)((d.nP2 * d.nA2 + 255) / 256), (unsigned)(d.nH2 * d.nA2));
-    ti_kernel<<<grid, 256, 0, st>>>(z, w.W1 + w.w1n, w.gA, w.Ti);
+    ti_kernel<<<grid, 256, 0, st>>>(z, w.W1 + w.w1n, w.gA, w.Ti, all);
     DSRG_LAUNCH_CHECK(p);
   }
   if (!ints_ready) {
