@@ -42,7 +42,8 @@
  *     hole index (0..nC-1 core, nC..nH-1 active), a a particle index
  *     (0..nA-1 active, nA..nP-1 virtual); eps has length n = nC+nA+nV;
  *     gamma1 has nA*nA entries and lambda2 nA^4 (both may be NULL if nA == 0);
- *   - all work is queued on the plan's CUDA stream; energy and gradient calls
+ *   - all work is queued on the plan's CUDA stream (and, in between, on streams the
+ *     plan owns, joined before the results); energy and gradient calls
  *     do not allocate and do not synchronise (results land in device memory);
  *   - errors are returned as dsrg_status_t, never by abort or exception; a
  *     one-line detail is kept per plan (dsrg_plan_last_error). Conditions
@@ -71,7 +72,12 @@ typedef enum {
 
 /* Arithmetic of the pair contractions (the v_mn^ef products over Q of
  * Eq. (19) for diagrams F1 and F2, and the (A,A|V,V) integrals):
- *   DSRG_PREC_FP64    plain FP64 products and sums on CUDA cores;
+ *   DSRG_PREC_FP64    FP64: products as exact sums of integer digit products on
+ *                     the tensor cores, rounded once (each factor row as seven
+ *                     base-256 digits of its largest value, so within 2^-56 of
+ *                     that; a row with an infinity in FP64 FMAs, one with a NaN
+ *                     gives NaN), or FP64 FMAs on CUDA cores where the digits'
+ *                     workspace would be over 2/5 of the device's memory;
  *   DSRG_PREC_TF32X3  B = hi + lo split into two TF32 planes, products
  *                     hi*hi + hi*lo + lo*hi on tcgen05 tensor cores with FP32
  *                     accumulation (and lo*lo where both operands are the
@@ -301,7 +307,7 @@ dsrg_status_t dsrg_plan_time_ccvv(dsrg_plan_t *plan, const double *B, const doub
  * service to callers that cannot call cudaMalloc, e.g. code running inside a
  * memory pool it does not own or a host that forbids allocation on its hot
  * path). Same value as out[0] of dsrg_mrpt2_energy with a DSRG_PREC_FP64 plan
- * (same FP64 kernel; the final sum may differ in the last bits). B and eps are
+ * (by FP64 FMAs on CUDA cores: equal to within their rounding). B and eps are
  * device arrays as above, out_dev one device double, work queued on
  * cuda_stream. Scratch (work lists and per-item partial sums) lives in a fixed
  * device array of 147456 doubles (1.125 MiB) inside the library, held on every
@@ -378,10 +384,11 @@ dsrg_status_t dsrg_plan_branch_counts(dsrg_plan_t *plan, uint64_t counts[DSRG_NC
  *                                on every index (only if lambda3 != NULL);
  *   U_out       [n][n]           U (may be NULL).
  * All arrays are caller-owned device arrays, 8-byte aligned. The plan owns its
- * workspace (about naux*n*(nH+1) + 2*naux*nH*nP + 6 n^2 doubles). The
- * semicanonicalisation synchronises the plan's stream (the Jacobi sweeps stop
- * on a convergence test read by the host, ||offdiag||^2 <= 1e-30 ||A||^2, at
- * most 30 sweeps) and is not meant to be captured in a graph. */
+ * workspace (about naux*n*(nH+1) + 2*naux*nH*nP + 7 n^2 doubles, partial exchange
+ * matrices and up to 512 MiB for the products' digits). The semicanonicalisation
+ * synchronises the plan's stream at its end (the Jacobi sweeps run in one launch per
+ * block and stop at ||offdiag||^2 <= 1e-30 ||A||^2, at most 30 sweeps) and is not meant
+ * to be captured in a graph. */
 typedef struct dsrg_sc_plan dsrg_sc_plan_t;
 /* sz->ncore, nactive, nvirt >= 0 (n >= 1), naux >= 1, nactive <= 8. */
 dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t **plan, const dsrg_sizes_t *sz, void *cuda_stream);
