@@ -10,8 +10,9 @@
 //         (F2), CCAV (F3) and the active block's integrals read it.
 //
 // The FP64 CUDA-core kernels these replace ran at the FP64 pipe's rate: 101.6 ms for
-// CCVV and 16 ms for CAVV at the cc-pVTZ size (24/2/372/1200); here 4.2 ms and 0.4 ms (plus 0.9 ms for the
-// shared GEMM of the rest).
+// CCVV and 16 ms for CAVV at the cc-pVTZ size (24/2/372/1200); here 4.7 ms (products 3.3,
+// regulators 1.4) and 0.35 ms, and 0.64 ms for the product of the rest. Regulators beside
+// the next group's product would need registers that its kernel leaves no room for.
 // The regulators are what is left on that pipe: about 25 FP64 instructions each.
 #include "internal.cuh"
 #include "oz_gemm.cuh"
