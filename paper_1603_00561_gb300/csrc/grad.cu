@@ -1053,7 +1053,7 @@ __device__ __forceinline__ void dacc_warp(double* sacc, int o, double v) {
 // A thread takes one (I,U,A) and the X its spin allows (W1 is zero elsewhere): the sums
 // of an orbital's derivatives stay in registers or are added over the warp, where an
 // atomic per element on the few active orbitals took most of the time (127 us at
-// 10/4/60/200 and 289 us at 24/2/372/1200, 43 us and 57 us now).
+// 10/4/60/200 and 289 us at 24/2/372/1200, 42 us and 62 us now).
 __global__ void __launch_bounds__(128) adj_w1_chain_kernel(ActAdjArgs a) {
   extern __shared__ double sacc_[];
   dacc_init(sacc_, a.z.n);
