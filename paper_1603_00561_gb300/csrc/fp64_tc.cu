@@ -25,6 +25,7 @@ struct Fp64Tc {
   OzRows rows{};               // p (B) is filled per call
   __nv_bfloat16* planes = nullptr;
   int* rexp = nullptr;
+  void* mask = nullptr;        // of the products of a group, or of Y
   int group = 0;               // core pairs per buffer
   double* V = nullptr;         // [group][nV][nV]
   double* Y = nullptr;         // [xrow0 + nH nA][ldy]
@@ -309,7 +310,7 @@ __global__ void gather_y_fp64_kernel(const double* __restrict__ Y, long long ldy
 // product just wrote from it.
 constexpr size_t V_BYTES = (size_t)96 << 20;
 
-// The slices take 14 bytes per value of B and Y one FP64 per (hole, virtual) and active
+// The slices and the check plane take 16 bytes per value of B and Y one FP64 per (hole, virtual) and active
 // pair: sizes whose workspace would be over 2/5 of the device's memory stay with the
 // CUDA-core kernels, which need none (they run for hours there, but they run).
 bool fp64_tc_alloc(dsrg_plan* p) {
@@ -317,7 +318,7 @@ bool fp64_tc_alloc(dsrg_plan* p) {
   {
     const double nvp = (z.nV + OZ_ROW_PAD - 1) / OZ_ROW_PAD * (double)OZ_ROW_PAD;
     const double rows = z.nH * nvp + z.nH * z.nA + OZ_ROW_PAD;
-    const double bytes = rows * (14.0 * oz_kpad(z.Q) + 8.0 * (z.nA * nvp + z.nH * z.nA));
+    const double bytes = rows * (16.0 * oz_kpad(z.Q) + 8.0 * (z.nA * nvp + z.nH * z.nA));
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
     if (bytes > 0.4 * (double)total_b || rows > 2.0e9) return true;
@@ -342,8 +343,11 @@ bool fp64_tc_alloc(dsrg_plan* p) {
   const size_t per = (size_t)z.nV * z.nV * sizeof(double);
   const size_t fit = V_BYTES / per;
   w->group = (int)(fit < 1 ? 1 : (fit > (size_t)p->n_pairs ? (size_t)p->n_pairs : fit));
+  const size_t mask_v = oz_mask_bytes(z.nV, z.nV, w->group);
+  const size_t mask_y = oz_mask_bytes(w->xrow0 + z.nH * z.nA, w->xc + z.nH * z.nA, 1);
   return plan_alloc(p, (void**)&w->planes, oz_plane_bytes(r.total, z.Q)) &&
-         plan_alloc(p, (void**)&w->rexp, (size_t)r.total * sizeof(int)) &&
+         plan_alloc(p, (void**)&w->rexp, (size_t)r.total * OZ_ROW_INFO) &&
+         plan_alloc(p, &w->mask, mask_v > mask_y ? mask_v : mask_y) &&
          plan_alloc(p, (void**)&w->V, per * w->group) &&
          (z.nA == 0 ||
           plan_alloc(p, (void**)&w->Y, (size_t)(w->xrow0 + z.nH * z.nA) * w->ldy * sizeof(double)));
@@ -379,6 +383,7 @@ static OzArgs pair_args(const dsrg_plan* p, const double* B) {
   a.astep = a.bstep = w->nVpad;
   a.alpha = 1.0;
   a.accumulate = 0;
+  a.mask = w->mask;
   return a;
 }
 
@@ -397,7 +402,7 @@ cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps
     const int n = left < w->group ? left : w->group;
     a.p0 = p0;
     if ((e = oz_multiply(p->stream, w->planes, w->planes, a, n)) != cudaSuccess) return e;
-    ++p->launches;
+    p->launches += 3;
     ccvv_reg_fp64_kernel<<<(unsigned)(n * p->n_tp_ccvv), 256, 0, p->stream>>>(
         w->V, eps, s, z, p->d_pairs, p0, p->shard_world, p->d_tp_ccvv, p->n_tp_ccvv,
         p->d_partials + sg.begin);
@@ -419,7 +424,7 @@ cudaError_t launch_ccvv_adj_fp64_tc(dsrg_plan* p, const double* B, const double*
     const int n = p->n_pairs - p0 < w->group ? p->n_pairs - p0 : w->group;
     a.p0 = p0;
     if ((e = oz_multiply(p->stream, w->planes, w->planes, a, n)) != cudaSuccess) return e;
-    ++p->launches;
+    p->launches += 3;
     ccvv_adj_v_kernel<<<(unsigned)(n * p->n_tp_ccvv), 256, sm, p->stream>>>(
         w->V, eps, s, p->z, p->d_pairs, p0, p->d_tp_ccvv, p->n_tp_ccvv, nVp, W, deps, ds);
     DSRG_LAUNCH_CHECK(p);
@@ -462,8 +467,9 @@ cudaError_t launch_rest_fp64_tc(dsrg_plan* p, const double* B, const double* eps
   a.astep = a.bstep = 0;
   a.alpha = 1.0;
   a.accumulate = 0;
+  a.mask = w->mask;
   if ((e = oz_multiply(st, w->planes, w->planes, a, 1)) != cudaSuccess) return e;
-  ++p->launches;
+  p->launches += 3;
   const Segment &s2 = p->segs[p->seg_cavv], &s3 = p->segs[p->seg_ccav];
   const size_t sm2 = (size_t)z.nA * FT * (FT + 1) * 8, sm3 = (size_t)z.nC * z.nC * z.nA * 8;
 #define REST_CASE(NA_)                                                                            \

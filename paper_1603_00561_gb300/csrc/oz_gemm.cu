@@ -14,12 +14,20 @@
 // first dropped weight is 2^-78 of the scales). After every 128 K values the
 // epilogue takes the eight integer sums out of TMEM and adds them into a 96-bit
 // integer per element; one conversion and one rounding to FP64 end the tile. The
-// result does not depend on the order of anything. Its error, set by the slicing
-// (2^-56 of the row scale per value) and that rounding, is below that of a chain of
-// FP64 FMAs (tests/test_gpu_oz_gemm.py).
+// result does not depend on the order of anything.
 //
-// A row with a NaN gives NaN; a row with an infinity is multiplied by FP64 FMAs in the
-// epilogue, so that infinities propagate as in a plain FP64 product.
+// Error. A value is off by at most 2^-56 of its row's scale, so with x_k = |a_k| / 2^Ea and
+// y_k = |b_k| / 2^Eb the digits give c within 2^-56 2^{Ea+Eb} (sum x + sum y), whatever the
+// size of the products (and the dropped weights within K 2^-61.6): much is lost where a row
+// of A is large where the row of B is small (badly scaled auxiliary functions, orbitals on
+// different fragments). A chain of FP64 FMAs gives c within K 2^-53 2^{Ea+Eb} S, S = sum x y.
+// So every element is checked: an extra product of the leading eight bits of the magnitudes
+// gives S from below (oz_check_kernel), and elements with 8 K S < sum x + sum y + K / 50 are
+// formed by FP64 FMAs (oz_fma_kernel). S = 0 is exact (no K index has both factors). The bound is then no
+// larger than that of the FMA chain for any element of any input. On N(0, 1) e^{-0.02 Q}
+// factors no element fails the check, on the products of the Fock and DF steps 1e-3 and
+// fewer; with an unnormalised auxiliary basis (metric diagonal over 1e11) 9 in 10 of the
+// product with the inverse factor do, and it runs at the FP64 pipe's rate.
 //
 // Kernel (one CTA per SM, persistent, tiles 128 x 64):
 //   warp 0      producer: bulk copies of the seven slices of 128 A rows (56 KB, one
@@ -32,6 +40,8 @@
 // [slice][row % 128][64 bytes, swizzled]: as K-major planes behind a tensor map a stage
 // was 1344 rows of 64 bytes and took 4400 clocks to arrive, twice what its MMAs take.
 #include <cuda_bf16.h>
+
+#include <climits>
 
 #include "internal.cuh"
 #include "oz_gemm.cuh"
@@ -49,6 +59,7 @@ constexpr int OZ_STAGE_BYTES = OZ_A_BYTES + OZ_B_BYTES;
 constexpr int OZ_THREADS = 320, OZ_EPI_WARPS = 8;
 constexpr int OZ_EXP_INF = 0x7ff;             // "exponent" of a row with an infinity
 constexpr int OZ_EXP_NAN = 0x800;             // ... with a NaN
+constexpr long long OZ_TINY = LLONG_MIN;      // a value that is not 0 but is as a fixed-point number
 
 // ------------------------------- row scales -------------------------------
 // Biased exponent of the largest magnitude of every row, by atomicMax (rexp starts
@@ -84,11 +95,12 @@ __global__ void __launch_bounds__(256) oz_rowmax_kernel(OzRows s, int* __restric
 }
 
 // ------------------------------- slices -------------------------------
-// x as a fixed-point integer of the row scale: round(x 2^{55 - E}), |.| <= 2^55.
+// x as a fixed-point integer of the row scale: round(x 2^{55 - E}), |.| <= 2^55, or OZ_TINY.
 __device__ __forceinline__ long long oz_fixed(double x, int rowexp) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(u >> 52) & 0x7ff;
-  if (e == 0 || rowexp >= OZ_EXP_INF) return 0;  // zeros and values below 2^-1022; see the epilogue
+  if (rowexp >= OZ_EXP_INF || (u << 1) == 0) return 0;  // see the epilogue; zero
+  if (e == 0) return OZ_TINY;                           // below 2^-1022
   unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
   const int sh = rowexp - e - 2;  // right shift of the 53-bit significand
   if (sh <= 0)
@@ -97,6 +109,7 @@ __device__ __forceinline__ long long oz_fixed(double x, int rowexp) {
     m = (m + (1ull << (sh - 1))) >> sh;
   else
     m = 0;
+  if (m == 0) return OZ_TINY;
   return (u >> 63) ? -(long long)m : (long long)m;
 }
 
@@ -108,9 +121,19 @@ __device__ __forceinline__ size_t oz_off(int row, int l, int sl, int nkb) {
   return (blk * 128 + r) * 64 + (size_t)((((l >> 3) & 3) ^ ((r >> 1) & 3)) * 16);
 }
 
-// 64 rows x 64 K values per CTA through shared memory.
+// ... and of a row of the check plane (one slice).
+__device__ __forceinline__ size_t oz_check_off(int row, int l, int nkb) {
+  const int r = row & 127;
+  return (((size_t)(row >> 7) * nkb + (l >> 5)) * 128 + r) * 64 +
+         (size_t)((((l >> 3) & 3) ^ ((r >> 1) & 3)) * 16);
+}
+
+// 64 rows x 64 K values per CTA through shared memory. The check plane (after the slices)
+// holds the leading eight bits of |x| / 2^E, 2^-60 for OZ_TINY; rsum its sum over the row in
+// 2^-24 units, rounded up (integers: the order of the atomics does not matter).
 template <bool KCONT>
 __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __restrict__ rexp,
+                                                       unsigned long long* __restrict__ rsum,
                                                        __nv_bfloat16* __restrict__ planes, int Kp) {
   __shared__ long long t[64][65];
   const int r0 = blockIdx.x * 64, l0 = blockIdx.y * 64, K = s.L1 * s.L2;
@@ -124,11 +147,34 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __re
   }
   __syncthreads();
   const int rr = threadIdx.x >> 2, c0 = (threadIdx.x & 3) * 16;
-  if (r0 + rr >= s.total || l0 + c0 >= Kp) return;
+  const bool on = r0 + rr < s.total && l0 + c0 < Kp;
   const int nkb = Kp / OZ_KB;
   long long v[16];
+  unsigned long long sum = 0;
+  uint32_t cw[8];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = t[rr][c0 + k];
+  for (int k = 0; k < 16; k += 2) {
+    float x[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const long long w = t[rr][c0 + k + i];
+      v[k + i] = w == OZ_TINY ? 0 : w;
+      const unsigned long long m = (unsigned long long)llabs(v[k + i]);
+      sum += (m >> 31) + (w != 0);
+      x[i] = w == OZ_TINY ? 0x1p-60f : __ull2float_rz(m) * 0x1p-55f;
+    }
+    const __nv_bfloat162 h = __halves2bfloat162(__float2bfloat16_rz(x[0]), __float2bfloat16_rz(x[1]));
+    cw[k / 2] = *(const uint32_t*)&h;
+  }
+  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  if (!on) return;
+  if ((threadIdx.x & 3) == 0 && sum) atomicAdd(&rsum[r0 + rr], sum);
+  {
+    uint8_t* o = (uint8_t*)planes + (size_t)OZ_S * s.total * Kp * sizeof(__nv_bfloat16);
+    *(uint4*)(o + oz_check_off(r0 + rr, l0 + c0, nkb)) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
+    *(uint4*)(o + oz_check_off(r0 + rr, l0 + c0 + 8, nkb)) = make_uint4(cw[4], cw[5], cw[6], cw[7]);
+  }
 #pragma unroll
   for (int sl = OZ_S - 1; sl >= 0; --sl) {
     uint32_t w[8];
@@ -347,6 +393,15 @@ __device__ __forceinline__ OzTile oz_tile(const OzArgs& a, int it) {
   return t;
 }
 
+// The mask words [128 rows][2 x 32 columns] of an item, and the bytes that say whether the
+// epilogue warps of the check set any.
+__device__ __forceinline__ uint32_t* oz_mask(const OzArgs& a, int it) {
+  return (uint32_t*)a.mask + (size_t)it * 256;
+}
+__device__ __forceinline__ uint8_t* oz_mask_any(const OzArgs& a, int it) {
+  return (uint8_t*)a.mask + (size_t)a.n_items * 1024 + (size_t)it * 8;
+}
+
 // An element whose row of A or B is not finite.
 static __device__ __noinline__ double oz_not_finite(const OzArgs& a, int ra, int rb, int e) {
   if (e >= OZ_EXP_NAN) return __longlong_as_double(0x7ff8000000000000ll);
@@ -540,11 +595,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       if (i < a.M) {
         // value = (hi + lo 2^-32) 2^-38 2^{Ea + Eb}, E = exponent field - 1022
         const int ra = t.arow + quarter * 32 + lane, ea = a.aexp[ra];
+        // elements of oz_fma_kernel
+        const uint32_t skip = oz_mask(a, it)[(quarter * 32 + lane) * 2 + ch];
         double* crow = a.C + t.coff + (long long)i * a.ci;
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
           const int j = t.j0 + ch * 32 + c;
-          if (j < a.N) {
+          if (j < a.N && !(skip >> c & 1u)) {
             double d = fma((double)lo[c], 2.3283064365386962890625e-10, (double)hi[c]);
             const int rb = t.brow + ch * 32 + c, eb = a.bexp[rb];
             const int e = ea + eb - 2 * 1022 - 38;
@@ -575,19 +632,301 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
 }
 
+// ------------------------------- the check -------------------------------
+// S of every element (see the head of the file) in one FP32 accumulation over all of K, and
+// its mask bit. One BF16 product against the 34 of the slices, bound by its operands' copies:
+// 4 stages of up to 128 K values.
+constexpr int OC_KB = 4;  // blocks of 32 K values per stage
+constexpr int OC_STAGES = 4;
+constexpr int OC_STAGE_BYTES = OC_KB * (OZ_A_SLICE + OZ_B_SLICE);
+
+__global__ void __launch_bounds__(OZ_THREADS, 1)
+    oz_check_kernel(const uint8_t* __restrict__ pa, const uint8_t* __restrict__ pb,
+                    const __grid_constant__ OzArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + OC_STAGES * OC_STAGE_BYTES);
+  uint64_t* empty = full + OC_STAGES;
+  uint64_t* tfull = empty + OC_STAGES;  // [2]
+  uint64_t* tempty = tfull + 2;         // [2]
+  uint64_t* drain = tempty + 2;
+  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < OC_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(&tfull[t], 1);
+      mbar_init(&tempty[t], OZ_EPI_WARPS);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     su32(tmem_slot)),
+                 "r"(128u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int nst = (a.kstages + OC_KB - 1) / OC_KB;
+
+  if (warp == 0) {
+    const uint32_t leader = tc_elect();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; ok && it < a.n_items; it += gridDim.x) {
+      const OzTile t = oz_tile(a, it);
+      const uint8_t* ga = pa + (size_t)(t.arow >> 7) * a.kstages * OZ_A_SLICE;
+      const uint8_t* gb = pb + (size_t)(t.brow >> 7) * a.kstages * OZ_A_SLICE + (t.brow & 64) * 64;
+      for (int ks = 0; ks < nst; ++ks) {
+        if (!TC_WARP_WAIT(&empty[stage], phase ^ 1u, abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        uint8_t* st = smem + stage * OC_STAGE_BYTES;
+        const int k0 = ks * OC_KB, nk = min(OC_KB, a.kstages - k0);
+        mbar_expect_tx_if(leader, &full[stage], (uint32_t)(nk * (OZ_A_SLICE + OZ_B_SLICE)));
+        if (leader) {
+          oz_bulk(st, ga + (size_t)k0 * OZ_A_SLICE, (uint32_t)(nk * OZ_A_SLICE), &full[stage]);
+          for (int k = 0; k < nk; ++k)
+            oz_bulk(st + OC_KB * OZ_A_SLICE + k * OZ_B_SLICE, gb + (size_t)(k0 + k) * OZ_A_SLICE, OZ_B_SLICE,
+                    &full[stage]);
+        }
+        __syncwarp();
+        if (++stage == OC_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    if (!ok && leader) {
+      int s = stage;
+      uint32_t ph = phase;
+      for (int k = 0; k < OC_STAGES; ++k) {
+        if (--s < 0) {
+          s = OC_STAGES - 1;
+          ph ^= 1u;
+        }
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try(&full[s], ph) && gtimer() - t0 < TC_WAIT_NS) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    const uint32_t leader = tc_elect();
+    const uint32_t tm = tc_uniform(tmem), base_lo = tc_uniform(desc_sw64_lo(su32(smem)));
+    constexpr uint32_t idesc = idesc_128xn<true>(OZ_BN);
+    int stage = 0, tb = 0;
+    uint32_t phase = 0, tphase = 0;
+    bool ok = true, issued = false;
+    for (int it = blockIdx.x; ok && it < a.n_items; it += gridDim.x) {
+      if (!TC_WARP_WAIT(&tempty[tb], tphase ^ 1u, abort_flag, a.status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      for (int ks = 0; ks < nst; ++ks) {
+        if (!TC_WARP_WAIT(&full[stage], phase, abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t sa = base_lo + (uint32_t)(stage * (OC_STAGE_BYTES / 16));
+        const uint32_t sb = sa + OC_KB * OZ_A_SLICE / 16;
+        const int nk = min(OC_KB, a.kstages - ks * OC_KB);
+        for (int k = 0; k < nk; ++k)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            tc_mma_if<true>(leader, tm + (uint32_t)(tb * OZ_BN), sa + k * (OZ_A_SLICE / 16) + 2 * h,
+                            sb + k * (OZ_B_SLICE / 16) + 2 * h, idesc, (ks | k | h) ? 1u : 0u);
+        issued = true;
+        tc_commit_if(leader, &empty[stage]);
+        if (++stage == OC_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+      if (!ok) break;
+      tc_commit_if(leader, &tfull[tb]);
+      if (++tb == 2) {
+        tb = 0;
+        tphase ^= 1u;
+      }
+    }
+    if (!ok && issued && leader) {
+      tc_commit(drain);
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(drain, 0) && gtimer() - t0 < TC_WAIT_NS) {
+      }
+    }
+  } else {
+    const int quarter = warp & 3, ch = (warp - 2) >> 2;  // TMEM lanes and column half
+    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ch * 32);
+    const unsigned long long* asum = (const unsigned long long*)(a.aexp + a.a.total);
+    const unsigned long long* bsum = (const unsigned long long*)(a.bexp + a.b.total);
+    const float K = (float)(a.a.L1 * a.a.L2), K8 = 8.0f * K;
+    int tb = 0;
+    uint32_t tphase = 0;
+    for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
+      const OzTile t = oz_tile(a, it);
+      const bool ok = mbar_wait(&tfull[tb], tphase, abort_flag, a.status);
+      tc_fence_after();
+      uint32_t r[2][16];
+      if (ok) {
+        tmem_ld16(tl + (uint32_t)(tb * OZ_BN), r[0]);
+        tmem_ld16(tl + (uint32_t)(tb * OZ_BN + 16), r[1]);
+        tmem_ld_wait();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[tb]);
+      if (++tb == 2) {
+        tb = 0;
+        tphase ^= 1u;
+      }
+      const int row = quarter * 32 + lane, i = t.i0 + row;
+      uint32_t word = 0;
+      if (ok && i < a.M) {
+        const float sa = (float)asum[t.arow + row] * 0x1p-24f + 0.02f * K;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const int j = ch * 32 + c;
+          if (t.j0 + j < a.N) {
+            const float S = __uint_as_float(r[c >> 4][c & 15]);
+            if (S > 0.0f && K8 * S < sa + (float)bsum[t.brow + j] * 0x1p-24f) word |= 1u << c;
+          }
+        }
+      }
+      oz_mask(a, it)[row * 2 + ch] = word;
+      const bool any = __any_sync(0xffffffffu, word != 0);
+      if (lane == 0) oz_mask_any(a, it)[warp - 2] = any;
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128u)
+                 : "memory");
+  }
+}
+
+// The elements the check set, from the FP64 operands: a warp each, its lanes along K, where
+// a quarter of a 64 x 64 half tile or less is set, else the half tile in chunks of 16 K
+// values (the chain of gemm_fp64_kernel in grad.cu).
+constexpr int OF_FEW = 1024;
+__global__ void __launch_bounds__(256) oz_fma_kernel(const __grid_constant__ OzArgs a) {
+  __shared__ double sA[16][OZ_BN + 1], sB[16][OZ_BN + 1];
+  __shared__ uint32_t sm[128];  // mask words of a half tile: [64 rows][2]
+  __shared__ unsigned short list[OF_FEW];
+  __shared__ unsigned char work[256];
+  __shared__ int cnt;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int L1 = a.a.L1, L2 = a.a.L2, K = L1 * L2;
+  auto put = [&](double* p, double d) { *p = a.accumulate ? fma(a.alpha, d, *p) : a.alpha * d; };
+  for (long long base = blockIdx.x; base < a.n_items; base += 256ll * gridDim.x) {
+    // 256 items at a time: which of them have any
+    const long long mine = base + (long long)tid * gridDim.x;
+    work[tid] = mine < a.n_items && *(const unsigned long long*)oz_mask_any(a, (int)mine) != 0;
+    if (!__syncthreads_or(work[tid])) continue;
+    for (int w = 0; w < 512; ++w) {
+      if (!work[w >> 1]) continue;
+      const int it = (int)(base + (long long)(w >> 1) * gridDim.x), h = w & 1;
+      __syncthreads();  // the previous half tile is done
+      if (tid == 0) cnt = 0;
+      if (tid < 128) sm[tid] = oz_mask(a, it)[h * 128 + tid];
+      __syncthreads();
+      if (tid < 128 && sm[tid]) atomicAdd(&cnt, __popc(sm[tid]));
+      __syncthreads();
+      const int n = cnt;
+      if (n == 0) continue;
+      const OzTile t = oz_tile(a, it);
+      const int i0 = t.i0 + 64 * h, ar = t.arow + 64 * h;
+      double* C = a.C + t.coff;
+      if (n <= OF_FEW) {
+        __syncthreads();
+        if (tid == 0) cnt = 0;
+        __syncthreads();
+        if (tid < 128)
+          for (uint32_t m = sm[tid]; m; m &= m - 1)
+            list[atomicAdd(&cnt, 1)] = (unsigned short)((tid >> 1) << 6 | (tid & 1) << 5 | (__ffs(m) - 1));
+        __syncthreads();
+        for (int e = warp; e < n; e += 8) {  // (whatever the order of the list)
+          const int r = list[e] >> 6, c = list[e] & 63;
+          long long oa, ob;
+          oz_row(a.a, ar + r, oa);
+          oz_row(a.b, t.brow + c, ob);
+          double d = 0.0;
+#pragma unroll 4
+          for (int l = lane; l < K; l += 32)
+            d = fma(a.a.p[oa + oz_k(a.a, l)], a.b.p[ob + oz_k(a.b, l)], d);
+          for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+          if (lane == 0) put(C + (long long)(i0 + r) * a.ci + (long long)(t.j0 + c) * a.cj, d);
+        }
+        continue;
+      }
+      const int ty = tid >> 4, tx = tid & 15;
+      double acc[4][4] = {};
+      for (int l0 = 0; l0 < K; l0 += 16) {
+        for (int e = tid; e < 16 * 64; e += 256) {
+          const int l = l0 + (e >> 6), c = e & 63;
+          double va = 0.0, vb = 0.0;
+          if (l < K) {
+            long long o;
+            if (i0 + c < a.M && oz_row(a.a, ar + c, o)) va = a.a.p[o + oz_k(a.a, l)];
+            if (t.j0 + c < a.N && oz_row(a.b, t.brow + c, o)) vb = a.b.p[o + oz_k(a.b, l)];
+          }
+          sA[e >> 6][c] = va;
+          sB[e >> 6][c] = vb;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int l = 0; l < 16; ++l)
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] = fma(sA[l][ty * 4 + r], sB[l][tx * 4 + c], acc[r][c]);
+        __syncthreads();
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int i = ty * 4 + r, j = tx * 4 + c;
+          if (sm[i * 2 + (j >> 5)] >> (j & 31) & 1u)
+            put(C + (long long)(i0 + i) * a.ci + (long long)(t.j0 + j) * a.cj, acc[r][c]);
+        }
+    }
+    __syncthreads();
+  }
+}
+
 // ------------------------------- host side -------------------------------
 cudaError_t oz_pack(cudaStream_t st, const OzRows& s, __nv_bfloat16* planes, int* rexp) {
   const int Kp = oz_kpad((long long)s.L1 * s.L2);
   const dim3 grid((unsigned)((s.total + 63) / 64), (unsigned)((Kp + 63) / 64));
-  cudaError_t e = cudaMemsetAsync(rexp, 0, (size_t)s.total * sizeof(int), st);
+  cudaError_t e = cudaMemsetAsync(rexp, 0, (size_t)s.total * OZ_ROW_INFO, st);
   if (e != cudaSuccess) return e;
+  unsigned long long* rsum = (unsigned long long*)(rexp + s.total);
   // lanes along K when K is the unit-stride index, else along the rows
   if ((s.L2 == 1 ? s.k1 : s.k2) == 1 && s.ri != 1) {
     oz_rowmax_kernel<true><<<grid, 256, 0, st>>>(s, rexp);
-    oz_slice_kernel<true><<<grid, 256, 0, st>>>(s, rexp, planes, Kp);
+    oz_slice_kernel<true><<<grid, 256, 0, st>>>(s, rexp, rsum, planes, Kp);
   } else {
     oz_rowmax_kernel<false><<<grid, 256, 0, st>>>(s, rexp);
-    oz_slice_kernel<false><<<grid, 256, 0, st>>>(s, rexp, planes, Kp);
+    oz_slice_kernel<false><<<grid, 256, 0, st>>>(s, rexp, rsum, planes, Kp);
   }
   return cudaGetLastError();
 }
@@ -605,21 +944,27 @@ cudaError_t oz_multiply(cudaStream_t st, const __nv_bfloat16* pa, const __nv_bfl
   int dev = 0, nsm = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const unsigned grid = (unsigned)(items < nsm ? items : nsm);
+  const size_t smc = (size_t)OC_STAGES * OC_STAGE_BYTES + 1024 + 256;
+  raise_smem_limit((const void*)oz_check_kernel, smc);
+  oz_check_kernel<<<grid, OZ_THREADS, smc, st>>>((const uint8_t*)(pa + (size_t)OZ_S * a.a.total * Kp),
+                                                 (const uint8_t*)(pb + (size_t)OZ_S * a.b.total * Kp), a);
   const size_t sm = (size_t)OZ_STAGES * OZ_STAGE_BYTES + 1024 + 256;
   raise_smem_limit((const void*)oz_gemm_kernel, sm);
-  oz_gemm_kernel<<<(unsigned)(items < nsm ? items : nsm), OZ_THREADS, sm, st>>>(
-      (const uint8_t*)pa, (const uint8_t*)pb, a);
+  oz_gemm_kernel<<<grid, OZ_THREADS, sm, st>>>((const uint8_t*)pa, (const uint8_t*)pb, a);
+  oz_fma_kernel<<<(unsigned)(items < 4ll * nsm ? items : 4ll * nsm), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 // ------------------------------- generic GEMM -------------------------------
 static long long oz_up(long long x, long long m) { return (x + m - 1) / m * m; }
-static size_t oz_row_bytes(long long K) { return (size_t)OZ_S * oz_kpad(K) * 2 + sizeof(int); }
+static size_t oz_row_bytes(long long K) { return oz_plane_bytes(1, K) + OZ_ROW_INFO; }
 
 size_t oz_work_bytes(long long M, long long N, long long K, long long nb, bool shared_a, bool shared_b) {
   const long long mp = oz_up(M, OZ_ROW_PAD), np = oz_up(N, OZ_ROW_PAD);
-  const size_t need = ((shared_a ? mp : mp * nb) + (shared_b ? np : np * nb)) * oz_row_bytes(K);
-  const size_t one = (mp + np) * oz_row_bytes(K);
+  const size_t mask = oz_mask_bytes(mp, np, 1);  // (rows padded to whole blocks: either side may be M)
+  const size_t need = ((shared_a ? mp : mp * nb) + (shared_b ? np : np * nb)) * oz_row_bytes(K) + nb * mask;
+  const size_t one = (mp + np) * oz_row_bytes(K) + mask;
   const size_t cap = need < OZ_WS_CAP ? need : OZ_WS_CAP;
   return (cap > one ? cap : (one < 4 * OZ_WS_CAP ? one : 4 * OZ_WS_CAP)) + 4096;
 }
@@ -660,17 +1005,18 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
   const bool share_m = g.nb > 1 && zm == 0, share_n = g.nb > 1 && zn == 0;
   const size_t rb = oz_row_bytes(K);
   const size_t avail = w.bytes > 2048 ? w.bytes - 2048 : 0;
+  const size_t mb128 = oz_mask_bytes(OZ_BM, n, 1);  // mask of 128 rows
   const long long np = oz_up(n, OZ_ROW_PAD);
   long long mb = oz_up(m, OZ_ROW_PAD);  // rows of the 128-row side at a time
   // problems at a time
   const size_t fixed = ((share_m ? mb : 0) + (share_n ? np : 0)) * rb;
-  const size_t per = ((share_m ? 0 : mb) + (share_n ? 0 : np)) * rb;
+  const size_t per = ((share_m ? 0 : mb) + (share_n ? 0 : np)) * rb + mb / OZ_BM * mb128;
   long long zb = fixed + per <= avail ? (long long)((avail - fixed) / per) : 0;
   if (zb > g.nb) zb = g.nb;
   if (zb < 1) {
     // not even one problem: a problem's rows in blocks
-    const long long rows = avail / rb > (size_t)np ? (long long)(avail / rb) - np : 0;
-    mb = rows / OZ_ROW_PAD * OZ_ROW_PAD;
+    const size_t left = avail > np * rb ? avail - np * rb : 0;
+    mb = (long long)(left / (OZ_ROW_PAD * rb + mb128)) * OZ_ROW_PAD;
     if (mb < OZ_ROW_PAD) return launch_gemm_fp64(st, g0);
     zb = 1;
   }
@@ -679,7 +1025,8 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
   __nv_bfloat16* plm = (__nv_bfloat16*)base;
   __nv_bfloat16* pln = (__nv_bfloat16*)(base + oz_up(oz_plane_bytes(m_rows, K), 256));
   int* xm = (int*)((uint8_t*)pln + oz_up(oz_plane_bytes(n_rows, K), 256));
-  int* xn = xm + m_rows;
+  int* xn = (int*)((uint8_t*)xm + m_rows * OZ_ROW_INFO);
+  void* mask = (uint8_t*)xn + n_rows * OZ_ROW_INFO;  // (row counts are multiples of 128)
   cudaError_t e;
   for (long long z0 = 0; z0 < g.nb; z0 += zb) {
     const int nz = (int)(g.nb - z0 < zb ? g.nb - z0 : zb);
@@ -710,6 +1057,7 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
       a.bstep = share_n ? 0 : a.b.rpad;
       a.alpha = g.alpha;
       a.accumulate = g.accumulate;
+      a.mask = mask;
       if ((e = oz_multiply(st, plm, pln, a, nz)) != cudaSuccess) return e;
     }
   }

@@ -1,4 +1,5 @@
-// FP64 products on the tensor cores from exact integer slices (oz_gemm.cu).
+// FP64 products on the tensor cores from exact integer slices, checked element by element
+// against the error of FP64 FMAs (oz_gemm.cu).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -63,7 +64,7 @@ inline OzRows oz_rows(const double* p, int nb, int rows, int rpad, long long ri,
 // y * bstep, (x, y) = pairs[p0 + p * pstep] (pairs null: (p, p)); its C starts at p * sc.
 struct OzArgs {
   OzRows a, b;
-  const int* aexp;  // row exponents by plane row (oz_pack)
+  const int* aexp;  // row scales and sums by plane row (oz_pack)
   const int* bexp;
   int* status;
   double* C;
@@ -74,19 +75,28 @@ struct OzArgs {
   int arow0, astep, brow0, bstep;
   double alpha;
   int accumulate;
+  void* mask;       // oz_mask_bytes(M, N, problems), 8-byte aligned: elements left to FP64 FMAs
   // filled by oz_multiply
   int mt, nt, band, kstages, n_items;
 };
 
 constexpr int OZ_ROW_PAD = 128;  // plane rows of a problem are a multiple, so that tiles start in it
 __host__ __device__ inline int oz_kpad(long long K) { return (int)((K + 31) / 32 * 32); }
+// Seven slices and the plane of leading digits for the check.
 inline size_t oz_plane_bytes(long long rows, long long K) {
-  return (size_t)OZ_S * rows * oz_kpad(K) * sizeof(__nv_bfloat16);
+  return (size_t)(OZ_S + 1) * rows * oz_kpad(K) * sizeof(__nv_bfloat16);
 }
-// Row exponents rexp[total] and slices (oz_plane_bytes(total, K); oz_off) of one operand,
-// total a multiple of OZ_ROW_PAD.
+// Per plane row: exponent of its scale, and the sum of its scaled magnitudes (2^-24 units).
+constexpr size_t OZ_ROW_INFO = sizeof(int) + sizeof(unsigned long long);
+// A bit per element of every 128 x 64 tile, and a byte per epilogue warp of the check.
+inline size_t oz_mask_bytes(long long M, long long N, long long problems) {
+  return (size_t)((M + 127) / 128) * ((N + 63) / 64) * problems * (128 * 8 + 8);
+}
+// Row scales and sums (OZ_ROW_INFO * total bytes at rexp) and slices (oz_plane_bytes(total,
+// K); oz_off) of one operand, total a multiple of OZ_ROW_PAD.
 cudaError_t oz_pack(cudaStream_t st, const OzRows& s, __nv_bfloat16* planes, int* rexp);
-// The product of two packed operands (a.a, a.b: their rows).
+// The product of two packed operands (a.a, a.b: their rows as packed; the FP64 values at
+// a.a.p and a.b.p are read again where the check finds the slices short of bits).
 cudaError_t oz_multiply(cudaStream_t st, const __nv_bfloat16* pa, const __nv_bfloat16* pb, OzArgs a,
                         int n_prob);
 

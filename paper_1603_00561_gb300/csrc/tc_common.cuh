@@ -162,6 +162,21 @@ __device__ __forceinline__ void tc_mma3_if(uint32_t leader, uint32_t d, uint32_t
 #undef DSRG_LL
 #undef DSRG_MMA3
 }
+// One MMA D (+)= A B by the leader lane of a whole converged warp.
+template <bool BF16>
+__device__ __forceinline__ void tc_mma_if(uint32_t leader, uint32_t d, uint32_t a, uint32_t b,
+                                          uint32_t idesc, uint32_t acc) {
+#define DSRG_MMA1(KIND)                                                                      \
+  asm volatile("{\n .reg .pred p, q;\n .reg .b64 x, y;\n"                                    \
+               " setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"                            \
+               " mov.b64 x, {%1, %6};\n mov.b64 y, {%2, %6};\n"                              \
+               " @q tcgen05.mma.cta_group::1.kind::" KIND " [%0], x, y, %3, p;\n}\n" ::"r"(d), \
+               "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(leader), "r"(DESC_SW64_HI)          \
+               : "memory")
+  if (BF16) DSRG_MMA1("f16");
+  else DSRG_MMA1("tf32");
+#undef DSRG_MMA1
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15},"
