@@ -23,7 +23,8 @@
 // different fragments). A chain of FP64 FMAs gives c within K 2^-53 2^{Ea+Eb} S, S = sum x y.
 // So every element is checked: an extra product of the leading eight bits of the magnitudes
 // gives S from below (oz_check_kernel), and elements with 8 K S < sum x + sum y + K / 50 are
-// formed by FP64 FMAs (oz_fma_kernel). S = 0 is exact (no K index has both factors). The bound is then no
+// formed by FP64 FMAs (oz_fma_kernel). So are those of rows with a NaN or an infinity, which
+// have no scale. S = 0 is exact (no K index has both factors). The bound is then no
 // larger than that of the FMA chain for any element of any input. On N(0, 1) e^{-0.02 Q}
 // factors no element fails the check, on the products of the Fock and DF steps 1e-3 and
 // fewer; with an unnormalised auxiliary basis (metric diagonal over 1e11) 9 in 10 of the
@@ -57,8 +58,8 @@ constexpr int OZ_A_SLICE = OZ_BM * 64, OZ_B_SLICE = OZ_BN * 64;
 constexpr int OZ_A_BYTES = OZ_S * OZ_A_SLICE, OZ_B_BYTES = OZ_S * OZ_B_SLICE;
 constexpr int OZ_STAGE_BYTES = OZ_A_BYTES + OZ_B_BYTES;
 constexpr int OZ_THREADS = 320, OZ_EPI_WARPS = 8;
-constexpr int OZ_EXP_INF = 0x7ff;             // "exponent" of a row with an infinity
-constexpr int OZ_EXP_NAN = 0x800;             // ... with a NaN
+constexpr int OZ_EXP_INF = 0x7ff;             // exponent field of a row with an infinity or a NaN
+constexpr unsigned long long OZ_SUM_INF = 1ull << 62;  // its sum (others: below 2^49)
 constexpr long long OZ_TINY = LLONG_MIN;      // a value that is not 0 but is as a fixed-point number
 
 // ------------------------------- row scales -------------------------------
@@ -80,7 +81,6 @@ __global__ void __launch_bounds__(256) oz_rowmax_kernel(OzRows s, int* __restric
     if (oz_row(s, r0 + rr, off) && l < K) {
       const double x = s.p[off + oz_k(s, l)];
       e = (__double2hiint(x) >> 20) & 0x7ff;
-      if (x != x) e = OZ_EXP_NAN;
     }
     if (KCONT) {
       for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) oz_rowmax_kernel(OzRows s, int* __restric
 __device__ __forceinline__ long long oz_fixed(double x, int rowexp) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(u >> 52) & 0x7ff;
-  if (rowexp >= OZ_EXP_INF || (u << 1) == 0) return 0;  // see the epilogue; zero
+  if (rowexp == OZ_EXP_INF || (u << 1) == 0) return 0;
   if (e == 0) return OZ_TINY;                           // below 2^-1022
   unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
   const int sh = rowexp - e - 2;  // right shift of the 53-bit significand
@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __re
   sum += __shfl_xor_sync(0xffffffffu, sum, 1);
   sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   if (!on) return;
+  if (l0 + c0 == 0 && rexp[r0 + rr] == OZ_EXP_INF) sum = OZ_SUM_INF;
   if ((threadIdx.x & 3) == 0 && sum) atomicAdd(&rsum[r0 + rr], sum);
   {
     uint8_t* o = (uint8_t*)planes + (size_t)OZ_S * s.total * Kp * sizeof(__nv_bfloat16);
@@ -402,17 +403,6 @@ __device__ __forceinline__ uint8_t* oz_mask_any(const OzArgs& a, int it) {
   return (uint8_t*)a.mask + (size_t)a.n_items * 1024 + (size_t)it * 8;
 }
 
-// An element whose row of A or B is not finite.
-static __device__ __noinline__ double oz_not_finite(const OzArgs& a, int ra, int rb, int e) {
-  if (e >= OZ_EXP_NAN) return __longlong_as_double(0x7ff8000000000000ll);
-  long long oa, ob;
-  oz_row(a.a, ra, oa);
-  oz_row(a.b, rb, ob);
-  double d = 0.0;
-  for (int l = 0; l < a.a.L1 * a.a.L2; ++l) d = fma(a.a.p[oa + oz_k(a.a, l)], a.b.p[ob + oz_k(a.b, l)], d);
-  return d;
-}
-
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm_kernel(const uint8_t* __restrict__ pa, const uint8_t* __restrict__ pb,
                    const __grid_constant__ OzArgs a) {
@@ -606,9 +596,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             const int rb = t.brow + ch * 32 + c, eb = a.bexp[rb];
             const int e = ea + eb - 2 * 1022 - 38;
             const int hw = __double2hiint(d), ef = (hw >> 20) & 0x7ff;
-            if (max(ea, eb) >= OZ_EXP_INF) {
-              d = oz_not_finite(a, ra, rb, max(ea, eb));
-            } else if (ef != 0) {
+            if (ef != 0) {
               if (ef + e > 0 && ef + e < 0x7ff)
                 d = __hiloint2double(hw + (e << 20), __double2loint(d));
               else
@@ -804,7 +792,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           const int j = ch * 32 + c;
           if (t.j0 + j < a.N) {
             const float S = __uint_as_float(r[c >> 4][c & 15]);
-            if (S > 0.0f && K8 * S < sa + (float)bsum[t.brow + j] * 0x1p-24f) word |= 1u << c;
+            const float sums = sa + (float)bsum[t.brow + j] * 0x1p-24f;
+            if ((S > 0.0f && K8 * S < sums) || sums > (float)(OZ_SUM_INF >> 25)) word |= 1u << c;
           }
         }
       }

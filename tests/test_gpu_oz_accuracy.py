@@ -217,3 +217,43 @@ def test_digits_at_the_most_negative(pk):
         D = eC[0] + eC[1] - eV[:, None] - eV[None, :]
         ref = np.sum(w * w * -np.expm1(-np.longdouble(1.0) * D * D) / D)
         assert abs(e[0, 1] / ref - 1) <= 16 * 2.0 ** -52
+
+
+def test_infinite_rows_of_a_long_product(pk):
+    """A row with an infinity (or a NaN) goes through FP64 FMAs element by element; of the
+    exchange product's 31 000-long sums that is no reason to run into the bound of the
+    kernels' waits. Rows and columns of the other orbitals are not touched."""
+    import time
+    import torch
+    nC, nA, nV, Q = 24, 2, 130, 1200
+    n = nC + nA + nV
+    r = np.random.default_rng(9)
+    B = torch.as_tensor(r.standard_normal((Q, n, n)) * np.exp(-0.02 * np.arange(Q))[:, None, None]).cuda()
+    B = 0.5 * (B + B.transpose(1, 2)).contiguous()
+    h, G = _dev(np.zeros((n, n))), _dev(np.diag([1.25, 0.75]))
+    sc = pk.SemicanonicalPlan(nC, nA, nV, Q)
+    good = sc.fock(h, B, G).clone()
+    hit = [40, 41, 100]
+    B[7, 30, hit] = float("inf")  # orbital 30 is virtual: only f[30, :] and f[:, hit] ...
+    B[7, hit, 30] = float("inf")
+    B[9, 50, 60] = float("nan")
+    B[9, 60, 50] = float("nan")
+    torch.cuda.synchronize()
+    f = sc.fock(h, B, G)
+    # J reads every pair: the pairs' own elements; K only hole columns, which are finite
+    fine = torch.ones((n, n), dtype=torch.bool, device="cuda")
+    for a, b in [(30, k) for k in hit] + [(50, 60)]:
+        fine[a, b] = fine[b, a] = False
+    assert not torch.isfinite(f[~fine]).any()
+    assert torch.equal(f[fine], good[fine])
+    # an infinity in a hole column: the whole row and column of that orbital, in K
+    B[7, 3, 77] = B[7, 77, 3] = float("inf")
+    torch.cuda.synchronize()
+    t0 = time.time()
+    f = sc.fock(h, B, G)
+    torch.cuda.synchronize()
+    assert time.time() - t0 < 1.0
+    fine[77, :] = fine[:, 77] = False
+    fine[3, :] = fine[:, 3] = False
+    assert not torch.isfinite(f[77]).any()
+    assert torch.equal(f[fine], good[fine])
