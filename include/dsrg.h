@@ -393,7 +393,9 @@ typedef struct dsrg_sc_plan dsrg_sc_plan_t;
 /* sz->ncore, nactive, nvirt >= 0 (n >= 1), naux >= 1, nactive <= 8. */
 dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t **plan, const dsrg_sizes_t *sz, void *cuda_stream);
 dsrg_status_t dsrg_sc_plan_destroy(dsrg_sc_plan_t *plan);
-/* f_dev [n][n]: the generalized Fock matrix (asynchronous, on the plan's stream). */
+/* f_dev [n][n]: the generalized Fock matrix (asynchronous, on the plan's stream). If a
+ * bounded wait of its product on the tensor cores runs out, f_dev is all NaN, and the next
+ * dsrg_sc_sync or dsrg_semicanonicalize returns DSRG_ERR_TIMEOUT. */
 dsrg_status_t dsrg_generalized_fock(dsrg_sc_plan_t *plan, const double *h, const double *Bfull,
                                     const double *gamma1, double *f_dev);
 dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t *plan, const double *h, const double *Bfull,
@@ -401,6 +403,12 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t *plan, const double *h, const
                                     const double *lambda3, double *eps_out, double *B_out,
                                     double *f1_out, double *gamma1_out, double *lambda2_out,
                                     double *lambda3_out, double *U_out);
+/* Wait for the plan's stream and report a device-side wait that ran out since the last
+ * report (DSRG_ERR_TIMEOUT), then clear it. */
+dsrg_status_t dsrg_sc_sync(dsrg_sc_plan_t *plan);
+/* Self-test of that path, as dsrg_plan_selftest_wait_timeout: queues a wait on the plan's
+ * stream that runs out after about 2 s. */
+dsrg_status_t dsrg_sc_selftest_wait_timeout(dsrg_sc_plan_t *plan);
 /* Jacobi sweeps of the slowest-converging block in the last call. */
 int32_t dsrg_sc_last_sweeps(const dsrg_sc_plan_t *plan);
 const char *dsrg_sc_last_error(const dsrg_sc_plan_t *plan);

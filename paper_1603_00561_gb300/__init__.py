@@ -373,6 +373,10 @@ class SemicanonicalPlan:
         self._check(st, "dsrg_semicanonicalize")
         return out
 
+    def sync(self):
+        """Wait for the plan's stream; raises if a device-side wait ran out (``dsrg_sc_sync``)."""
+        self._check(self.lib.dsrg_sc_sync(self.h), "dsrg_sc_sync")
+
     def last_sweeps(self) -> int:
         return int(self.lib.dsrg_sc_last_sweeps(self.h))
 

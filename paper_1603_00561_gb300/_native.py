@@ -28,7 +28,8 @@ EXPORTS = [
     "dsrg_plan_time_ccvv", "dsrg_plan_set_item_order", "dsrg_batch_set_item_order",
     "dsrg_plan_selftest_wait_timeout", "dsrg_plan_branch_counts", "dsrg_mrpt2_energy_ext",
     "dsrg_mrpt2_energy_grad_ext", "dsrg_sc_plan_create", "dsrg_sc_plan_destroy", "dsrg_generalized_fock",
-    "dsrg_semicanonicalize", "dsrg_sc_last_sweeps", "dsrg_sc_last_error",
+    "dsrg_semicanonicalize", "dsrg_sc_sync", "dsrg_sc_selftest_wait_timeout",
+    "dsrg_sc_last_sweeps", "dsrg_sc_last_error",
     "dsrg_df_mo_transform_work_bytes", "dsrg_df_mo_transform", "dsrg_cd_factors_work_bytes",
     "dsrg_cd_factors", "dsrg_plan_set_shard", "dsrg_shard_pairs", "dsrg_batch_branches",
     "dsrg_batch_set_branches", "dsrg_batch_autotune_branches", "dsrg_tune_cache_get",
@@ -88,6 +89,10 @@ def load(path: str = LIB_PATH) -> C.CDLL:
     lib.dsrg_generalized_fock.restype = st
     lib.dsrg_semicanonicalize.argtypes = [vp] + [vp] * 12
     lib.dsrg_semicanonicalize.restype = st
+    lib.dsrg_sc_sync.argtypes = [vp]
+    lib.dsrg_sc_sync.restype = st
+    lib.dsrg_sc_selftest_wait_timeout.argtypes = [vp]
+    lib.dsrg_sc_selftest_wait_timeout.restype = st
     lib.dsrg_sc_last_sweeps.argtypes = [vp]
     lib.dsrg_sc_last_sweeps.restype = C.c_int32
     i32 = C.c_int32

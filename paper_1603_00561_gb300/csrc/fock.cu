@@ -22,6 +22,7 @@
 //   on every active index.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -34,7 +35,9 @@ namespace dsrg {
 struct JacState {
   GridBar bar;
   int sweeps;  // of the slowest block so far
-  int wait;    // status word of the products' bounded waits
+  // status word of the products' bounded waits: kept until a call reports it (the Fock
+  // build alone is asynchronous and cannot)
+  int wait;
 };
 }  // namespace dsrg
 
@@ -131,10 +134,11 @@ __global__ void fock_x_kernel(const double* __restrict__ B, const double* __rest
   X[k] = v;
 }
 
-// f = h + J - K / 2 (K in nk parts), symmetrised (the two halves round differently only in K)
+// f = h + J - K / 2 (K in nk parts), symmetrised (the two halves round differently only in
+// K); NaN if a wait of the product that forms K ran out (its tiles are then not written)
 __global__ void fock_sum_kernel(const double* __restrict__ h, const double* __restrict__ J,
                                 const double* __restrict__ K, int nk, int n,
-                                double* __restrict__ f) {
+                                const int* __restrict__ wait, double* __restrict__ f) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nn = (size_t)n * n;
   if (k >= nn) return;
   const int p = (int)(k / n), q = (int)(k % n);
@@ -146,7 +150,7 @@ __global__ void fock_sum_kernel(const double* __restrict__ h, const double* __re
   }
   const double a = fma(-0.5, ka, h[k] + J[k]);
   const double b = fma(-0.5, kb, h[kt] + J[kt]);
-  f[k] = 0.5 * (a + b);
+  f[k] = *wait ? __longlong_as_double(0x7ff8000000000000ll) : 0.5 * (a + b);
 }
 
 // ---------------------------- Jacobi eigensolver ----------------------------
@@ -434,6 +438,22 @@ cudaError_t sc_check(dsrg_sc_plan* p) {
   return e;
 }
 
+// Waits for the plan's stream, reads its words and reports a wait that ran out since the
+// last report (the barrier's word is that of the last semicanonicalisation alone).
+dsrg_status_t sc_wait(dsrg_sc_plan* p, JacState* js) {
+  cudaStream_t st = p->stream;
+  if (cudaMemcpyAsync(js, p->jac, sizeof(*js), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return DSRG_ERR_CUDA;
+  if (!js->bar.abort && !js->wait) return DSRG_OK;
+  p->last_error = "a device-side wait ran out";
+  if (cudaMemsetAsync(&p->jac->bar.abort, 0, sizeof(int), st) != cudaSuccess ||
+      cudaMemsetAsync(&p->jac->wait, 0, sizeof(int), st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return DSRG_ERR_CUDA;
+  return DSRG_ERR_TIMEOUT;
+}
+
 // Diagonalise the block [lo, lo + m) of f (symmetric); writes U and eps there.
 cudaError_t jacobi_block(dsrg_sc_plan* p, int lo, int m, double* eps) {
   if (m == 0) return cudaSuccess;
@@ -482,7 +502,7 @@ cudaError_t build_fock(dsrg_sc_plan* p, const double* h, const double* B, const 
   if (rest && (e = launch_gemm(st, part(full * qc, rest, p->K + (size_t)full * nn), p->oz)) != cudaSuccess)
     return e;
   fock_sum_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(h, p->J, p->K, full + (rest ? 1 : 0), z.n,
-                                                               p->f);
+                                                               &p->jac->wait, p->f);
   return sc_check(p);
 }
 
@@ -597,7 +617,7 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
   cudaStream_t st = p->stream;
   const size_t nn = (size_t)z.n * z.n;
   p->sweeps_last = 0;
-  if (cudaMemsetAsync(p->jac, 0, sizeof(JacState), st) != cudaSuccess) return DSRG_ERR_CUDA;
+  if (cudaMemsetAsync(p->jac, 0, offsetof(JacState, wait), st) != cudaSuccess) return DSRG_ERR_CUDA;
   if (build_fock(p, h, Bfull, gamma1) != cudaSuccess) return DSRG_ERR_CUDA;
   if (cudaMemsetAsync(p->U, 0, nn * 8, st) != cudaSuccess) return DSRG_ERR_CUDA;
   if (jacobi_block(p, 0, z.nC, eps_out) != cudaSuccess ||
@@ -649,15 +669,20 @@ dsrg_status_t dsrg_semicanonicalize(dsrg_sc_plan_t* p, const double* h, const do
   if (U_out && cudaMemcpyAsync(U_out, p->U, nn * 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return DSRG_ERR_CUDA;
   JacState js{};
-  if (cudaMemcpyAsync(&js, p->jac, sizeof(js), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return DSRG_ERR_CUDA;
+  const dsrg_status_t status = sc_wait(p, &js);
   p->sweeps_last = js.sweeps;
-  if (js.bar.abort || js.wait) {
-    p->last_error = "a device-side wait ran out";
-    return DSRG_ERR_TIMEOUT;
-  }
-  return DSRG_OK;
+  return status;
+}
+
+dsrg_status_t dsrg_sc_sync(dsrg_sc_plan_t* p) {
+  if (!p) return DSRG_ERR_INVALID_ARG;
+  JacState js{};
+  return sc_wait(p, &js);
+}
+
+dsrg_status_t dsrg_sc_selftest_wait_timeout(dsrg_sc_plan_t* p) {
+  if (!p) return DSRG_ERR_INVALID_ARG;
+  return launch_wait_selftest(p->stream, &p->jac->wait) == cudaSuccess ? DSRG_OK : DSRG_ERR_CUDA;
 }
 
 }  // extern "C"

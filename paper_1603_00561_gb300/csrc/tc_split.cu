@@ -1425,10 +1425,9 @@ __global__ void wait_selftest_kernel(int* status) {
   if (threadIdx.x == 0) (void)mbar_wait(&bar, 0u, (volatile int*)&abort_flag, status);
 }
 
-cudaError_t launch_wait_selftest(dsrg_plan* p) {
-  wait_selftest_kernel<<<1, 32, 0, p->stream>>>(p->d_status);
-  DSRG_LAUNCH_CHECK(p);
-  return cudaSuccess;
+cudaError_t launch_wait_selftest(cudaStream_t st, int* status) {
+  wait_selftest_kernel<<<1, 32, 0, st>>>(status);
+  return cudaGetLastError();
 }
 
 size_t split_mol_desc_bytes() { return sizeof(MolDesc); }
