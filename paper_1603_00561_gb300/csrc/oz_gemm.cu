@@ -129,8 +129,8 @@ __device__ __forceinline__ size_t oz_check_off(int row, int l, int nkb) {
 }
 
 // 64 rows x 64 K values per CTA through shared memory. The check plane (after the slices)
-// holds the leading eight bits of |x| / 2^E, 2^-60 for OZ_TINY; rsum its sum over the row in
-// 2^-24 units, rounded up (integers: the order of the atomics does not matter).
+// holds the leading eight bits of |x| / 2^E (2^-60 where they are all 0, but x is not); rsum
+// the sum of |x| / 2^E over the row in 2^-24 units, rounded up (integers: the order of the atomics does not matter).
 template <bool KCONT>
 __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __restrict__ rexp,
                                                        unsigned long long* __restrict__ rsum,
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __re
   const bool on = r0 + rr < s.total && l0 + c0 < Kp;
   const int nkb = Kp / OZ_KB;
   long long v[16];
-  unsigned long long sum = 0;
+  uint32_t sum = 0;  // below 2^29
   uint32_t cw[8];
 #pragma unroll
   for (int k = 0; k < 16; k += 2) {
@@ -159,18 +159,20 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzRows s, const int* __re
     for (int i = 0; i < 2; ++i) {
       const long long w = t[rr][c0 + k + i];
       v[k + i] = w == OZ_TINY ? 0 : w;
-      const unsigned long long m = (unsigned long long)llabs(v[k + i]);
-      sum += (m >> 31) + (w != 0);
-      x[i] = w == OZ_TINY ? 0x1p-60f : __ull2float_rz(m) * 0x1p-55f;
+      // |x| in 2^-24 units, rounded down (by up to 2 units): the complement of a negative
+      const int hi = (int)(v[k + i] >> 31), m = hi ^ (hi >> 31);
+      sum += m + (w != 0);
+      x[i] = w == 0 ? 0.0f : fmaxf((float)m * 0x1p-24f, 0x1p-60f);
     }
-    const __nv_bfloat162 h = __halves2bfloat162(__float2bfloat16_rz(x[0]), __float2bfloat16_rz(x[1]));
-    cw[k / 2] = *(const uint32_t*)&h;
+    cw[k / 2] = __byte_perm(__float_as_uint(x[0]), __float_as_uint(x[1]), 0x7632);  // upper halves
   }
   sum += __shfl_xor_sync(0xffffffffu, sum, 1);
   sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   if (!on) return;
-  if (l0 + c0 == 0 && rexp[r0 + rr] == OZ_EXP_INF) sum = OZ_SUM_INF;
-  if ((threadIdx.x & 3) == 0 && sum) atomicAdd(&rsum[r0 + rr], sum);
+  if ((threadIdx.x & 3) == 0) {
+    const bool inf = l0 == 0 && rexp[r0 + rr] == OZ_EXP_INF;
+    if (inf || sum) atomicAdd(&rsum[r0 + rr], inf ? OZ_SUM_INF : (unsigned long long)sum);
+  }
   {
     uint8_t* o = (uint8_t*)planes + (size_t)OZ_S * s.total * Kp * sizeof(__nv_bfloat16);
     *(uint4*)(o + oz_check_off(r0 + rr, l0 + c0, nkb)) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
