@@ -321,9 +321,18 @@ __global__ void __launch_bounds__(JT * JT) jac_run_kernel(double* __restrict__ A
   if (blockIdx.x == 0 && tid == 0) st->sweeps = max(st->sweeps, sweep);
 }
 
+// Whether eigenvalue x of index i comes before dc of index c: ascending, a NaN above every
+// number, equal values and NaNs by index. A total order: the places of m eigenvalues are a
+// permutation whatever they are, so that every column is written, by one CTA.
+__device__ __forceinline__ bool jac_before(double x, int i, double dc, int c) {
+  const bool xn = isnan(x), cn = isnan(dc);
+  if (xn || cn) return xn == cn ? i < c : cn;
+  return x < dc || (x == dc && i < c);
+}
+
 // U block and eps from the eigenvalues diag and V, one CTA per column: column c of V
-// becomes column lo + rank of U, rank = its place in ascending order (equal values in
-// index order), with its largest-magnitude component made positive (first one on ties).
+// becomes column lo + rank of U, rank = its place in ascending order (jac_before),
+// with its largest-magnitude component made positive (first one on ties).
 __global__ void __launch_bounds__(128) jac_store_kernel(const double* __restrict__ diag,
                                                         const double* __restrict__ V, int m, int n,
                                                         int lo, double* __restrict__ U,
@@ -338,8 +347,7 @@ __global__ void __launch_bounds__(128) jac_store_kernel(const double* __restrict
   int below = 0, imax = 0;
   double vmax = -1.0;
   for (int i = tid; i < m; i += 128) {
-    const double x = diag[i];
-    below += x < dc || (x == dc && i < c);
+    below += jac_before(diag[i], i, dc, c);
     const double a = fabs(V[(size_t)i * m + c]);
     if (a > vmax) {
       vmax = a;
