@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(JT * JT) jac_run_kernel(double* __restrict__ A
     }
     const double off = sh0[0], all = sh1[0];
     __syncthreads();
-    if (off <= 1e-30 * all || off == 0.0 || sweep >= max_sweeps) break;
+    // (an infinite norm is no convergence)
+    if ((off <= 1e-30 * all && all < INFINITY) || off == 0.0 || sweep >= max_sweeps) break;
     for (int t = 0; t < mp - 1; ++t) {
       for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
         const int tp = tile / nt, tr = tile % nt;

@@ -47,7 +47,7 @@ def test_a_wait_that_ran_out_is_reported(pk):
     sc.close()
 
 
-@pytest.mark.parametrize("block,bad", [("virtual", "nan"), ("core", "nan"), ("all", "nan")])
+@pytest.mark.parametrize("block,bad", [("virtual", "nan"), ("virtual", "inf"), ("core", "nan"), ("all", "nan")])
 def test_a_fock_matrix_that_is_not_finite(pk, block, bad):
     """Every output is written: the block's orbital energies and columns of U are not finite, those
     of the other blocks are what they are without it."""
