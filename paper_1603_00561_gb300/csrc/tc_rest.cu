@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 
 #include "ff.cuh"
+#include "index.cuh"
 #include "internal.cuh"
 #include "regulators.cuh"
 #include "tc_common.cuh"
@@ -889,9 +890,9 @@ __global__ void act_gather_kernel(const float* __restrict__ Y, long long ldy, in
     K3[r] = Gxx[r];
   } else if (k < 2 * n12 + n3 + nm) {
     const size_t r = k - 2 * n12 - n3;
-    const size_t xu = r / ((size_t)z.nV * z.nV);
-    const unsigned ef = (unsigned)(r - xu * z.nV * z.nV);
-    const int f = (int)(ef % z.nV), e = (int)(ef / z.nV), u = (int)xu % nA, x = (int)xu / nA;
+    int xu, e, f;
+    split_xu_ef(r, z.nV, xu, e, f);
+    const int u = xu % nA, x = xu / nA;
     M[r] = (double)Y[(size_t)((nC + x) * nVpad + e) * ldy + (size_t)u * nVpad + f];
   }
 }
