@@ -315,6 +315,7 @@ constexpr size_t V_BYTES = (size_t)96 << 20;
 // CUDA-core kernels, which need none (they run for hours there, but they run).
 bool fp64_tc_alloc(dsrg_plan* p) {
   const Sizes& z = p->z;
+  if (z.Q > OZ_MAX_K) return true;
   {
     const double nvp = (z.nV + OZ_ROW_PAD - 1) / OZ_ROW_PAD * (double)OZ_ROW_PAD;
     const double rows = z.nH * nvp + z.nH * z.nA + OZ_ROW_PAD;

@@ -980,7 +980,7 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
   }
   const long long K = (long long)g.L1 * g.L2;
   const double flops = 2.0 * g.M * g.N * (double)K * g.nb;
-  if (!w.mem || !oz_worthwhile(flops) || K > (1 << 21)) return launch_gemm_fp64(st, g0);
+  if (!w.mem || !oz_worthwhile(flops) || K > OZ_MAX_K) return launch_gemm_fp64(st, g0);
   // the operand on the 128-row side: the one that wastes less of the tiles
   auto tiles = [](long long m, long long n) {
     return oz_up(m, OZ_BM) * oz_up(n, OZ_BN);

@@ -80,6 +80,7 @@ struct OzArgs {
   int mt, nt, band, kstages, n_items;
 };
 
+constexpr long long OZ_MAX_K = 1ll << 21;  // limit of oz_pack's grid and of the integer sums' headroom
 constexpr int OZ_ROW_PAD = 128;  // plane rows of a problem are a multiple, so that tiles start in it
 __host__ __device__ inline int oz_kpad(long long K) { return (int)((K + 31) / 32 * 32); }
 // Seven slices and the plane of leading digits for the check.
