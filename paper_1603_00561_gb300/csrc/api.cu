@@ -33,6 +33,14 @@ bool plan_alloc(dsrg_plan* p, void** ptr, size_t bytes) {
   return true;
 }
 
+void plan_release(dsrg_plan* p, size_t n_allocs, size_t ws_bytes) {
+  while (p->allocs.size() > n_allocs) {
+    cudaFree(p->allocs.back());
+    p->allocs.pop_back();
+  }
+  p->ws_bytes = ws_bytes;
+}
+
 cudaError_t raise_smem_limit(const void* func, size_t bytes) {
   static std::mutex mu;
   static std::map<std::pair<const void*, int>, size_t> cur;
@@ -239,7 +247,6 @@ dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precis
   if (ok && prec != DSRG_PREC_FP64)
     ok = share ? split_alloc_at(p, share->hi, share->lo, share->Qld, share->row_base, nullptr, nullptr)
                : split_alloc(p);
-  if (ok && prec == DSRG_PREC_FP64) ok = fp64_tc_alloc(p);
   if (ok && p->rest_tc) ok = rest_alloc(p, share ? share->y : nullptr);
   if (ok && (flags & DSRG_PLAN_GRAD)) ok = grad_alloc(p);
   if (ok && !share) ok = plan_fork_alloc(p);
@@ -272,6 +279,11 @@ dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precis
     free_all(p);
     delete p;
     return DSRG_ERR_OOM;
+  }
+  // what the plan can do without comes last
+  if (prec == DSRG_PREC_FP64) {
+    fp64_tc_alloc(p);
+    grad_alloc_products(p);
   }
   cudaError_t e = cudaSuccess;
   e = cudaMemcpy(p->d_pairs, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice);

@@ -14,6 +14,8 @@
 // regulators 1.4) and 0.35 ms, and 0.64 ms for the product of the rest. Regulators beside
 // the next group's product would need registers that its kernel leaves no room for.
 // The regulators are what is left on that pipe: about 25 FP64 instructions each.
+#include <new>
+
 #include "internal.cuh"
 #include "oz_gemm.cuh"
 #include "regulators.cuh"
@@ -310,25 +312,24 @@ __global__ void gather_y_fp64_kernel(const double* __restrict__ Y, long long ldy
 // product just wrote from it.
 constexpr size_t V_BYTES = (size_t)96 << 20;
 
-// The slices and the check plane take 16 bytes per value of B and Y one FP64 per (hole, virtual) and active
-// pair: sizes whose workspace would be over 2/5 of the device's memory stay with the
-// CUDA-core kernels, which need none (they run for hours there, but they run).
-bool fp64_tc_alloc(dsrg_plan* p) {
+// The slices and the check plane take 16 bytes per value of B, Y one FP64 per (hole,
+// virtual) and active pair, the pair buffer at least one pair's integrals. A plan takes them
+// only where they are at most 2/5 of the memory free at its creation, and can be had: others
+// run on the CUDA-core kernels, which need none of it (they run for hours there, but they run).
+void fp64_tc_alloc(dsrg_plan* p) {
   const Sizes& z = p->z;
-  if (z.Q > OZ_MAX_K) return true;
-  {
-    const double nvp = (z.nV + OZ_ROW_PAD - 1) / OZ_ROW_PAD * (double)OZ_ROW_PAD;
-    const double rows = z.nH * nvp + z.nH * z.nA + OZ_ROW_PAD;
-    const double bytes = rows * (16.0 * oz_kpad(z.Q) + 8.0 * (z.nA * nvp + z.nH * z.nA));
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-    if (bytes > 0.4 * (double)total_b || rows > 2.0e9) return true;
-  }
-  Fp64Tc* w = new Fp64Tc();
-  p->f64 = w;
-  w->nVpad = (z.nV + OZ_ROW_PAD - 1) / OZ_ROW_PAD * OZ_ROW_PAD;
+  if (z.Q > OZ_MAX_K) return;
+  const long long nVpad = (z.nV + OZ_ROW_PAD - 1ll) / OZ_ROW_PAD * OZ_ROW_PAD;
+  const long long XR = (z.nH * z.nA + OZ_ROW_PAD - 1ll) / OZ_ROW_PAD * OZ_ROW_PAD;
+  const long long rows = z.nH * nVpad + XR;
+  const size_t per = (size_t)z.nV * z.nV * sizeof(double);
+  size_t free_b = 0, total_b = 0;
+  if (rows > 2000000000ll || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
+  Fp64Tc* w = new (std::nothrow) Fp64Tc();
+  if (!w) return;
+  w->nVpad = (int)nVpad;
   w->xrow0 = z.nH * w->nVpad;
-  w->XR = (z.nH * z.nA + OZ_ROW_PAD - 1) / OZ_ROW_PAD * OZ_ROW_PAD;
+  w->XR = (int)XR;
   OzRows& r = w->rows;
   // B[(q nH + h) nP + a], rows (h, nA + e) and then (h, x)
   r = oz_rows(nullptr, z.nH, z.nV, w->nVpad, 1, z.nP, 1, z.Q, 0, (long long)z.nH * z.nP);
@@ -341,17 +342,23 @@ bool fp64_tc_alloc(dsrg_plan* p) {
   r.xri = 1;
   w->xc = (long long)z.nA * w->nVpad;
   w->ldy = w->xc + (z.nH * z.nA + 7) / 8 * 8;
-  const size_t per = (size_t)z.nV * z.nV * sizeof(double);
   const size_t fit = V_BYTES / per;
   w->group = (int)(fit < 1 ? 1 : (fit > (size_t)p->n_pairs ? (size_t)p->n_pairs : fit));
   const size_t mask_v = oz_mask_bytes(z.nV, z.nV, w->group);
   const size_t mask_y = oz_mask_bytes(w->xrow0 + z.nH * z.nA, w->xc + z.nH * z.nA, 1);
-  return plan_alloc(p, (void**)&w->planes, oz_plane_bytes(r.total, z.Q)) &&
-         plan_alloc(p, (void**)&w->rexp, (size_t)r.total * OZ_ROW_INFO) &&
-         plan_alloc(p, &w->mask, mask_v > mask_y ? mask_v : mask_y) &&
-         plan_alloc(p, (void**)&w->V, per * w->group) &&
-         (z.nA == 0 ||
-          plan_alloc(p, (void**)&w->Y, (size_t)(w->xrow0 + z.nH * z.nA) * w->ldy * sizeof(double)));
+  const size_t mask = mask_v > mask_y ? mask_v : mask_y;
+  const size_t y = z.nA == 0 ? 0 : (size_t)(w->xrow0 + z.nH * z.nA) * w->ldy * sizeof(double);
+  const size_t need = oz_plane_bytes(r.total, z.Q) + (size_t)r.total * OZ_ROW_INFO + mask + per * w->group + y;
+  const size_t n_allocs = p->allocs.size(), ws = p->ws_bytes;
+  if ((double)need <= 0.4 * (double)free_b &&
+      plan_alloc(p, (void**)&w->planes, oz_plane_bytes(r.total, z.Q)) &&
+      plan_alloc(p, (void**)&w->rexp, (size_t)r.total * OZ_ROW_INFO) && plan_alloc(p, &w->mask, mask) &&
+      plan_alloc(p, (void**)&w->V, per * w->group) && (y == 0 || plan_alloc(p, (void**)&w->Y, y))) {
+    p->f64 = w;
+    return;
+  }
+  plan_release(p, n_allocs, ws);
+  delete w;
 }
 
 void fp64_tc_free(dsrg_plan* p) {

@@ -1324,10 +1324,6 @@ bool grad_alloc(dsrg_plan* p) {
     const size_t kmax = ((size_t)2 << 30) / per_w;
     g->kgroup = (int)(kmax < 1 ? 1 : (kmax > (size_t)z.nC ? (size_t)z.nC : kmax));
     ok = plan_alloc(p, (void**)&g->Wk, per_w * g->kgroup);
-    // the largest product: dB of a group of rows from W
-    g->oz.bytes = oz_work_bytes(z.Q, z.nV, (long long)z.nC * z.nV, g->kgroup, true, false);
-    ok = ok && plan_alloc(p, &g->oz.mem, g->oz.bytes);
-    g->oz.status = p->d_status;
   } else {
     // split plans: S and B^T planes of the tensor-core assembly (tc_adjoint.cu)
     ok = tc_adj_alloc(p);
@@ -1351,6 +1347,20 @@ bool grad_alloc(dsrg_plan* p) {
          plan_alloc(p, (void**)&g->dM, (size_t)z.nA * z.nA * z.nV * z.nV * 8);
   }
   return ok;
+}
+
+// Workspace of the largest product, dB of a group of rows from W; without it the products
+// are FP64 FMAs.
+void grad_alloc_products(dsrg_plan* p) {
+  GradWs* g = p->grad;
+  if (!g) return;
+  const Sizes& z = p->z;
+  const size_t bytes = oz_work_bytes(z.Q, z.nV, (long long)z.nC * z.nV, g->kgroup, true, false);
+  size_t free_b = 0, total_b = 0;
+  g->oz.status = p->d_status;
+  if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && (double)bytes <= 0.4 * (double)free_b &&
+      plan_alloc(p, &g->oz.mem, bytes))
+    g->oz.bytes = bytes;
 }
 
 void grad_free(dsrg_plan* p) {

@@ -133,6 +133,8 @@ namespace dsrg {
 
 // Allocation helper: records the pointer in the plan; returns false on failure.
 bool plan_alloc(dsrg_plan* p, void** ptr, size_t bytes);
+// Back to the first n_allocs allocations (ws_bytes: what the plan owned then).
+void plan_release(dsrg_plan* p, size_t n_allocs, size_t ws_bytes);
 
 // Raise (never lower) a kernel's dynamic shared-memory limit on the current
 // device. A launch captured in a CUDA graph keeps its own size; lowering the
@@ -147,8 +149,8 @@ inline cudaStream_t side_stream(const dsrg_plan* p) { return p->forked ? p->call
 
 // Launchers (each returns cudaSuccess or the launch error; adds to p->launches).
 // FP64 plans: tensor-core products (fp64_tc.cu) when their workspace is a small enough
-// part of the device's memory (then p->f64 is set), else the CUDA-core kernels.
-bool fp64_tc_alloc(dsrg_plan* p);
+// part of the free memory and can be had (then p->f64 is set), else the CUDA-core kernels.
+void fp64_tc_alloc(dsrg_plan* p);
 void fp64_tc_free(dsrg_plan* p);
 cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps, double s);
 cudaError_t launch_rest_fp64_tc(dsrg_plan* p, const double* B, const double* eps, const double* G,
@@ -298,6 +300,7 @@ std::string tune_size_class(const Sizes& z, int kblocks, int world);
 
 // Gradient (grad.cu).
 bool grad_alloc(dsrg_plan* p);
+void grad_alloc_products(dsrg_plan* p);  // FP64 plans: the digits' workspace, if it can be had
 void grad_free(dsrg_plan* p);
 cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const double* G,
                         const double* L, const double* L3, const double* F1, double s, double* dB,

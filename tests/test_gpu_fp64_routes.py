@@ -35,3 +35,67 @@ def test_very_long_auxiliary_basis(pk, naux):
     v = float((B * B).sum())
     ref = v * v * -np.expm1(-9.0) / -3.0
     assert abs(e[4] / ref - 1.0) <= 1e-10
+
+
+def _gradient_errors(plan, pk, p):
+    l3, f1 = pk.extra_to_device(p)
+    out, dB, de, ds = plan.energy_grad(*pk.to_device(p), p.s, lambda3=l3, f1=f1)
+    plan.sync()
+    ref = odsrg.energy_and_grad(p.B, p.eps, p.gamma1, p.lambda2, p.s, p.ncore, p.nactive, p.nvirt,
+                                lambda3=p.lambda3, f1=p.f1)
+    worst = abs(float(out[4].cpu()) / ref["total"] - 1.0)
+    for got, want in ((dB, ref["dB"]), (de, ref["deps"]), (ds, np.asarray([ref["ds"]]))):
+        worst = max(worst, np.abs(got.cpu().numpy() - want).max() / np.abs(want).max())
+    return worst
+
+
+def test_workspace_that_cannot_be_allocated(pk, monkeypatch):
+    """Only what the CUDA-core kernels need as well may make a plan fail: where the digits'
+    workspace cannot be had, the plan runs without it."""
+    from paper_1603_00561_gb300 import _native
+    sizes = (6, 2, 70, 40)
+    p = make_problem(*sizes, s=0.5, seed=5)
+    full = pk.Plan(*sizes, precision="fp64", grad=True)
+    assert _gradient_errors(full, pk, p) <= 1e-10
+    made, smallest = 0, None
+    for k in range(80):
+        monkeypatch.setenv("DSRG_FAIL_ALLOC_AFTER", str(k))
+        try:
+            plan = pk.Plan(*sizes, precision="fp64", grad=True)
+        except pk.DSRGError as e:
+            assert e.status == _native.ERR_OOM and made == 0
+            continue
+        made += 1
+        smallest = plan.workspace_bytes() if smallest is None else smallest
+        assert _gradient_errors(plan, pk, p) <= 1e-10
+        if plan.workspace_bytes() == full.workspace_bytes():
+            break
+    assert made > 1 and smallest < full.workspace_bytes()
+
+
+def _leave_free(torch, nbytes):
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+
+
+def test_little_free_memory(pk):
+    """A plan on a GPU that others have filled takes at most 2/5 of what is left, or does without."""
+    import torch
+    sizes = (8, 2, 600, 2400)
+    p = make_problem(*sizes, s=0.5, seed=6)
+    dev = pk.to_device(p)
+    plan = pk.Plan(*sizes, precision="fp64")
+    ref, need = plan.energy(*dev, p.s).cpu().numpy(), plan.workspace_bytes()
+    plan.close()
+    filler = _leave_free(torch, 300 << 20)
+    try:
+        plan = pk.Plan(*sizes, precision="fp64")
+        assert plan.workspace_bytes() <= (300 << 20) * 0.5 < need
+        e = plan.energy(*dev, p.s).cpu().numpy()
+        plan.sync()
+        plan.close()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert np.abs(e / ref - 1.0).max() <= 1e-12
