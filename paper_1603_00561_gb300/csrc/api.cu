@@ -41,6 +41,19 @@ void plan_release(dsrg_plan* p, size_t n_allocs, size_t ws_bytes) {
   p->ws_bytes = ws_bytes;
 }
 
+size_t digits_limit() {
+  size_t free_b = 0, total_b = 0;
+  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess ? free_b / 5 * 2 : 0;
+}
+
+void plan_alloc_digits(dsrg_plan* p, size_t& limit) {
+  if (p->prec != DSRG_PREC_FP64) return;
+  const size_t ws = p->ws_bytes;
+  fp64_tc_alloc(p, limit);
+  grad_alloc_products(p, limit - (p->ws_bytes - ws));
+  limit -= p->ws_bytes - ws;
+}
+
 cudaError_t raise_smem_limit(const void* func, size_t bytes) {
   static std::mutex mu;
   static std::map<std::pair<const void*, int>, size_t> cur;
@@ -163,7 +176,7 @@ size_t dsrg_plan_workspace_bytes(const dsrg_plan_t* plan) { return plan ? plan->
 
 namespace dsrg {
 dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precision_t prec,
-                          void* cuda_stream, uint32_t flags, const SplitShare* share) {
+                          void* cuda_stream, uint32_t flags, const SplitShare* share, bool digits) {
   if (!out) return DSRG_ERR_INVALID_ARG;
   *out = nullptr;
   if (!sz) return DSRG_ERR_INVALID_ARG;
@@ -281,9 +294,9 @@ dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precis
     return DSRG_ERR_OOM;
   }
   // what the plan can do without comes last
-  if (prec == DSRG_PREC_FP64) {
-    fp64_tc_alloc(p);
-    grad_alloc_products(p);
+  if (digits) {
+    size_t limit = digits_limit();
+    plan_alloc_digits(p, limit);
   }
   cudaError_t e = cudaSuccess;
   e = cudaMemcpy(p->d_pairs, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice);
@@ -314,7 +327,7 @@ extern "C" {
 
 dsrg_status_t dsrg_df_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precision_t prec,
                            void* cuda_stream, uint32_t flags) {
-  return create_plan(out, sz, prec, cuda_stream, flags, nullptr);
+  return create_plan(out, sz, prec, cuda_stream, flags, nullptr, true);
 }
 
 dsrg_status_t dsrg_plan_destroy(dsrg_plan_t* plan) {

@@ -199,13 +199,18 @@ dsrg_status_t dsrg_batch_plan(dsrg_batch_t** out, int32_t nmol, const dsrg_sizes
     sh.row_base = row_base[m];
     sh.y = b->ybuf ? b->ybuf + (m % b->max_branches) * (b->ybytes / sizeof(float)) : nullptr;
     dsrg_status_t st =
-        dsrg::create_plan(&b->plans[m], &sizes[m], prec, b->cap_stream, flags, split ? &sh : nullptr);
+        dsrg::create_plan(&b->plans[m], &sizes[m], prec, b->cap_stream, flags, split ? &sh : nullptr, false);
     if (st != DSRG_OK) {
       bfree(b);
       delete b;
       return st;
     }
-    b->ws_bytes += dsrg_plan_workspace_bytes(b->plans[m]);
+  }
+  // FP64 molecules: digits for as many, in order, as fit 2/5 of what all of them leave free
+  size_t limit = dsrg::digits_limit();
+  for (dsrg_plan* p : b->plans) {
+    dsrg::plan_alloc_digits(p, limit);
+    b->ws_bytes += dsrg_plan_workspace_bytes(p);
   }
   if (split) {
     const size_t mdb = dsrg::split_mol_desc_bytes();

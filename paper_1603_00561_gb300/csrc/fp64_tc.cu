@@ -314,17 +314,16 @@ constexpr size_t V_BYTES = (size_t)96 << 20;
 
 // The slices and the check plane take 16 bytes per value of B, Y one FP64 per (hole,
 // virtual) and active pair, the pair buffer at least one pair's integrals. A plan takes them
-// only where they are at most 2/5 of the memory free at its creation, and can be had: others
-// run on the CUDA-core kernels, which need none of it (they run for hours there, but they run).
-void fp64_tc_alloc(dsrg_plan* p) {
+// only where they are within `limit` and can be had: others run on the CUDA-core kernels,
+// which need none of it (they run for hours there, but they run).
+void fp64_tc_alloc(dsrg_plan* p, size_t limit) {
   const Sizes& z = p->z;
   if (z.Q > OZ_MAX_K) return;
   const long long nVpad = (z.nV + OZ_ROW_PAD - 1ll) / OZ_ROW_PAD * OZ_ROW_PAD;
   const long long XR = (z.nH * z.nA + OZ_ROW_PAD - 1ll) / OZ_ROW_PAD * OZ_ROW_PAD;
   const long long rows = z.nH * nVpad + XR;
   const size_t per = (size_t)z.nV * z.nV * sizeof(double);
-  size_t free_b = 0, total_b = 0;
-  if (rows > 2000000000ll || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
+  if (rows > 2000000000ll) return;
   Fp64Tc* w = new (std::nothrow) Fp64Tc();
   if (!w) return;
   w->nVpad = (int)nVpad;
@@ -350,7 +349,7 @@ void fp64_tc_alloc(dsrg_plan* p) {
   const size_t y = z.nA == 0 ? 0 : (size_t)(w->xrow0 + z.nH * z.nA) * w->ldy * sizeof(double);
   const size_t need = oz_plane_bytes(r.total, z.Q) + (size_t)r.total * OZ_ROW_INFO + mask + per * w->group + y;
   const size_t n_allocs = p->allocs.size(), ws = p->ws_bytes;
-  if ((double)need <= 0.4 * (double)free_b &&
+  if (need <= limit &&
       plan_alloc(p, (void**)&w->planes, oz_plane_bytes(r.total, z.Q)) &&
       plan_alloc(p, (void**)&w->rexp, (size_t)r.total * OZ_ROW_INFO) && plan_alloc(p, &w->mask, mask) &&
       plan_alloc(p, (void**)&w->V, per * w->group) && (y == 0 || plan_alloc(p, (void**)&w->Y, y))) {

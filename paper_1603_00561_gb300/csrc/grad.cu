@@ -1351,16 +1351,13 @@ bool grad_alloc(dsrg_plan* p) {
 
 // Workspace of the largest product, dB of a group of rows from W; without it the products
 // are FP64 FMAs.
-void grad_alloc_products(dsrg_plan* p) {
+void grad_alloc_products(dsrg_plan* p, size_t limit) {
   GradWs* g = p->grad;
   if (!g) return;
   const Sizes& z = p->z;
   const size_t bytes = oz_work_bytes(z.Q, z.nV, (long long)z.nC * z.nV, g->kgroup, true, false);
-  size_t free_b = 0, total_b = 0;
   g->oz.status = p->d_status;
-  if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && (double)bytes <= 0.4 * (double)free_b &&
-      plan_alloc(p, &g->oz.mem, bytes))
-    g->oz.bytes = bytes;
+  if (bytes <= limit && plan_alloc(p, &g->oz.mem, bytes)) g->oz.bytes = bytes;
 }
 
 void grad_free(dsrg_plan* p) {

@@ -149,8 +149,11 @@ inline cudaStream_t side_stream(const dsrg_plan* p) { return p->forked ? p->call
 
 // Launchers (each returns cudaSuccess or the launch error; adds to p->launches).
 // FP64 plans: tensor-core products (fp64_tc.cu) when their workspace is a small enough
-// part of the free memory and can be had (then p->f64 is set), else the CUDA-core kernels.
-void fp64_tc_alloc(dsrg_plan* p);
+// part of the free memory (digits_limit, when the plan or batch is made) and can be had (then
+// p->f64 is set), else the CUDA-core kernels.
+size_t digits_limit();
+void plan_alloc_digits(dsrg_plan* p, size_t& limit);  // takes it off the limit
+void fp64_tc_alloc(dsrg_plan* p, size_t limit);
 void fp64_tc_free(dsrg_plan* p);
 cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps, double s);
 cudaError_t launch_rest_fp64_tc(dsrg_plan* p, const double* B, const double* eps, const double* G,
@@ -201,7 +204,7 @@ struct SplitShare {
   float* y;  // GEMM output of tc_rest.cu shared by the molecules (NULL: the plan owns one)
 };
 dsrg_status_t create_plan(dsrg_plan_t** out, const dsrg_sizes_t* sz, dsrg_precision_t prec,
-                          void* cuda_stream, uint32_t flags, const SplitShare* share);
+                          void* cuda_stream, uint32_t flags, const SplitShare* share, bool digits);
 dsrg_status_t run_rest(dsrg_plan* p, const double* B, const double* eps, const double* G,
                        const double* L, const double* L3, const double* F1, double s, double* out);
 dsrg_status_t run_blocks(dsrg_plan* p, const double* B, const double* eps, const double* G,
@@ -300,7 +303,7 @@ std::string tune_size_class(const Sizes& z, int kblocks, int world);
 
 // Gradient (grad.cu).
 bool grad_alloc(dsrg_plan* p);
-void grad_alloc_products(dsrg_plan* p);  // FP64 plans: the digits' workspace, if it can be had
+void grad_alloc_products(dsrg_plan* p, size_t limit);  // FP64 plans: the products' workspace, if it can be had
 void grad_free(dsrg_plan* p);
 cudaError_t launch_grad(dsrg_plan* p, const double* B, const double* eps, const double* G,
                         const double* L, const double* L3, const double* F1, double s, double* dB,

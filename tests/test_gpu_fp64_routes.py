@@ -99,3 +99,31 @@ def test_little_free_memory(pk):
         del filler
         torch.cuda.empty_cache()
     assert np.abs(e / ref - 1.0).max() <= 1e-12
+
+
+def test_batch_under_little_free_memory(pk):
+    """The molecules of an FP64 batch share 2/5 of the free memory: those that find no room for
+    digits run without. The same energies as plans by themselves."""
+    import torch
+    sizes = [(8, 2, 300, 1500)] * 5 + [(3, 1, 40, 60)]
+    ps = [make_problem(*sz, s=0.5, seed=k) for k, sz in enumerate(sizes)]
+    dev = [pk.to_device(p) for p in ps]
+    ref = []
+    for sz, d, p in zip(sizes, dev, ps):
+        plan = pk.Plan(*sz, precision="fp64")
+        ref.append(plan.energy(*d, p.s).cpu().numpy())
+        plan.close()
+    filler = _leave_free(torch, 500 << 20)
+    try:
+        free0, _ = torch.cuda.mem_get_info()
+        batch = pk.Batch(sizes, precision="fp64")
+        free1, _ = torch.cuda.mem_get_info()
+        e = batch.energy(dev, [p.s for p in ps]).cpu().numpy()
+        batch.sync()
+        batch.close()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    # 300 MB or so would not have been left by five digits' workspaces of over 130 MB
+    assert free1 >= 0.5 * free0
+    assert np.abs(e / np.array(ref) - 1.0).max() <= 1e-12
