@@ -426,10 +426,13 @@ const char *dsrg_sc_last_error(const dsrg_sc_plan_t *plan);
  *   C      [nbf][nmo]        MO coefficients;
  *   metric [naux][naux]      two-centre integrals J_PQ, symmetric positive definite;
  *   B_out  [naux][np][nq];
- *   work   caller-owned device scratch of dsrg_df_mo_transform_work_bytes() bytes.
+ *   work   caller-owned device scratch of dsrg_df_mo_transform_work_bytes() bytes, or of
+ *          any number from dsrg_df_mo_transform_min_work_bytes() up: with less room
+ *          the products run in parts or as FP64 FMAs (slower; the same accuracy).
  * Synchronous (it reads back the positivity check of the metric):
  * DSRG_ERR_INVALID_ARG if the metric is not positive definite. */
 size_t dsrg_df_mo_transform_work_bytes(int32_t nbf, int32_t naux, int32_t np, int32_t nq);
+size_t dsrg_df_mo_transform_min_work_bytes(int32_t nbf, int32_t naux, int32_t np, int32_t nq);
 dsrg_status_t dsrg_df_mo_transform(const double *ao3, const double *C, const double *metric,
                                    int32_t nbf, int32_t nmo, int32_t naux, int32_t p0, int32_t np,
                                    int32_t q0, int32_t nq, double *B_out, double *work,

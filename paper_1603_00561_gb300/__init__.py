@@ -416,7 +416,11 @@ def df_mo_transform(ao3, C, metric, p0: int = 0, np_: int | None = None, q0: int
     nq = nmo - q0 if nq is None else nq
     out = torch.empty((naux, np_, nq), dtype=torch.float64, device=ao3.device)
     wb = int(lib.dsrg_df_mo_transform_work_bytes(nbf, naux, np_, nq))
-    work = torch.empty((wb + 7) // 8, dtype=torch.float64, device=ao3.device)
+    try:
+        work = torch.empty((wb + 7) // 8, dtype=torch.float64, device=ao3.device)
+    except torch.cuda.OutOfMemoryError:  # without room for the digits of the products
+        wb = int(lib.dsrg_df_mo_transform_min_work_bytes(nbf, naux, np_, nq))
+        work = torch.empty((wb + 7) // 8, dtype=torch.float64, device=ao3.device)
     st = lib.dsrg_df_mo_transform(_ptr(ao3), _ptr(C), _ptr(metric), nbf, nmo, naux, p0, np_, q0, nq,
                                   _ptr(out), _ptr(work), wb,
                                   C_.c_void_p(torch.cuda.current_stream().cuda_stream))

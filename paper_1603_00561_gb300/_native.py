@@ -30,7 +30,8 @@ EXPORTS = [
     "dsrg_mrpt2_energy_grad_ext", "dsrg_sc_plan_create", "dsrg_sc_plan_destroy", "dsrg_generalized_fock",
     "dsrg_semicanonicalize", "dsrg_sc_sync", "dsrg_sc_selftest_wait_timeout",
     "dsrg_sc_last_sweeps", "dsrg_sc_last_error",
-    "dsrg_df_mo_transform_work_bytes", "dsrg_df_mo_transform", "dsrg_cd_factors_work_bytes",
+    "dsrg_df_mo_transform_work_bytes", "dsrg_df_mo_transform_min_work_bytes", "dsrg_df_mo_transform",
+    "dsrg_cd_factors_work_bytes",
     "dsrg_cd_factors", "dsrg_plan_set_shard", "dsrg_shard_pairs", "dsrg_batch_branches",
     "dsrg_batch_set_branches", "dsrg_batch_autotune_branches", "dsrg_tune_cache_get",
     "dsrg_tune_cache_put",
@@ -98,6 +99,8 @@ def load(path: str = LIB_PATH) -> C.CDLL:
     i32 = C.c_int32
     lib.dsrg_df_mo_transform_work_bytes.argtypes = [i32, i32, i32, i32]
     lib.dsrg_df_mo_transform_work_bytes.restype = C.c_size_t
+    lib.dsrg_df_mo_transform_min_work_bytes.argtypes = [i32, i32, i32, i32]
+    lib.dsrg_df_mo_transform_min_work_bytes.restype = C.c_size_t
     lib.dsrg_df_mo_transform.argtypes = [vp, vp, vp, i32, i32, i32, i32, i32, i32, i32, vp, vp,
                                          C.c_size_t, vp]
     lib.dsrg_df_mo_transform.restype = st

@@ -346,8 +346,7 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
     return DSRG_ERR_INVALID_ARG;
   if (((uintptr_t)ao3 | (uintptr_t)C | (uintptr_t)metric | (uintptr_t)B_out | (uintptr_t)work) & 7u)
     return DSRG_ERR_INVALID_ARG;
-  const size_t need = dsrg_df_mo_transform_work_bytes(nbf, naux, np, nq);
-  if (work_bytes < need) return DSRG_ERR_INVALID_ARG;
+  if (work_bytes < dsrg_df_mo_transform_min_work_bytes(nbf, naux, np, nq)) return DSRG_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   double* Y = work;                                        // [naux][np][nbf]
   double* Z = Y + (size_t)naux * np * nbf;                 // [naux][np][nq]
@@ -355,8 +354,14 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   double* Li = Lm + (size_t)naux * naux;                   // [naux][naux] L^{-1}
   int* bad = (int*)(Li + (size_t)naux * naux);             // and the waits' status word
   OzWork ow;
-  ow.mem = (uint8_t*)(((uintptr_t)(bad + 8) + 255) & ~(uintptr_t)255);
-  ow.bytes = df_gemm_bytes(nbf, naux, np, nq);
+  // what is left of the work array holds the digits of the products; FP64 FMAs where it is short
+  uint8_t* end = (uint8_t*)work + work_bytes;
+  uint8_t* mem = (uint8_t*)(((uintptr_t)(bad + 8) + 255) & ~(uintptr_t)255);
+  if (mem < end) {
+    const size_t left = (size_t)(end - mem), most = df_gemm_bytes(nbf, naux, np, nq);
+    ow.mem = mem;
+    ow.bytes = left < most ? left : most;
+  }
   ow.status = bad + 1;
   if (cudaMemsetAsync(bad, 0, 2 * sizeof(int), st) != cudaSuccess) return DSRG_ERR_CUDA;
   cudaError_t e;
@@ -399,9 +404,12 @@ dsrg_status_t dsrg_df_mo_transform(const double* ao3, const double* C, const dou
   return hbad[0] ? DSRG_ERR_INVALID_ARG : DSRG_OK;
 }
 
+size_t dsrg_df_mo_transform_min_work_bytes(int32_t nbf, int32_t naux, int32_t np, int32_t nq) {
+  return ((size_t)naux * np * nbf + (size_t)naux * np * nq + 2 * (size_t)naux * naux) * 8 + 64;
+}
+
 size_t dsrg_df_mo_transform_work_bytes(int32_t nbf, int32_t naux, int32_t np, int32_t nq) {
-  return ((size_t)naux * np * nbf + (size_t)naux * np * nq + 2 * (size_t)naux * naux) * 8 + 512 +
-         df_gemm_bytes(nbf, naux, np, nq);
+  return dsrg_df_mo_transform_min_work_bytes(nbf, naux, np, nq) + 448 + df_gemm_bytes(nbf, naux, np, nq);
 }
 
 dsrg_status_t dsrg_cd_factors(const double* F, int32_t nfac, int32_t n, double tau,
