@@ -447,8 +447,9 @@ dsrg_status_t dsrg_df_mo_transform(const double *ao3, const double *C, const dou
  * small basis or a finer factorisation). Output: L_out [max_rank][n][n], of
  * which the first *rank_out are the Cholesky vectors B^Q_pq; every integral
  * of M - sum_Q B^Q (B^Q)^T is below tau in magnitude. FP64. work: caller-owned
- * device scratch of dsrg_cd_factors_work_bytes(n) bytes. Synchronous (the rank
- * is read back). */
+ * device scratch of dsrg_cd_factors_work_bytes(n) bytes (from 8 n^2 + 88 on the
+ * call finds itself what little more it needs). Synchronous (the rank is read
+ * back). */
 size_t dsrg_cd_factors_work_bytes(int32_t n);
 dsrg_status_t dsrg_cd_factors(const double *F, int32_t nfac, int32_t n, double tau,
                               int32_t max_rank, double *L_out, int32_t *rank_out, double *work,

@@ -200,6 +200,25 @@ struct CdSlot {
   long long i;
 };
 constexpr int CD_SLOTS = 2048;  // CTAs of the decomposition, at most
+constexpr size_t CD_MIN_EXTRA = 88;  // bytes a work array has beyond the diagonal, at least
+static_assert(sizeof(CdState) <= CD_MIN_EXTRA, "the state lies there");
+
+// Stream-ordered memory for the scope.
+struct StreamAlloc {
+  cudaStream_t st;
+  void* p = nullptr;
+  explicit StreamAlloc(cudaStream_t s) : st(s) {}
+  void* get(size_t bytes) {
+    if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return p;
+  }
+  ~StreamAlloc() {
+    if (p) cudaFreeAsync(p, st);
+  }
+};
 
 // d[p] = M_pp = sum_k F[k][p]^2 (p over the N = n^2 pairs)
 __global__ void cd_diag_kernel(const double* __restrict__ F, int K0, size_t N, double* __restrict__ d) {
@@ -419,11 +438,14 @@ dsrg_status_t dsrg_cd_factors(const double* F, int32_t nfac, int32_t n, double t
     return DSRG_ERR_INVALID_ARG;
   if (((uintptr_t)F | (uintptr_t)L_out | (uintptr_t)work) & 7u) return DSRG_ERR_INVALID_ARG;
   const size_t N = (size_t)n * n;
-  if (work_bytes < dsrg_cd_factors_work_bytes(n)) return DSRG_ERR_INVALID_ARG;
+  if (work_bytes < N * 8 + CD_MIN_EXTRA) return DSRG_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   double* d = work;
   CdState* cs = (CdState*)(d + N);
   CdSlot* slots = (CdSlot*)(((uintptr_t)(cs + 1) + 15) & ~(uintptr_t)15);
+  StreamAlloc own(st);  // the slots, for a work array that has no room for them
+  if (work_bytes < dsrg_cd_factors_work_bytes(n) && !(slots = (CdSlot*)own.get(2 * CD_SLOTS * sizeof(CdSlot))))
+    return DSRG_ERR_OOM;
   if (cudaMemsetAsync(cs, 0, sizeof(CdState), st) != cudaSuccess) return DSRG_ERR_CUDA;
   cd_diag_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(F, nfac, N, d);
   if (cudaGetLastError() != cudaSuccess) return DSRG_ERR_CUDA;

@@ -85,3 +85,23 @@ def test_df_transform_with_little_free_memory(pk):
         del filler
         torch.cuda.empty_cache()
     assert (B - ref).abs().max() <= 1e-12 * ref.abs().max()
+
+
+@pytest.mark.parametrize("n,nfac", [(3, 4), (30, 120)])
+def test_cholesky_in_a_work_array_of_the_former_size(pk, n, nfac):
+    """8 n^2 + 88 bytes: the same vectors, bit for bit, as with all that the call asks for."""
+    import torch
+    from paper_1603_00561_gb300 import _native
+    lib = _native.load()
+    F = _dev(make_eri_factors(n, nfac, seed=2))
+    ref = pk.cd_factors(F, 1e-7)
+    ptr = lambda t: C.c_void_p(t.data_ptr())
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    for wb, want in ((8 * n * n + 88, _native.OK), (8 * n * n + 80, _native.ERR_INVALID_ARG)):
+        L = torch.zeros((n * n, n, n), dtype=torch.float64, device="cuda")
+        work = torch.full((wb + 512,), 0x5A, dtype=torch.uint8, device="cuda")
+        rank = C.c_int32(-1)
+        assert lib.dsrg_cd_factors(ptr(F), nfac, n, 1e-7, n * n, ptr(L), C.byref(rank), ptr(work), wb, stream) == want
+        assert (work[wb:] == 0x5A).all()
+        if want == _native.OK:
+            assert rank.value == ref.shape[0] and torch.equal(L[: rank.value], ref)
