@@ -384,8 +384,9 @@ dsrg_status_t dsrg_plan_branch_counts(dsrg_plan_t *plan, uint64_t counts[DSRG_NC
  *                                on every index (only if lambda3 != NULL);
  *   U_out       [n][n]           U (may be NULL).
  * All arrays are caller-owned device arrays, 8-byte aligned. The plan owns its
- * workspace (about naux*n*(nH+1) + 2*naux*nH*nP + 7 n^2 doubles, partial exchange
- * matrices and up to 512 MiB for the products' digits). The semicanonicalisation
+ * workspace (about naux*n*(nH+1) + 2*naux*nH*nP + 7 n^2 doubles; and, where the memory
+ * free at its creation allows, partial exchange matrices and up to 512 MiB, or one
+ * product's need, for the products' digits). The semicanonicalisation
  * synchronises the plan's stream at its end (the Jacobi sweeps run in one launch per
  * block and stop at ||offdiag||^2 <= 1e-30 ||A||^2, at most 30 sweeps) and is not meant
  * to be captured in a graph. */

@@ -54,10 +54,9 @@ struct dsrg_sc_plan {
   double *X = nullptr;      // [naux][n][nH]
   double *f = nullptr;      // [n][n]
   double *U = nullptr;      // [n][n]
-  double *T = nullptr;      // [n][n]
+  double *T = nullptr;      // [n][n]; the other copy of A during the Jacobi sweeps
   double *A = nullptr;      // [mmax][mmax] Jacobi work matrix
   double *V = nullptr;      // [mmax][mmax] Jacobi eigenvectors
-  double *A2 = nullptr;     // [mmax][mmax] its other copy
   double *diag = nullptr;   // [mmax] eigenvalues in matrix order
   double2 *slots = nullptr; // [JAC_SLOTS] partial norms
   dsrg::JacState *jac = nullptr;
@@ -83,6 +82,12 @@ bool sc_alloc(dsrg_sc_plan* p, void** ptr, size_t bytes) {
   p->allocs.push_back(*ptr);
   p->ws_bytes += bytes;
   return true;
+}
+
+// ... of at most 2/5 of the free memory.
+bool sc_alloc_spare(dsrg_sc_plan* p, void** ptr, size_t bytes) {
+  *ptr = nullptr;
+  return bytes <= digits_limit() && sc_alloc(p, ptr, bytes);
 }
 
 // w_Q = sum_rs B^Q_rs D_rs = 2 sum_m B^Q_mm + sum_uv B^Q_{nC+u, nC+v} G_uv (one warp per Q).
@@ -478,7 +483,7 @@ cudaError_t jacobi_block(dsrg_sc_plan* p, int lo, int m, double* eps) {
   int max_sweeps = m > 1 ? 30 : 0;
   e = cudaMemsetAsync(&p->jac->bar.count, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  void* args[] = {&p->A, &p->A2, &p->V, &m, &mp, &max_sweeps, &p->slots, &p->diag, &p->jac};
+  void* args[] = {&p->A, &p->T, &p->V, &m, &mp, &max_sweeps, &p->slots, &p->diag, &p->jac};
   e = cudaLaunchCooperativeKernel((const void*)jac_run_kernel, dim3(grid), dim3(JT * JT), args, 0, st);
   if (e != cudaSuccess) return e;
   jac_store_kernel<<<m, 128, 0, st>>>(p->diag, p->V, m, n, lo, p->U, eps);
@@ -562,15 +567,15 @@ dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t** out, const dsrg_sizes_t* sz, 
     p->oz.bytes = b;
   }
   bool ok = sc_alloc(p, (void**)&p->w, (size_t)z.Q * 8) && sc_alloc(p, (void**)&p->J, nn * 8) &&
-            sc_alloc(p, (void**)&p->K, p->nk * nn * 8) &&
+            sc_alloc(p, (void**)&p->K, nn * 8) &&
             sc_alloc(p, (void**)&p->X, (size_t)z.Q * z.n * z.nH * 8) &&
             sc_alloc(p, (void**)&p->f, nn * 8) && sc_alloc(p, (void**)&p->U, nn * 8) &&
             sc_alloc(p, (void**)&p->T, nn * 8) && sc_alloc(p, (void**)&p->A, mm * 8) &&
             sc_alloc(p, (void**)&p->V, mm * 8) &&
-            sc_alloc(p, (void**)&p->A2, mm * 8) && sc_alloc(p, (void**)&p->diag, (size_t)p->mmax * 8) &&
+            sc_alloc(p, (void**)&p->diag, (size_t)p->mmax * 8) &&
             sc_alloc(p, (void**)&p->slots, JAC_SLOTS * sizeof(double2)) &&
             sc_alloc(p, (void**)&p->jac, sizeof(JacState)) && sc_alloc(p, (void**)&p->Bhp, nhp * 8) &&
-            sc_alloc(p, (void**)&p->Bt, nhp * 8) && sc_alloc(p, &p->oz.mem, p->oz.bytes);
+            sc_alloc(p, (void**)&p->Bt, nhp * 8);
   ok = ok && cudaMemset(p->jac, 0, sizeof(JacState)) == cudaSuccess;
   if (ok) p->oz.status = &p->jac->wait;
   size_t n3 = 1;
@@ -581,6 +586,14 @@ dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t** out, const dsrg_sizes_t* sz, 
     delete p;
     return DSRG_ERR_OOM;
   }
+  // what the plan can do without: the digits of the products (FP64 FMAs then) and the
+  // partial exchange matrices (one then)
+  if (!sc_alloc_spare(p, &p->oz.mem, p->oz.bytes)) p->oz.bytes = 0;
+  void* parts = nullptr;
+  if (p->nk > 1 && sc_alloc_spare(p, &parts, p->nk * nn * 8))
+    p->K = (double*)parts;
+  else
+    p->nk = 1;
   *out = p;
   return DSRG_OK;
 }

@@ -105,3 +105,32 @@ def test_cholesky_in_a_work_array_of_the_former_size(pk, n, nfac):
         assert (work[wb:] == 0x5A).all()
         if want == _native.OK:
             assert rank.value == ref.shape[0] and torch.equal(L[: rank.value], ref)
+
+
+def test_semicanonical_plan_with_little_free_memory(pk):
+    """Without room for digits and partial exchange matrices the plan is made all the same."""
+    import torch
+    nC, nA, nV, Q = 8, 2, 200, 1500
+    n, nH, nP = nC + nA + nV, nC + nA, nA + nV
+    p = make_fock_problem(nC, nA, nV, Q, seed=5)
+    args = [_dev(x) for x in (p.h, p.Bfull, p.gamma1, p.lambda2)]
+    sc = pk.SemicanonicalPlan(nC, nA, nV, Q)
+    ref = sc.semicanonicalize(*args)
+    f = sc.fock(*args[:3])
+    sc.close()
+    # the arrays that the plan is documented to need, in 2 MiB granules, and its outputs
+    need = 8 * (Q * n * (nH + 1) + 2 * Q * nH * nP + 7 * n * n) + (40 << 20)
+    out = 8 * (Q * nH * nP + 3 * n * n) + (60 << 20)
+    filler = _leave_free(torch, need + out)
+    try:
+        sc = pk.SemicanonicalPlan(nC, nA, nV, Q)
+        got = sc.semicanonicalize(*args)
+        f2 = sc.fock(*args[:3])
+        sc.sync()
+        sc.close()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert (f2 - f).abs().max() <= 1e-12 * f.abs().max()
+    assert (got["eps"] - ref["eps"]).abs().max() <= 1e-12 * f.abs().max()
+    assert (got["B"] - ref["B"]).abs().max() <= 1e-9 * ref["B"].abs().max()
