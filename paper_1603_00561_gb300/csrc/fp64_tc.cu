@@ -401,7 +401,7 @@ cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps
   cudaError_t e;
   OzArgs a = pair_args(p, B);
   if ((e = oz_pack(p->stream, a.a, w->planes, w->rexp)) != cudaSuccess) return e;
-  p->launches += 2;
+  p->launches += OZ_PACK_LAUNCHES;
   const Segment& sg = p->segs[p->seg_ccvv];
   a.pstep = p->shard_world;
   for (int p0 = p->shard_rank; p0 < p->n_pairs; p0 += w->group * p->shard_world) {
@@ -409,7 +409,7 @@ cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps
     const int n = left < w->group ? left : w->group;
     a.p0 = p0;
     if ((e = oz_multiply(p->stream, w->planes, w->planes, a, n)) != cudaSuccess) return e;
-    p->launches += 3;
+    p->launches += OZ_MULTIPLY_LAUNCHES;
     ccvv_reg_fp64_kernel<<<(unsigned)(n * p->n_tp_ccvv), 256, 0, p->stream>>>(
         w->V, eps, s, z, p->d_pairs, p0, p->shard_world, p->d_tp_ccvv, p->n_tp_ccvv,
         p->d_partials + sg.begin);
@@ -431,7 +431,7 @@ cudaError_t launch_ccvv_adj_fp64_tc(dsrg_plan* p, const double* B, const double*
     const int n = p->n_pairs - p0 < w->group ? p->n_pairs - p0 : w->group;
     a.p0 = p0;
     if ((e = oz_multiply(p->stream, w->planes, w->planes, a, n)) != cudaSuccess) return e;
-    p->launches += 3;
+    p->launches += OZ_MULTIPLY_LAUNCHES;
     ccvv_adj_v_kernel<<<(unsigned)(n * p->n_tp_ccvv), 256, sm, p->stream>>>(
         w->V, eps, s, p->z, p->d_pairs, p0, p->d_tp_ccvv, p->n_tp_ccvv, nVp, W, deps, ds);
     DSRG_LAUNCH_CHECK(p);
@@ -476,7 +476,7 @@ cudaError_t launch_rest_fp64_tc(dsrg_plan* p, const double* B, const double* eps
   a.accumulate = 0;
   a.mask = w->mask;
   if ((e = oz_multiply(st, w->planes, w->planes, a, 1)) != cudaSuccess) return e;
-  p->launches += 3;
+  p->launches += OZ_MULTIPLY_LAUNCHES;
   const Segment &s2 = p->segs[p->seg_cavv], &s3 = p->segs[p->seg_ccav];
   const size_t sm2 = (size_t)z.nA * FT * (FT + 1) * 8, sm3 = (size_t)z.nC * z.nC * z.nA * 8;
 #define REST_CASE(NA_)                                                                            \

@@ -129,10 +129,7 @@ cudaError_t launch_gemm_fp64(cudaStream_t st, const GemmArgs& g) {
 // The FP64 plans' GEMMs (split plans assemble dB on the tensor cores).
 static cudaError_t gemm(dsrg_plan* p, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  const cudaError_t e = launch_gemm(p->stream, g, p->grad->oz);
-  if (e != cudaSuccess) return e;
-  p->launches++;
-  return cudaSuccess;
+  return launch_gemm(p->stream, g, p->grad->oz, &p->launches);
 }
 
 // ---------------------------------------------------------------------------

@@ -965,9 +965,10 @@ size_t oz_work_bytes(long long M, long long N, long long K, long long nb, bool s
 // operations the two are about even (58 MFLOP: 120 us against 60).
 static bool oz_worthwhile(double flops) { return flops >= 1e8; }
 
-cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
+cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w, int* launches) {
   GemmArgs g = g0;
   if (g.M <= 0 || g.N <= 0 || g.nb <= 0) return cudaSuccess;
+  int none = 0, &count = launches ? *launches : none;
   // batches that are one matrix: the shared operand's problems follow one another
   if (g.nb > 1 && g.sb == 0 && g.sa == (long long)g.M * g.ai && g.sc == (long long)g.M * g.ci &&
       (long long)g.M * g.nb < (1ll << 30)) {
@@ -980,7 +981,10 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
   }
   const long long K = (long long)g.L1 * g.L2;
   const double flops = 2.0 * g.M * g.N * (double)K * g.nb;
-  if (!w.mem || !oz_worthwhile(flops) || K > OZ_MAX_K) return launch_gemm_fp64(st, g0);
+  if (!w.mem || !oz_worthwhile(flops) || K > OZ_MAX_K) {
+    ++count;
+    return launch_gemm_fp64(st, g0);
+  }
   // the operand on the 128-row side: the one that wastes less of the tiles
   auto tiles = [](long long m, long long n) {
     return oz_up(m, OZ_BM) * oz_up(n, OZ_BN);
@@ -1008,7 +1012,10 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
     // not even one problem: a problem's rows in blocks
     const size_t left = avail > np * rb ? avail - np * rb : 0;
     mb = (long long)(left / (OZ_ROW_PAD * rb + mb128)) * OZ_ROW_PAD;
-    if (mb < OZ_ROW_PAD) return launch_gemm_fp64(st, g0);
+    if (mb < OZ_ROW_PAD) {
+      ++count;
+      return launch_gemm_fp64(st, g0);
+    }
     zb = 1;
   }
   uint8_t* base = (uint8_t*)w.mem;
@@ -1023,14 +1030,18 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
     const int nz = (int)(g.nb - z0 < zb ? g.nb - z0 : zb);
     OzArgs a;
     a.b = oz_rows(pn + z0 * zn, share_n ? 1 : nz, n, (int)np, rn, zn, g.L1, g.L2, n1, n2);
-    if (z0 == 0 || !share_n)
+    if (z0 == 0 || !share_n) {
       if ((e = oz_pack(st, a.b, pln, xn)) != cudaSuccess) return e;
+      count += OZ_PACK_LAUNCHES;
+    }
     for (long long r0 = 0; r0 < m; r0 += mb) {
       const int mr = (int)(m - r0 < mb ? m - r0 : mb);
       a.a = oz_rows(pm + z0 * zm + r0 * rm, share_m ? 1 : nz, mr, (int)(mb < m ? oz_up(mr, OZ_ROW_PAD) : mb),
                     rm, zm, g.L1, g.L2, m1, m2);
-      if (z0 == 0 || !share_m || mb < m)
+      if (z0 == 0 || !share_m || mb < m) {
         if ((e = oz_pack(st, a.a, plm, xm)) != cudaSuccess) return e;
+        count += OZ_PACK_LAUNCHES;
+      }
       a.aexp = xm;
       a.bexp = xn;
       a.status = w.status;
@@ -1050,6 +1061,7 @@ cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w) {
       a.accumulate = g.accumulate;
       a.mask = mask;
       if ((e = oz_multiply(st, plm, pln, a, nz)) != cudaSuccess) return e;
+      count += OZ_MULTIPLY_LAUNCHES;
     }
   }
   return cudaSuccess;

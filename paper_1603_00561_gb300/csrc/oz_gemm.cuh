@@ -95,6 +95,7 @@ inline size_t oz_mask_bytes(long long M, long long N, long long problems) {
 }
 // Row scales and sums (OZ_ROW_INFO * total bytes at rexp) and slices (oz_plane_bytes(total,
 // K); oz_off) of one operand, total a multiple of OZ_ROW_PAD.
+constexpr int OZ_PACK_LAUNCHES = 2, OZ_MULTIPLY_LAUNCHES = 3;
 cudaError_t oz_pack(cudaStream_t st, const OzRows& s, __nv_bfloat16* planes, int* rexp);
 // The product of two packed operands (a.a, a.b: their rows as packed; the FP64 values at
 // a.a.p and a.b.p are read again where the check finds the slices short of bits).
@@ -110,7 +111,8 @@ struct OzWork {
   int* status = nullptr;  // device status word of the bounded waits
 };
 struct GemmArgs;
-cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g, const OzWork& w);
+// The kernels queued are added to *launches (may be null).
+cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g, const OzWork& w, int* launches = nullptr);
 // Workspace that lets launch_gemm run nb problems of M x N x K at once, at most OZ_WS_CAP
 // (the problems then run in turns).
 constexpr size_t OZ_WS_CAP = (size_t)512 << 20;
