@@ -1375,7 +1375,6 @@ GemmArgs mk(int M, int N, int L1, int L2, const double* A, long long ai, long lo
   g.accumulate = 1;
   g.nb = 1;
   g.sa = g.sb = g.sc = 0;
-  g.A32 = g.B32 = nullptr;
   return g;
 }
 

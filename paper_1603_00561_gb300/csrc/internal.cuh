@@ -282,9 +282,6 @@ struct GemmArgs {
   int accumulate;
   int nb;                // independent problems in one launch (blockIdx.z);
   long long sa, sb, sc;  // their offsets of A, Bm, C
-  // FP32 copies of A and Bm (same element offsets) for the FP32 GEMM, or null
-  const float* A32;
-  const float* B32;
 };
 GemmArgs mk(int M, int N, int L1, int L2, const double* A, long long ai, long long a1, long long a2,
             const double* Bm, long long b1, long long b2, long long bj, double* C, long long ci,

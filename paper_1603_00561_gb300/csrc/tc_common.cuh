@@ -23,10 +23,6 @@ __device__ __forceinline__ uint32_t su32(const void* p) {
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes)
-               : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
 }
@@ -60,15 +56,7 @@ static __device__ __noinline__ bool mbar_wait(uint64_t* b, uint32_t parity, vola
     }
   }
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0,
-                                            int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
-      "%4}], [%2];" ::"r"(su32(dst)),
-      "l"((unsigned long long)map), "r"(su32(bar)), "r"(c0), "r"(c1)
-      : "memory");
-}
-// ... of a whole converged warp, issued by its leader lane (tc_elect).
+// Expected bytes and a TMA load of a whole converged warp, by its leader lane (tc_elect).
 __device__ __forceinline__ void mbar_expect_tx_if(uint32_t leader, uint64_t* b, uint32_t bytes) {
   asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
                " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(su32(b)),

@@ -933,8 +933,6 @@ size_t rest_y_bytes(const Sizes& z) {
   return (size_t)z.nH * st.nVpad * st.ldy * sizeof(float);
 }
 
-bool rest_split_used(const dsrg_plan* p) { return p->prec != DSRG_PREC_FP64 && p->z.nA > 0; }
-
 int rest_cavv_blocks(const dsrg_plan* p) {
   RestState st;
   rest_dims(p->z, &st);
