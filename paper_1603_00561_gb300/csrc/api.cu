@@ -68,6 +68,14 @@ cudaError_t raise_smem_limit(const void* func, size_t bytes) {
   return e;
 }
 
+int sm_count() {
+  int dev = 0, n = 0;
+  return cudaGetDevice(&dev) == cudaSuccess &&
+                 cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0
+             ? n
+             : 1;
+}
+
 static void tile_pairs(int n, int tile, std::vector<int2>& out) {
   const int nt = (n + tile - 1) / tile;
   out.clear();

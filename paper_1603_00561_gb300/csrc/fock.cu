@@ -555,7 +555,7 @@ dsrg_status_t dsrg_sc_plan_create(dsrg_sc_plan_t** out, const dsrg_sizes_t* sz, 
     // the exchange matrix has few tiles and a long sum: parts of it over Q, so that about
     // two tiles per SM run, each part at least 512 long
     const long long tiles = ((z.n + 127) / 128) * (long long)((z.n + 63) / 64);
-    long long nk = 304 / tiles, most = (long long)z.Q * z.nH / 512;
+    long long nk = 2 * sm_count() / tiles, most = (long long)z.Q * z.nH / 512;
     nk = nk > 16 ? 16 : nk;
     nk = nk > most ? most : nk;
     p->nk = nk < 1 ? 1 : (int)(nk > z.Q ? z.Q : nk);

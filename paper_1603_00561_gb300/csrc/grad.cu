@@ -116,10 +116,10 @@ cudaError_t launch_gemm_fp64(cudaStream_t st, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   auto grid = [&](int t) { return dim3((g.N + t - 1) / t, (g.M + t - 1) / t, g.nb); };
   auto ctas = [&](int t) { const dim3 d = grid(t); return (double)d.x * d.y * d.z; };
-  constexpr double FILL = 2.0 * 152;
-  if (ctas(64) >= FILL || (g.M + 15) / 16 > 65535)
+  const double fill = 2.0 * sm_count();
+  if (ctas(64) >= fill || (g.M + 15) / 16 > 65535)
     gemm_fp64_kernel<4><<<grid(64), 256, 0, st>>>(g);
-  else if (ctas(32) >= FILL)
+  else if (ctas(32) >= fill)
     gemm_fp64_kernel<2><<<grid(32), 256, 0, st>>>(g);
   else
     gemm_fp64_kernel<1><<<grid(16), 256, 0, st>>>(g);

@@ -141,6 +141,9 @@ void plan_release(dsrg_plan* p, size_t n_allocs, size_t ws_bytes);
 // limit afterwards for a smaller problem would invalidate that launch.
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
 
+// SMs of the current device.
+int sm_count();
+
 // The plan's chain stream and events (false: out of resources), a wait of stream `to` for
 // what `from` holds, and the stream of the kernels beside the chain.
 bool plan_fork_alloc(dsrg_plan* p);

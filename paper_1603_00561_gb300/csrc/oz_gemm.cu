@@ -932,9 +932,7 @@ cudaError_t oz_multiply(cudaStream_t st, const __nv_bfloat16* pa, const __nv_bfl
   const long long items = (long long)a.mt * a.nt * n_prob;
   if (items <= 0 || items > 0x7fffffff) return cudaErrorInvalidValue;
   a.n_items = (int)items;
-  int dev = 0, nsm = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nsm = sm_count();
   const unsigned grid = (unsigned)(items < nsm ? items : nsm);
   const size_t smc = (size_t)OC_STAGES * OC_STAGE_BYTES + 1024 + 256;
   raise_smem_limit((const void*)oz_check_kernel, smc);
