@@ -59,7 +59,7 @@ constexpr int OZ_A_BYTES = OZ_S * OZ_A_SLICE, OZ_B_BYTES = OZ_S * OZ_B_SLICE;
 constexpr int OZ_STAGE_BYTES = OZ_A_BYTES + OZ_B_BYTES;
 constexpr int OZ_THREADS = 320, OZ_EPI_WARPS = 8;
 constexpr int OZ_EXP_INF = 0x7ff;             // exponent field of a row with an infinity or a NaN
-constexpr unsigned long long OZ_SUM_INF = 1ull << 62;  // its sum (others: below 2^49)
+constexpr unsigned long long OZ_SUM_INF = 1ull << 46;  // its sum (others: at most K (2^24 + 1) < 2^46)
 constexpr long long OZ_TINY = LLONG_MIN;      // a value that is not 0 but is as a fixed-point number
 
 // ------------------------------- row scales -------------------------------
@@ -624,8 +624,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
 // ------------------------------- the check -------------------------------
 // S of every element (see the head of the file) in one FP32 accumulation over all of K, and
-// its mask bit. One BF16 product against the 34 of the slices, bound by its operands' copies:
-// 4 stages of up to 128 K values.
+// its mask bit. One BF16 product against the 34 of the slices, bound by its operands' copies
+// and the epilogue: 4 stages of up to 128 K values. 36 us beside 780 us for the products of
+// 86 pairs at 24/2/372/1200, 17 beside 190 us (K = 398) in the DF transform.
 constexpr int OC_KB = 4;  // blocks of 32 K values per stage
 constexpr int OC_STAGES = 4;
 constexpr int OC_STAGE_BYTES = OC_KB * (OZ_A_SLICE + OZ_B_SLICE);
@@ -788,14 +789,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       const int row = quarter * 32 + lane, i = t.i0 + row;
       uint32_t word = 0;
       if (ok && i < a.M) {
-        const float sa = (float)asum[t.arow + row] * 0x1p-24f + 0.02f * K;
+        // (sums in 2^-9 units, rounded up: a conversion from 64 bits would be one of the FP64 pipe)
+        const float sa = (float)(uint32_t)(asum[t.arow + row] >> 15) * 0x1p-9f + 0x1p-8f + 0.02f * K;
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
           const int j = ch * 32 + c;
           if (t.j0 + j < a.N) {
             const float S = __uint_as_float(r[c >> 4][c & 15]);
-            const float sums = sa + (float)bsum[t.brow + j] * 0x1p-24f;
-            if ((S > 0.0f && K8 * S < sums) || sums > (float)(OZ_SUM_INF >> 25)) word |= 1u << c;
+            const float sums = sa + (float)(uint32_t)(bsum[t.brow + j] >> 15) * 0x1p-9f;
+            if ((S > 0.0f && K8 * S < sums) || sums >= (float)(OZ_SUM_INF >> 24)) word |= 1u << c;
           }
         }
       }
@@ -814,46 +816,56 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
 }
 
-// The elements the check set, from the FP64 operands: a warp each, its lanes along K, where
-// a quarter of a 64 x 64 half tile or less is set, else the half tile in chunks of 16 K
-// values (the chain of gemm_fp64_kernel in grad.cu).
-constexpr int OF_FEW = 1024;
+// The elements the check set, from the FP64 operands, in units of 16 rows x 64 columns (as
+// 64 x 64 ones, few products filled the chip: 110, 72 and 105 us in the triangular inverse
+// at naux = 1200, 35, 53 and 84 us now): a warp each, its lanes along K, where an eighth of a
+// unit or less is set, else the unit in chunks of 16 K values (the chain of
+// gemm_fp64_kernel in grad.cu). Bound by the FP64 pipe where much is set: the DF transform at
+// 398 functions and naux = 1200 takes 33 ms with auxiliary functions scaled by 2^-20 .. 2^20
+// (8.5 ms as drawn; 143 ms with FP64 FMAs alone). With none set the launch takes 4 us.
+constexpr int OF_ROWS = 16, OF_UNITS = OZ_BM / OF_ROWS, OF_FEW = 128;
 __global__ void __launch_bounds__(256) oz_fma_kernel(const __grid_constant__ OzArgs a) {
-  __shared__ double sA[16][OZ_BN + 1], sB[16][OZ_BN + 1];
-  __shared__ uint32_t sm[128];  // mask words of a half tile: [64 rows][2]
+  __shared__ double sA[16][OF_ROWS + 1], sB[16][OZ_BN + 1];
+  __shared__ uint32_t sm[2 * OF_ROWS];  // the unit's mask words
   __shared__ unsigned short list[OF_FEW];
   __shared__ unsigned char work[256];
   __shared__ int cnt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int L1 = a.a.L1, L2 = a.a.L2, K = L1 * L2;
   auto put = [&](double* p, double d) { *p = a.accumulate ? fma(a.alpha, d, *p) : a.alpha * d; };
-  for (long long base = blockIdx.x; base < a.n_items; base += 256ll * gridDim.x) {
-    // 256 items at a time: which of them have any
+  const long long units = (long long)a.n_items * OF_UNITS;
+  for (long long base = blockIdx.x; base < units; base += 256ll * gridDim.x) {
+    // 256 units at a time: which of them may have any
     const long long mine = base + (long long)tid * gridDim.x;
-    work[tid] = mine < a.n_items && *(const unsigned long long*)oz_mask_any(a, (int)mine) != 0;
-    if (!__syncthreads_or(work[tid])) continue;
-    for (int w = 0; w < 512; ++w) {
-      if (!work[w >> 1]) continue;
-      const int it = (int)(base + (long long)(w >> 1) * gridDim.x), h = w & 1;
-      __syncthreads();  // the previous half tile is done
+    bool any = false;
+    if (mine < units) {
+      // bytes of the warps that had the rows' TMEM quarter: q = warp & 3, warps 2 to 9
+      const int b = (((int)(mine % OF_UNITS) >> 1) + 2) & 3;
+      const uint8_t* m = oz_mask_any(a, (int)(mine / OF_UNITS));
+      any = m[b] | m[b + 4];
+    }
+    work[tid] = any;
+    if (!__syncthreads_or(any)) continue;
+    for (int w = 0; w < 256; ++w) {
+      if (!work[w]) continue;
+      const long long u = base + (long long)w * gridDim.x;
+      const int it = (int)(u / OF_UNITS), r0 = (int)(u % OF_UNITS) * OF_ROWS;
+      __syncthreads();  // the previous unit is done
       if (tid == 0) cnt = 0;
-      if (tid < 128) sm[tid] = oz_mask(a, it)[h * 128 + tid];
+      if (tid < 2 * OF_ROWS) sm[tid] = oz_mask(a, it)[r0 * 2 + tid];
       __syncthreads();
-      if (tid < 128 && sm[tid]) atomicAdd(&cnt, __popc(sm[tid]));
+      if (tid < 2 * OF_ROWS)
+        for (uint32_t m = sm[tid]; m; m &= m - 1) {
+          const int k = atomicAdd(&cnt, 1);
+          if (k < OF_FEW) list[k] = (unsigned short)((tid >> 1) << 6 | (tid & 1) << 5 | (__ffs(m) - 1));
+        }
       __syncthreads();
       const int n = cnt;
       if (n == 0) continue;
       const OzTile t = oz_tile(a, it);
-      const int i0 = t.i0 + 64 * h, ar = t.arow + 64 * h;
+      const int i0 = t.i0 + r0, ar = t.arow + r0;
       double* C = a.C + t.coff;
       if (n <= OF_FEW) {
-        __syncthreads();
-        if (tid == 0) cnt = 0;
-        __syncthreads();
-        if (tid < 128)
-          for (uint32_t m = sm[tid]; m; m &= m - 1)
-            list[atomicAdd(&cnt, 1)] = (unsigned short)((tid >> 1) << 6 | (tid & 1) << 5 | (__ffs(m) - 1));
-        __syncthreads();
         for (int e = warp; e < n; e += 8) {  // (whatever the order of the list)
           const int r = list[e] >> 6, c = list[e] & 63;
           long long oa, ob;
@@ -868,37 +880,32 @@ __global__ void __launch_bounds__(256) oz_fma_kernel(const __grid_constant__ OzA
         }
         continue;
       }
-      const int ty = tid >> 4, tx = tid & 15;
-      double acc[4][4] = {};
+      const int r = tid >> 4, cx = tid & 15;  // columns cx, + 16, + 32, + 48 of row r
+      double acc[4] = {};
       for (int l0 = 0; l0 < K; l0 += 16) {
-        for (int e = tid; e < 16 * 64; e += 256) {
-          const int l = l0 + (e >> 6), c = e & 63;
-          double va = 0.0, vb = 0.0;
-          if (l < K) {
-            long long o;
-            if (i0 + c < a.M && oz_row(a.a, ar + c, o)) va = a.a.p[o + oz_k(a.a, l)];
-            if (t.j0 + c < a.N && oz_row(a.b, t.brow + c, o)) vb = a.b.p[o + oz_k(a.b, l)];
+        {
+          const int l = l0 + cx;  // K along 16 lanes, a row each
+          long long o;
+          sA[cx][r] = l < K && i0 + r < a.M && oz_row(a.a, ar + r, o) ? a.a.p[o + oz_k(a.a, l)] : 0.0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int c = r + 16 * k;
+            sB[cx][c] = l < K && t.j0 + c < a.N && oz_row(a.b, t.brow + c, o) ? a.b.p[o + oz_k(a.b, l)] : 0.0;
           }
-          sA[e >> 6][c] = va;
-          sB[e >> 6][c] = vb;
         }
         __syncthreads();
-#pragma unroll 4
+#pragma unroll
         for (int l = 0; l < 16; ++l)
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = fma(sA[l][ty * 4 + r], sB[l][tx * 4 + c], acc[r][c]);
+          for (int k = 0; k < 4; ++k) acc[k] = fma(sA[l][r], sB[l][cx + 16 * k], acc[k]);
         __syncthreads();
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int i = ty * 4 + r, j = tx * 4 + c;
-          if (sm[i * 2 + (j >> 5)] >> (j & 31) & 1u)
-            put(C + (long long)(i0 + i) * a.ci + (long long)(t.j0 + j) * a.cj, acc[r][c]);
-        }
+      for (int k = 0; k < 4; ++k) {
+        const int c = cx + 16 * k;
+        if (sm[r * 2 + (c >> 5)] >> (c & 31) & 1u)
+          put(C + (long long)(i0 + r) * a.ci + (long long)(t.j0 + c) * a.cj, acc[k]);
+      }
     }
     __syncthreads();
   }
@@ -941,7 +948,8 @@ cudaError_t oz_multiply(cudaStream_t st, const __nv_bfloat16* pa, const __nv_bfl
   const size_t sm = (size_t)OZ_STAGES * OZ_STAGE_BYTES + 1024 + 256;
   raise_smem_limit((const void*)oz_gemm_kernel, sm);
   oz_gemm_kernel<<<grid, OZ_THREADS, sm, st>>>((const uint8_t*)pa, (const uint8_t*)pb, a);
-  oz_fma_kernel<<<(unsigned)(items < 4ll * nsm ? items : 4ll * nsm), 256, 0, st>>>(a);
+  const long long units = items * OF_UNITS;
+  oz_fma_kernel<<<(unsigned)(units < 4ll * nsm ? units : 4ll * nsm), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
