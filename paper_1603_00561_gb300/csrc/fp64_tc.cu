@@ -404,9 +404,11 @@ cudaError_t launch_ccvv_fp64_tc(dsrg_plan* p, const double* B, const double* eps
   p->launches += OZ_PACK_LAUNCHES;
   const Segment& sg = p->segs[p->seg_ccvv];
   a.pstep = p->shard_world;
-  for (int p0 = p->shard_rank; p0 < p->n_pairs; p0 += w->group * p->shard_world) {
-    const int left = (p->n_pairs - p0 + p->shard_world - 1) / p->shard_world;
-    const int n = left < w->group ? left : w->group;
+  // (64 bits: a world may be as large as an int, and group times that is not)
+  const long long world = p->shard_world;
+  for (long long q0 = p->shard_rank; q0 < p->n_pairs; q0 += w->group * world) {
+    const long long left = (p->n_pairs - q0 + world - 1) / world;
+    const int p0 = (int)q0, n = (int)(left < w->group ? left : w->group);
     a.p0 = p0;
     if ((e = oz_multiply(p->stream, w->planes, w->planes, a, n)) != cudaSuccess) return e;
     p->launches += OZ_MULTIPLY_LAUNCHES;

@@ -127,3 +127,22 @@ def test_batch_under_little_free_memory(pk):
     # 300 MB or so would not have been left by five digits' workspaces of over 130 MB
     assert free1 >= 0.5 * free0
     assert np.abs(e / np.array(ref) - 1.0).max() <= 1e-12
+
+
+@pytest.mark.parametrize("world", [20, 21, 22, 1000, 30_000_000, 100_000_000, 2 ** 31 - 1])
+def test_shards_of_a_world_with_more_ranks_than_pairs(pk, world):
+    """21 core pairs: from 21 ranks on a rank has one pair or none, however many there are."""
+    nC = 6
+    p = make_problem(nC, 0, 70, 40, s=0.5, seed=8)
+    dev = pk.to_device(p)
+    plan = pk.Plan(nC, 0, 70, 40, precision="fp64")
+    pairs = plan.pair_energies(dev[0], dev[1], p.s).cpu().numpy()
+    iu = [(i, j) for i in range(nC) for j in range(i, nC)]
+    for rank in (0, 3, 19, 20, world - 1):
+        if rank >= world:
+            continue
+        plan.set_shard(rank, world)
+        e = plan.energy(*dev, p.s).cpu().numpy()
+        plan.sync()
+        want = sum((1.0 if i == j else 2.0) * pairs[i, j] for k, (i, j) in enumerate(iu) if k % world == rank)
+        assert abs(e[0] - want) <= 1e-12 * abs(pairs).sum()
