@@ -341,7 +341,8 @@ void fp64_tc_alloc(dsrg_plan* p, size_t limit) {
   r.xri = 1;
   w->xc = (long long)z.nA * w->nVpad;
   w->ldy = w->xc + (z.nH * z.nA + 7) / 8 * 8;
-  const size_t fit = V_BYTES / per;
+  const size_t mask_1 = oz_mask_bytes(z.nV, z.nV, 1);  // whole tiles: larger than `per` for a few virtuals
+  const size_t fit = V_BYTES / (per > mask_1 ? per : mask_1);
   w->group = (int)(fit < 1 ? 1 : (fit > (size_t)p->n_pairs ? (size_t)p->n_pairs : fit));
   const size_t mask_v = oz_mask_bytes(z.nV, z.nV, w->group);
   const size_t mask_y = oz_mask_bytes(w->xrow0 + z.nH * z.nA, w->xc + z.nH * z.nA, 1);
