@@ -74,10 +74,13 @@ typedef enum {
  * Eq. (19) for diagrams F1 and F2, and the (A,A|V,V) integrals):
  *   DSRG_PREC_FP64    FP64: products as exact sums of integer digit products on
  *                     the tensor cores, rounded once (each factor row as seven
- *                     base-256 digits of its largest value, so within 2^-56 of
- *                     that; a row with an infinity in FP64 FMAs, one with a NaN
- *                     gives NaN), or FP64 FMAs on CUDA cores where the digits'
- *                     workspace would be over 2/5 of the device's memory;
+ *                     base-256 digits of its largest value). Elements for which
+ *                     the digits' error bound, 2^-56 of the rows' scales, is above
+ *                     that of a chain of FP64 FMAs, naux 2^-53 sum_Q |B_r B_c|, and
+ *                     rows with an infinity or a NaN, are formed by FP64 FMAs. So
+ *                     are all where the digits' workspace, about 16 bytes per value
+ *                     of B and a buffer of pairs, is over 2/5 of the memory free
+ *                     when the plan is made, or naux over 2^21;
  *   DSRG_PREC_TF32X3  B = hi + lo split into two TF32 planes, products
  *                     hi*hi + hi*lo + lo*hi on tcgen05 tensor cores with FP32
  *                     accumulation (and lo*lo where both operands are the
@@ -163,8 +166,8 @@ dsrg_status_t dsrg_ccvv_pair_energies(dsrg_plan_t *plan, const double *B, const 
  * deps_dev [n], ds_dev [1]. Outputs are overwritten, not accumulated. Needs a
  * plan created with DSRG_PLAN_GRAD (else DSRG_ERR_INVALID_ARG). The adjoint is
  * the derivative of the energy expression (Table 1, Table 2, Eqs. (12)-(15),
- * (23)) evaluated in FP64 for every precision mode; each core row recomputes
- * its pair integrals v^{kj} instead of storing them. dB is bit-reproducible;
+ * (23)) in the plan's precision; the pair integrals v^{ij} are recomputed, not
+ * kept from the energy. dB is bit-reproducible;
  * deps and ds are summed with FP64 atomics. */
 dsrg_status_t dsrg_mrpt2_energy_grad(dsrg_plan_t *plan, const double *B, const double *eps,
                                      const double *gamma1, const double *lambda2, double s,
@@ -336,14 +339,14 @@ dsrg_status_t dsrg_ccvv_energy_noalloc(const dsrg_sizes_t *sz, const double *B, 
  *                             large that exp(-2 s Delta^2) < 2^-63, evaluated as
  *                             1/Delta;
  *   DSRG_COUNT_CCVV_FACTORED  blocks with every |Delta| >= 1/4 of a pair whose
- *                             factorised exponentials stay in range (the energy
- *                             forms exp(-2 s Delta^2) directly, the gradient from
- *                             the factors);
+ *                             factorised exponentials would stay in range (energy
+ *                             and gradient form 1 - exp(-2 s Delta^2) directly, in
+ *                             pairs of FP32 numbers);
  *   DSRG_COUNT_CCVV_DIRECT    blocks with some |Delta| < 1/4 (or of a pair whose
- *                             factors could overflow), evaluated with expm1 per
+ *                             factors would overflow), evaluated with expm1 per
  *                             element (R(0) = 0) and the exchange combination in FP64;
  *   DSRG_COUNT_CCVV_UNFACTORABLE work items (core pair x tile pair) of pairs whose
- *                             factors could overflow;
+ *                             factors would overflow;
  *   DSRG_COUNT_CAVV_NEAR      CAVV positions (core m, e, f) with some |Delta_u| < 1/4
  *                             (or a non-factorisable (m, u)), evaluated in FP64 with
  *                             expm1;

@@ -462,7 +462,8 @@ __global__ void __launch_bounds__(256) actvv_kernel(const double* __restrict__ e
 // nA^4 products P1 += (M_xu Rv_xu)(M_yv Rt_yv), P2 += (M_xu Rv_xu)(M_vy Rt_yv).
 // F32 (split-precision plans, as actvv_gen_kernel): the regulated factors are
 // rounded to FP32 and each thread's sums over up to ACTVV_CH positions run in
-// FP32 with round-to-nearest, the chunk sums in FP64; the regulators stay FP64.
+// FP32 with round-to-nearest, the chunk sums in FP64; the regulators are pairs of FP32
+// numbers (FP64 near D = 0).
 template <int NA, bool F32>
 __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restrict__ eps, double s,
                                                           Sizes z, const double* __restrict__ M,
@@ -611,7 +612,8 @@ __global__ void __launch_bounds__(256) actvv_small_kernel(const double* __restri
 //
 // F32 (split-precision plans): the regulated factors are rounded to FP32 and each
 // 64-term chunk of the sum over (e, f) runs in FP32 on CUDA cores (round to
-// nearest), the chunk sums in FP64; the regulators themselves stay FP64.
+// nearest), the chunk sums in FP64; the regulators are pairs of FP32 numbers (FP64
+// near D = 0).
 template <int NA, bool F32>
 __global__ void __launch_bounds__(256) actvv_gen_kernel(const double* __restrict__ eps, double s,
                                                         Sizes z, const double* __restrict__ M,

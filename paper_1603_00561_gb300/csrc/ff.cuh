@@ -7,8 +7,8 @@
 // regulator in FP32 pairs is about 90 FP32 instructions, under 6 us.
 //
 // Accuracy: a pair carries 48 bits; 1/D and 1 - exp(-k D^2) below have relative
-// errors under 2^-41 (tests/test_ff.py compares them with FP64 over the range
-// of arguments), as had the FP64 form, whose 1/D came from a 20-bit
+// errors under 2^-40 (at most 2^-40.8 in tests/test_ff.py, which compares them with
+// FP64 over the range of arguments), as had the FP64 form, whose 1/D came from a 20-bit
 // seed and one Newton-Raphson step.
 //
 // The error-free sums and products are Knuth's and Dekker's (T. J. Dekker,

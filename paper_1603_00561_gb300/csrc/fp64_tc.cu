@@ -1,5 +1,6 @@
 // The FP64 plans' pair contractions on the tensor cores (oz_gemm.cu: exact integer
-// slices, error below that of FP64 FMAs) with FP64 regulators and sums.
+// slices, elements checked against the error bound of FP64 FMAs) with FP64 regulators
+// and sums.
 //
 // Plane rows as in the split plans: (h, e) for every hole h and virtual e (nVpad rows
 // per hole), then (h, x) for every hole and active particle.

@@ -1,15 +1,16 @@
 // Adjoint of the DSRG-MRPT2 energy: dE_total/dB, dE_total/deps, dE_total/ds.
 //
-// FP64 plans: all adjoint arithmetic is FP64 on CUDA cores. Pair quantities
-// are recomputed per core row rather than stored: for a fixed core orbital k
-// the kernel forms v^{kj} for every j tile by tile and keeps only
-// W^{kj} = dE/dv^{kj}, which a GEMM turns into dB.
+// FP64 plans: regulators and sums are FP64 on CUDA cores, products digit products on the
+// tensor cores (oz_gemm.cu) or FP64 FMAs. Pair quantities are recomputed rather than
+// stored: v^{ij} of every pair as digit products, or, where W of all rows does not fit,
+// on a shard or without the digits' workspace, v^{kj} of one core row k after another;
+// W^{kj} = dE/dv^{kj} is kept, which a GEMM turns into dB.
 // Split-precision plans: the CCVV pair blocks are recomputed on the tensor
 // cores by the CCVV kernel's adjoint epilogue (tc_split.cu), the CAVV / CCAV
 // integrals X, Z in FP32 (round to nearest) on CUDA cores; the adjoints of all
 // integrals then form one symmetric matrix S and one tensor-core GEMM turns it
-// into dB (tc_adjoint.cu). Regulators, their derivatives and every epilogue
-// stay FP64. dB is assembled with one thread per element (fixed order,
+// into dB (tc_adjoint.cu). The regulators of F1 and F2, their derivatives and the sums of
+// deps and ds are pairs of FP32 numbers away from D = 0 (ff.cuh), all others FP64. dB is assembled with one thread per element (fixed order,
 // bit-reproducible); deps and ds use FP64 atomics.
 //
 // Derivatives (closed-shell spin-adapted forms of Table 2, Eqs. (12)-(15), (23)):

@@ -17,9 +17,10 @@
 //     columns XC + h*nA + x ->  (ge|hx): Z_u[m,n,e] = (me|nu) of F3, and the
 //                               virtual parts of (ia|ux), (ix|ua)
 // (Sec. III step 4: the integrals with active indices are formed explicitly,
-// then contracted). FP64 kernels then evaluate the F2 and F3 energies with
-// FP64 regulators, and gather the active-block integrals; (hx|h'y), which
-// has no virtual index, is formed in FP64 from B directly.
+// then contracted). CUDA-core kernels then evaluate the F2 and F3 energies, with
+// regulators and sums in pairs of FP32 numbers away from D = 0 and in FP64 near it, and
+// gather the active-block integrals; (hx|h'y), which has no virtual index, is
+// formed in FP64 from B directly.
 //
 // The GEMM kernel (one CTA per SM, persistent, tiles 128 x 256):
 //   warp 0      TMA producer (the whole warp runs the loop, an elected lane issues)
@@ -343,8 +344,8 @@ __global__ void xx_gram_kernel(const double* __restrict__ Xq, int T, int Q, doub
 // One CTA per (m, 32 x 32 tile pair E <= F); for E < F each position (e,f) also
 // adds its mirror (f,e), whose X_u[f,e] is the same CTA's transposed tile.
 // Away from D = 0 the regulators and sums are pairs of FP32 numbers (ff.cuh);
-// |D_u| < 1/4 (or a pair whose factored exponentials could overflow, which the
-// gradient's kernels share) takes expm1 and an FP64 divide.
+// |D_u| < 1/4 (or a pair without the flag of pair_info_kernel) takes expm1 and an FP64
+// divide.
 //
 // Bound by FP32 issue: about 120 FP32 instructions per position and active orbital.
 // cc-pV5Z size (24/2/1214/3400): 386 us; with the FP64 regulator from factor tables

@@ -1,5 +1,5 @@
 // Split-precision CCVV (diagram F1, Eq. (23)) on the 5th-generation tensor
-// cores: TMA -> shared memory -> tcgen05.mma -> TMEM -> FP64 epilogue.
+// cores: TMA -> shared memory -> tcgen05.mma -> TMEM -> epilogue in FP32 pairs.
 //
 // The DF factors of the core x virtual block are split once per call into
 // two planes, B = hi + lo (TF32 or BF16), laid out K-major (K = the auxiliary
@@ -13,14 +13,13 @@
 // its bias would otherwise be set by the largest partial sums. Then it adds
 //     w * sum_ab (x^2 - x y + y^2) R_ab,   R = (1 - exp(-2 s D^2)) / D,
 // D = e_i + e_j - e_a - e_b, w = (2 if i<j) * (2 if A<B); for i = j only x is
-// formed (y = x). The energy's regulator and sums are pairs of FP32 numbers
-// (48 bits, ff.cuh): the FP64 pipe, 2 FMAs per SM and clock, took longer for the
-// regulators of an item than the tensor cores for its products. Positions with
-// |D| < 1/4 (never the case for core -> virtual excitations of a normal spectrum)
-// take expm1 and the exchange combination in FP64 instead. The adjoint's regulators
-// are FP64: exp(-2 s D^2) is the product of four exponentials (one per pair, one
-// per row, one per column, one pair-independent table), 1/D a seed refined by one
-// Newton-Raphson step.
+// formed (y = x). Regulators and sums of the energy and of the adjoint are pairs of
+// FP32 numbers (48 bits, ff.cuh): the FP64 pipe, 2 FMAs per SM and clock, took longer for
+// the regulators of an item than the tensor cores for its products. The energies' errors
+// against 64 bits are those of the FP64 epilogue (the split products set them). Positions
+// with |D| < 1/4 (never the case for core -> virtual excitations of a normal spectrum)
+// take expm1 and the exchange combination in FP64 instead; so does the adjoint's R where
+// the pair does not settle its rounding to FP32 (adjoint_chunk).
 //
 // Measured on one GB300 (this kernel alone, BF16x3): cc-pVTZ size (24/2/372/1200)
 // 855 us with the FP64 regulator and row-per-lane tail sums, 475 us with FP32 pairs,
@@ -272,7 +271,7 @@ __device__ __forceinline__ void store_split16(uint16_t* hi, uint16_t* lo, long l
 //
 // The regulators and sums are FP32 pairs (ff.cuh), P and Q FP32 with R rounded once, as
 // S keeps 16 bits of them. A last bit of R that differs moves a few of the 16-bit tails:
-// where the pair (relative error under 2^-41) is so close to the middle of two FP32
+// where the pair (relative error under 2^-40) is so close to the middle of two FP32
 // numbers that it does not settle the rounding, R is taken in FP64 (one element in 2^14).
 // 1536 us for the kernel at 24/2/372/1200 with FP64 regulators, 944 us now; what is left
 // above the energy kernel's 454 us is the row-per-lane tail sums and the stores of S.
@@ -968,9 +967,11 @@ __global__ void __launch_bounds__(256) split_planes_kernel(const double* __restr
 
 // E_mu of the orbital pairs mu and whether exp(-c D^2) factorises: with
 // D = E - e_a - e_b, whether the partial products of exp(-c E^2) exp(2 c E e_a)
-// exp(2 c E e_b) exp(-c (e_a + e_b)^2) stay within exp(+-700) (past that the regulators
-// take expm1). One CTA and launch: the largest |e_v| first, then the pairs, of `pairs`
-// or (m, u) = (mu / nA, nC + mu % nA).
+// exp(2 c E e_b) exp(-c (e_a + e_b)^2) stay within exp(+-700). No kernel forms these factors
+// any more (ff_one_minus_exp takes any c D^2): the flag is what the *_UNFACTORABLE
+// counters of dsrg_plan_branch_counts are defined by, and pairs without it keep the FP64
+// path that these and the DIRECT and NEAR counters stand for. One CTA and launch: the
+// largest |e_v| first, then the pairs, of `pairs` or (m, u) = (mu / nA, nC + mu % nA).
 __global__ void __launch_bounds__(1024) pair_info_kernel(const double* __restrict__ eps, double c,
                                                          Sizes z, const int2* __restrict__ pairs,
                                                          int n, double2* __restrict__ pinfo) {
@@ -985,8 +986,8 @@ __global__ void __launch_bounds__(1024) pair_info_kernel(const double* __restric
   for (int mu = threadIdx.x; mu < n; mu += 1024) {
     const int2 ij = pairs ? pairs[mu] : make_int2(mu / z.nA, z.nC + mu % z.nA);
     const double E = eps[ij.x] + eps[ij.y];
-    // the factors multiply left to right: for E e > 0 the partial products grow past each
-    // single factor's exponent, so the sum of their magnitudes is bounded
+    // (multiplied left to right: for E e > 0 the partial products grow past each single
+    // factor's exponent, so the sum of their magnitudes is bounded)
     const bool ok = (c * E * E + 4.0 * c * fabs(E) * m <= 700.0) && (4.0 * c * m * m <= 700.0);
     pinfo[mu] = make_double2(E, ok ? 1.0 : 0.0);
   }
