@@ -966,9 +966,11 @@ size_t oz_work_bytes(long long M, long long N, long long K, long long nb, bool s
   return (cap > one ? cap : (one < 4 * OZ_WS_CAP ? one : 4 * OZ_WS_CAP)) + 4096;
 }
 
-// The tensor-core form costs about six launches and the slicing, about 120 us for the
-// smallest products; the FP64 pipe does 1.1 TFLOP/s on tiles that fill the chip. At 1e8
-// operations the two are about even (58 MFLOP: 120 us against 60).
+// The tensor-core form is seven launches, 100 to 130 us for the smallest products; the FP64
+// pipe does 1.1 TFLOP/s on tiles that fill the chip, and less on others. Whole DF calls whose
+// last product alone is past the line, digits against FMAs: 1128 / 1090 us at 1.0e8 operations,
+// 1488 / 1500 at 1.8e8, 1811 / 1884 at 2.4e8; with three products of 1.1e8 to 2.2e8 of
+// which two have a side of 8: 1038 / 2619 us. So the line lies where full tiles lose 40 us.
 static bool oz_worthwhile(double flops) { return flops >= 1e8; }
 
 cudaError_t launch_gemm(cudaStream_t st, const GemmArgs& g0, const OzWork& w, int* launches) {
