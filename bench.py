@@ -49,16 +49,16 @@ FP64_PRODUCTS = 34  # BF16 digit products of one FP64 product (csrc/oz_gemm.cu)
 # keyed by (workload, precision, item order); summaries under profiles/. Any
 # other combination, or a kernel changed since the capture, reports null.
 TRAFFIC = {
-    # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch of the current CCVV kernel,
-    # whole tiles without prefetch (profiles/ccvv_dram_per_order_naphthyne-v5z-1240.md); other
-    # codes report null
-    ("naphthyne-v5z-1240", "bf16x3", 0): 18808265472 + 3898368,
-    ("naphthyne-v5z-1240", "bf16x3", 4): 9346629376 + 3872768,
-    ("naphthyne-v5z-1240", "bf16x3", 8): 14072587776 + 3752960,
-    ("naphthyne-v5z-1240", "bf16x3", 16): 19147768320 + 3742464,
-    ("naphthyne-v5z-1240", "bf16x3", 9): 15875443200 + 3923712,
-    ("naphthyne-v5z-1240", "bf16x3", 17): 14867894528 + 3962880,
-    ("naphthyne-v5z-1240", "bf16x3", 128): 20477330176 + 3740928,
+    # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch of the CCVV kernel with
+    # the FP32-pair epilogue and MMA blocks, whole tiles without prefetch
+    # (profiles/ccvv_dram_per_order_naphthyne-v5z-1240.md); other codes report null
+    ("naphthyne-v5z-1240", "bf16x3", 0): 16910911488 + 3521792,
+    ("naphthyne-v5z-1240", "bf16x3", 4): 20112961792 + 3554304,
+    ("naphthyne-v5z-1240", "bf16x3", 8): 16465344000 + 3780864,
+    ("naphthyne-v5z-1240", "bf16x3", 16): 21923124736 + 3529472,
+    ("naphthyne-v5z-1240", "bf16x3", 9): 18030274816 + 3641088,
+    ("naphthyne-v5z-1240", "bf16x3", 17): 18581475840 + 3993344,
+    ("naphthyne-v5z-1240", "bf16x3", 128): 22056651264 + 3974912,
 }
 
 

@@ -12,7 +12,7 @@
 //
 // The FP64 CUDA-core kernels these replace ran at the FP64 pipe's rate: 101.6 ms for
 // CCVV and 16 ms for CAVV at the cc-pVTZ size (24/2/372/1200); here 4.7 ms (products 3.3,
-// regulators 1.4) and 0.35 ms, and 0.64 ms for the product of the rest. Regulators beside
+// their check 0.1, regulators 1.4) and 0.35 ms, and 0.65 ms for the product of the rest. Regulators beside
 // the next group's product would need registers that its kernel leaves no room for.
 // The regulators are what is left on that pipe: about 25 FP64 instructions each.
 #include <new>

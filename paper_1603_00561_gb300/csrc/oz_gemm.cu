@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // ------------------------------- the check -------------------------------
 // S of every element (see the head of the file) in one FP32 accumulation over all of K, and
 // its mask bit. One BF16 product against the 34 of the slices, bound by its operands' copies
-// and the epilogue: 4 stages of up to 128 K values. 36 us beside 780 us for the products of
+// and the epilogue: 4 stages of up to 128 K values. 33 us beside 780 us for the products of
 // 86 pairs at 24/2/372/1200, 17 beside 190 us (K = 398) in the DF transform.
 constexpr int OC_KB = 4;  // blocks of 32 K values per stage
 constexpr int OC_STAGES = 4;
