@@ -24,8 +24,8 @@
 // So every element is checked: an extra product of the leading eight bits of the magnitudes
 // gives S from below (oz_check_kernel), and elements with 8 K S < sum x + sum y + K / 50 are
 // formed by FP64 FMAs (oz_fma_kernel). So are those of rows with a NaN or an infinity, which
-// have no scale. S = 0 is exact (no K index has both factors). The bound is then no
-// larger than that of the FMA chain for any element of any input. On N(0, 1) e^{-0.02 Q}
+// have no scale. S = 0 is exact (no K index has both factors). Up to the rounding to
+// FP64 the bound is then no larger than that of the FMA chain, for any element of any input. On N(0, 1) e^{-0.02 Q}
 // factors no element fails the check, on the products of the Fock and DF steps 1e-3 and
 // fewer; with an unnormalised auxiliary basis (metric diagonal over 1e11) 9 in 10 of the
 // product with the inverse factor do, and it runs at the FP64 pipe's rate.

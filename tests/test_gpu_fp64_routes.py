@@ -146,3 +146,22 @@ def test_shards_of_a_world_with_more_ranks_than_pairs(pk, world):
         plan.sync()
         want = sum((1.0 if i == j else 2.0) * pairs[i, j] for k, (i, j) in enumerate(iu) if k % world == rank)
         assert abs(e[0] - want) <= 1e-12 * abs(pairs).sum()
+
+
+@pytest.mark.parametrize("sizes", [(1, 1, 3, 5), (3, 3, 33, 20), (2, 5, 17, 9), (2, 8, 40, 30), (5, 0, 65, 17)])
+def test_plan_without_digits(pk, monkeypatch, sizes):
+    """The CUDA-core kernels for every kind of active space, with the inputs of the full Table 1:
+    the plan of the first allocation count that suffices."""
+    p = make_problem(*sizes, s=0.6, seed=11, with_lambda3=sizes[1] > 0, with_f1=True)
+    for k in range(80):
+        monkeypatch.setenv("DSRG_FAIL_ALLOC_AFTER", str(k))
+        try:
+            plan = pk.Plan(*sizes, precision="fp64", grad=True)
+            break
+        except pk.DSRGError:
+            continue
+    monkeypatch.delenv("DSRG_FAIL_ALLOC_AFTER")
+    full = pk.Plan(*sizes, precision="fp64", grad=True)
+    assert plan.workspace_bytes() < full.workspace_bytes()
+    assert _gradient_errors(plan, pk, p) <= 1e-10
+    assert _gradient_errors(full, pk, p) <= 1e-10
